@@ -165,7 +165,7 @@ size_t split_grad_layout(const fq_plan* p, void* base, SplitGradWs* out) {
   w.nslots = s * L + 1;
   w.bstride = (size_t)w.np * w.np;
   w.astride = (size_t)w.ncp * w.kp;
-  const int bn = p->tile_n == 128 ? 128 : 64;
+  const int bn = fq_split_shape(p).n == 128 ? 128 : 64;
   w.ncta = (w.np / bn) * (w.ncp / BM);
   char* b = (char*)base;
   size_t off = 0;
@@ -403,7 +403,7 @@ fq_status fq_grad_split(fq_plan* p, const double* d_f, const void* d_W, double* 
   r.s = s;
   split_grad_layout(p, d_ws, &r.w);
   SplitGradWs& w = r.w;
-  r.c = GemmCtx{p->n, w.np, w.kp, w.ncp, w.ns, p->tile_n == 128 ? 128 : 64, w.bstride, w.astride};
+  r.c = GemmCtx{p->n, w.np, w.kp, w.ncp, w.ns, fq_split_shape(p).n == 128 ? 128 : 64, w.bstride, w.astride};
   const int n = p->n, M = p->steps, L = p->L, S = p->stride;
   const size_t plane_bytes = sizeof(float) * (size_t)n * w.ldm;
 

@@ -74,6 +74,21 @@ __global__ void k_split_omega6(Omega6Split a, __nv_bfloat16* os, __nv_bfloat16* 
 // ------------------------------------------------------------------------- orchestration
 static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Largest N whose default tile is 64 wide, for BF16X3 and BF16X6: up to there the 128-wide tiles of a
+// product are at most one wave (144 and 121 tiles on 152 SMs), and twice as many narrow ones fill the
+// chip better.  A product in us with 64- / 128-wide tiles: BF16X3 N = 400 18 / 29, 1000 28 / 48, 1536
+// 61 / 70, 2048 136 / 127; BF16X6 N = 1000 45 / 76, 1300 82 / 99, 1536 117 / 112.  The rule looks at N
+// alone, so that a block of columns and the whole U_T take the same tiles and agree bit for bit.
+constexpr int SPLIT_NARROW_MAX_N_X3 = 1536;
+constexpr int SPLIT_NARROW_MAX_N_X6 = 1408;
+
+// Tile shape of a split plan: its own (chosen by the caller or by floquet_autotune), or by size.
+fq_tile_shape fq_split_shape(const fq_plan* p) {
+  const int narrow = p->precision == FQ_BF16X6 ? SPLIT_NARROW_MAX_N_X6 : SPLIT_NARROW_MAX_N_X3;
+  if (p->tile_auto && p->n <= narrow) return fq_tile_shape{64, p->tile_k};
+  return fq_tile_shape{p->tile_n, p->tile_k};
+}
+
 size_t fq_split_workspace(const fq_plan* p, int nc, void* base, void* out) {
   const int NS = p->precision == FQ_BF16X6 ? 3 : 2;
   SplitWs w{};
@@ -238,12 +253,13 @@ fq_status fq_split_propagate(fq_plan* p, const double* x0, double* x, int nc, in
                              int transpose_out, void* ws, cudaStream_t s) {
   // (slices, tile width, K per stage): 64-byte swizzle stages where 128-byte ones would not fit
   // more than two stages in shared memory
-  const bool wide = p->tile_n == 128;
+  const fq_tile_shape shape = fq_split_shape(p);
+  const bool wide = shape.n == 128;
   if (p->precision == FQ_BF16X6)
     return wide ? run_split<3, 128, 32>(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s)
                 : run_split<3, 64, 32>(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s);
   if (wide) return run_split<2, 128, 32>(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s);
-  return p->tile_k == 32 ? run_split<2, 64, 32>(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s)
+  return shape.k == 32 ? run_split<2, 64, 32>(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s)
                          : run_split<2, 64, 64>(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s);
 }
 
@@ -273,6 +289,8 @@ static fq_status floquet_autotune_body(fq_plan* p, void* ws, size_t bytes, void*
   float best = 1e30f;
   Shape pick = cand[0];
   const Shape before{p->tile_n, p->tile_k};
+  const bool auto_before = p->tile_auto;
+  p->tile_auto = false;
   cudaEvent_t a = nullptr, b = nullptr;
   cudaError_t e = cudaEventCreate(&a);
   if (e == cudaSuccess) e = cudaEventCreate(&b);
@@ -302,6 +320,7 @@ static fq_status floquet_autotune_body(fq_plan* p, void* ws, size_t bytes, void*
   if (b) cudaEventDestroy(b);
   p->tile_n = st == FQ_OK ? pick.n : before.n;  // on failure the plan keeps the shape it had
   p->tile_k = st == FQ_OK ? pick.k : before.k;
+  if (st != FQ_OK) p->tile_auto = auto_before;
   if (st == FQ_OK && tile_n) *tile_n = pick.n;
   return st;
 }

@@ -40,6 +40,11 @@ struct fq_ktimer {
   cudaError_t err = cudaSuccess;  // first failure since the last read
 };
 
+// Output tile width and K elements a stage (0: the width's default) of a split plan's products.
+struct fq_tile_shape {
+  int n, k;
+};
+
 struct fq_plan {
   // problem
   int n = 0, steps = 0, format = 0, precision = 0, drive_kind = 0, stride = 16, L = 0;
@@ -67,6 +72,7 @@ struct fq_plan {
   std::vector<double> band6;
   double* d_cm = nullptr;      // K0 .. KK1: 8 matrices n*n after d_k (= K)
   int tile_n = 128;          // split path: output tile width of the tensor-core kernel (autotuned)
+  bool tile_auto = false;    // neither the caller nor floquet_autotune chose it: fq_split_shape decides
   int tile_k = 0;            // split path, 64-wide BF16X3 tiles: K elements a stage (32 or 64; 0 = 64)
   int device = 0;
   // device copies (owned by the plan)
@@ -237,6 +243,7 @@ fq_status fq_ozaki_propagate(fq_plan* p, const double* x0, double* x, int nc, in
                              int transpose_out, void* ws, cudaStream_t s);
 // split-precision dense path (dense_split.cu)
 size_t fq_split_workspace(const fq_plan* p, int nc, void* base, void* out);
+fq_tile_shape fq_split_shape(const fq_plan* p);
 // batched scan as one persistent launch (scan.cu): whether the plans qualify, the bytes it needs
 // beyond the plans' own workspaces, and the graph (counter reset + the launch) writing d_U[i];
 // plan i's workspace at ws + off[i], the scan's region at ws + extra_off

@@ -531,6 +531,7 @@ fq_status fq_host_plan(const fq_problem* p, fq_plan* plan, bool defer_dense_boun
     return FQ_EINVAL;
   }
   plan->tile_n = p->tile_n ? p->tile_n : 128;
+  plan->tile_auto = p->tile_n == 0;
   if (p->tile_k != 0 && p->tile_k != 32 && p->tile_k != 64) {
     fq_set_error("tile_k must be 0, 32 or 64 (got %d)", p->tile_k);
     return FQ_EINVAL;

@@ -13,14 +13,14 @@
 // CTAs take units from a device counter, so cheap and costly instances balance.  Units are taken in
 // increasing order and each waits only on earlier ones, so the scan always advances, whether or not
 // every CTA is resident.  In each CTA a TMA producer thread takes the units and hands them through
-// a ring of SCAN_RING slots in shared memory to the MMA thread, four epilogue warps and four
+// a ring of SCAN_RING slots in shared memory to the MMA thread, eight epilogue warps and four
 // builder warps.  The term units run as in k_split_chain (two accumulator buffers in tensor memory,
 // the epilogue of one tile overlapping the MMAs of the next); the builder warps do the B and W
 // units beside them, so that their memory latency stays off the tensor cores' path.
 // Dependencies (monotonic counters in global memory, bounded acquire spins):
 //   T(i, m, p, tile of state block tj): every B(i, m, *) done (a counter per buffer parity: Omega~_m
 //     lives in buffer m & 1), and term p - 1 of step m (term L - 1 of step m - 1 when p = 0) done on
-//     state block tj (its four epilogue warps per tile, counted per (i, p, tj) across the steps);
+//     state block tj (its epilogue warps, EPI_WARPS per tile, counted per (i, p, tj) across the steps);
 //   B(i, m, *), m >= 2: step m - 2 done on every state block (its buffer has been read);
 //   W(i, b): step M - 1 done on the state block of its 16 states.
 // The arithmetic of every unit is that of the one-instance path (dense_split.cu) with the same tile
@@ -36,7 +36,8 @@ namespace {
 
 constexpr int SCAN_MAXL = 32;    // Chebyshev terms per step an instance may have
 constexpr int SCAN_RING = 8;     // units handed from the producer to the MMA thread and the warps
-constexpr int SCAN_THREADS = 320;  // producer, MMA, four epilogue warps, four builder warps
+constexpr int SCAN_BUILDERS = 4;  // warps of the B and W units
+constexpr int SCAN_THREADS = PTHREADS + 32 * SCAN_BUILDERS;  // producer, MMA, epilogue warps, builder warps
 constexpr int BLOCK_ROWS = 16;   // rows of a B or W unit
 constexpr int SCAN_TAIL = 512;   // barriers, tensor-memory slot, abort flag and ring after the stages
 
@@ -266,7 +267,8 @@ __device__ void scan_store_rows(const ScanInst& I, int j0, int tid) {
 template <int NS, int BN, int BKE>
 struct ScanCfg {
   using Split = SplitCfg<NS, BN, BKE, true>;
-  static constexpr size_t SMEM = (size_t)Split::STAGES * Split::STAGE_BYTES + 1024 + SCAN_TAIL;
+  static constexpr size_t SMEM = (size_t)Split::STAGES * Split::STAGE_BYTES + 1024 + SCAN_TAIL + EPI_WARPS * EPI_STAGE_BYTES;
+  static_assert(SMEM <= 232448, "shared memory of one CTA");
 };
 
 template <int NS, int BN, int BKE>
@@ -274,7 +276,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
   using Cfg = SplitCfg<NS, BN, BKE, true>;
   constexpr int STAGES = Cfg::STAGES;
   constexpr int R = SCAN_RING;
-  constexpr uint32_t BUF_COLS = 2 * BN;
+  constexpr uint32_t BUF_COLS = Cfg::ACC_COLS;
   constexpr uint32_t TMEM_COLS = 2 * BUF_COLS;
   static_assert((2 * STAGES + 5 + 2 * R) * 8 + 8 + R * 5 * 4 <= SCAN_TAIL, "shared tail");
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -298,12 +300,12 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull0 + 8 * b, 1);
-      mbar_init(tempty0 + 8 * b, 4);
+      mbar_init(tempty0 + 8 * b, EPI_WARPS);
     }
     mbar_init(done, 1);
     for (int s = 0; s < R; ++s) {
       mbar_init(ufull0 + 8 * s, 1);
-      mbar_init(uempty0 + 8 * s, 9);  // the MMA thread, the four epilogue and the four builder warps
+      mbar_init(uempty0 + 8 * s, 1 + EPI_WARPS + SCAN_BUILDERS);  // MMA thread, epilogue and builder warps
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -350,12 +352,12 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
         if (d.type != SU_TERM) continue;
         const ScanInst& I = a.inst[d.inst];
         const int tj = d.t / I.tiles_i, j0 = tj * BM, i0 = (d.t - tj * I.tiles_i) * BN;
-        ok = scan_wait(I.omegacnt + (d.m & 1), 4u * I.nblk * (unsigned)(d.m / 2 + 1), a.abort);
+        const unsigned per_term = (unsigned)EPI_WARPS * I.tiles_i;  // counts of one term in a state block
+        ok = scan_wait(I.omegacnt + (d.m & 1), (unsigned)SCAN_BUILDERS * I.nblk * (unsigned)(d.m / 2 + 1), a.abort);
         if (ok && d.p > 0)
-          ok = scan_wait(I.termcnt + (size_t)(d.p - 1) * I.tiles_j + tj, 4u * I.tiles_i * (unsigned)(d.m + 1),
-                         a.abort);
+          ok = scan_wait(I.termcnt + (size_t)(d.p - 1) * I.tiles_j + tj, per_term * (unsigned)(d.m + 1), a.abort);
         if (ok && d.p == 0 && d.m > 0)
-          ok = scan_wait(I.termcnt + (size_t)(I.L - 1) * I.tiles_j + tj, 4u * I.tiles_i * (unsigned)d.m, a.abort);
+          ok = scan_wait(I.termcnt + (size_t)(I.L - 1) * I.tiles_j + tj, per_term * (unsigned)d.m, a.abort);
         if (!ok) break;
         fence_proxy_async_global();  // the epilogues' generic stores, before this thread's TMA reads
         const int av = ((d.m * (I.L & 1)) & 1) ^ (d.p & 1);
@@ -375,13 +377,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
           const uint32_t bar = full0 + 8 * s;
           mbar_expect_tx(bar, Cfg::STAGE_BYTES);
           const int kx = kb * BKE;
-#pragma unroll
-          for (int q = 0; q < NS; ++q) {
-            tma_load_2d(st + q * Cfg::A_BYTES, &la[q], bar, kx, j0);
-            tma_load_2d(st + (NS + q) * Cfg::A_BYTES, &la[q], bar, I.np + kx, j0);
-            tma_load_2d(st + 2 * NS * Cfg::A_BYTES + q * Cfg::B_BYTES, &ros[q], bar, kx, i0);
-            tma_load_2d(st + 2 * NS * Cfg::A_BYTES + (NS + q) * Cfg::B_BYTES, &roa[q], bar, kx, i0);
-          }
+          split_load_stage<NS, BN, BKE, true>(st, bar, la, ros, roa, kx, I.np, j0, i0);
           ++g;
         }
         if (!ok) break;
@@ -392,9 +388,6 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
     }
   } else if (warp == 1) {
     if (lane == 0) {  // ---------------- MMA issuer (as k_split_chain)
-      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                                 ((uint32_t)(BM >> 4) << 24);
-      constexpr uint32_t idesc_neg = idesc | (1u << 13);
       int g = 0, k = 0;
       bool ok = true;
       for (int i = 0;; ++i) {
@@ -413,23 +406,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
           if (!(ok = mbar_wait_or(full0 + 8 * s, (g / STAGES) & 1, abort_flag))) break;
           tc_fence_after();
           const uint32_t st = base + s * Cfg::STAGE_BYTES;
-#pragma unroll
-          for (int pp = 0; pp < Pairs<NS>::N; ++pp) {
-            const uint32_t pr = st + Pairs<NS>::a(pp) * Cfg::A_BYTES;
-            const uint32_t pi = st + (NS + Pairs<NS>::a(pp)) * Cfg::A_BYTES;
-            const uint32_t os = st + 2 * NS * Cfg::A_BYTES + Pairs<NS>::b(pp) * Cfg::B_BYTES;
-            const uint32_t oa = st + 2 * NS * Cfg::A_BYTES + (NS + Pairs<NS>::b(pp)) * Cfg::B_BYTES;
-#pragma unroll
-            for (int kk = 0; kk < BKE / 16; ++kk) {
-              const uint32_t first = (kb == 0 && pp == 0 && kk == 0) ? 0u : 1u;
-              const uint64_t dpr = smem_desc<Cfg::ROWB>(pr + 32 * kk), dpi = smem_desc<Cfg::ROWB>(pi + 32 * kk);
-              const uint64_t dos = smem_desc<Cfg::ROWB>(os + 32 * kk), doa = smem_desc<Cfg::ROWB>(oa + 32 * kk);
-              mma_bf16(acc, dpr, dos, idesc, first);
-              mma_bf16(acc, dpi, doa, idesc_neg, 1u);
-              mma_bf16(acc + BN, dpr, doa, idesc, first);
-              mma_bf16(acc + BN, dpi, dos, idesc, 1u);
-            }
-          }
+          split_issue_stage<NS, BN, BKE, true>(acc, st, kb == 0);
           mma_commit(empty0 + 8 * s);
         }
         if (!ok) break;
@@ -440,8 +417,10 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
       mma_commit(done);  // every MMA issued above has completed once this arrives
       mbar_wait(done, 0);
     }
-  } else if (warp < 6) {  // ---------------- epilogue warps 2-5: the term units' epilogues
+  } else if (warp < 2 + EPI_WARPS) {  // ---------------- epilogue warps: the term units' epilogues
     const int quarter = warp & 3;
+    float* stage =
+        reinterpret_cast<float*>(gbase + STAGES * Cfg::STAGE_BYTES + SCAN_TAIL + (warp - 2) * EPI_STAGE_BYTES);
     bool ok = true;
     int k = 0;
     for (int i = 0;; ++i) {
@@ -474,26 +453,23 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
       else ld_acquire_u32(I.omegacnt);  // the initial masters, written by the prologue's B units
       SplitEpi e;
       scan_epi(I, d.m, d.p, e);
-      const int j = j0 + quarter * 32 + lane;
       const uint32_t trow = tmem + (uint32_t)b * BUF_COLS + ((uint32_t)(quarter * 32) << 16);
       bool bad = false;
       double dsr = 0.0, dsi = 0.0;
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 16) {
-        float yr[16], yi[16];
-        tmem_ld16(trow + c0, yr);
-        tmem_ld16(trow + BN + c0, yi);
-        tmem_wait_ld();
-        const int ib = i0 + c0;
-        if (j >= e.nc || ib >= e.n) continue;
-        epi_chunk<NS, EPI_FWD>(e, yr, yi, j, ib, bad, dsr, dsi);
+      for (int c0 = epi_begin<BN>(warp), c1 = c0 + BN * 4 / EPI_WARPS; c0 < c1; c0 += 32) {
+        float yr[32], yi[32];
+        split_load_y<NS, BN, BKE, true>(trow, c0, stage, lane, yr, yi);
+        if (c0 + 32 >= c1) {  // this warp's sums are read: the buffer's next MMAs may start
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tempty0 + 8 * b);
+        }
+        if (i0 + c0 < e.n) epi_block<NS, EPI_FWD, 2>(e, yr, yi, j0 + quarter * 32, i0 + c0, lane, bad, dsr, dsi);
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tempty0 + 8 * b);
       if (bad) atomicOr(I.status, FQ_BIT_BOUND);
       // this warp's stores of the tile made visible (to the async proxy too), then one release per
-      // warp: a state block is done when the four epilogue warps of each of its tiles have counted
+      // warp: a state block is done when the epilogue warps of each of its tiles have counted
       fence_proxy_async_global();
       __threadfence();
       __syncwarp();
@@ -501,8 +477,8 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
       ++k;
     }
     if (!ok) fail();
-  } else {  // ---------------- builder warps 6-9: the B and W units
-    const int tid = threadIdx.x - 192;
+  } else {  // ---------------- builder warps: the B and W units
+    const int tid = threadIdx.x - PTHREADS;
     bool ok = true;
     for (int i = 0;; ++i) {
       const int slot = i % R;
@@ -522,7 +498,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
         if (d.m >= 2) {  // buffer m & 1 was read by step m - 2: wait until it has finished everywhere
           bool w = true;
           for (int tj = lane; tj < I.tiles_j && w; tj += 32)
-            w = scan_wait(I.termcnt + (size_t)(I.L - 1) * I.tiles_j + tj, 4u * I.tiles_i * (unsigned)(d.m - 1),
+            w = scan_wait(I.termcnt + (size_t)(I.L - 1) * I.tiles_j + tj, (unsigned)EPI_WARPS * I.tiles_i * (unsigned)(d.m - 1),
                           a.abort);
           if (!__all_sync(0xffffffffu, w)) {
             ok = false;
@@ -539,7 +515,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
       if (d.type == SU_STORE) {
         const int j0 = d.t * BLOCK_ROWS;
         if (!__all_sync(0xffffffffu, scan_wait(I.termcnt + (size_t)(I.L - 1) * I.tiles_j + j0 / BM,
-                                                4u * I.tiles_i * (unsigned)I.steps, a.abort))) {
+                                                (unsigned)EPI_WARPS * I.tiles_i * (unsigned)I.steps, a.abort))) {
           ok = false;
           break;
         }

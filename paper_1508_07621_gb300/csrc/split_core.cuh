@@ -4,16 +4,16 @@
 // One product on a block of state rows: Y^T = Psi^T Omega~^T with Omega~ = S + i A (S real
 // symmetric, A real antisymmetric), i.e. with X.B := sum_k X[j][k] B[i][k]
 //   Yr = Psi_r.S - Psi_i.A,   Yi = Psi_r.A + Psi_i.S       (HAS_A; A = 0 drops two streams).
-// Each K stage loads the Psi_r, Psi_i tiles and one S (and one A) tile, and four MMA streams
-// (the minus sign through the instruction's negate-A bit) use every tile twice.  Every operand
+// Each K stage loads the Psi_r, Psi_i tiles and one S (and one A) tile, and every tile is used twice
+// (split_issue_stage).  Every operand
 // is held as NS BF16 slices (x = x_0 + x_1 + ..., x_s = bf16 of the remainder), and the products
 // x_a y_b with a + b < NS (3 for NS = 2, 6 for NS = 3) are summed in FP32 in tensor memory.
-// The epilogue (epi_chunk) is one of: the Chebyshev term (recurrence psi_{l+1} = -2i Y +
+// The epilogue (epi_block) is one of: the Chebyshev term (recurrence psi_{l+1} = -2i Y +
 // psi_{l-1}, Bessel accumulation and step phase on FP32 masters, Eqs. 10 and 12), the adjoint
 // term, or the gradient dot; the first two also write the next product's slices.
 //
 // k_split_term: one 128-row x BN-column tile per CTA of 128 threads.  k_split_persist: one CTA
-// per SM walks its tiles with a dedicated TMA warp, MMA warp and four epilogue warps, and two
+// per SM walks its tiles with a dedicated TMA warp, MMA warp and eight epilogue warps, and two
 // tensor-memory buffers so that a tile's epilogue overlaps the next tile's MMAs.  Tiles are
 // rasterized in groups of 8 row blocks so that co-running CTAs share operands in L2.  TMA loads
 // are K-major with 128- or 64-byte swizzle; stages and buffers are handed over by mbarriers.
@@ -37,6 +37,10 @@ namespace {
 constexpr int BM = 128;      // state rows per tile (tcgen05 M)
 constexpr int NTHREADS = 128;
 constexpr int RASTER_GROUP = 8;
+// Epilogue warps of the persistent kernels: two per tensor-memory lane quarter, each taking half of
+// the tile's columns, with a transposing stage (epi_transpose) of its own.
+constexpr int EPI_WARPS = 8;
+constexpr int EPI_STAGE_BYTES = 4096;
 constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz
 
 // ------------------------------------------------------------------------- PTX wrappers
@@ -240,10 +244,78 @@ struct SplitCfg {
   static constexpr int A_BYTES = BM * ROWB;           // one slice of Psi_r or Psi_i, one stage
   static constexpr int B_BYTES = BN * ROWB;           // one slice of S or A, one stage
   static constexpr int STAGE_BYTES = 2 * NS * A_BYTES + (HAS_A ? 2 : 1) * NS * B_BYTES;
-  static constexpr int STAGES = (215040 / STAGE_BYTES) > 4 ? 4 : (215040 / STAGE_BYTES);
-  static constexpr int TMEM_COLS = 2 * BN <= 32 ? 32 : (2 * BN <= 64 ? 64 : (2 * BN <= 128 ? 128 : 256));
-  static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 256;
+  static constexpr int STAGES = (198000 / STAGE_BYTES) > 4 ? 4 : (198000 / STAGE_BYTES);
+  // 64-wide complex tiles multiply each left tile by the stacked [S; A] rows in one N = 128 MMA
+  // (split_issue_stage); other tiles take S and A in MMAs of their own
+  static constexpr bool STACKED = HAS_A && BN == 64;
+  static constexpr int ACC_COLS = STACKED ? 4 * BN : 2 * BN;  // tensor-memory columns of one tile's sums
+  static constexpr int TMEM_COLS = ACC_COLS <= 128 ? 128 : 256;
+  // stages, their alignment, barriers, then the epilogue warps' transposing stages
+  static constexpr size_t TAIL = 256;
+  static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + TAIL + EPI_WARPS * EPI_STAGE_BYTES;
+  static_assert(SMEM <= 232448, "shared memory of one CTA");
+  // one stage in shared memory: Psi_r slices, Psi_i slices, then S_q (and A_q) of slice q side by side
+  static __device__ __forceinline__ uint32_t right(uint32_t st, int q, int part) {
+    return st + 2 * NS * A_BYTES + ((HAS_A ? 2 : 1) * q + part) * B_BYTES;
+  }
 };
+
+// TMA loads of one stage (columns kx .. kx + BKE of the left rows j0 .. and the right rows i0 ..).
+template <int NS, int BN, int BKE, bool HAS_A>
+__device__ __forceinline__ void split_load_stage(uint32_t st, uint32_t bar, const CUtensorMap* left,
+                                                 const CUtensorMap* os, const CUtensorMap* oa, int kx, int np, int j0,
+                                                 int i0) {
+  using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
+#pragma unroll
+  for (int q = 0; q < NS; ++q) {
+    tma_load_2d(st + q * Cfg::A_BYTES, left + q, bar, kx, j0);              // Psi_r
+    tma_load_2d(st + (NS + q) * Cfg::A_BYTES, left + q, bar, np + kx, j0);  // Psi_i
+    tma_load_2d(Cfg::right(st, q, 0), os + q, bar, kx, i0);                 // S
+    if (HAS_A) tma_load_2d(Cfg::right(st, q, 1), oa + q, bar, kx, i0);      // A
+  }
+}
+
+// The MMAs of one stage into the accumulators at acc (fresh: the tile's first stage overwrites them).
+//  STACKED: Psi_r.[S; A] -> columns [0, 2 BN) and Psi_i.[S; A] -> columns [2 BN, 4 BN), two MMAs of
+//    N = 128 per slice pair and 16 values of k: an MMA's operands then cost 8 KB of shared-memory
+//    reads per 64 tensor cycles.  Four MMAs of N = 64 read 6 KB per 32 cycles, more than the 128
+//    bytes a cycle of shared memory: 43 -> 35 us a product at N = 1000 (BF16X3, K stages of 64).
+//    split_load_y forms Yr and Yi from the four sums.
+//  other complex tiles: Yr += Psi_r.S - Psi_i.A, Yi += Psi_r.A + Psi_i.S (negate-A bit);
+//  real right operand: Yr += Psi_r.S, Yi += Psi_i.S.
+template <int NS, int BN, int BKE, bool HAS_A>
+__device__ __forceinline__ void split_issue_stage(uint32_t acc, uint32_t st, bool fresh) {
+  using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
+  constexpr int MN = Cfg::STACKED ? 2 * BN : BN;
+  constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(MN >> 3) << 17) |
+                             ((uint32_t)(BM >> 4) << 24);
+  constexpr uint32_t idesc_neg = idesc | (1u << 13);  // negate the left operand
+#pragma unroll
+  for (int p = 0; p < Pairs<NS>::N; ++p) {
+    const uint32_t pr = st + Pairs<NS>::a(p) * Cfg::A_BYTES;
+    const uint32_t pi = st + (NS + Pairs<NS>::a(p)) * Cfg::A_BYTES;
+    const uint32_t os = Cfg::right(st, Pairs<NS>::b(p), 0), oa = Cfg::right(st, Pairs<NS>::b(p), 1);
+#pragma unroll
+    for (int kk = 0; kk < BKE / 16; ++kk) {
+      const uint32_t first = (fresh && p == 0 && kk == 0) ? 0u : 1u;
+      const uint64_t dpr = smem_desc<Cfg::ROWB>(pr + 32 * kk), dpi = smem_desc<Cfg::ROWB>(pi + 32 * kk);
+      const uint64_t dos = smem_desc<Cfg::ROWB>(os + 32 * kk);
+      if constexpr (Cfg::STACKED) {
+        mma_bf16(acc, dpr, dos, idesc, first);
+        mma_bf16(acc + 2 * BN, dpi, dos, idesc, first);
+      } else if constexpr (HAS_A) {
+        const uint64_t doa = smem_desc<Cfg::ROWB>(oa + 32 * kk);
+        mma_bf16(acc, dpr, dos, idesc, first);
+        mma_bf16(acc, dpi, doa, idesc_neg, 1u);
+        mma_bf16(acc + BN, dpr, doa, idesc, first);
+        mma_bf16(acc + BN, dpi, dos, idesc, 1u);
+      } else {
+        mma_bf16(acc, dpr, dos, idesc, first);
+        mma_bf16(acc + BN, dpi, dos, idesc, first);
+      }
+    }
+  }
+}
 
 __device__ __forceinline__ void store_f4(float* p, const float* v) {
   *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
@@ -253,151 +325,197 @@ __device__ __forceinline__ void load_f4(const float* p, float* v) {
   v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
 }
 
-// Loads cnt (<= 16) FP32 entries at p + idx (zero beyond cnt; all zero when p is NULL).
-__device__ __forceinline__ void load16(const float* p, size_t idx, int cnt, float (&v)[16]) {
-  if (p && cnt == 16) {
-#pragma unroll
-    for (int q = 0; q < 16; q += 4) load_f4(p + idx + q, v + q);
+// Loads cnt (<= 4) FP32 entries at p + idx (zero beyond cnt; all zero when p is NULL).
+__device__ __forceinline__ void load4(const float* p, size_t idx, int cnt, float (&v)[4]) {
+  if (p && cnt >= 4) {
+    load_f4(p + idx, v);
   } else {
 #pragma unroll
-    for (int q = 0; q < 16; ++q) v[q] = (p && q < cnt) ? p[idx + q] : 0.f;
+    for (int q = 0; q < 4; ++q) v[q] = (p && q < cnt) ? p[idx + q] : 0.f;
   }
 }
 
-__device__ __forceinline__ void store16(float* p, size_t idx, int cnt, const float (&v)[16]) {
-  if (cnt == 16) {
-#pragma unroll
-    for (int q = 0; q < 16; q += 4) store_f4(p + idx + q, v + q);
+__device__ __forceinline__ void store4(float* p, size_t idx, int cnt, const float (&v)[4]) {
+  if (cnt >= 4) {
+    store_f4(p + idx, v);
   } else {
 #pragma unroll
-    for (int q = 0; q < 16; ++q)
+    for (int q = 0; q < 4; ++q)
       if (q < cnt) p[idx + q] = v[q];
   }
 }
 
-// NS BF16 slices of 16 new complex entries into the next left operand (row j, columns ib..ib+cnt):
+// NS BF16 slices of 4 new complex entries into the next left operand (row j, columns ib..ib+cnt):
 // the real parts at column ib, the imaginary parts at column np + ib of each slice.
 template <int NS>
-__device__ __forceinline__ void store_slices(const SplitEpi& e, int j, int ib, int cnt, const float (&o_r)[16],
-                                             const float (&o_i)[16]) {
-  uint32_t wre[NS][8], wim[NS][8];  // two bf16 per word, element 2w in the low half
-#pragma unroll
-  for (int q = 0; q < 16; q += 2) {
-    __nv_bfloat16 r0[NS], r1[NS], m0[NS], m1[NS];
-    split_f32<NS>(o_r[q], r0);
-    split_f32<NS>(o_r[q + 1], r1);
-    split_f32<NS>(o_i[q], m0);
-    split_f32<NS>(o_i[q + 1], m1);
-#pragma unroll
-    for (int t = 0; t < NS; ++t) {
-      wre[t][q / 2] = (uint32_t)__bfloat16_as_ushort(r0[t]) | ((uint32_t)__bfloat16_as_ushort(r1[t]) << 16);
-      wim[t][q / 2] = (uint32_t)__bfloat16_as_ushort(m0[t]) | ((uint32_t)__bfloat16_as_ushort(m1[t]) << 16);
-    }
-  }
+__device__ __forceinline__ void store_slices(const SplitEpi& e, int j, int ib, int cnt, const float (&o_r)[4],
+                                             const float (&o_i)[4]) {
   const size_t srow = (size_t)j * e.kp + ib;
-  if (cnt == 16) {
+#pragma unroll
+  for (int part = 0; part < 2; ++part) {
+    __nv_bfloat16 s[4][NS];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) split_f32<NS>(part ? o_i[q] : o_r[q], s[q]);
 #pragma unroll
     for (int t = 0; t < NS; ++t) {
-      uint4* dr = reinterpret_cast<uint4*>(e.slice_out + t * e.slice_stride + srow);
-      uint4* di = reinterpret_cast<uint4*>(e.slice_out + t * e.slice_stride + srow + e.np);
-      dr[0] = make_uint4(wre[t][0], wre[t][1], wre[t][2], wre[t][3]);
-      dr[1] = make_uint4(wre[t][4], wre[t][5], wre[t][6], wre[t][7]);
-      di[0] = make_uint4(wim[t][0], wim[t][1], wim[t][2], wim[t][3]);
-      di[1] = make_uint4(wim[t][4], wim[t][5], wim[t][6], wim[t][7]);
-    }
-  } else {
+      __nv_bfloat16* d = e.slice_out + t * e.slice_stride + srow + (part ? e.np : 0);
+      if (cnt >= 4) {  // two bf16 per word, element 2w in the low half
+        const uint32_t lo = (uint32_t)__bfloat16_as_ushort(s[0][t]) | ((uint32_t)__bfloat16_as_ushort(s[1][t]) << 16);
+        const uint32_t hi = (uint32_t)__bfloat16_as_ushort(s[2][t]) | ((uint32_t)__bfloat16_as_ushort(s[3][t]) << 16);
+        *reinterpret_cast<uint2*>(d) = make_uint2(lo, hi);
+      } else {
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      if (q < cnt) {
-#pragma unroll
-        for (int t = 0; t < NS; ++t) {
-          const uint32_t wr = wre[t][q / 2] >> (16 * (q & 1)), wi = wim[t][q / 2] >> (16 * (q & 1));
-          e.slice_out[t * e.slice_stride + srow + q] = __ushort_as_bfloat16((unsigned short)(wr & 0xFFFFu));
-          e.slice_out[t * e.slice_stride + srow + e.np + q] = __ushort_as_bfloat16((unsigned short)(wi & 0xFFFFu));
-        }
+        for (int q = 0; q < 4; ++q)
+          if (q < cnt) d[q] = s[q][t];
       }
     }
   }
 }
 
-// Epilogue of one 16-column chunk of row j: Y entries yr, yi of columns ib .. ib + 15 (cnt valid).
-template <int NS, int EPI>
-__device__ __forceinline__ void epi_chunk(const SplitEpi& e, const float (&yr)[16], const float (&yi)[16], int j,
-                                          int ib, bool& bad, double& dsr, double& dsi) {
+// Epilogue stage of a warp: 32 rows x 32 columns of FP32 (4 KB), 16-byte units XOR-swizzled by row.
+static_assert(EPI_STAGE_BYTES == 32 * 32 * sizeof(float), "one 32 x 32 block a warp");
+
+// Turns a warp's 32 x 32 block from the tensor-memory layout (lane = row, v = its 32 columns) into
+// rows spread over lanes: out[4 p .. 4 p + 3] = columns 4 (lane % 8) .. of row 4 p + lane / 8, so that
+// the warp's global accesses cover four rows of 128 contiguous bytes.  Without it every lane walks a
+// row of its own: 32 lines an instruction, and the load/store unit (one line a cycle) set the
+// epilogue's time, 5.5 us per 16 columns of a 128-row tile at N = 200.  A BF16X3 product with it, 128 /
+// 64-wide tiles: N = 200 34 -> 24 / 20 -> 15 us, N = 1000 60 -> 48 / 35 -> 28 us, N = 2048 145 -> 127 /
+// 148 -> 136 us.
+__device__ __forceinline__ void epi_transpose(float* stage, int lane, const float (&v)[32], float (&out)[32]) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) store_f4(stage + lane * 32 + 4 * (c ^ (lane & 7)), v + 4 * c);
+  __syncwarp();
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    const int row = 4 * p + (lane >> 3);
+    load_f4(stage + row * 32 + 4 * ((lane & 7) ^ (row & 7)), out + 4 * p);
+  }
+  __syncwarp();
+}
+
+// Yr and Yi of 32 columns at c0 of this warp's 32 rows (trow: the tile's sums at the warp's lanes), in
+// the row-contiguous layout of epi_transpose.
+template <int NS, int BN, int BKE, bool HAS_A>
+__device__ __forceinline__ void split_load_y(uint32_t trow, int c0, float* stage, int lane, float (&yr)[32],
+                                             float (&yi)[32]) {
+#pragma unroll
+  for (int part = 0; part < 2; ++part) {
+    float v[2][16];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) tmem_ld16(trow + part * BN + c0 + 16 * h, v[h]);
+    if constexpr (SplitCfg<NS, BN, BKE, HAS_A>::STACKED) {
+      float w[2][16];  // Psi_i.A for Yr, Psi_i.S for Yi
+#pragma unroll
+      for (int h = 0; h < 2; ++h) tmem_ld16(trow + (part ? 2 : 3) * BN + c0 + 16 * h, w[h]);
+      tmem_wait_ld();
+#pragma unroll
+      for (int q = 0; q < 32; ++q) v[q >> 4][q & 15] += part ? w[q >> 4][q & 15] : -w[q >> 4][q & 15];
+    } else {
+      tmem_wait_ld();
+    }
+    float u[32];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) u[q] = v[q >> 4][q & 15];
+    epi_transpose(stage, lane, u, part ? yi : yr);
+  }
+}
+
+// Epilogue of one 32-row x 32-column block (rows jb .., columns ib0 ..) in the layout of
+// epi_transpose; BATCH row groups' operands are loaded together.
+template <int NS, int EPI, int BATCH>
+__device__ __forceinline__ void epi_block(const SplitEpi& e, const float (&yr)[32], const float (&yi)[32], int jb,
+                                          int ib0, int lane, bool& bad, double& dsr, double& dsi) {
   const float c0f = (float)e.t.coef0, cf = (float)e.t.coef, pr_ = (float)e.t.ph_re, pi_ = (float)e.t.ph_im;
   const float b2 = (float)e.t.bound2;
-  const int cnt = min(16, e.n - ib);
-  const size_t idx = (size_t)j * e.ldm + ib;
-  if (EPI == EPI_DOT) {
-    float br[16], bi[16];
-    load16(e.cur_re, idx, cnt, br);
-    load16(e.cur_im, idx, cnt, bi);
+  const int ib = ib0 + 4 * (lane & 7), cnt = min(4, e.n - ib);
+  if (cnt <= 0) return;
+#pragma unroll
+  for (int g = 0; g < 8; g += BATCH) {
+    float x_r[BATCH][4], x_i[BATCH][4], z_r[BATCH][4], z_i[BATCH][4];
     float sr = 0.f, si = 0.f;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {  // conj(b) Y; entries beyond cnt are zero in b
-      sr = fmaf(br[q], yr[q], fmaf(bi[q], yi[q], sr));
-      si = fmaf(br[q], yi[q], fmaf(-bi[q], yr[q], si));
+    for (int u = 0; u < BATCH; ++u) {
+      const int j = jb + 4 * (g + u) + (lane >> 3);
+      const int c = j < e.nc ? cnt : 0;
+      const size_t idx = (size_t)j * e.ldm + ib;
+      if (EPI == EPI_FWD) {
+        load4(e.t.first ? e.cur_re : e.prev_re, idx, c, x_r[u]);
+        load4(e.t.first ? e.cur_im : e.prev_im, idx, c, x_i[u]);
+        load4(e.t.first ? nullptr : e.acc_re, idx, c, z_r[u]);
+        load4(e.t.first ? nullptr : e.acc_im, idx, c, z_i[u]);
+      } else {
+        load4(e.cur_re, idx, c, x_r[u]);
+        load4(e.cur_im, idx, c, x_i[u]);
+        if (EPI == EPI_ADJ) {
+          load4(e.prev_re, idx, c, z_r[u]);
+          load4(e.prev_im, idx, c, z_i[u]);
+        }
+      }
     }
-    dsr += (double)sr;
-    dsi += (double)si;
-    return;
-  }
-  float o_r[16], o_i[16];
-  if (EPI == EPI_ADJ) {  // out = cpa g + i cw Y + b2
-    float g_r[16], g_i[16], p_r[16], p_i[16];
-    load16(e.cur_re, idx, cnt, g_r);
-    load16(e.cur_im, idx, cnt, g_i);
-    load16(e.prev_re, idx, cnt, p_r);
-    load16(e.prev_im, idx, cnt, p_i);
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      o_r[q] = e.cpa_re * g_r[q] - e.cpa_im * g_i[q] - e.cw * yi[q] + p_r[q];
-      o_i[q] = e.cpa_re * g_i[q] + e.cpa_im * g_r[q] + e.cw * yr[q] + p_i[q];
-      bad |= q < cnt && !(o_r[q] * o_r[q] + o_i[q] * o_i[q] <= b2);
-    }
-    store16(e.out_re, idx, cnt, o_r);
-    store16(e.out_im, idx, cnt, o_i);
-    store_slices<NS>(e, j, ib, cnt, o_r, o_i);
-    return;
-  }
-  // EPI_FWD
-  float a_r[16], a_i[16], p_r[16], p_i[16];
-  load16(e.t.first ? e.cur_re : e.prev_re, idx, cnt, p_r);
-  load16(e.t.first ? e.cur_im : e.prev_im, idx, cnt, p_i);
-  load16(e.t.first ? nullptr : e.acc_re, idx, cnt, a_r);
-  load16(e.t.first ? nullptr : e.acc_im, idx, cnt, a_i);
+    for (int u = 0; u < BATCH; ++u) {
+      const int j = jb + 4 * (g + u) + (lane >> 3);
+      const size_t idx = (size_t)j * e.ldm + ib;
+      const float* vr = yr + 4 * (g + u);
+      const float* vi = yi + 4 * (g + u);
+      if (EPI == EPI_DOT) {  // conj(b) Y; entries beyond the block are zero in b
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    float nr, ni, sr, si;
-    if (e.t.first) {  // psi_1 = -i Y, acc = a_0 psi_0 + a_1 psi_1
-      nr = yi[q];
-      ni = -yr[q];
-      sr = c0f * p_r[q] + cf * nr;
-      si = c0f * p_i[q] + cf * ni;
-    } else {  // psi_{l+1} = -2i Y + psi_{l-1}, acc += a_{l+1} psi_{l+1}
-      nr = 2.f * yi[q] + p_r[q];
-      ni = -2.f * yr[q] + p_i[q];
-      sr = a_r[q] + cf * nr;
-      si = a_i[q] + cf * ni;
+        for (int q = 0; q < 4; ++q) {
+          sr = fmaf(x_r[u][q], vr[q], fmaf(x_i[u][q], vi[q], sr));
+          si = fmaf(x_r[u][q], vi[q], fmaf(-x_i[u][q], vr[q], si));
+        }
+        continue;
+      }
+      if (j >= e.nc) continue;
+      float o_r[4], o_i[4];
+      if (EPI == EPI_ADJ) {  // out = cpa g + i cw Y + b2
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          o_r[q] = e.cpa_re * x_r[u][q] - e.cpa_im * x_i[u][q] - e.cw * vi[q] + z_r[u][q];
+          o_i[q] = e.cpa_re * x_i[u][q] + e.cpa_im * x_r[u][q] + e.cw * vr[q] + z_i[u][q];
+          bad |= q < cnt && !(o_r[q] * o_r[q] + o_i[q] * o_i[q] <= b2);
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          float nr, ni, ar, ai;
+          if (e.t.first) {  // psi_1 = -i Y, acc = a_0 psi_0 + a_1 psi_1
+            nr = vi[q];
+            ni = -vr[q];
+            ar = c0f * x_r[u][q] + cf * nr;
+            ai = c0f * x_i[u][q] + cf * ni;
+          } else {  // psi_{l+1} = -2i Y + psi_{l-1}, acc += a_{l+1} psi_{l+1}
+            nr = 2.f * vi[q] + x_r[u][q];
+            ni = -2.f * vr[q] + x_i[u][q];
+            ar = z_r[u][q] + cf * nr;
+            ai = z_i[u][q] + cf * ni;
+          }
+          bad |= q < cnt && !(nr * nr + ni * ni <= b2);
+          if (e.t.last) {  // X = e^{-i beta h} (acc + a_L psi_L)
+            o_r[q] = pr_ * ar - pi_ * ai;
+            o_i[q] = pr_ * ai + pi_ * ar;
+          } else {
+            o_r[q] = nr;
+            o_i[q] = ni;
+          }
+          z_r[u][q] = ar;
+          z_i[u][q] = ai;
+        }
+        if (!e.t.last) {
+          store4(e.acc_re, idx, cnt, z_r[u]);
+          store4(e.acc_im, idx, cnt, z_i[u]);
+        }
+      }
+      store4(e.out_re, idx, cnt, o_r);
+      store4(e.out_im, idx, cnt, o_i);
+      store_slices<NS>(e, j, ib, cnt, o_r, o_i);
     }
-    bad |= q < cnt && !(nr * nr + ni * ni <= b2);
-    if (e.t.last) {  // X = e^{-i beta h} (acc + a_L psi_L)
-      o_r[q] = pr_ * sr - pi_ * si;
-      o_i[q] = pr_ * si + pi_ * sr;
-    } else {
-      o_r[q] = nr;
-      o_i[q] = ni;
+    if (EPI == EPI_DOT) {
+      dsr += (double)sr;
+      dsi += (double)si;
     }
-    a_r[q] = sr;
-    a_i[q] = si;
   }
-  store16(e.out_re, idx, cnt, o_r);
-  store16(e.out_im, idx, cnt, o_i);
-  if (!e.t.last) {
-    store16(e.acc_re, idx, cnt, a_r);
-    store16(e.acc_im, idx, cnt, a_i);
-  }
-  store_slices<NS>(e, j, ib, cnt, o_r, o_i);
 }
 
 // One split GEMM on a 128-row x BN-column tile of Y = left . right^T:
@@ -465,14 +583,7 @@ k_split_term(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int ti
       const uint32_t bar = full0 + 8 * s;
       mbar_expect_tx(bar, Cfg::STAGE_BYTES);
       const int kx = kb * BKE;
-#pragma unroll
-      for (int q = 0; q < NS; ++q) {
-        tma_load_2d(st + q * Cfg::A_BYTES, &maps.a[q], bar, kx, j0);                       // Psi_r
-        tma_load_2d(st + (NS + q) * Cfg::A_BYTES, &maps.a[q], bar, e.np + kx, j0);         // Psi_i
-        tma_load_2d(st + 2 * NS * Cfg::A_BYTES + q * Cfg::B_BYTES, &maps.os[q], bar, kx, i0);  // S
-        if (HAS_A)
-          tma_load_2d(st + 2 * NS * Cfg::A_BYTES + (NS + q) * Cfg::B_BYTES, &maps.oa[q], bar, kx, i0);  // A
-      }
+      split_load_stage<NS, BN, BKE, HAS_A>(st, bar, maps.a, maps.os, maps.oa, kx, e.np, j0, i0);
       issued = kb + 1;
     }
     if (!ok) {
@@ -496,29 +607,7 @@ k_split_term(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int ti
       }
       tc_fence_after();
       const uint32_t st = base + s * Cfg::STAGE_BYTES;
-#pragma unroll
-      for (int p = 0; p < Pairs<NS>::N; ++p) {
-        const uint32_t pr = st + Pairs<NS>::a(p) * Cfg::A_BYTES;
-        const uint32_t pi = st + (NS + Pairs<NS>::a(p)) * Cfg::A_BYTES;
-        const uint32_t os = st + 2 * NS * Cfg::A_BYTES + Pairs<NS>::b(p) * Cfg::B_BYTES;
-        const uint32_t oa = st + 2 * NS * Cfg::A_BYTES + (NS + Pairs<NS>::b(p)) * Cfg::B_BYTES;
-#pragma unroll
-        for (int kk = 0; kk < BKE / 16; ++kk) {
-          const uint32_t first = (kb == 0 && p == 0 && kk == 0) ? 0u : 1u;
-          const uint64_t dpr = smem_desc<Cfg::ROWB>(pr + 32 * kk), dpi = smem_desc<Cfg::ROWB>(pi + 32 * kk);
-          const uint64_t dos = smem_desc<Cfg::ROWB>(os + 32 * kk);
-          if (HAS_A) {
-            const uint64_t doa = smem_desc<Cfg::ROWB>(oa + 32 * kk);
-            mma_bf16(tmem, dpr, dos, idesc, first);
-            mma_bf16(tmem, dpi, doa, idesc_neg, 1u);
-            mma_bf16(tmem + BN, dpr, doa, idesc, first);
-            mma_bf16(tmem + BN, dpi, dos, idesc, 1u);
-          } else {
-            mma_bf16(tmem, dpr, dos, idesc, first);
-            mma_bf16(tmem + BN, dpi, dos, idesc, first);
-          }
-        }
-      }
+      split_issue_stage<NS, BN, BKE, HAS_A>(tmem, st, kb == 0);
       mma_commit(empty0 + 8 * s);  // stage s free once these MMAs have read it
     }
     if (!ok) {
@@ -534,19 +623,16 @@ k_split_term(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int ti
   tc_fence_after();
   if (!got) atomicOr(e.t.status, FQ_BIT_TIMEOUT);
   const bool run = got && !*(volatile int*)abort_flag;
-  const int j = j0 + warp * 32 + lane;
+  float* stage = reinterpret_cast<float*>(gbase + STAGES * Cfg::STAGE_BYTES + Cfg::TAIL + warp * EPI_STAGE_BYTES);
   const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
   bool bad = false;
   double dsr = 0.0, dsi = 0.0;  // DOT partial of this thread
 #pragma unroll 1
-  for (int c0 = 0; c0 < BN; c0 += 16) {
-    float yr[16], yi[16];
-    tmem_ld16(trow + c0, yr);
-    tmem_ld16(trow + BN + c0, yi);
-    tmem_wait_ld();
-    const int ib = i0 + c0;
-    if (!run || j >= e.nc || ib >= e.n) continue;
-    epi_chunk<NS, EPI>(e, yr, yi, j, ib, bad, dsr, dsi);
+  for (int c0 = 0; c0 < BN; c0 += 32) {
+    float yr[32], yi[32];
+    split_load_y<NS, BN, BKE, HAS_A>(trow, c0, stage, lane, yr, yi);
+    if (!run || i0 + c0 >= e.n) continue;
+    epi_block<NS, EPI, 4>(e, yr, yi, j0 + warp * 32, i0 + c0, lane, bad, dsr, dsi);
   }
   if (bad) atomicOr(e.t.status, FQ_BIT_BOUND);
   if (EPI == EPI_DOT) {
@@ -572,11 +658,14 @@ k_split_term(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int ti
 
 // Persistent form of k_split_term for the forward and adjoint epilogues: one CTA per SM walks
 // the tiles blockIdx.x, blockIdx.x + gridDim.x, ...  Warp 0 (one thread) streams TMA stages,
-// warp 1 (one thread) issues the MMAs of tile i into tensor-memory buffer i & 1, and warps 2-5
-// run the epilogue of tile i from its buffer while tile i + 1 accumulates in the other one.
+// warp 1 (one thread) issues the MMAs of tile i into tensor-memory buffer i & 1, and the
+// epilogue warps run the epilogue of tile i from its buffer while tile i + 1 accumulates in the other one.
 // Buffers are handed over by mbarriers (tfull: MMAs of a tile done; tempty: its accumulators
 // read).  Every wait is bounded as in k_split_term.
-constexpr int PTHREADS = 192;
+constexpr int PTHREADS = 64 + 32 * EPI_WARPS;
+// column range [begin, end) of epilogue warp `warp` (2 .. 1 + EPI_WARPS) of a BN-wide tile
+template <int BN>
+__device__ __forceinline__ int epi_begin(int warp) { return ((warp - 2) >> 2) * (BN * 4 / EPI_WARPS); }
 
 template <int NS, int BN, int BKE, int EPI, bool HAS_A>
 __global__ void __launch_bounds__(PTHREADS, 1)
@@ -584,7 +673,7 @@ k_split_persist(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int
   static_assert(EPI != EPI_DOT, "the gradient dot keeps the one-tile kernel (per-CTA partials)");
   using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
   constexpr int STAGES = Cfg::STAGES;
-  constexpr uint32_t BUF_COLS = 2 * BN;             // Yr and Yi of one tile
+  constexpr uint32_t BUF_COLS = Cfg::ACC_COLS;      // one tile's sums
   constexpr uint32_t TMEM_COLS = 2 * BUF_COLS;      // two buffers (<= 512)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -606,7 +695,7 @@ k_split_persist(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull0 + 8 * b, 1);
-      mbar_init(tempty0 + 8 * b, 4);
+      mbar_init(tempty0 + 8 * b, EPI_WARPS);
     }
     mbar_init(done, 1);
     *abort_flag = 0;
@@ -648,14 +737,7 @@ k_split_persist(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int
           const uint32_t bar = full0 + 8 * s;
           mbar_expect_tx(bar, Cfg::STAGE_BYTES);
           const int kx = kb * BKE;
-#pragma unroll
-          for (int q = 0; q < NS; ++q) {
-            tma_load_2d(st + q * Cfg::A_BYTES, &maps.a[q], bar, kx, j0);
-            tma_load_2d(st + (NS + q) * Cfg::A_BYTES, &maps.a[q], bar, e.np + kx, j0);
-            tma_load_2d(st + 2 * NS * Cfg::A_BYTES + q * Cfg::B_BYTES, &maps.os[q], bar, kx, i0);
-            if (HAS_A)
-              tma_load_2d(st + 2 * NS * Cfg::A_BYTES + (NS + q) * Cfg::B_BYTES, &maps.oa[q], bar, kx, i0);
-          }
+          split_load_stage<NS, BN, BKE, HAS_A>(st, bar, maps.a, maps.os, maps.oa, kx, e.np, j0, i0);
           ++g;
         }
       }
@@ -668,9 +750,6 @@ k_split_persist(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int
     }
   } else if (warp == 1) {
     if (lane == 0) {  // ---------------- MMA issuer
-      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                                 ((uint32_t)(BM >> 4) << 24);
-      constexpr uint32_t idesc_neg = idesc | (1u << 13);
       int g = 0, i = 0;
       bool ok = true;
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++i) {
@@ -686,29 +765,7 @@ k_split_persist(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int
           }
           tc_fence_after();
           const uint32_t st = base + s * Cfg::STAGE_BYTES;
-#pragma unroll
-          for (int p = 0; p < Pairs<NS>::N; ++p) {
-            const uint32_t pr = st + Pairs<NS>::a(p) * Cfg::A_BYTES;
-            const uint32_t pi = st + (NS + Pairs<NS>::a(p)) * Cfg::A_BYTES;
-            const uint32_t os = st + 2 * NS * Cfg::A_BYTES + Pairs<NS>::b(p) * Cfg::B_BYTES;
-            const uint32_t oa = st + 2 * NS * Cfg::A_BYTES + (NS + Pairs<NS>::b(p)) * Cfg::B_BYTES;
-#pragma unroll
-            for (int kk = 0; kk < BKE / 16; ++kk) {
-              const uint32_t first = (kb == 0 && p == 0 && kk == 0) ? 0u : 1u;
-              const uint64_t dpr = smem_desc<Cfg::ROWB>(pr + 32 * kk), dpi = smem_desc<Cfg::ROWB>(pi + 32 * kk);
-              const uint64_t dos = smem_desc<Cfg::ROWB>(os + 32 * kk);
-              if (HAS_A) {
-                const uint64_t doa = smem_desc<Cfg::ROWB>(oa + 32 * kk);
-                mma_bf16(acc, dpr, dos, idesc, first);
-                mma_bf16(acc, dpi, doa, idesc_neg, 1u);
-                mma_bf16(acc + BN, dpr, doa, idesc, first);
-                mma_bf16(acc + BN, dpi, dos, idesc, 1u);
-              } else {
-                mma_bf16(acc, dpr, dos, idesc, first);
-                mma_bf16(acc + BN, dpi, dos, idesc, first);
-              }
-            }
-          }
+          split_issue_stage<NS, BN, BKE, HAS_A>(acc, st, kb == 0);
           mma_commit(empty0 + 8 * s);
         }
         if (!ok) break;
@@ -721,8 +778,10 @@ k_split_persist(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int
       mma_commit(done);  // every MMA issued above has completed once this arrives
       mbar_wait(done, 0);
     }
-  } else {  // ---------------- epilogue warps 2-5: tensor-memory lane quarter warp % 4
+  } else {  // ---------------- epilogue warps: tensor-memory lane quarter warp % 4
     const int quarter = warp & 3;
+    float* stage =
+        reinterpret_cast<float*>(gbase + STAGES * Cfg::STAGE_BYTES + Cfg::TAIL + (warp - 2) * EPI_STAGE_BYTES);
     bool bad = false, ok = true;
     double dsr = 0.0, dsi = 0.0;
     int i = 0;
@@ -737,21 +796,18 @@ k_split_persist(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int
       }
       int j0, i0;
       coords(t, j0, i0);
-      const int j = j0 + quarter * 32 + lane;
       const uint32_t trow = tmem + (uint32_t)b * BUF_COLS + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 16) {
-        float yr[16], yi[16];
-        tmem_ld16(trow + c0, yr);
-        tmem_ld16(trow + BN + c0, yi);
-        tmem_wait_ld();
-        const int ib = i0 + c0;
-        if (j >= e.nc || ib >= e.n) continue;
-        epi_chunk<NS, EPI>(e, yr, yi, j, ib, bad, dsr, dsi);
+      for (int c0 = epi_begin<BN>(warp), c1 = c0 + BN * 4 / EPI_WARPS; c0 < c1; c0 += 32) {
+        float yr[32], yi[32];
+        split_load_y<NS, BN, BKE, HAS_A>(trow, c0, stage, lane, yr, yi);
+        if (c0 + 32 >= c1) {  // this warp's sums are read: the buffer's next MMAs may start
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tempty0 + 8 * b);
+        }
+        if (i0 + c0 < e.n) epi_block<NS, EPI, 4>(e, yr, yi, j0 + quarter * 32, i0 + c0, lane, bad, dsr, dsi);
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tempty0 + 8 * b);
     }
     if (!ok) {
       atomicExch(abort_flag, 1);
@@ -784,7 +840,7 @@ struct ChainArgs {
   CUtensorMap left[CHAIN_MAXP][3]; // left operand slices of product p
   SplitEpi epi[CHAIN_MAXP];        // epilogue of product p (slice_out = product p+1's left operand)
   int nprod, nk, tiles_j, tiles_i;
-  unsigned int* flags;             // [nprod][tiles_j]: finished epilogue warps (4 a tile) of product p in
+  unsigned int* flags;             // [nprod][tiles_j]: finished epilogue warps (EPI_WARPS a tile) of product p in
                                    // row block tj (zeroed before the launch)
 };
 
@@ -814,7 +870,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
   static_assert(EPI != EPI_DOT, "chains of forward or adjoint terms only");
   using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
   constexpr int STAGES = Cfg::STAGES;
-  constexpr uint32_t BUF_COLS = 2 * BN;
+  constexpr uint32_t BUF_COLS = Cfg::ACC_COLS;
   constexpr uint32_t TMEM_COLS = 2 * BUF_COLS;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -838,7 +894,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull0 + 8 * b, 1);
-      mbar_init(tempty0 + 8 * b, 4);
+      mbar_init(tempty0 + 8 * b, EPI_WARPS);
     }
     mbar_init(done, 1);
     *abort_flag = 0;
@@ -871,7 +927,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
         int p, tj, j0, i0;
         unit(u, p, tj, j0, i0);
         if (p > 0) {
-          if (!(ok = wait_count(args.flags + (size_t)(p - 1) * args.tiles_j + tj, 4u * args.tiles_i))) break;
+          if (!(ok = wait_count(args.flags + (size_t)(p - 1) * args.tiles_j + tj, (unsigned)EPI_WARPS * args.tiles_i))) break;
           fence_proxy_async_global();  // the epilogues' generic stores, before this thread's TMA reads
         }
         const int np_ = args.epi[p].np;
@@ -886,14 +942,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
           const uint32_t bar = full0 + 8 * s;
           mbar_expect_tx(bar, Cfg::STAGE_BYTES);
           const int kx = kb * BKE;
-#pragma unroll
-          for (int q = 0; q < NS; ++q) {
-            tma_load_2d(st + q * Cfg::A_BYTES, &args.left[p][q], bar, kx, j0);
-            tma_load_2d(st + (NS + q) * Cfg::A_BYTES, &args.left[p][q], bar, np_ + kx, j0);
-            tma_load_2d(st + 2 * NS * Cfg::A_BYTES + q * Cfg::B_BYTES, &args.rmaps.os[q], bar, kx, i0);
-            if (HAS_A)
-              tma_load_2d(st + 2 * NS * Cfg::A_BYTES + (NS + q) * Cfg::B_BYTES, &args.rmaps.oa[q], bar, kx, i0);
-          }
+          split_load_stage<NS, BN, BKE, HAS_A>(st, bar, args.left[p], args.rmaps.os, args.rmaps.oa, kx, np_, j0, i0);
           ++g;
         }
       }
@@ -905,9 +954,6 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
     }
   } else if (warp == 1) {
     if (lane == 0) {  // ---------------- MMA issuer (as k_split_persist)
-      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                                 ((uint32_t)(BM >> 4) << 24);
-      constexpr uint32_t idesc_neg = idesc | (1u << 13);
       int g = 0, i = 0;
       bool ok = true;
       for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x, ++i) {
@@ -923,29 +969,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
           }
           tc_fence_after();
           const uint32_t st = base + s * Cfg::STAGE_BYTES;
-#pragma unroll
-          for (int pp = 0; pp < Pairs<NS>::N; ++pp) {
-            const uint32_t pr = st + Pairs<NS>::a(pp) * Cfg::A_BYTES;
-            const uint32_t pi = st + (NS + Pairs<NS>::a(pp)) * Cfg::A_BYTES;
-            const uint32_t os = st + 2 * NS * Cfg::A_BYTES + Pairs<NS>::b(pp) * Cfg::B_BYTES;
-            const uint32_t oa = st + 2 * NS * Cfg::A_BYTES + (NS + Pairs<NS>::b(pp)) * Cfg::B_BYTES;
-#pragma unroll
-            for (int kk = 0; kk < BKE / 16; ++kk) {
-              const uint32_t first = (kb == 0 && pp == 0 && kk == 0) ? 0u : 1u;
-              const uint64_t dpr = smem_desc<Cfg::ROWB>(pr + 32 * kk), dpi = smem_desc<Cfg::ROWB>(pi + 32 * kk);
-              const uint64_t dos = smem_desc<Cfg::ROWB>(os + 32 * kk);
-              if (HAS_A) {
-                const uint64_t doa = smem_desc<Cfg::ROWB>(oa + 32 * kk);
-                mma_bf16(acc, dpr, dos, idesc, first);
-                mma_bf16(acc, dpi, doa, idesc_neg, 1u);
-                mma_bf16(acc + BN, dpr, doa, idesc, first);
-                mma_bf16(acc + BN, dpi, dos, idesc, 1u);
-              } else {
-                mma_bf16(acc, dpr, dos, idesc, first);
-                mma_bf16(acc + BN, dpi, dos, idesc, first);
-              }
-            }
-          }
+          split_issue_stage<NS, BN, BKE, HAS_A>(acc, st, kb == 0);
           mma_commit(empty0 + 8 * s);
         }
         if (!ok) break;
@@ -958,8 +982,10 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
       mma_commit(done);
       mbar_wait(done, 0);
     }
-  } else {  // ---------------- epilogue warps 2-5; then the unit's completion for its row block
+  } else {  // ---------------- epilogue warps; then the unit's completion for its row block
     const int quarter = warp & 3;
+    float* stage =
+        reinterpret_cast<float*>(gbase + STAGES * Cfg::STAGE_BYTES + Cfg::TAIL + (warp - 2) * EPI_STAGE_BYTES);
     bool bad = false, ok = true;
     double dsr = 0.0, dsi = 0.0;
     int i = 0;
@@ -977,23 +1003,20 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
       // the previous product's outputs this epilogue reads (prev, acc) were released with its counter
       if (p > 0) ld_acquire_u32(args.flags + (size_t)(p - 1) * args.tiles_j + tj);
       const SplitEpi& e = args.epi[p];
-      const int j = j0 + quarter * 32 + lane;
       const uint32_t trow = tmem + (uint32_t)b * BUF_COLS + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 16) {
-        float yr[16], yi[16];
-        tmem_ld16(trow + c0, yr);
-        tmem_ld16(trow + BN + c0, yi);
-        tmem_wait_ld();
-        const int ib = i0 + c0;
-        if (j >= e.nc || ib >= e.n) continue;
-        epi_chunk<NS, EPI>(e, yr, yi, j, ib, bad, dsr, dsi);
+      for (int c0 = epi_begin<BN>(warp), c1 = c0 + BN * 4 / EPI_WARPS; c0 < c1; c0 += 32) {
+        float yr[32], yi[32];
+        split_load_y<NS, BN, BKE, HAS_A>(trow, c0, stage, lane, yr, yi);
+        if (c0 + 32 >= c1) {  // this warp's sums are read: the buffer's next MMAs may start
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tempty0 + 8 * b);
+        }
+        if (i0 + c0 < e.n) epi_block<NS, EPI, 4>(e, yr, yi, j0 + quarter * 32, i0 + c0, lane, bad, dsr, dsi);
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tempty0 + 8 * b);
       // this warp's stores of the unit made visible (to the async proxy too), then one release per
-      // warp: a tile is done when its four epilogue warps have counted
+      // warp: a tile is done when its epilogue warps have counted
       fence_proxy_async_global();
       __threadfence();
       __syncwarp();

@@ -60,6 +60,37 @@ def test_split_goe64_build(fq, prec, ns, tile, tk):
     assert err <= tol
 
 
+@pytest.mark.parametrize("n", [1, 3, 31, 33, 66, 127, 129, 161])
+@pytest.mark.parametrize("prec,ns,tile,tk", SHAPES)
+def test_split_tile_edges(fq, prec, ns, tile, tk, n):
+    """U_T at the edges of the epilogue's 32-column blocks and 4-column units and of the 64- and
+    128-wide tiles, every shape, with a drive of nonzero phase (A of Omega~ = S + i A not small)."""
+    M = 10
+    h0, h1 = fi.goe(n, 1311), fi.goe(n, 1312)
+    drv = fi.Drive(0.2, 1.3, 1.1, 0.6)
+    plan = fq.Plan.dense(h0, h1, omega=drv.omega, f_ac=drv.f_ac, f_dc=drv.f_dc, phi0=drv.phi0, steps=M,
+                         precision=prec, tile_n=tile, tile_k=tk)
+    U = plan.build_UT().cpu().numpy()
+    assert plan.check_status() == fq.FQ_OK
+    ref = o.build_ut_dense(h0, h1, o.plan_for_drive_dense(h0, h1, drv, M))
+    assert np.max(np.abs(U - ref)) <= tol_split(M, plan.info.L, plan.info.R, ns)
+
+
+@pytest.mark.parametrize("prec", [2, 3])
+def test_split_default_tile(fq, prec):
+    """Below the line of the default rule a plan without a tile width runs the 64-wide tiles, bit for
+    bit as a plan that asks for them, whole and in column blocks."""
+    import torch
+    n = 150
+    kw = dict(omega=1.3, f_ac=1.1, steps=6, precision=prec)
+    h0, h1 = fi.goe(n, 1313), fi.goe(n, 1314)
+    plan = fq.Plan.dense(h0, h1, **kw)
+    U = plan.build_UT()
+    assert torch.equal(U, fq.Plan.dense(h0, h1, tile_n=64, **kw).build_UT())
+    X = plan.propagate(torch.eye(n, dtype=torch.complex128, device="cuda")[17:20].contiguous())
+    assert torch.equal(X.transpose(0, 1), U[:, 17:20])
+
+
 @pytest.mark.parametrize("prec,ns,tile,tk", SHAPES)
 def test_split_ragged_propagate(fq, prec, ns, tile, tk):
     """N = 200 (K' padded to 512, output tiles ragged), 37 states (one partial 128-row tile),
