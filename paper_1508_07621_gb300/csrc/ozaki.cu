@@ -97,8 +97,12 @@ fq_status fq_ozaki_propagate(fq_plan* p, const double* x0, double* x, int nc, in
   if (m_end > m_begin)
     k_oz_slice_left<<<w.ncp, 256, 0, s>>>(w.m[0][0], w.m[0][1], 1.0, 0.0, nullptr, nullptr, n, nc, w.np, w.astride,
                                           w.left, w.es);
-  const int tiles_i = w.np / OZ_BN, tiles_j = w.ncp / BM;
-  const int nk = w.np / OZ_BKE;
+  // output columns and values of k beyond N are zero: their tiles and stages are left out.  The
+  // cluster size looks at N alone, so that a block of columns agrees with the whole U_T bit for bit.
+  const int tiles_i = (n + OZ_BN - 1) / OZ_BN, tiles_j = w.ncp / BM;
+  const int nk = (n + OZ_BKE - 1) / OZ_BKE;
+  const int csize = oz_cluster(tiles_i * ((n + BM - 1) / BM), nk);
+  OzLaunch launch(tiles_i * tiles_j, csize, OzCfg::SMEM, s);
   fq_term t{};
   t.coef0 = p->cheb[0];
   t.ph_re = p->phase_re;
@@ -127,8 +131,8 @@ fq_status fq_ozaki_propagate(fq_plan* p, const double* x0, double* x, int nc, in
       e.es = w.es;
       e.et = w.et;
       e.t = t;
-      k_oz_term<<<tiles_i * tiles_j, OZ_THREADS, OzCfg::SMEM, s>>>(maps, nk, tiles_j, tiles_i,
-                                                                                        w.np, e);
+      cudaError_t le = cudaLaunchKernelEx(&launch.cfg, k_oz_term, maps, nk, tiles_j, tiles_i, w.np, csize, e);
+      if (le != cudaSuccess) return fq_cuda_fail(le, "FP64-emulation term launch");
       if (!(t.last && m == m_end - 1))
         k_oz_slice_left<<<w.ncp, 256, 0, s>>>(w.m[out][0], w.m[out][1], 1.0, 0.0, nullptr, nullptr, n, nc, w.np,
                                               w.astride, w.left, w.es);

@@ -33,6 +33,18 @@
 // the four accumulators (128 columns each), so the MMAs wait for each drain.  Every wait is
 // bounded; a wait that gives up records FQ_BIT_TIMEOUT, drains this CTA's own copies and MMAs,
 // frees tensor memory and returns.
+//
+// Split K.  Where a product has fewer tiles than half the SMs (oz_cluster), a cluster of 2 or 4 CTAs
+// shares a tile: each takes a range of k, the double-float sums stay in shared memory, and each
+// CTA folds all of them (double-float again, as the chunks of one CTA are folded) for its share of
+// the 64 columns and runs the epilogue there.
+//
+// Epilogue.  GB300 runs 2 FP64 multiply-adds a cycle and SM, so an FP64 instruction of a warp costs
+// 16 cycles and the epilogue is bound by their number: it had 15 a complex entry (30 us a tile) and
+// has 6.  The double-float sums are scaled and widened to FP64 by integer work on the bit patterns
+// (oz_value), and the bound check compares high words first (oz_outside).  The sums are staged
+// column-major in the idle stages, and a warp then takes 32 consecutive columns of a row, so that
+// every global access is a contiguous 256 bytes.
 #pragma once
 
 #include "split_core.cuh"
@@ -49,7 +61,9 @@ constexpr int OZ_EPI_WARPS = 16;
 constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;
 constexpr int OZ_A_BYTES = BM * OZ_ROWB;                   // one slice of Psi_r or Psi_i
 constexpr uint32_t OZ_TMEM_COLS = 512;      // 4 accumulators x (Yr | Yi) x 64 columns
-constexpr int OZ_XS_BYTES = 64 * 4 * 32 * OZ_EPI_WARPS;   // drained sums staged for the epilogue
+constexpr int OZ_EPI_ROWS = 4;              // rows of the epilogue a thread loads together
+constexpr int OZ_XS_LD = 129;               // staged sums: [column][row] planes, padded against bank conflicts
+constexpr int OZ_XS_PLANE = OZ_XS_LD * OZ_BN;
 
 // Stage layout of the complex product (Omega~ = S + i A): one right slice is the [-A; S; A] rows
 // of a 64-row block.  (Products with a real right operand use ozaki_real.cuh.)
@@ -59,7 +73,7 @@ struct OzCfg {
   static constexpr int STAGE_BYTES = 2 * OZ_S * OZ_A_BYTES + OZ_S * R_BYTES;
   static constexpr int STAGES = 2;
   static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 256;
-  static_assert((size_t)STAGES * STAGE_BYTES >= OZ_XS_BYTES + 16 * sizeof(double2), "epilogue staging");
+  static_assert((size_t)STAGES * STAGE_BYTES >= 4 * OZ_XS_PLANE * sizeof(float), "epilogue staging");
 };
 
 struct OzMaps {
@@ -128,7 +142,69 @@ __device__ __forceinline__ void dd_add2(float2& h, float2& l, float2 v) {
   h = h2;
 }
 
+// (h, l) += (h2, l2), both double-float
+__device__ __forceinline__ void dd_add(float& h, float& l, float h2, float l2) {
+  const float s = __fadd_rn(h, h2);
+  const float bb = __fsub_rn(s, h);
+  const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(h2, bb));
+  const float lo = __fadd_rn(__fadd_rn(l, l2), e);
+  h = __fadd_rn(s, lo);
+  l = __fsub_rn(lo, __fsub_rn(h, s));
+}
+
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
+
+// x 2^ex as FP64 for |ex| <= 800, by integer work on the bit pattern (FP64 conversions and
+// multiplications run at the FP64 rate).  x is zero or a multiple of 2^-56 below 2^24, as every
+// staged sum is: FP32 subnormals do not occur.
+__device__ __forceinline__ double oz_scaled(float x, int ex) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7FFFFFFFu;
+  if (m == 0) return 0.0;
+  const unsigned hi = (u & 0x80000000u) | ((m >> 3) + (unsigned)((896 + ex) << 20));
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+
+// (h + l) 2^ex in FP64, one addition; exponents outside +-800 take the conversions and a product
+// (below 2^-1022 the product is below 2^-1022 too)
+__device__ __forceinline__ double oz_value(float h, float l, int ex) {
+  if (ex < -800 || ex > 800) return ((double)h + (double)l) * pow2(ex < -1022 ? -1022 : ex);
+  return oz_scaled(h, ex) + oz_scaled(l, ex);
+}
+
+// !(re^2 + im^2 <= bound2) for bound2 >= 1; both parts below 2^-1/2 in magnitude (their high words
+// compare as integers, NaN and infinity above every finite value) need no FP64 arithmetic
+__device__ __forceinline__ bool oz_outside(double re, double im, double bound2) {
+  const int a = __double2hiint(re) & 0x7FFFFFFF, b = __double2hiint(im) & 0x7FFFFFFF;
+  if (a < 0x3FE6A09E && b < 0x3FE6A09E) return false;
+  return !(re * re + im * im <= bound2);
+}
+
+// Shared-memory float at the same offset in cluster CTA `rank`
+__device__ __forceinline__ float ld_cluster(const float* local, unsigned rank) {
+  unsigned ra;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(smem_u32(local)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(ra) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void oz_cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Sum of the staged double-float value at plane offset `at` (high part; low part `lo` floats on) over
+// the cluster's CTAs, in rank order.
+__device__ __forceinline__ void oz_fold(const float* xs, int at, int lo, int csize, float& h, float& l) {
+  if (csize == 1) {
+    h = xs[at];
+    l = xs[at + lo];
+    return;
+  }
+  h = ld_cluster(xs + at, 0);
+  l = ld_cluster(xs + at + lo, 0);
+  for (int r = 1; r < csize; ++r) dd_add(h, l, ld_cluster(xs + at, r), ld_cluster(xs + at + lo, r));
+}
 
 // |x| as an ordered integer key (the bit pattern of a non-negative double orders like its value)
 __device__ __forceinline__ unsigned long long abs_key(double x) {
@@ -347,9 +423,10 @@ __global__ void k_oz_real(const double* __restrict__ h0, const double* __restric
   if (threadIdx.x == 0) et[i] = e;
 }
 
-// One Chebyshev term (OZ_FWD) on a 128-state x 64-column tile (see the file comment).
+// One Chebyshev term (OZ_FWD) on a 128-state x 64-column tile per cluster of `csize` CTAs (see the
+// file comment).
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    k_oz_term(const __grid_constant__ OzMaps maps, int nk, int tiles_j, int tiles_i, int np, OzEpi e) {
+    k_oz_term(const __grid_constant__ OzMaps maps, int nk, int tiles_j, int tiles_i, int np, int csize, OzEpi e) {
   using Cfg = OzCfg;
   constexpr int OZ_STAGES = Cfg::STAGES;
   constexpr int OZ_STAGE_BYTES = Cfg::STAGE_BYTES;
@@ -366,11 +443,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   const uint32_t tfull = smem_u32(bars + 2 * OZ_STAGES), tempty0 = smem_u32(bars + 2 * OZ_STAGES + 1);
   const uint32_t done = smem_u32(bars + 2 * OZ_STAGES + 5);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nchunks = nk / OZ_KB_PER_DRAIN;
+  // this CTA's K stages kb0 .. kb0 + nkr
+  const int rank = blockIdx.x % csize;
+  const int kb0 = nk * rank / csize, nkr = nk * (rank + 1) / csize - kb0;
+  const int nchunks = (nkr + OZ_KB_PER_DRAIN - 1) / OZ_KB_PER_DRAIN;
 
   int tj, ti;
   {
-    const int b = blockIdx.x, per = RASTER_GROUP * tiles_i, g = b / per;
+    const int b = blockIdx.x / csize, per = RASTER_GROUP * tiles_i, g = b / per;
     const int gj = min(RASTER_GROUP, tiles_j - g * RASTER_GROUP), r = b - g * per;
     tj = g * RASTER_GROUP + r % gj;
     ti = r / gj;
@@ -403,7 +483,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     if (lane == 0) {  // ---------------- TMA producer
       int issued = 0;
       bool ok = true;
-      for (int kb = 0; kb < nk && ok; ++kb) {
+      for (int kb = 0; kb < nkr && ok; ++kb) {
         const int s = kb % OZ_STAGES;
         if (kb >= OZ_STAGES && !(ok = mbar_wait(empty0 + 8 * s, ((kb / OZ_STAGES) - 1) & 1))) break;
         if (*(volatile int*)abort_flag) {
@@ -413,7 +493,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const uint32_t st = base + s * OZ_STAGE_BYTES;
         const uint32_t bar = full0 + 8 * s;
         mbar_expect_tx(bar, OZ_STAGE_BYTES);
-        const int kx = kb * OZ_BKE;
+        const int kx = (kb0 + kb) * OZ_BKE;
 #pragma unroll
         for (int q = 0; q < OZ_S; ++q) {
           tma_load_2d(st + (2 * q) * OZ_A_BYTES, &maps.a[q], bar, kx, j0);           // Psi_r
@@ -436,7 +516,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       bool ok = true;
       int kb = 0;
       for (int c = 0; c < nchunks && ok; ++c) {
-        for (int kq = 0; kq < OZ_KB_PER_DRAIN && ok; ++kq, ++kb) {
+        for (int kq = 0; kq < OZ_KB_PER_DRAIN && kb < nkr; ++kq, ++kb) {
           const int s = kb % OZ_STAGES;
           ok = mbar_wait(full0 + 8 * s, (kb / OZ_STAGES) & 1);
           if (!ok || *(volatile int*)abort_flag) {
@@ -469,6 +549,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             mma_bf16(acc, d0 + (uint64_t)(((2 * a + 1) * OZ_A_BYTES) >> 4), d0 + (uint64_t)(rb >> 4), idesc,
                      1u);            // Psi_i . [-A; S]
           }
+          if (!ok) break;
           mma_commit(empty0 + 8 * s);
         }
         if (!ok) break;
@@ -483,7 +564,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     }
   } else {  // ---------------- drain warps 2-17
     const int quarter = warp & 3, part = (warp - 2) >> 2;
-    const int j = j0 + quarter * 32 + lane;
     const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * 16);
     float2 hr[8], lr[8], hi[8], li[8];  // double-float sums of columns (2p, 2p + 1)
 #pragma unroll
@@ -523,72 +603,119 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     if (!ok) {
       atomicExch(abort_flag, 1);
       atomicOr(e.t.status, FQ_BIT_TIMEOUT);
-    } else if (j < e.nc) {
-      // ---------------- epilogue in FP64 (as in the plain FP64 path).  The stages are idle now
-      // (the last MMAs have completed): the sums wait there, one column per pass.
-      float* xs = reinterpret_cast<float*>(gbase) + (threadIdx.x - 64);
-      constexpr int XS = 32 * OZ_EPI_WARPS;
+    } else {
+      // the stages are idle now (the last MMAs have completed, every copy has landed): the sums wait
+      // there as planes hr, lr, hi, li of [column][row]
+      float* xw = reinterpret_cast<float*>(gbase) + part * 16 * OZ_XS_LD + quarter * 32 + lane;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        xs[(8 * q) * XS] = hr[q].x;
-        xs[(8 * q + 1) * XS] = lr[q].x;
-        xs[(8 * q + 2) * XS] = hi[q].x;
-        xs[(8 * q + 3) * XS] = li[q].x;
-        xs[(8 * q + 4) * XS] = hr[q].y;
-        xs[(8 * q + 5) * XS] = lr[q].y;
-        xs[(8 * q + 6) * XS] = hi[q].y;
-        xs[(8 * q + 7) * XS] = li[q].y;
-      }
-      const fq_term& t = e.t;
-      const int ej = e.es[j];
-      bool bad = false;
-#pragma unroll 1
       for (int q = 0; q < 16; ++q) {
-        const int i = i0 + part * 16 + q;
-        if (i >= e.n) break;
-        const int ex = ej + e.et[i];
-        const double sc = pow2(ex < -1022 ? -1022 : ex);  // below that the product is below 2^-1022
-        const int b = 8 * (q >> 1) + 4 * (q & 1);  // slots of column q: hr, lr, hi, li
-        const double yr = ((double)xs[b * XS] + (double)xs[(b + 1) * XS]) * sc;
-        const double yi = ((double)xs[(b + 2) * XS] + (double)xs[(b + 3) * XS]) * sc;
-        const size_t idx = (size_t)j * e.n + i;
-        double pr, pi;
-        if (t.first) {
-          pr = yi;
-          pi = -yr;
-        } else {
-          pr = fma(2.0, yi, e.prev_re[idx]);
-          pi = fma(-2.0, yr, e.prev_im[idx]);
-        }
-        bad |= !(pr * pr + pi * pi <= t.bound2);
-        double ar, ai;
-        if (t.first) {
-          ar = fma(t.coef, pr, t.coef0 * e.cur_re[idx]);
-          ai = fma(t.coef, pi, t.coef0 * e.cur_im[idx]);
-        } else {
-          ar = fma(t.coef, pr, e.acc_re[idx]);
-          ai = fma(t.coef, pi, e.acc_im[idx]);
-        }
-        if (t.last) {
-          e.out_re[idx] = t.ph_re * ar - t.ph_im * ai;
-          e.out_im[idx] = t.ph_re * ai + t.ph_im * ar;
-        } else {
-          e.out_re[idx] = pr;
-          e.out_im[idx] = pi;
-          e.acc_re[idx] = ar;
-          e.acc_im[idx] = ai;
-        }
+        xw[q * OZ_XS_LD] = q & 1 ? hr[q >> 1].y : hr[q >> 1].x;
+        xw[q * OZ_XS_LD + OZ_XS_PLANE] = q & 1 ? lr[q >> 1].y : lr[q >> 1].x;
+        xw[q * OZ_XS_LD + 2 * OZ_XS_PLANE] = q & 1 ? hi[q >> 1].y : hi[q >> 1].x;
+        xw[q * OZ_XS_LD + 3 * OZ_XS_PLANE] = q & 1 ? li[q >> 1].y : li[q >> 1].x;
       }
-      if (bad) atomicOr(t.status, FQ_BIT_BOUND);
     }
   }
   tc_fence_before();
   __syncthreads();
+  if (csize > 1) oz_cluster_sync();
+  if (warp >= 2 && !*(volatile int*)abort_flag) {
+    // ---------------- epilogue in FP64 (as in the plain FP64 path): this CTA's share of the columns,
+    // consecutive threads on consecutive columns of a row
+    const float* xs = reinterpret_cast<const float*>(gbase);
+    const fq_term& t = e.t;
+    const int w = OZ_BN / csize, tt = threadIdx.x - 64;
+    const int cc = rank * w + tt % w, i = i0 + cc;
+    bool bad = false;
+    if (i < e.n) {
+      const int ei = e.et[i];
+      // OZ_EPI_ROWS rows' operands are loaded together (the stores may alias them for the compiler)
+      const int step = 32 * OZ_EPI_WARPS / w;
+      for (int row0 = tt / w; row0 < BM && j0 + row0 < e.nc; row0 += OZ_EPI_ROWS * step) {
+        double xr[OZ_EPI_ROWS], xi[OZ_EPI_ROWS], zr[OZ_EPI_ROWS], zi[OZ_EPI_ROWS];
+        int ej[OZ_EPI_ROWS];
+#pragma unroll
+        for (int u = 0; u < OZ_EPI_ROWS; ++u) {
+          const int row = row0 + u * step, j = j0 + row;
+          const bool in = row < BM && j < e.nc;
+          const size_t idx = (size_t)j * e.n + i;
+          xr[u] = !in ? 0.0 : t.first ? e.cur_re[idx] : e.prev_re[idx];
+          xi[u] = !in ? 0.0 : t.first ? e.cur_im[idx] : e.prev_im[idx];
+          zr[u] = in && !t.first ? e.acc_re[idx] : 0.0;
+          zi[u] = in && !t.first ? e.acc_im[idx] : 0.0;
+          ej[u] = in ? e.es[j] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < OZ_EPI_ROWS; ++u) {
+          const int row = row0 + u * step, j = j0 + row;
+          if (row >= BM || j >= e.nc) break;
+          const int ex = ej[u] + ei, at = cc * OZ_XS_LD + row;
+          const size_t idx = (size_t)j * e.n + i;
+          float h0, l0, h1, l1;
+          oz_fold(xs, at, OZ_XS_PLANE, csize, h0, l0);
+          oz_fold(xs, at + 2 * OZ_XS_PLANE, OZ_XS_PLANE, csize, h1, l1);
+          const double yr = oz_value(h0, l0, ex), yi = oz_value(h1, l1, ex);
+          double pr, pi, ar, ai;
+          if (t.first) {
+            pr = yi;
+            pi = -yr;
+            ar = fma(t.coef, pr, t.coef0 * xr[u]);
+            ai = fma(t.coef, pi, t.coef0 * xi[u]);
+          } else {
+            pr = fma(2.0, yi, xr[u]);
+            pi = fma(-2.0, yr, xi[u]);
+            ar = fma(t.coef, pr, zr[u]);
+            ai = fma(t.coef, pi, zi[u]);
+          }
+          bad |= oz_outside(pr, pi, t.bound2);
+          if (t.last) {
+            e.out_re[idx] = t.ph_re * ar - t.ph_im * ai;
+            e.out_im[idx] = t.ph_re * ai + t.ph_im * ar;
+          } else {
+            e.out_re[idx] = pr;
+            e.out_im[idx] = pi;
+            e.acc_re[idx] = ar;
+            e.acc_im[idx] = ai;
+          }
+        }
+      }
+    }
+    if (bad) atomicOr(t.status, FQ_BIT_BOUND);
+  }
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OZ_TMEM_COLS) : "memory");
   }
+  if (csize > 1) oz_cluster_sync();  // no CTA leaves while a peer may still read its sums
 }
+
+// CTAs that share a tile's K range: as many of 4, 2, 1 as keep a product of `tiles` tiles within one
+// wave, and no more than its K stages.  A term (product and slicing pass) in us before and now, the
+// shorter epilogue included: N = 64 56 -> 32 and 200 94 -> 48 and 414 121 -> 58 (clusters of four), 777
+// 175 -> 139, 1536 546 -> 464 and 2600 2287 -> 2028 (no clusters: more tiles than half the SMs; a
+// second wave of half tiles would cost what it saves).
+int oz_cluster(int tiles, int nk) {
+  const int sms = fq_sm_count();
+  return tiles * 4 <= sms && nk >= 4 ? 4 : (tiles * 2 <= sms && nk >= 2 ? 2 : 1);
+}
+
+// Launch configuration of `tiles` tiles of `csize` CTAs.
+struct OzLaunch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  OzLaunch(int tiles, int csize, size_t smem, cudaStream_t s) {
+    cfg.gridDim = dim3((unsigned)(tiles * csize));
+    cfg.blockDim = dim3(OZ_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)csize;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = csize > 1 ? 1 : 0;
+  }
+};
 
 
 }  // namespace

@@ -119,9 +119,16 @@ fq_status oz_gemm(const OzGradWs& w, const __nv_bfloat16* left, size_t lstride, 
                                          (int)OZR_SMEM);
     if (r != cudaSuccess) return fq_cuda_fail(r, "FP64-emulation gradient kernel shared-memory attribute");
   }
-  const int tiles_i = w.np / OZ_BN, tiles_j = rows / OZR_BM;
-  k_oz_real_term<EPI><<<tiles_i * tiles_j, OZ_THREADS, OZR_SMEM, s>>>(maps, w.np / OZ_BKE, tiles_j, tiles_i, w.np, e);
-  return FQ_OK;
+  // values of k (and, but for the dot's stacked blocks with their partial per tile, rows and columns)
+  // beyond N are zero and left out
+  const bool dot = EPI == OZ_DOT;
+  const int tiles_i = dot ? w.np / OZ_BN : (e.n + OZ_BN - 1) / OZ_BN;
+  const int tiles_j = dot ? rows / OZR_BM : (e.n + OZR_BM - 1) / OZR_BM;
+  const int nk = (e.n + OZ_BKE - 1) / OZ_BKE;
+  const int csize = dot ? 1 : oz_cluster(tiles_i * tiles_j, nk);
+  OzLaunch launch(tiles_i * tiles_j, csize, OZR_SMEM, s);
+  cudaError_t le = cudaLaunchKernelEx(&launch.cfg, k_oz_real_term<EPI>, maps, nk, tiles_j, tiles_i, w.np, csize, e);
+  return le == cudaSuccess ? FQ_OK : fq_cuda_fail(le, "FP64-emulation gradient product");
 }
 
 struct Runner {

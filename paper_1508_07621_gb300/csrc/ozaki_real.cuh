@@ -11,8 +11,9 @@
 //
 // Warp 0 streams TMA stages (K = 16 per stage: the two 64-row halves of each left slice and the
 // 64 rows of each right slice), warp 1 issues the MMAs, warps 2-17 drain (four per lane quarter,
-// 16 columns each) and finally run the FP64 epilogue on 8 columns of one state each.  Every wait
-// is bounded as in the other tensor-core kernels.
+// 16 columns each) and finally run the FP64 epilogue.  Clusters split K where tiles are few, and the
+// epilogue is kept short, as in ozaki_core.cuh.  Every wait is bounded as in the other tensor-core
+// kernels.
 #pragma once
 
 #include "ozaki_core.cuh"
@@ -26,14 +27,13 @@ constexpr int OZR_STAGE_BYTES = OZ_S * (OZR_A_BYTES + OZR_B_BYTES);
 constexpr int OZR_STAGES = 4;
 constexpr int OZR_KB_PER_DRAIN = 16;              // 256 values of k per chunk
 constexpr int OZR_BUF_COLS = 4 * OZ_BN;           // four groups of 64 columns
-constexpr int OZR_XS_LD = 129;                    // staged sums: [col][row], padded against bank conflicts
-constexpr int OZR_XS_BYTES = 2 * OZR_XS_LD * OZ_BN * 4;  // hi, then lo
+constexpr int OZR_XS_BYTES = 2 * OZ_XS_PLANE * 4;  // staged sums: hi, then lo
 constexpr size_t OZR_SMEM = (size_t)OZR_STAGES * OZR_STAGE_BYTES + 1024 + 256;
 static_assert((size_t)OZR_STAGES * OZR_STAGE_BYTES >= OZR_XS_BYTES + 16 * sizeof(double2), "epilogue staging");
 
 template <int EPI>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    k_oz_real_term(const __grid_constant__ OzMaps maps, int nk, int tiles_j, int tiles_i, int np, OzEpi e) {
+    k_oz_real_term(const __grid_constant__ OzMaps maps, int nk, int tiles_j, int tiles_i, int np, int csize, OzEpi e) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -46,11 +46,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   const uint32_t tfull0 = smem_u32(bars + 2 * OZR_STAGES), tempty0 = smem_u32(bars + 2 * OZR_STAGES + 2);
   const uint32_t done = smem_u32(bars + 2 * OZR_STAGES + 4);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nchunks = (nk + OZR_KB_PER_DRAIN - 1) / OZR_KB_PER_DRAIN;
+  const int rank = blockIdx.x % csize;
+  const int kb0 = nk * rank / csize, nkr = nk * (rank + 1) / csize - kb0;  // this CTA's K stages
+  const int nchunks = (nkr + OZR_KB_PER_DRAIN - 1) / OZR_KB_PER_DRAIN;
 
   int tj, ti;
   {
-    const int b = blockIdx.x, per = RASTER_GROUP * tiles_i, g = b / per;
+    const int b = blockIdx.x / csize, per = RASTER_GROUP * tiles_i, g = b / per;
     const int gj = min(RASTER_GROUP, tiles_j - g * RASTER_GROUP), r = b - g * per;
     tj = g * RASTER_GROUP + r % gj;
     ti = r / gj;
@@ -85,7 +87,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     if (lane == 0) {  // ---------------- TMA producer
       int issued = 0;
       bool ok = true;
-      for (int kb = 0; kb < nk && ok; ++kb) {
+      for (int kb = 0; kb < nkr && ok; ++kb) {
         const int s = kb % OZR_STAGES;
         if (kb >= OZR_STAGES && !(ok = mbar_wait(empty0 + 8 * s, ((kb / OZR_STAGES) - 1) & 1))) break;
         if (*(volatile int*)abort_flag) {
@@ -95,7 +97,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const uint32_t st = base + s * OZR_STAGE_BYTES;
         const uint32_t bar = full0 + 8 * s;
         mbar_expect_tx(bar, OZR_STAGE_BYTES);
-        const int kx = kb * OZ_BKE;
+        const int kx = (kb0 + kb) * OZ_BKE;
 #pragma unroll
         for (int q = 0; q < OZ_S; ++q) {
           tma_load_2d(st + q * OZR_A_BYTES, &maps.a[q], bar, kx, j0);                                // Re rows
@@ -122,7 +124,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         if (c >= 2 && !(ok = mbar_wait(tempty0 + 8 * b, ((c >> 1) - 1) & 1))) break;
         tc_fence_after();
         const uint32_t accb = tmem + (uint32_t)(b * OZR_BUF_COLS);
-        for (int kq = 0; kq < OZR_KB_PER_DRAIN && kb < nk; ++kq, ++kb) {
+        for (int kq = 0; kq < OZR_KB_PER_DRAIN && kb < nkr; ++kq, ++kb) {
           const int s = kb % OZR_STAGES;
           ok = mbar_wait(full0 + 8 * s, (kb / OZR_STAGES) & 1);
           if (!ok || *(volatile int*)abort_flag) {
@@ -192,81 +194,102 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     }
     // stage the sums column-major (xs[col][row], hi then lo) in the idle stages: the last MMAs
     // have completed, and every stage's copies have landed
-    float* xs = reinterpret_cast<float*>(gbase);
-    constexpr int LO = OZR_XS_LD * OZ_BN;
+    if (ok) {
+      float* xw = reinterpret_cast<float*>(gbase) + part * 16 * OZ_XS_LD + row;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int c0 = part * 16 + 2 * q;
-      xs[c0 * OZR_XS_LD + row] = h[q].x;
-      xs[(c0 + 1) * OZR_XS_LD + row] = h[q].y;
-      xs[LO + c0 * OZR_XS_LD + row] = l[q].x;
-      xs[LO + (c0 + 1) * OZR_XS_LD + row] = l[q].y;
+      for (int q = 0; q < 16; ++q) {
+        xw[q * OZ_XS_LD] = q & 1 ? h[q >> 1].y : h[q >> 1].x;
+        xw[q * OZ_XS_LD + OZ_XS_PLANE] = q & 1 ? l[q >> 1].y : l[q >> 1].x;
+      }
     }
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * OZ_EPI_WARPS) : "memory");  // the drain warps only
-    // ---------------- FP64 epilogue: thread t -> state t / 8, columns 8 (t % 8) .. + 7
-    const int t = threadIdx.x - 64, srow = t >> 3, cb = (t & 7) * 8;
-    const int j = j0 + srow;
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (csize > 1) oz_cluster_sync();
+  if (warp >= 2) {
+    // ---------------- FP64 epilogue: this CTA's share of the columns, consecutive threads on
+    // consecutive columns of a state
+    const bool ok = !*(volatile int*)abort_flag;
+    const float* xs = reinterpret_cast<const float*>(gbase);
+    const int wd = OZ_BN / csize, t = threadIdx.x - 64;
+    const int cc = rank * wd + t % wd, i = i0 + cc;
     double dsr = 0.0, dsi = 0.0;
     bool bad = false;
-    if (ok && j < e.nc) {
+    if (ok && i < e.n) {
       const fq_term& tt = e.t;
-      const int ej = e.es[j];
-#pragma unroll 1
-      for (int q = 0; q < 8; ++q) {
-        const int cc = cb + q, i = i0 + cc;
-        if (i >= e.n) break;
-        const int ex = ej + e.et[i];
-        const double sc = pow2(ex < -1022 ? -1022 : ex);
-        const double yr = ((double)xs[cc * OZR_XS_LD + srow] + (double)xs[LO + cc * OZR_XS_LD + srow]) * sc;
-        const double yi =
-            ((double)xs[cc * OZR_XS_LD + 64 + srow] + (double)xs[LO + cc * OZR_XS_LD + 64 + srow]) * sc;
-        const size_t idx = (size_t)j * e.n + i;
-        if (EPI == OZ_DOT) {  // conj(b) Y
-          const double br = e.cur_re[idx], bi = e.cur_im[idx];
-          dsr = fma(br, yr, fma(bi, yi, dsr));
-          dsi = fma(br, yi, fma(-bi, yr, dsi));
-        } else if (EPI == OZ_ADJ) {  // out = cpa g + i cw Y + b2
-          const double gr = e.cur_re[idx], gi = e.cur_im[idx];
-          double orr = e.cpa_re * gr - e.cpa_im * gi - e.cw * yi;
-          double oi = e.cpa_re * gi + e.cpa_im * gr + e.cw * yr;
-          if (e.prev_re) {
-            orr += e.prev_re[idx];
-            oi += e.prev_im[idx];
-          }
-          bad |= !(orr * orr + oi * oi <= tt.bound2);
-          e.out_re[idx] = orr;
-          e.out_im[idx] = oi;
-        } else {  // Chebyshev term (as in the plain FP64 path)
-          double pr, pi;
-          if (tt.first) {
-            pr = yi;
-            pi = -yr;
-          } else {
-            pr = fma(2.0, yi, e.prev_re[idx]);
-            pi = fma(-2.0, yr, e.prev_im[idx]);
-          }
-          bad |= !(pr * pr + pi * pi <= tt.bound2);
-          double ar, ai;
-          if (tt.first) {
-            ar = fma(tt.coef, pr, tt.coef0 * e.cur_re[idx]);
-            ai = fma(tt.coef, pi, tt.coef0 * e.cur_im[idx]);
-          } else {
-            ar = fma(tt.coef, pr, e.acc_re[idx]);
-            ai = fma(tt.coef, pi, e.acc_im[idx]);
-          }
-          if (tt.last) {
-            e.out_re[idx] = tt.ph_re * ar - tt.ph_im * ai;
-            e.out_im[idx] = tt.ph_re * ai + tt.ph_im * ar;
-          } else {
-            e.out_re[idx] = pr;
-            e.out_im[idx] = pi;
-            e.acc_re[idx] = ar;
-            e.acc_im[idx] = ai;
+      const int ei = e.et[i];
+      const bool first = EPI == OZ_FWD && tt.first;
+      const double* src_re = EPI == OZ_FWD && !first ? e.prev_re : e.cur_re;
+      const double* src_im = EPI == OZ_FWD && !first ? e.prev_im : e.cur_im;
+      const double* add_re = EPI == OZ_ADJ ? e.prev_re : e.acc_re;  // ADJ: b2 (may be absent); FWD: acc
+      const double* add_im = EPI == OZ_ADJ ? e.prev_im : e.acc_im;
+      const bool add = EPI != OZ_DOT && !first && add_re;
+      const int step = 32 * OZ_EPI_WARPS / wd;
+      for (int row0 = t / wd; row0 < OZR_BM && j0 + row0 < e.nc; row0 += OZ_EPI_ROWS * step) {
+        double xr[OZ_EPI_ROWS], xi[OZ_EPI_ROWS], zr[OZ_EPI_ROWS], zi[OZ_EPI_ROWS];
+        int ej[OZ_EPI_ROWS];
+#pragma unroll
+        for (int u = 0; u < OZ_EPI_ROWS; ++u) {
+          const int srow = row0 + u * step, j = j0 + srow;
+          const bool in = srow < OZR_BM && j < e.nc;
+          const size_t idx = (size_t)j * e.n + i;
+          xr[u] = in ? src_re[idx] : 0.0;
+          xi[u] = in ? src_im[idx] : 0.0;
+          zr[u] = in && add ? add_re[idx] : 0.0;
+          zi[u] = in && add ? add_im[idx] : 0.0;
+          ej[u] = in ? e.es[j] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < OZ_EPI_ROWS; ++u) {
+          const int srow = row0 + u * step, j = j0 + srow;
+          if (srow >= OZR_BM || j >= e.nc) break;
+          const int ex = ej[u] + ei, at = cc * OZ_XS_LD + srow;
+          const size_t idx = (size_t)j * e.n + i;
+          float h0, l0, h1, l1;
+          oz_fold(xs, at, OZ_XS_PLANE, csize, h0, l0);
+          oz_fold(xs, at + OZR_BM, OZ_XS_PLANE, csize, h1, l1);
+          const double yr = oz_value(h0, l0, ex), yi = oz_value(h1, l1, ex);
+          if (EPI == OZ_DOT) {  // conj(b) Y
+            dsr = fma(xr[u], yr, fma(xi[u], yi, dsr));
+            dsi = fma(xr[u], yi, fma(-xi[u], yr, dsi));
+          } else if (EPI == OZ_ADJ) {  // out = cpa g + i cw Y + b2
+            double orr = e.cpa_re * xr[u] - e.cpa_im * xi[u] - e.cw * yi;
+            double oi = e.cpa_re * xi[u] + e.cpa_im * xr[u] + e.cw * yr;
+            if (add) {
+              orr += zr[u];
+              oi += zi[u];
+            }
+            bad |= oz_outside(orr, oi, tt.bound2);
+            e.out_re[idx] = orr;
+            e.out_im[idx] = oi;
+          } else {  // Chebyshev term (as in the plain FP64 path)
+            double pr, pi, ar, ai;
+            if (first) {
+              pr = yi;
+              pi = -yr;
+              ar = fma(tt.coef, pr, tt.coef0 * xr[u]);
+              ai = fma(tt.coef, pi, tt.coef0 * xi[u]);
+            } else {
+              pr = fma(2.0, yi, xr[u]);
+              pi = fma(-2.0, yr, xi[u]);
+              ar = fma(tt.coef, pr, zr[u]);
+              ai = fma(tt.coef, pi, zi[u]);
+            }
+            bad |= oz_outside(pr, pi, tt.bound2);
+            if (tt.last) {
+              e.out_re[idx] = tt.ph_re * ar - tt.ph_im * ai;
+              e.out_im[idx] = tt.ph_re * ai + tt.ph_im * ar;
+            } else {
+              e.out_re[idx] = pr;
+              e.out_im[idx] = pi;
+              e.acc_re[idx] = ar;
+              e.acc_im[idx] = ai;
+            }
           }
         }
       }
-      if (bad) atomicOr(tt.status, FQ_BIT_BOUND);
     }
+    if (bad) atomicOr(e.t.status, FQ_BIT_BOUND);
     if (EPI == OZ_DOT) {  // per-CTA partial in a fixed order (bit-reproducible)
       double2* red = reinterpret_cast<double2*>(gbase + OZR_XS_BYTES);
 #pragma unroll
@@ -286,12 +309,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       }
     }
   }
-  tc_fence_before();
-  __syncthreads();
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OZ_TMEM_COLS) : "memory");
   }
+  if (csize > 1) oz_cluster_sync();  // no CTA leaves while a peer may still read its sums
 }
 
 }  // namespace

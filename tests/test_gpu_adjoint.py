@@ -180,7 +180,8 @@ def test_fidelity_loss_autograd(fq):
 
 
 # ------------------------------------------------------------------ FP64 emulation (FQ_OZAKI)
-@pytest.mark.parametrize("n,M,stride", [(12, 20, 6), (33, 7, 1), (200, 12, 5), (130, 9, 16)])
+@pytest.mark.parametrize("n,M,stride", [(12, 20, 6), (33, 7, 1), (200, 12, 5), (130, 9, 16), (400, 4, 2), (530, 3, 3),
+                                        (600, 2, 1)])
 def test_ozaki_grad_matches_oracle(fq, n, M, stride):
     """Gradient with every product in FP64 emulation on the tensor cores against the FP64 oracle,
     held to the FP64 criterion (1e-9 of max |g|, loss to 1e-11): ragged tiles, ragged checkpoint

@@ -63,6 +63,39 @@ def test_ozaki_ragged_propagate(fq, n, nc):
     assert err <= TOL
 
 
+@pytest.mark.parametrize("n,nc", [(1, 1), (5, 5), (16, 3), (17, 17), (49, 49), (64, 64), (65, 65), (127, 127),
+                                  (130, 129), (513, 40), (576, 130), (640, 9), (705, 2), (770, 131)])
+def test_ozaki_shared_tiles(fq, n, nc):
+    """Tiles shared by clusters of four (N up to 576 on 152 SMs), two (640, 705) and one CTA (770);
+    values of k that end inside a 16-wide stage or a 128-wide chunk; column tiles and state tiles with a
+    single column or state."""
+    M = 3
+    h0, h1 = fi.goe(n, 1411), fi.goe(n, 1412)
+    drv = fi.Drive(0.2, 1.3, 1.1, 0.6)
+    x0 = fi.ginibre(max(n, nc), 1413)[:nc, :n]
+    x0 = x0 / np.linalg.norm(x0, axis=1, keepdims=True)
+    plan = fq.Plan.dense(h0, h1, omega=drv.omega, f_ac=drv.f_ac, f_dc=drv.f_dc, phi0=drv.phi0, steps=200,
+                         precision=fq.FQ_OZAKI)
+    X = plan.propagate(cuda_c128(x0), 1, 1 + M).cpu().numpy()
+    assert plan.check_status() == fq.FQ_OK
+    ref = o.propagate_dense(h0, h1, o.plan_for_drive_dense(h0, h1, drv, 200), x0.T, 1, 1 + M).T
+    assert np.max(np.abs(X - ref)) <= 1e-12  # a few 2^-44 over three steps of at most a dozen products
+
+
+def test_ozaki_scales_beyond_the_integer_widening(fq):
+    """States scaled by 2^-850: the epilogue's exponents leave the range of its integer widening.  The
+    chain is linear, and nothing here underflows, so the result is the unscaled one times 2^-850."""
+    n, s = 60, 2.0 ** -850
+    h0, h1 = fi.goe(n, 1421), fi.goe(n, 1422)
+    x0 = fi.ginibre(n, 1423)[:7]
+    x0 /= np.linalg.norm(x0, axis=1, keepdims=True)
+    plan = fq.Plan.dense(h0, h1, omega=1.1, f_ac=1.3, steps=24, precision=fq.FQ_OZAKI)
+    a = plan.propagate(cuda_c128(x0), 0, 4).cpu().numpy()
+    b = plan.propagate(cuda_c128(x0 * s), 0, 4).cpu().numpy()
+    assert plan.check_status() == fq.FQ_OK
+    assert np.max(np.abs(b / s - a)) <= 1e-15
+
+
 def test_ozaki_magnus6(fq):
     n, M = 40, 16
     h0, h1 = fi.goe(n, 1501), fi.goe(n, 1502)
