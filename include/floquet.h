@@ -142,7 +142,7 @@ typedef struct fq_problem {
                                dense FP64); ignored by the split precisions */
   int32_t tile_n;           /* split path: tensor-core output tile width 64 or 128; 0 = by N (64 where
                                the 128-wide tiles of a product would leave SMs idle, else 128)
-                               until floquet_autotune picks one; in a persistent scan 0 counts as 128 */
+                               until floquet_autotune picks one */
   int32_t magnus_order;     /* 4 (default, also 0) or 6: Eq. 14 in full with its alphas taken as
                                3-point Gauss-Legendre moments (nine commutators of H0, H1 computed
                                once: on the device for FQ_DENSE, on the host as bands for

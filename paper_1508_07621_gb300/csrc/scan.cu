@@ -537,12 +537,13 @@ size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 int scan_ns(const fq_plan* p) { return p->precision == FQ_BF16X6 ? 3 : 2; }
 
-// Tile width of the scan: the one the plans' (autotuned) widths favour, weighted by their work.
+// Tile width of the scan: the one the plans' widths (their own or fq_split_shape's) favour, weighted
+// by their work.
 int scan_bn(fq_plan* const* plans, int count) {
   double w128 = 0, w64 = 0;
   for (int i = 0; i < count; ++i) {
     const double c = (double)plans[i]->n * plans[i]->n * plans[i]->n * plans[i]->steps * plans[i]->L;
-    (plans[i]->tile_n == 128 ? w128 : w64) += c;
+    (fq_split_shape(plans[i]).n == 128 ? w128 : w64) += c;
   }
   return w128 >= w64 ? 128 : 64;
 }
