@@ -1,13 +1,16 @@
-// Tiled tridiagonal chain (FP64 or FP32): one launch per step; each CTA carries one segment of one
-// state through all L products of the step on chip and writes it back, so HBM sees the state
-// once per step instead of five times per product.
+// Tiled tridiagonal chain (FP64 or FP32): each CTA carries one segment of one state through all L
+// products of a step on chip and writes it back, so HBM sees the state once per step instead of five
+// times per product.  Where one CTA holds a whole state, one launch runs every step and the state
+// stays on chip throughout; otherwise there is one launch per step.
 //
 // The step works in the real gauge frame of Omega~_m (gauge.cuh): X_m = D_m P(Omega'_m) D_m^+
 // X_{m-1} with P(x) = e^{-i beta h} sum_k c_k T_k(x), c_k = (-i)^k a_k (Eqs. 10 and 12), applied by
-// Clenshaw's backward recurrence.  A CTA holds NT * EPT consecutive rows: its segment of
-// seg = NT * EPT - 2L rows plus L halo rows on each side.  Every product can be wrong only one
-// row further in from the tile's edge (the rows beyond it are taken as zero), so after the L
-// products of a step the segment's rows are exact; only those are written.
+// Clenshaw's backward recurrence.  A CTA holds (threads x EPT) consecutive rows: its segment of seg
+// rows plus L halo rows on each side where the state goes on.  Every product can be wrong only one
+// row further in from such an edge (the rows beyond it are taken as zero), so after the L products
+// of a step the segment's rows are exact; only those are written.  An exact row takes the same
+// operations on the same numbers in every segmentation, so the split never changes a result's bits.
+// pick_tile chooses segments, threads and rows per thread for the state length and count.
 //
 // FQ_DF32 runs the same step in double-float arithmetic: every value is an unevaluated sum
 // hi + lo of two FP32 numbers (Dekker's splitting, Knuth's two-sum, and two-product by FMA), so
@@ -21,29 +24,89 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <cmath>
+
 #include "dfl.cuh"
 #include "gauge.cuh"
 #include "internal.h"
 
 namespace {
 
-constexpr int TILE_NT = 256;
-constexpr int TILE_EPT = 8;
-constexpr int TILE_ROWS = TILE_NT * TILE_EPT;
+constexpr int TILE_NT = 256;  // most threads of a CTA
+constexpr int TILE_NW = TILE_NT / 32;
 constexpr int TILE_MAXL = 128;
+
+// Rows base .. a CTA holds and the rows [first, last) of them it writes, for segment blockIdx.x.
+struct TileRows {
+  int first, last, base;
+  __device__ TileRows(int seg, int L, int n) {
+    first = blockIdx.x * seg;
+    last = min(first + seg, n);
+    base = max(0, first - L);
+  }
+};
+
+// FP64: rows of a CTA below which a product's time no longer falls, where the FP64 pipe's time for
+// that many rows (2 multiply-adds a cycle and SM) equals the latency of a product.
+constexpr int F64_FLOOR_ROWS = 128;
+
+// Segments per state, threads per CTA and rows per thread.
+struct TileShape {
+  int segs, seg, nt, ept;
+};
+
+// The shape for states of n rows, nc of them.  The arithmetic of a step is the rows the CTAs hold, halo
+// and padding included, so a CTA gets no more threads than its rows need, and as few segments as fit
+// (one segment has no halo and runs all steps in one launch).  FP64 (floor_rows > 0) is bound by its
+// pipe from 128 rows on, so there an SM's time is (CTAs on the fullest SM) x (rows of a CTA), and more
+// segments are taken where few states would leave SMs idle; the FP32 pipes need two dozen warps before
+// that pays.  Rows per thread: the smallest of `epts` that holds the rows with TILE_NT threads (many
+// warps of few rows hide latency best).
+// A step in us before (2048 rows a CTA in FP64 and FP32, 1024 in double-float, always) and now, states
+// x rows: FP64 36 x 36 43 -> 7, 24 x 501 66 -> 14, 501 x 501 245 -> 62, 24 x 3001 116 -> 49, 160 x 10001
+// 1317 -> 1141; double-float 36 x 36 16 -> 4.8, 501 x 501 48 -> 31, 1501 x 1501 253 -> 212; FP32 501 x 501
+// 19 -> 6.5.
+template <int NE>
+TileShape pick_tile(int n, int nc, int L, const int (&epts)[NE], int floor_rows) {
+  const int sms = fq_sm_count(), cap = TILE_NT * epts[NE - 1];
+  TileShape best{};
+  double cost = 0.0;
+  for (int segs = 1; segs <= n; ++segs) {
+    const int seg = (n + segs - 1) / segs;
+    const int halo = segs == 1 ? 0 : (segs == 2 ? L : 2 * L);
+    const int need = segs == 1 ? n : std::min(n, seg + halo);
+    if (need > cap) continue;
+    int ept = epts[NE - 1];
+    if (segs == 1 || floor_rows > 0)
+      for (int q = NE - 1; q >= 0; --q)
+        if (need <= TILE_NT * epts[q]) ept = epts[q];
+    const int nt = 32 * ((need + 32 * ept - 1) / (32 * ept));
+    const int real = (n + seg - 1) / seg;  // segments that hold rows
+    const double waves = std::ceil((double)nc * real / sms);
+    const double c = std::max(waves * nt * ept, (double)floor_rows);
+    if (best.segs == 0 || c < 0.999 * cost) {
+      best = TileShape{real, seg, nt, ept};
+      cost = c;
+    }
+    if (floor_rows == 0) break;
+    if ((double)nc * real >= 4.0 * sms || seg <= 2 * L) break;  // more segments only add halo from here
+  }
+  return best;
+}
 
 template <typename T>
 struct TileCoef {
   T c[TILE_MAXL + 1];  // |c_k|: c_k = c[k] for even k (real, sign included), i c[k] for odd k
 };
 
-template <typename T>
+template <typename T, int TILE_EPT>
 struct Tile {
   using T2 = typename V2<T>::t;
-  static constexpr int NW = TILE_NT / 32;
+  static constexpr int NW = TILE_NW;
   T2* slot_last;   // [2][NW]
   T2* slot_first;  // [2][NW]
-  int lane, warp;
+  int lane, warp, warps;
 
   // rows i0 - 1 and i0 + EPT of x (neighbouring threads; zero beyond the tile)
   __device__ __forceinline__ void halo(const T2 (&x)[TILE_EPT], int par, T2& left, T2& right) {
@@ -60,7 +123,7 @@ struct Tile {
       li = w.y;
     }
     if (lane == 31) {
-      const T2 w = warp < NW - 1 ? slot_first[par * NW + warp + 1] : T2{0, 0};
+      const T2 w = warp < warps - 1 ? slot_first[par * NW + warp + 1] : T2{0, 0};
       rr = w.x;
       ri = w.y;
     }
@@ -97,100 +160,108 @@ struct Tile {
   }
 };
 
-template <typename T>
+// `steps` steps of the chain (more than one only with a single segment per state).
+template <typename T, int TILE_EPT>
 __global__ void __launch_bounds__(TILE_NT)
 k_tri_tile(const typename V2<T>::t* __restrict__ cf, const typename V2<T>::t* __restrict__ rot,
            const T* __restrict__ xr, const T* __restrict__ xi, T* __restrict__ yr, T* __restrict__ yi, int n, int ld,
-           int L, int seg, TileCoef<T> coef, T ph_re, T ph_im, T bound2, unsigned int* status) {
+           int L, int seg, int steps, TileCoef<T> coef, T ph_re, T ph_im, T bound2, unsigned int* status) {
   using T2 = typename V2<T>::t;
-  __shared__ T2 slots[4 * Tile<T>::NW];
-  Tile<T> tl;
+  using Tl = Tile<T, TILE_EPT>;
+  __shared__ T2 slots[4 * Tl::NW];
+  Tl tl;
   tl.slot_last = slots;
-  tl.slot_first = slots + 2 * Tile<T>::NW;
+  tl.slot_first = slots + 2 * Tl::NW;
   tl.lane = threadIdx.x & 31;
   tl.warp = threadIdx.x >> 5;
+  tl.warps = blockDim.x >> 5;
   const size_t j = blockIdx.y;
-  const int first = blockIdx.x * seg;   // first row this CTA writes
-  const int i0 = first - L + (int)threadIdx.x * TILE_EPT;
+  const TileRows rows(seg, L, n);
+  const int i0 = rows.base + (int)threadIdx.x * TILE_EPT;
   T2 v[TILE_EPT], A[TILE_EPT], B[TILE_EPT];
   T d[TILE_EPT], e[TILE_EPT];
 #pragma unroll
   for (int q = 0; q < TILE_EPT; ++q) {
     const int i = i0 + q;
-    if (i >= 0 && i < n) {
-      const T x_r = xr[j * ld + i], x_i = xi[j * ld + i];
-      const T2 r = rot[i], c = cf[i];
-      v[q] = T2{r.x * x_r + r.y * x_i, r.x * x_i - r.y * x_r};  // D^+ x
+    A[q] = i < n ? T2{xr[j * ld + i], xi[j * ld + i]} : T2{0, 0};
+  }
+  bool bad = false;
+  int par = 0;
+  const T cL = coef.c[L];
+  for (int m = 0; m < steps; ++m, cf += ld, rot += ld) {
+#pragma unroll
+    for (int q = 0; q < TILE_EPT; ++q) {
+      const int i = i0 + q;
+      const T2 r = i < n ? rot[i] : T2{0, 0}, c = i < n ? cf[i] : T2{0, 0};
+      v[q] = T2{fma(r.x, A[q].x, r.y * A[q].y), fma(r.x, A[q].y, -(r.y * A[q].x))};  // D^+ x
       d[q] = c.x;
       e[q] = c.y;
-    } else {
-      v[q] = T2{0, 0};
-      d[q] = 0;
-      e[q] = 0;
+    }
+    // e' of the row before this thread's first row (constant over the step)
+    T el0 = __shfl_up_sync(0xffffffffu, e[TILE_EPT - 1], 1);
+    if (tl.lane == 0) el0 = i0 > 0 && i0 - 1 < n ? cf[i0 - 1].y : (T)0;
+    // b_L = c_L v, b_{L+1} = 0
+#pragma unroll
+    for (int q = 0; q < TILE_EPT; ++q) {
+      A[q] = (L & 1) ? T2{-cL * v[q].y, cL * v[q].x} : T2{cL * v[q].x, cL * v[q].y};
+      B[q] = T2{0, 0};
+    }
+    int k = L - 1;
+    // b_k = c_k v + 2 Omega' b_{k+1} - b_{k+2}; two per iteration so the array roles stay static
+    while (k >= 2) {
+      if (k & 1) tl.template apply<true, false>(A, B, v, d, e, el0, coef.c[k], par);
+      else tl.template apply<false, false>(A, B, v, d, e, el0, coef.c[k], par);
+      par ^= 1;
+      --k;
+      if (k & 1) tl.template apply<true, false>(B, A, v, d, e, el0, coef.c[k], par);
+      else tl.template apply<false, false>(B, A, v, d, e, el0, coef.c[k], par);
+      par ^= 1;
+      --k;
+    }
+    if (k == 1) {  // b_1 into B, then sum = c_0 v + Omega' b_1 - b_2 into A
+      tl.template apply<true, false>(A, B, v, d, e, el0, coef.c[1], par);
+      par ^= 1;
+      tl.template apply<false, true>(B, A, v, d, e, el0, coef.c[0], par);
+    } else {  // b_1 in A, b_2 in B: sum into B, then moved to A
+      tl.template apply<false, true>(A, B, v, d, e, el0, coef.c[0], par);
+#pragma unroll
+      for (int q = 0; q < TILE_EPT; ++q) A[q] = B[q];
+    }
+    par ^= 1;
+    // X = D e^{-i beta h} sum on this CTA's own rows
+#pragma unroll
+    for (int q = 0; q < TILE_EPT; ++q) {
+      const int i = i0 + q;
+      if (i < rows.first || i >= rows.last) {
+        A[q] = T2{0, 0};
+        continue;
+      }
+      const T2 y = T2{fma(ph_re, A[q].x, -(ph_im * A[q].y)), fma(ph_re, A[q].y, ph_im * A[q].x)};
+      const T2 r = rot[i];
+      A[q] = T2{fma(r.x, y.x, -(r.y * y.y)), fma(r.x, y.y, r.y * y.x)};
+      bad |= !(A[q].x * A[q].x + A[q].y * A[q].y <= bound2);
     }
   }
-  // e' of the row before this thread's first row (constant over the step)
-  T el0 = __shfl_up_sync(0xffffffffu, e[TILE_EPT - 1], 1);
-  if (tl.lane == 0) {
-    el0 = 0;
-    if (i0 > 0 && i0 - 1 < n) el0 = cf[i0 - 1].y;
-  }
-  // b_L = c_L v, b_{L+1} = 0
-  const T cL = coef.c[L];
-#pragma unroll
-  for (int q = 0; q < TILE_EPT; ++q) {
-    A[q] = (L & 1) ? T2{-cL * v[q].y, cL * v[q].x} : T2{cL * v[q].x, cL * v[q].y};
-    B[q] = T2{0, 0};
-  }
-  int k = L - 1, par = 0;
-  // b_k = c_k v + 2 Omega' b_{k+1} - b_{k+2}; two per iteration so the array roles stay static
-  while (k >= 2) {
-    if (k & 1) tl.template apply<true, false>(A, B, v, d, e, el0, coef.c[k], par);
-    else tl.template apply<false, false>(A, B, v, d, e, el0, coef.c[k], par);
-    par ^= 1;
-    --k;
-    if (k & 1) tl.template apply<true, false>(B, A, v, d, e, el0, coef.c[k], par);
-    else tl.template apply<false, false>(B, A, v, d, e, el0, coef.c[k], par);
-    par ^= 1;
-    --k;
-  }
-  if (k == 1) {  // b_1 into B, then sum = c_0 v + Omega' b_1 - b_2 into A
-    tl.template apply<true, false>(A, B, v, d, e, el0, coef.c[1], par);
-    par ^= 1;
-    tl.template apply<false, true>(B, A, v, d, e, el0, coef.c[0], par);
-  } else {  // b_1 in A, b_2 in B: sum into B, then moved to A
-    tl.template apply<false, true>(A, B, v, d, e, el0, coef.c[0], par);
-#pragma unroll
-    for (int q = 0; q < TILE_EPT; ++q) A[q] = B[q];
-  }
-  // X = D e^{-i beta h} sum on this CTA's own rows
-  bool bad = false;
 #pragma unroll
   for (int q = 0; q < TILE_EPT; ++q) {
     const int i = i0 + q;
-    if (i >= first && i < first + seg && i < n) {
-      const T2 y = T2{ph_re * A[q].x - ph_im * A[q].y, ph_re * A[q].y + ph_im * A[q].x};
-      const T2 r = rot[i];
-      const T o_r = r.x * y.x - r.y * y.y, o_i = r.x * y.y + r.y * y.x;
-      bad |= !(o_r * o_r + o_i * o_i <= bound2);
-      yr[j * ld + i] = o_r;
-      yi[j * ld + i] = o_i;
+    if (i >= rows.first && i < rows.last) {
+      yr[j * ld + i] = A[q].x;
+      yi[j * ld + i] = A[q].y;
     }
   }
   if (bad) atomicOr(status, FQ_BIT_BOUND);
 }
 
 // ---------------------------------------------------------------------------- double-float
-// 4 rows a thread and an 80-register cap (a few spills) let three CTAs (24 warps) share an SM:
-// the double-float FMA chains are long, and latency, not the FP32 pipe, limits fewer warps.
-constexpr int DFL_NT = 256;
-constexpr int DFL_EPT = 4;
-constexpr int DFL_ROWS = DFL_NT * DFL_EPT;
+// At most 4 rows a thread and an 80-register cap (a few spills) let three CTAs (24 warps) share an
+// SM: the double-float FMA chains are long, and latency, not the FP32 pipe, limits fewer warps.
+template <int DFL_EPT>
 struct DflTile {
-  static constexpr int NW = DFL_NT / 32;
+  static constexpr int NW = TILE_NW;
   dflc* slot_last;   // [2][NW]
   dflc* slot_first;  // [2][NW]
-  int lane, warp;
+  int lane, warp, warps;
 
   __device__ __forceinline__ static dflc shfl(dflc a, bool up) {
     dflc r;
@@ -216,7 +287,7 @@ struct DflTile {
     __syncthreads();
     const dflc z = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     if (lane == 0) l = warp > 0 ? slot_last[par * NW + warp - 1] : z;
-    if (lane == 31) r = warp < NW - 1 ? slot_first[par * NW + warp + 1] : z;
+    if (lane == 31) r = warp < warps - 1 ? slot_first[par * NW + warp + 1] : z;
     left = l;
     right = r;
   }
@@ -247,88 +318,108 @@ struct DflCoef {
   dfl c[TILE_MAXL + 1];  // as TileCoef: c_k = c[k] (even k) or i c[k] (odd k)
 };
 
-// One step of the double-float tiled chain; states FP64 planar in HBM.
-__global__ void __launch_bounds__(DFL_NT, 3)
+// One step of the double-float tiled chain, or `steps` of them (MULTI: a single segment per state);
+// states FP64 planar in HBM, and FP64 between the steps of a launch.
+template <int DFL_EPT, bool MULTI>
+__global__ void __launch_bounds__(TILE_NT, 3)
 k_tri_tile_dfl(const dfl2* __restrict__ cf, const dfl2* __restrict__ rot, const double* __restrict__ xr,
                const double* __restrict__ xi, double* __restrict__ yr, double* __restrict__ yi, int n, int ld, int L,
-               int seg, DflCoef coef, double ph_re, double ph_im, double bound2, unsigned int* status) {
-  __shared__ dflc slots[4 * DflTile::NW];
-  DflTile tl;
+               int seg, int steps, DflCoef coef, double ph_re, double ph_im, double bound2, unsigned int* status) {
+  using Tl = DflTile<DFL_EPT>;
+  __shared__ dflc slots[4 * Tl::NW];
+  Tl tl;
   tl.slot_last = slots;
-  tl.slot_first = slots + 2 * DflTile::NW;
+  tl.slot_first = slots + 2 * Tl::NW;
   tl.lane = threadIdx.x & 31;
   tl.warp = threadIdx.x >> 5;
+  tl.warps = blockDim.x >> 5;
   const size_t j = blockIdx.y;
-  const int first = blockIdx.x * seg;
-  const int i0 = first - L + (int)threadIdx.x * DFL_EPT;
+  const TileRows rows(seg, L, n);
+  const int i0 = rows.base + (int)threadIdx.x * DFL_EPT;
   const dfl zero = {0.f, 0.f};
   const dflc zc = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  dflc v[DFL_EPT], A[DFL_EPT], B[DFL_EPT];
-  dfl d[DFL_EPT], e[DFL_EPT];
+  const dfl cL = coef.c[L];
+  double o_r[DFL_EPT], o_i[DFL_EPT];  // MULTI: the state between steps
+  if (MULTI) {
 #pragma unroll
-  for (int q = 0; q < DFL_EPT; ++q) {
-    const int i = i0 + q;
-    if (i >= 0 && i < n) {
-      const double x_r = xr[j * ld + i], x_i = xi[j * ld + i];
-      const dfl2 r = rot[i], c = cf[i];
-      const double rc = dfl_value(r.x), rs = dfl_value(r.y);
-      const dfl vr = dfl_of(rc * x_r + rs * x_i), vi = dfl_of(rc * x_i - rs * x_r);  // D^+ x in FP64
-      v[q] = {make_float2(vr.h, vi.h), make_float2(vr.l, vi.l)};
-      d[q] = c.x;
-      e[q] = c.y;
-    } else {
-      v[q] = zc;
-      d[q] = zero;
-      e[q] = zero;
+    for (int q = 0; q < DFL_EPT; ++q) {
+      const int i = i0 + q;
+      o_r[q] = i < n ? xr[j * ld + i] : 0.0;
+      o_i[q] = i < n ? xi[j * ld + i] : 0.0;
     }
   }
-  dfl el0;
-  el0.h = __shfl_up_sync(0xffffffffu, e[DFL_EPT - 1].h, 1);
-  el0.l = __shfl_up_sync(0xffffffffu, e[DFL_EPT - 1].l, 1);
-  if (tl.lane == 0) {
-    el0 = zero;
-    if (i0 > 0 && i0 - 1 < n) el0 = cf[i0 - 1].y;
-  }
-  // b_L = c_L v (L odd: i cL v)
-  const dfl cL = coef.c[L];
-#pragma unroll
-  for (int q = 0; q < DFL_EPT; ++q) {
-    A[q] = (L & 1) ? dflc_ifma(cL, v[q], zc) : dflc_fma(cL, v[q], zc);
-    B[q] = zc;
-  }
-  int k = L - 1, par = 0;
-  while (k >= 2) {
-    if (k & 1) tl.apply<true, false>(A, B, v, d, e, el0, coef.c[k], par);
-    else tl.apply<false, false>(A, B, v, d, e, el0, coef.c[k], par);
-    par ^= 1;
-    --k;
-    if (k & 1) tl.apply<true, false>(B, A, v, d, e, el0, coef.c[k], par);
-    else tl.apply<false, false>(B, A, v, d, e, el0, coef.c[k], par);
-    par ^= 1;
-    --k;
-  }
-  if (k == 1) {
-    tl.apply<true, false>(A, B, v, d, e, el0, coef.c[1], par);
-    par ^= 1;
-    tl.apply<false, true>(B, A, v, d, e, el0, coef.c[0], par);
-  } else {
-    tl.apply<false, true>(A, B, v, d, e, el0, coef.c[0], par);
-#pragma unroll
-    for (int q = 0; q < DFL_EPT; ++q) A[q] = B[q];
-  }
   bool bad = false;
+  int par = 0;
+  for (int m = 0; m < (MULTI ? steps : 1); ++m, cf += ld, rot += ld) {
+    dflc v[DFL_EPT], A[DFL_EPT], B[DFL_EPT];
+    dfl d[DFL_EPT], e[DFL_EPT];
 #pragma unroll
-  for (int q = 0; q < DFL_EPT; ++q) {
-    const int i = i0 + q;
-    if (i >= first && i < first + seg && i < n) {
+    for (int q = 0; q < DFL_EPT; ++q) {
+      const int i = i0 + q;
+      if (i < n) {
+        const dfl2 r = rot[i], c = cf[i];
+        const double rc = dfl_value(r.x), rs = dfl_value(r.y);
+        const double x_r = MULTI ? o_r[q] : xr[j * ld + i], x_i = MULTI ? o_i[q] : xi[j * ld + i];
+        const dfl vr = dfl_of(fma(rc, x_r, rs * x_i)), vi = dfl_of(fma(rc, x_i, -(rs * x_r)));  // D^+ x
+        v[q] = {make_float2(vr.h, vi.h), make_float2(vr.l, vi.l)};
+        d[q] = c.x;
+        e[q] = c.y;
+      } else {
+        v[q] = zc;
+        d[q] = zero;
+        e[q] = zero;
+      }
+    }
+    dfl el0;
+    el0.h = __shfl_up_sync(0xffffffffu, e[DFL_EPT - 1].h, 1);
+    el0.l = __shfl_up_sync(0xffffffffu, e[DFL_EPT - 1].l, 1);
+    if (tl.lane == 0) {
+      el0 = zero;
+      if (i0 > 0 && i0 - 1 < n) el0 = cf[i0 - 1].y;
+    }
+    // b_L = c_L v (L odd: i cL v)
+#pragma unroll
+    for (int q = 0; q < DFL_EPT; ++q) {
+      A[q] = (L & 1) ? dflc_ifma(cL, v[q], zc) : dflc_fma(cL, v[q], zc);
+      B[q] = zc;
+    }
+    int k = L - 1;
+    while (k >= 2) {
+      if (k & 1) tl.template apply<true, false>(A, B, v, d, e, el0, coef.c[k], par);
+      else tl.template apply<false, false>(A, B, v, d, e, el0, coef.c[k], par);
+      par ^= 1;
+      --k;
+      if (k & 1) tl.template apply<true, false>(B, A, v, d, e, el0, coef.c[k], par);
+      else tl.template apply<false, false>(B, A, v, d, e, el0, coef.c[k], par);
+      par ^= 1;
+      --k;
+    }
+    if (k == 1) {
+      tl.template apply<true, false>(A, B, v, d, e, el0, coef.c[1], par);
+      par ^= 1;
+      tl.template apply<false, true>(B, A, v, d, e, el0, coef.c[0], par);
+    } else {
+      tl.template apply<false, true>(A, B, v, d, e, el0, coef.c[0], par);
+#pragma unroll
+      for (int q = 0; q < DFL_EPT; ++q) A[q] = B[q];
+    }
+    par ^= 1;
+#pragma unroll
+    for (int q = 0; q < DFL_EPT; ++q) {
+      const int i = i0 + q;
+      if (MULTI) o_r[q] = o_i[q] = 0.0;
+      if (i < rows.first || i >= rows.last) continue;  // FP64 arithmetic on this CTA's own rows only
       const double sr = (double)A[q].h.x + (double)A[q].l.x, si = (double)A[q].h.y + (double)A[q].l.y;
-      const double y_r = ph_re * sr - ph_im * si, y_i = ph_re * si + ph_im * sr;
+      const double y_r = fma(ph_re, sr, -(ph_im * si)), y_i = fma(ph_re, si, ph_im * sr);
       const dfl2 r = rot[i];
       const double rc = dfl_value(r.x), rs = dfl_value(r.y);
-      const double o_r = rc * y_r - rs * y_i, o_i = rc * y_i + rs * y_r;
-      bad |= !(o_r * o_r + o_i * o_i <= bound2);
-      yr[j * ld + i] = o_r;
-      yi[j * ld + i] = o_i;
+      o_r[q] = fma(rc, y_r, -(rs * y_i));
+      o_i[q] = fma(rc, y_i, rs * y_r);
+      bad |= !(o_r[q] * o_r[q] + o_i[q] * o_i[q] <= bound2);
+      if (!MULTI || m == steps - 1) {
+        yr[j * ld + i] = o_r[q];
+        yi[j * ld + i] = o_i[q];
+      }
     }
   }
   if (bad) atomicOr(status, FQ_BIT_BOUND);
@@ -337,7 +428,6 @@ k_tri_tile_dfl(const dfl2* __restrict__ cf, const dfl2* __restrict__ rot, const 
 fq_status dfl_chain(fq_plan* p, const double* x0, double* x, int nc, int m_begin, int m_end, int identity,
                     int transpose_out, void* ws, cudaStream_t s) {
   const int n = p->n, ld = (n + 3) & ~3, nsteps = m_end - m_begin, L = p->L;
-  const int seg = DFL_ROWS - 2 * L;
   dfl2* cf = (dfl2*)ws;
   dfl2* rot = cf + (size_t)nsteps * ld;
   double* bufs = (double*)(rot + (size_t)nsteps * ld);
@@ -354,17 +444,31 @@ fq_status dfl_chain(fq_plan* p, const double* x0, double* x, int nc, int m_begin
     const float h = (float)c;
     coef.c[k] = {h, (float)(c - (double)h)};
   }
-  const int segs = (n + seg - 1) / seg;
+  const int epts[] = {1, 2, 4};
+  TileShape sh = pick_tile(n, nc, L, epts, 0);
+  // Three CTAs share an SM.  Where the CTAs are a wave and a part of one, segments as long as fit and a
+  // short last one (its FP64 rotations are few) fill the second wave better than equal ones: 160 x 3001
+  // 86 us a step against 95.
+  const double waves = (double)nc * sh.segs / (3.0 * fq_sm_count());
+  if (sh.segs > 1 && waves > 1.25 && waves < 2.0) {
+    sh.seg = 4 * TILE_NT - 2 * L;
+    sh.segs = (n + sh.seg - 1) / sh.seg;
+    sh.nt = TILE_NT;
+  }
+  const int per = sh.segs == 1 ? nsteps : 1;  // steps a launch
   int cur = 0;
-  for (int m = 0; m < nsteps; ++m) {
-    for (int r0 = 0; r0 < nc; r0 += 65535) {
+  for (int m = 0; m < nsteps; m += per) {
+    for (int r0 = 0; r0 < nc; r0 += 65535) {  // gridDim.y limit
       const int rows = nc - r0 < 65535 ? nc - r0 : 65535;
       const size_t o = (size_t)r0 * ld;
       fq_ktimer_start(p, s, "k_tri_tile_dfl");
-      k_tri_tile_dfl<<<dim3(segs, rows), DFL_NT, 0, s>>>(cf + (size_t)m * ld, rot + (size_t)m * ld, b[cur].re + o,
-                                                          b[cur].im + o, b[cur ^ 1].re + o, b[cur ^ 1].im + o, n, ld,
-                                                          L, seg, coef, p->phase_re, p->phase_im, 1.0 + 1e-9,
-                                                          p->d_status);
+      const auto kern = sh.segs > 1   ? k_tri_tile_dfl<4, false>
+                        : sh.ept == 1 ? k_tri_tile_dfl<1, true>
+                        : sh.ept == 2 ? k_tri_tile_dfl<2, true>
+                                      : k_tri_tile_dfl<4, true>;
+      kern<<<dim3(sh.segs, rows), sh.nt, 0, s>>>(cf + (size_t)m * ld, rot + (size_t)m * ld, b[cur].re + o,
+                                                 b[cur].im + o, b[cur ^ 1].re + o, b[cur ^ 1].im + o, n, ld, L, sh.seg,
+                                                 per, coef, p->phase_re, p->phase_im, 1.0 + 1e-9, p->d_status);
       fq_ktimer_stop(p, s);
     }
     cur ^= 1;
@@ -410,7 +514,6 @@ fq_status tile_chain(fq_plan* p, const double* x0, double* x, int nc, int m_begi
                      int transpose_out, void* ws, cudaStream_t s) {
   using T2 = typename V2<T>::t;
   const int n = p->n, ld = (n + 3) & ~3, nsteps = m_end - m_begin, L = p->L;
-  const int seg = TILE_ROWS - 2 * L;
   T2* cf = (T2*)ws;
   T2* rot = cf + (size_t)nsteps * ld;
   T* bufs = (T*)(rot + (size_t)nsteps * ld);
@@ -422,16 +525,18 @@ fq_status tile_chain(fq_plan* p, const double* x0, double* x, int nc, int m_begi
   else load_block(x0, b[0], nc, n, ld, s);
   const TileCoef<T> coef = tile_coef<T>(p);
   const T b2 = (T)(1.0 + (sizeof(T) == 8 ? 1e-9 : 2e-3));
-  const int segs = (n + seg - 1) / seg;
+  const int epts[] = {2, 4, 8};
+  const TileShape sh = pick_tile(n, nc, L, epts, sizeof(T) == 8 ? F64_FLOOR_ROWS : 0);
+  const int per = sh.segs == 1 ? nsteps : 1;  // steps a launch
   int cur = 0;
-  for (int m = 0; m < nsteps; ++m) {
+  for (int m = 0; m < nsteps; m += per) {
     for (int r0 = 0; r0 < nc; r0 += 65535) {  // gridDim.y limit
       const int rows = nc - r0 < 65535 ? nc - r0 : 65535;
       const size_t o = (size_t)r0 * ld;
-      k_tri_tile<T><<<dim3(segs, rows), TILE_NT, 0, s>>>(cf + (size_t)m * ld, rot + (size_t)m * ld,
-                                                         b[cur].re + o, b[cur].im + o, b[cur ^ 1].re + o,
-                                                         b[cur ^ 1].im + o, n, ld, L, seg, coef, (T)p->phase_re,
-                                                         (T)p->phase_im, b2, p->d_status);
+      const auto kern = sh.ept == 2 ? k_tri_tile<T, 2> : (sh.ept == 4 ? k_tri_tile<T, 4> : k_tri_tile<T, 8>);
+      kern<<<dim3(sh.segs, rows), sh.nt, 0, s>>>(cf + (size_t)m * ld, rot + (size_t)m * ld, b[cur].re + o,
+                                                 b[cur].im + o, b[cur ^ 1].re + o, b[cur ^ 1].im + o, n, ld, L, sh.seg,
+                                                 per, coef, (T)p->phase_re, (T)p->phase_im, b2, p->d_status);
     }
     cur ^= 1;
   }
@@ -443,7 +548,7 @@ fq_status tile_chain(fq_plan* p, const double* x0, double* x, int nc, int m_begi
 
 }  // namespace
 
-int fq_tile_supported(int L) { return L >= 1 && L <= TILE_MAXL && 2 * L < TILE_ROWS / 2; }
+int fq_tile_supported(int L) { return L >= 1 && L <= TILE_MAXL; }
 
 size_t fq_tile_workspace(const fq_plan* p, int nc, int nsteps) {
   const size_t ld = (p->n + 3) & ~3;

@@ -282,6 +282,42 @@ def test_paper_dimer_parameters(fq, precision, kernel):
     assert np.max(np.abs(X - ref)) <= tol
 
 
+def _drive_models(nb, steps=2000):
+    d = fi.config_dimer(nb=nb, steps=steps)
+    d.drive = fi.Drive(0.2, 1.5, 3.0, 0.4)
+    return d
+
+
+def _unit_states(n, count, seed):
+    x = np.exp(2j * np.pi * fi.uniform(seed, count * n).reshape(count, n)) * fi.uniform(seed + 1, count * n).reshape(count, n)
+    return x / np.linalg.norm(x, axis=1, keepdims=True)
+
+
+@pytest.mark.parametrize("precision", [0, 1, 4])
+@pytest.mark.parametrize("nb", [1, 30, 63, 64, 127, 128, 255, 256, 511, 512, 600, 1023, 1024, 1500, 2047, 2048, 3000])
+def test_tiled_shapes_agree(fq, precision, nb):
+    """Segments, threads and rows per thread follow the length and number of the states: one state, the
+    same state among 170 (at 3001 rows the double-float kernel's second wave), and step by step (one
+    launch runs every step where one CTA holds a state) give the same bits, at sizes around every rows-per-thread
+    limit, and the oracle's state."""
+    import torch
+    d = _drive_models(nb)
+    plan = dimer_plan(fq, d, precision, 3)
+    x0 = _unit_states(d.n, 170, 2301)
+    one = plan.propagate(cuda_c128(x0[:1]), 1, 4)
+    many = plan.propagate(cuda_c128(x0), 1, 4)
+    assert plan.check_status() == fq.FQ_OK
+    assert torch.equal(one[0], many[0])
+    step = cuda_c128(x0)
+    for m in range(1, 4):
+        step = plan.propagate(step, m, m + 1)
+    assert torch.equal(step, many)
+    refp = o.plan_for_drive_tridiag(d.h0_diag, d.h0_off, d.h1_diag, d.drive, d.steps)
+    ref = o.propagate_tridiag(d.h0_diag, d.h0_off, d.h1_diag, refp, x0[[0, 169]].T, 1, 4).T
+    tol = tol_f32(3, plan.info.L, plan.info.R) if precision == 1 else 1e-12
+    assert np.max(np.abs(to_np(many[[0, 169]]) - ref)) <= tol
+
+
 @pytest.mark.parametrize("precision,nb,m_end", [(0, 3000, 6), (1, 3000, 6), (0, 10000, 3), (1, 12000, 3),
                                                  (0, 2011, 4), (0, 2012, 4), (4, 3000, 6), (4, 10000, 3)])
 def test_dimer_tiled_kernel_segments(fq, precision, nb, m_end):
