@@ -185,7 +185,7 @@ fq_status propagate_impl(fq_plan* p, const double* x0, double* x, int nc, int m_
   StateWs w;
   layout(p, nc, nsteps, ws, &w);
   if (p->path == PATH_TRI_RESIDENT) {
-    fq_launch_gauge_coeffs(p, m_begin, nsteps, w.coeff, s);
+    fq_launch_gauge_coeffs(p, nc, m_begin, nsteps, w.coeff, s);
     st = fq_launch_resident(p, w.coeff, identity ? nullptr : x0, x, transpose_out, nc, m_begin, m_end, s);
     if (st != FQ_OK) return st;
     return cuda_ok(cudaGetLastError(), "resident chain");

@@ -225,7 +225,7 @@ fq_status fq_tile_propagate(fq_plan* p, const double* x0, double* x, int nc, int
                             int transpose_out, void* ws, cudaStream_t s);
 size_t fq_resident_coeff_bytes(int n, int steps);
 // per-step (2 d, 2 e') of the gauge-real operator and the frame rotations, into `coeff`
-void fq_launch_gauge_coeffs(const fq_plan* p, int m_begin, int nsteps, void* coeff, cudaStream_t s);
+void fq_launch_gauge_coeffs(const fq_plan* p, int nc, int m_begin, int nsteps, void* coeff, cudaStream_t s);
 fq_status fq_launch_resident(const fq_plan* p, const void* coeff, const double* x0, double* x, int transpose_out,
                              int nc, int m_begin, int m_end, cudaStream_t s);
 

@@ -119,7 +119,7 @@ static fq_status build_static(const fq_problem* prob, void* d_U, void* stream) {
   if (e == cudaSuccess && n > 1) e = cudaMemcpyAsync(p.d_k, kl.data(), (n - 1) * sizeof(double), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return fq_cuda_fail(e, "floquet_build_UT_static upload");
 
-  fq_launch_gauge_coeffs(&p, 0, M, coef, s);
+  fq_launch_gauge_coeffs(&p, n, 0, M, coef, s);
   st = fq_launch_resident(&p, coef, nullptr, (double*)d_U, 1, n, 0, M, s);
   if (st != FQ_OK) return st;
   // the host vectors above are staged by the copies; wait for the chain and read the check

@@ -16,17 +16,22 @@
 // which needs the same L products as the forward recurrence of Eq. 10 but only two live
 // vectors besides v.  Then X_m = e^{-i beta h} sum.
 //
-// Layout: NT threads (256 x 40 rows above 9216 rows, 512 x <= 18 below, 256 x 2 or 4 up to 1024);
-// thread t owns rows i = t*EPT .. t*EPT+EPT-1 (EPT even).  b_{k+1}, b_{k+2} live in registers as
-// (re, im) pairs; v and the step's (2 d, 2 e') pairs live in shared memory as float4 holding rows
-// (2p, 2p+1) of thread t at [p][t], so one conflict-free 16-byte access serves two rows.  The
-// per-step coefficient and rotation arrays are written in global memory in exactly that order
-// ("resident order"), so their loads are coalesced.  Each sweep over a thread's rows applies two
+// Layout: nt threads of EPT rows (res_config chooses both); thread t owns rows i = t*EPT ..
+// t*EPT+EPT-1 (EPT even).  b_{k+1}, b_{k+2} live in registers as (re, im) pairs; v and the step's
+// (2 d, 2 e') pairs live in shared memory as float4 holding rows (2p, 2p+1) of thread t, so one
+// conflict-free 16-byte access serves two rows at an offset known when compiling: at [p][t] where
+// nt is a template argument (the largest shapes: 3 % faster there), else at [t][p] with an odd row
+// length.  The per-step coefficient and rotation arrays are in global memory as
+// [p][t] ("resident order"), so their loads are coalesced.  Every row takes the same operations
+// whatever nt and EPT are, so they never change a result's bits.  Each sweep over a thread's rows applies two
 // products (Chain::pass); the two-row halo of b_{k+1} crosses lanes by warp shuffles and warps
 // through small double-buffered shared arrays (one __syncthreads per two products).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+
+#include <algorithm>
+#include <cmath>
 
 #include "gauge.cuh"
 #include "internal.h"
@@ -34,6 +39,9 @@
 namespace {
 
 constexpr int RES_MAXNW = 32;
+constexpr int RES_EPTS[] = {2, 4, 6, 8, 10, 12, 14, 16, 18, 20};  // rows per thread below 9217 rows
+// most threads of a CTA with `ept` rows a thread: the registers of two live vectors set it
+__host__ __device__ constexpr int res_max_threads(int ept) { return ept > 20 ? 256 : 512; }
 constexpr int RES_MAXL = 128;
 struct ResCoef {
   float cr[RES_MAXL + 1];  // c_k = (-i)^k a_k: real for even k, imaginary for odd k
@@ -48,6 +56,17 @@ struct ResShared {
   float lim_clenshaw;  // bound on |b_1 entry|^2
   unsigned int bad;    // set by any thread whose check failed
 };
+
+// dynamic shared memory: v and the operator pairs (odd pitch), exchange and halo rows, ResShared
+size_t res_smem(int nt, int ept) {
+  return sizeof(float4) * (2 * (size_t)((ept / 2) | 1) + 3) * nt + sizeof(ResShared);
+}
+
+// Model of a pass (two products), for res_config: its latency is RES_LAT + RES_LAT_ROW EPT, and every
+// warp on the SM takes RES_WARP + RES_ROW EPT of its issue slots (fitted to shapes timed from 41 to
+// 9201 rows, in units of 1.8 cycles); registers of a thread by EPT / 2 - 1.
+constexpr double RES_LAT = 284, RES_LAT_ROW = 22, RES_WARP = 24, RES_ROW = 4;
+constexpr int RES_REGS[] = {64, 88, 96, 104, 104, 112, 120, 120, 128, 128};
 
 // Position of row i in resident order (float2 units) for NT threads of EPT rows each.
 __host__ __device__ __forceinline__ size_t res_index(int i, int nt, int ept) {
@@ -134,16 +153,18 @@ __device__ __forceinline__ float2 row_half(float cc, float2 vv, float2 o, float 
   return __ffma2_rn(f2(0.5f, 0.5f), s, __ffma2_rn(f2(cc, cc), vv, f2(-o.x, -o.y)));
 }
 
-template <int NT, int EPT>
+// FNT: the number of threads where it is fixed, 0 where it is blockDim.x
+template <int EPT, int FNT>
 struct Chain {
-  static constexpr int NW = NT / 32;
   static constexpr int NP = EPT / 2;
-  const float4* v;   // [NP][NT] state in the step's frame, rows (2p, 2p+1)
-  const float4* cf;  // [NP][NT] (2 d, 2 e') of rows (2p, 2p+1), e'_i = Omega'[i+1][i]
-  float4* first2;    // [2][NT] first two rows of b_{k+1} per thread (exchange buffers)
-  float4* bhalo;     // [NT] (b_k at row i0-1, b_k at row i0+EPT) per thread, carried between passes
+  // float4 strides in shared memory between a thread's row pairs (ROW) and between threads (COL)
+  static constexpr int ROW = FNT ? FNT : 1, COL = FNT ? 1 : NP | 1;
+  const float4* v;   // state in the step's frame, rows (2p, 2p+1) at [p * ROW] from this thread's first
+  const float4* cf;  // (2 d, 2 e') of rows (2p, 2p+1), e'_i = Omega'[i+1][i], likewise
+  float4* first2;    // [2][nt] first two rows of b_{k+1} per thread (exchange buffers)
+  float4* bhalo;     // [nt] (b_k at row i0-1, b_k at row i0+EPT) per thread, carried between passes
   ResShared* sh;
-  int t, lane, warp;
+  int nt, t, lane, warp;
 
   // Publishes x's first two rows for the left neighbour (read back by right() after the sweep) and
   // returns rows i0-2, i0-1 (as (re, im, re, im)) of the left neighbour; zero before row 0.
@@ -155,14 +176,14 @@ struct Chain {
     l.z = __shfl_up_sync(0xffffffffu, x[EPT - 1].x, 1);
     l.w = __shfl_up_sync(0xffffffffu, x[EPT - 1].y, 1);
     if (lane == 31) sh->slot_last[par][warp] = make_float4(x[EPT - 2].x, x[EPT - 2].y, x[EPT - 1].x, x[EPT - 1].y);
-    first2[par * NT + t] = make_float4(x[0].x, x[0].y, x[1].x, x[1].y);
+    first2[par * nt + t] = make_float4(x[0].x, x[0].y, x[1].x, x[1].y);
     __syncthreads();
     if (lane == 0) l = warp > 0 ? sh->slot_last[par][warp - 1] : make_float4(0.f, 0.f, 0.f, 0.f);
     return l;
   }
   // rows i0+EPT, i0+EPT+1 as published by the right neighbour in exchange(); zero past the end
   __device__ __forceinline__ float4 right(int par) const {
-    return t < NT - 1 ? first2[par * NT + t + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
+    return t < nt - 1 ? first2[par * nt + t + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 
   // Two Clenshaw products in one sweep over the rows (Eqs. 10 and 12 in backward form):
@@ -180,8 +201,8 @@ struct Chain {
     const float4 al = FIRST ? z4 : exchange(A, par);
     const float2 am2 = lo2(al), am1 = hi2(al);
     // row i0-1: (., 2e'_{i0-2}, 2d_{i0-1}, 2e'_{i0-1}) and its v
-    const float4 cl = t > 0 ? cf[(NP - 1) * NT + t - 1] : z4;
-    const float2 vl = t > 0 ? hi2(v[(NP - 1) * NT + t - 1]) : z2;
+    const float4 cl = t > 0 ? cf[(NP - 1) * ROW - COL] : z4;
+    const float2 vl = t > 0 ? hi2(v[(NP - 1) * ROW - COL]) : z2;
     const float2 nbl =
         FIRST ? cvec<IM1>(c1, vl) : row<IM1>(c1, vl, lo2(bhalo[t]), cl.z, am1, cl.y, am2, cl.w, A[0]);
     float4 cp = cl;  // operator of rows 2p-2, 2p-1
@@ -189,8 +210,8 @@ struct Chain {
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       const int q = 2 * p;
-      const float4 c = cf[p * NT + t];
-      const float4 w = v[p * NT + t];
+      const float4 c = cf[p * ROW];
+      const float4 w = v[p * ROW];
       float2 b0, b1;
       if (FIRST) {
         b0 = cvec<IM1>(c1, lo2(w));
@@ -217,8 +238,8 @@ struct Chain {
       vp = hi2(w);
     }
     // row i0+EPT: (2d, 2e') of that row and its v
-    const float2 cr = t < NT - 1 ? lo2(cf[t + 1]) : z2;
-    const float2 vr = t < NT - 1 ? lo2(v[t + 1]) : z2;
+    const float2 cr = t < nt - 1 ? lo2(cf[COL]) : z2;
+    const float2 vr = t < nt - 1 ? lo2(v[COL]) : z2;
     float2 nbr;
     if (FIRST) {
       nbr = cvec<IM1>(c1, vr);
@@ -237,12 +258,12 @@ struct Chain {
   // The closing product alone (an even number L): B <- c0 v + Omega' A - B on own rows, A = b_1.
   __device__ __forceinline__ void single_final(const float2 (&A)[EPT], float2 (&B)[EPT], float c0, int par) {
     const float2 am1 = hi2(exchange(A, par));
-    float el = t > 0 ? cf[(NP - 1) * NT + t - 1].w : 0.f;
+    float el = t > 0 ? cf[(NP - 1) * ROW - COL].w : 0.f;
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       const int q = 2 * p;
-      const float4 c = cf[p * NT + t];
-      const float4 w = v[p * NT + t];
+      const float4 c = cf[p * ROW];
+      const float4 w = v[p * ROW];
       B[q] = row_half(c0, lo2(w), B[q], c.x, A[q], el, q == 0 ? am1 : A[q - 1], c.y, A[q + 1]);
       B[q + 1] =
           row_half(c0, hi2(w), B[q + 1], c.z, A[q + 1], c.y, A[q], c.w, q + 2 < EPT ? A[q + 2] : lo2(right(par)));
@@ -288,22 +309,26 @@ struct Chain {
   }
 };
 
-template <int NT, int EPT>
-__global__ void __launch_bounds__(NT, 1)
+template <int EPT, int FNT>
+__global__ void __launch_bounds__(FNT ? FNT : res_max_threads(EPT), 1)
 k_tri_resident(const float4* __restrict__ cf_all, const float4* __restrict__ rot_all, int n, int L, int nsteps,
                const double2* __restrict__ x0, double2* __restrict__ xout, int transpose_out, ResCoef coef,
                float ph_re, float ph_im, float clenshaw_bound, unsigned int* status) {
-  using Ch = Chain<NT, EPT>;
-  constexpr int NP = EPT / 2, NW = NT / 32;
+  using Ch = Chain<EPT, FNT>;
+  constexpr int NP = EPT / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4* sv = reinterpret_cast<float4*>(smem_raw);
-  float4* scf = sv + NP * NT;
+  const int NT = FNT ? FNT : (int)blockDim.x, NW = NT >> 5;
+  const int plane = (FNT ? NP : Ch::COL) * NT;
+  float4* sv = reinterpret_cast<float4*>(smem_raw) + threadIdx.x * Ch::COL;  // this thread's rows
+  float4* scf = sv + plane;
+  float4* tail = reinterpret_cast<float4*>(smem_raw) + 2 * plane;
   Ch C;
   C.v = sv;
   C.cf = scf;
-  C.first2 = sv + 2 * NP * NT;
-  C.bhalo = sv + 2 * NP * NT + 2 * NT;
-  C.sh = reinterpret_cast<ResShared*>(sv + 2 * NP * NT + 3 * NT);
+  C.first2 = tail;
+  C.bhalo = tail + 2 * NT;
+  C.sh = reinterpret_cast<ResShared*>(tail + 3 * NT);
+  C.nt = NT;
   C.t = threadIdx.x;
   C.lane = threadIdx.x & 31;
   C.warp = threadIdx.x >> 5;
@@ -362,9 +387,9 @@ k_tri_resident(const float4* __restrict__ cf_all, const float4* __restrict__ rot
       const int s = p * NT + t;
       const float4 c = cf_all[off + s];
       const float4 r = rot_all[off + s];
-      scf[s] = c;
+      scf[p * Ch::ROW] = c;
       const float2 a = A[2 * p], b = A[2 * p + 1];
-      sv[s] = make_float4(r.x * a.x - r.y * a.y, r.x * a.y + r.y * a.x, r.z * b.x - r.w * b.y, r.z * b.y + r.w * b.x);
+      sv[p * Ch::ROW] = make_float4(r.x * a.x - r.y * a.y, r.x * a.y + r.y * a.x, r.z * b.x - r.w * b.y, r.z * b.y + r.w * b.x);
     }
     C.check(A, C.sh->lim_state);  // X_{m-1} (or the initial state)
     __syncthreads();
@@ -414,73 +439,88 @@ k_tri_resident(const float4* __restrict__ cf_all, const float4* __restrict__ rot
   }
 }
 
-template <int NT, int EPT>
+template <int EPT, int FNT>
 fq_status launch_cfg(const fq_plan* p, const float4* cf, const float4* rot, const double* x0, double* x,
-                     int transpose_out, int nc, int nsteps, const ResCoef& coef, float bcl, cudaStream_t s) {
-  const size_t smem = sizeof(float4) * (EPT + 3) * NT + sizeof(ResShared);
+                     int transpose_out, int nc, int nsteps, const ResCoef& coef, float bcl, int nt, cudaStream_t s) {
+  const size_t smem = res_smem(nt, EPT);
   static std::atomic<unsigned> attr_set{0};
   if (fq_first_on_device(attr_set)) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_tri_resident<NT, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_tri_resident<EPT, FNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)res_smem(res_max_threads(EPT), EPT));
     if (e != cudaSuccess) return fq_cuda_fail(e, "resident kernel smem attribute");
   }
   fq_ktimer_start(p, s, "k_tri_resident");
-  k_tri_resident<NT, EPT><<<nc, NT, smem, s>>>(cf, rot, p->n, p->L, nsteps, (const double2*)x0, (double2*)x,
-                                                transpose_out, coef, (float)p->phase_re, (float)p->phase_im, bcl,
-                                                p->d_status);
+  k_tri_resident<EPT, FNT><<<nc, nt, smem, s>>>(cf, rot, p->n, p->L, nsteps, (const double2*)x0, (double2*)x, transpose_out,
+                                           coef, (float)p->phase_re, (float)p->phase_im, bcl, p->d_status);
   fq_ktimer_stop(p, s);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fq_cuda_fail(e, "resident kernel launch");
   return FQ_OK;
 }
 
-// (threads, rows per thread) for dimension n; 0 threads if the resident kernel does not apply.
-// Above 9216 rows, 256 x 40 (250 registers, no spills) beats 512 x 20, which has to fit in 128
-// registers and spills; 1024 x 10 would have to fit in 64.
-void res_config(int n, int* nt, int* ept) {
+// Rows the coefficient arrays are sized for: at least those of every shape res_config picks.
+int res_rows(int n) {
+  if (n <= 512) return 512;
+  if (n <= 1024) return 1024;
+  const int need = (n + 511) / 512;
+  return need > 20 ? 0 : (need > 18 ? 10240 : 512 * (need + (need & 1)));
+}
+
+// (threads, rows per thread) for nc states of n rows; 0 threads if the resident kernel does not apply.
+// Few threads of many rows do the least work a row (the two halo rows and the exchange are paid per
+// thread and warp, padding per 32 EPT rows); few states need many threads for their latency.  The
+// shapes were 256 x 2 or 4 up to 1024 rows and 512 x an even count above.  A pass of all N states in us
+// before and now: N = 201 0.57 -> 0.31, 501 0.99 -> 0.45, 1002 1.93 -> 1.12, 1301 5.65 -> 1.82, 2001 8.2 ->
+// 3.9, 3501 19.5 -> 12.0, 6501 45.1 -> 41.2; of 24 states: N = 1301 0.66 -> 0.41, 5001 0.91 -> 0.87.
+void res_config(int n, int nc, int* nt, int* ept) {
   *nt = 0;
   *ept = 0;
-  if (n <= 256 * 4) {
-    *nt = 256;
-    *ept = n <= 512 ? 2 : 4;
-    return;
-  }
-  const int need = (n + 511) / 512;
-  if (need > 20) return;
-  if (need > 18) {
+  const int cap = res_rows(n);
+  if (cap == 0) return;
+  if (cap == 10240) {
     *nt = 256;
     *ept = 40;
     return;
   }
-  *nt = 512;
-  *ept = need + (need & 1);
+  const double states = std::ceil((double)nc / fq_sm_count());  // on the fullest SM
+  double cost = 0.0;
+  for (int e : RES_EPTS) {
+    const int w = (n + 32 * e - 1) / (32 * e), t = 32 * w;  // warps and threads of a CTA
+    if (t > res_max_threads(e) || t * e > cap) continue;
+    // warps on an SM at a time, spread over its four schedulers
+    const int fit = std::max(1, std::min(65536 / (RES_REGS[e / 2 - 1] * t), (int)(232448 / (res_smem(t, e) + 1024))));
+    const double on = std::min(states, (double)std::min(fit, 2048 / t)) * w;
+    const double issue = states * w * (RES_WARP + RES_ROW * e) * (4.0 * std::ceil(on / 4.0) / on);
+    const double c = std::hypot(RES_LAT + RES_LAT_ROW * e, issue);
+    if (*nt == 0 || c < cost) {
+      *nt = t;
+      *ept = e;
+      cost = c;
+    }
+  }
 }
 
 }  // namespace
 
 int fq_resident_supported(int n, int L) {
-  int nt, ept;
-  res_config(n, &nt, &ept);
-  return nt > 0 && L <= RES_MAXL && L >= 1;
+  return res_rows(n) > 0 && L <= RES_MAXL && L >= 1;
 }
 
-// (2 nsteps + 1) blocks of nt * ept float2 in resident order: the operator pairs of every step,
-// then the frame rotation of every step plus the final one.
+// (2 nsteps + 1) blocks of float2 rows in resident order: the operator pairs of every step, then the
+// frame rotation of every step plus the final one.
 size_t fq_resident_coeff_bytes(int n, int steps) {
-  int nt, ept;
-  res_config(n, &nt, &ept);
-  return (2 * (size_t)steps + 1) * (size_t)nt * ept * sizeof(float2);
+  return (2 * (size_t)steps + 1) * (size_t)res_rows(n) * sizeof(float2);
 }
 
-void fq_launch_gauge_coeffs(const fq_plan* p, int m_begin, int nsteps, void* coeff, cudaStream_t s) {
+void fq_launch_gauge_coeffs(const fq_plan* p, int nc, int m_begin, int nsteps, void* coeff, cudaStream_t s) {
   const int ld = (p->n + 3) & ~3;
   int nt, ept;
-  res_config(p->n, &nt, &ept);
+  res_config(p->n, nc, &nt, &ept);
   float2* cf = (float2*)coeff;
   float2* rot = cf + (size_t)nsteps * nt * ept;
   // rows beyond ld (padding of the resident order) must hold cf = 0 and rot = 1: zero them
   // and let the kernel overwrite every row < ld; rot padding only multiplies zeros.
-  cudaMemsetAsync(coeff, 0, fq_resident_coeff_bytes(p->n, nsteps), s);
+  cudaMemsetAsync(coeff, 0, (2 * (size_t)nsteps + 1) * (size_t)nt * ept * sizeof(float2), s);
   GaugeArgs ga{p->n, p->steps, p->d_h0, p->d_h0o, p->d_h1, p->d_k, p->d_scal, p->sbeta};
   k_gauge_coeffs<<<nsteps + 1, GAUGE_NT, 0, s>>>(ga, ld, m_begin, nsteps, nt, ept, cf, rot);
 }
@@ -489,7 +529,7 @@ fq_status fq_launch_resident(const fq_plan* p, const void* coeff, const double* 
                              int nc, int m_begin, int m_end, cudaStream_t s) {
   const int nsteps = m_end - m_begin;
   int nt, ept;
-  res_config(p->n, &nt, &ept);
+  res_config(p->n, nc, &nt, &ept);
   const float4* cf = (const float4*)coeff;
   const float4* rot = cf + (size_t)nsteps * nt * ept / 2;
   ResCoef coef;
@@ -506,19 +546,25 @@ fq_status fq_launch_resident(const fq_plan* p, const void* coeff, const double* 
     }
   }
   const float b = (float)bcl;
-  if (nt == 256 && ept == 2) return launch_cfg<256, 2>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
-  if (nt == 256 && ept == 4) return launch_cfg<256, 4>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
-  if (nt == 256 && ept == 40) return launch_cfg<256, 40>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
+  if (nt == 512 && ept == 16)
+    return launch_cfg<16, 512>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
+  if (nt == 512 && ept == 18)
+    return launch_cfg<18, 512>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
   switch (ept) {
-    case 4: return launch_cfg<512, 4>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
-    case 6: return launch_cfg<512, 6>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
-    case 8: return launch_cfg<512, 8>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
-    case 10: return launch_cfg<512, 10>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
-    case 12: return launch_cfg<512, 12>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
-    case 14: return launch_cfg<512, 14>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
-    case 16: return launch_cfg<512, 16>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
-    case 18: return launch_cfg<512, 18>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
-    case 20: return launch_cfg<512, 20>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, s);
+#define FQ_RES_CASE(E) \
+  case E: return launch_cfg<E, 0>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
+    FQ_RES_CASE(2)
+    FQ_RES_CASE(4)
+    FQ_RES_CASE(6)
+    FQ_RES_CASE(8)
+    FQ_RES_CASE(10)
+    FQ_RES_CASE(12)
+    FQ_RES_CASE(14)
+    FQ_RES_CASE(16)
+    FQ_RES_CASE(18)
+    FQ_RES_CASE(20)
+    case 40: return launch_cfg<40, 256>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
+#undef FQ_RES_CASE
     default: fq_set_error("resident kernel: n = %d too large", p->n); return FQ_EUNSUPPORTED;
   }
 }

@@ -318,6 +318,24 @@ def test_tiled_shapes_agree(fq, precision, nb):
     assert np.max(np.abs(to_np(many[[0, 169]]) - ref)) <= tol
 
 
+@pytest.mark.parametrize("nb", [1, 31, 63, 64, 100, 127, 200, 255, 320, 383, 500, 511, 512, 700, 1000, 1023, 1024, 1300,
+                                1600, 2047, 2048, 2600, 3500, 5000, 6500, 8191, 8192, 9215])
+def test_resident_shapes_agree(fq, nb):
+    """Threads and rows per thread of the resident kernel follow the length and number of the states: one
+    state and the same state among 320 give the same bits, and the oracle's state."""
+    import torch
+    d = _drive_models(nb)
+    plan = dimer_plan(fq, d, 1, 2)
+    x0 = _unit_states(d.n, 3, 2311)
+    one = plan.propagate(cuda_c128(x0[:1]), 1, 5)
+    many = plan.propagate(cuda_c128(np.tile(x0, (107, 1))), 1, 5)
+    assert plan.check_status() == fq.FQ_OK
+    assert torch.equal(one[0], many[0]) and torch.equal(many[3:6], many[:3])
+    refp = o.plan_for_drive_tridiag(d.h0_diag, d.h0_off, d.h1_diag, d.drive, d.steps)
+    ref = o.propagate_tridiag(d.h0_diag, d.h0_off, d.h1_diag, refp, x0.T, 1, 5).T
+    assert np.max(np.abs(to_np(many[:3]) - ref)) <= tol_f32(4, plan.info.L, plan.info.R)
+
+
 @pytest.mark.parametrize("precision,nb,m_end", [(0, 3000, 6), (1, 3000, 6), (0, 10000, 3), (1, 12000, 3),
                                                  (0, 2011, 4), (0, 2012, 4), (4, 3000, 6), (4, 10000, 3)])
 def test_dimer_tiled_kernel_segments(fq, precision, nb, m_end):
