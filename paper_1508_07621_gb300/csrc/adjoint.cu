@@ -11,7 +11,7 @@
 // where psi_l are step m's forward Chebyshev vectors.  Seed: G_M = -tau W / N^2, tau = Tr(W^+ U_T).
 //
 // Memory: X_m is kept every s = checkpoint_stride steps; each segment is recomputed forward once,
-// keeping its psi_l, and then walked backward.  All matrices are stored as rows (row r = column r
+// keeping its psi_l, and then walked backward (the forward sweep itself keeps those of the last segment).  All matrices are stored as rows (row r = column r
 // of the column-state matrix), so every product is the dense FP64 tile Y^T = X^T Omega~^T.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -373,7 +373,16 @@ static fq_status floquet_grad_body(fq_plan* p, const double* d_f, const void* d_
   k_identity_rows<<<grid_n(nn), 256, 0, s>>>(w.ck(0).re, w.ck(0).im, n);
   Mat x = w.ck(0);
   int xi = 0;
+  const int m_last = (w.nseg - 1) * S;  // first step of the last segment
   for (int m = 0; m < M; ++m) {
+    if (m >= m_last) {  // the last segment is walked back first: its psi_l are kept right away
+      if (m == m_last) k_copy2<<<grid_n(nn), 256, 0, s>>>(x.re, x.im, nn, w.slot(0).re, w.slot(0).im);
+      std::vector<Mat> psi(L + 1);
+      for (int l = 0; l < L; ++l) psi[l] = w.slot((m - m_last) * L + l);
+      x = w.slot((m - m_last + 1) * L);
+      forward_step(p, w, d_f, m, psi[0], x, psi.data(), Mat{}, Mat{}, s);
+      continue;
+    }
     Mat out = w.x[xi];
     forward_step(p, w, d_f, m, x, out, nullptr, w.x[(xi + 1) % 3], w.x[(xi + 2) % 3], s);
     x = out;
@@ -393,9 +402,11 @@ static fq_status floquet_grad_body(fq_plan* p, const double* d_f, const void* d_
   const double cph_r = p->phase_re, cph_i = -p->phase_im;  // conj(e^{-i beta h})
   for (int k = w.nseg - 1; k >= 0; --k) {
     const int m0 = k * S, m1 = std::min(M, m0 + S);
-    // recompute the segment forward, keeping every psi_l (slot st*L + l; X_{m+1} at slot (st+1)*L)
-    k_copy2<<<grid_n(nn), 256, 0, s>>>(w.ck(k).re, w.ck(k).im, nn, w.slot(0).re, w.slot(0).im);
-    for (int st = 0; st < m1 - m0; ++st) {
+    // recompute the segment forward, keeping every psi_l (slot st*L + l; X_{m+1} at slot (st+1)*L);
+    // the forward sweep has done so for the last one
+    if (k < w.nseg - 1)
+      k_copy2<<<grid_n(nn), 256, 0, s>>>(w.ck(k).re, w.ck(k).im, nn, w.slot(0).re, w.slot(0).im);
+    for (int st = 0; st < m1 - m0 && k < w.nseg - 1; ++st) {
       std::vector<Mat> psi(L + 1);
       for (int l = 0; l < L; ++l) psi[l] = w.slot(st * L + l);
       forward_step(p, w, d_f, m0 + st, psi[0], w.slot((st + 1) * L), psi.data(), Mat{}, Mat{}, s);

@@ -13,7 +13,7 @@
 //   dL/df_m = 2 Re sum_l w_l D_l  (w_1 = -i, w_l = -2i).
 // Memory: FP32 masters of X every s = checkpoint_stride steps; each segment is recomputed once
 // with the slices of every psi_l kept (they are the left operands of the dot products) and then
-// walked backward.  The slots are stored slice-major ([slice][slot][row][k]) and bbar_1..bbar_L
+// walked backward; the forward sweep itself keeps those of the last segment.  The slots are stored slice-major ([slice][slot][row][k]) and bbar_1..bbar_L
 // of a step are kept as one stacked block, so the L gradient dots of a step run as one GEMM over
 // L x Np stacked rows.
 #include <vector>
@@ -420,7 +420,15 @@ fq_status fq_grad_split(fq_plan* p, const double* d_f, const void* d_W, double* 
   r.scale_slices(Master{nullptr, nullptr}, 1.f, 0.f, w.f[0], w.lsl[0], w.astride);
   cudaMemcpyAsync(w.ckpt(0, n).re, w.f[0].re, 2 * plane_bytes, cudaMemcpyDeviceToDevice, s);
   std::vector<__nv_bfloat16*> left(L + 1);
+  const size_t ss = w.slot_slice();
+  const int m_last = (w.nseg - 1) * S;  // first step of the last segment
   for (int m = 0; m < M; ++m) {
+    if (m >= m_last) {  // the last segment is walked back first: its slices are kept right away
+      if (m == m_last) r.scale_slices(w.f[xb], 1.f, 0.f, Master{nullptr, nullptr}, w.slot(0), ss);
+      for (int l = 0; l <= L; ++l) left[l] = w.slot((m - m_last) * L + l);
+      if ((st = r.step(m, &xb, left.data(), ss)) != FQ_OK) return st;
+      continue;
+    }
     for (int l = 0; l <= L; ++l) left[l] = w.lsl[l & 1];
     if ((st = r.step(m, &xb, left.data(), w.astride)) != FQ_OK) return st;
     // the last term wrote X_m's slices into left[L]; the next step reads them from lsl[0]
@@ -436,14 +444,17 @@ fq_status fq_grad_split(fq_plan* p, const double* d_f, const void* d_W, double* 
 
   // ---- backward, one checkpoint segment at a time
   const float cph_r = (float)p->phase_re, cph_i = (float)-p->phase_im;  // conj(e^{-i beta h})
-  const size_t ss = w.slot_slice();
   for (int k = w.nseg - 1; k >= 0; --k) {
     const int m0 = k * S, m1 = std::min(M, m0 + S);
-    // recompute the segment forward keeping the slices of every psi_l (slot st * L + l)
-    cudaMemcpyAsync(w.f[0].re, w.ckpt(k, n).re, 2 * plane_bytes, cudaMemcpyDeviceToDevice, s);
-    r.scale_slices(w.f[0], 1.f, 0.f, Master{nullptr, nullptr}, w.slot(0), ss);
-    xb = 0;
-    for (int st_ = 0; st_ < m1 - m0; ++st_) {
+    // recompute the segment forward keeping the slices of every psi_l (slot st * L + l); the forward
+    // sweep has done so for the last one
+    const int redo = k < w.nseg - 1 ? m1 - m0 : 0;
+    if (redo) {
+      cudaMemcpyAsync(w.f[0].re, w.ckpt(k, n).re, 2 * plane_bytes, cudaMemcpyDeviceToDevice, s);
+      r.scale_slices(w.f[0], 1.f, 0.f, Master{nullptr, nullptr}, w.slot(0), ss);
+      xb = 0;
+    }
+    for (int st_ = 0; st_ < redo; ++st_) {
       for (int l = 0; l <= L; ++l) left[l] = w.slot(st_ * L + l);
       if ((st = r.step(m0 + st_, &xb, left.data(), ss)) != FQ_OK) return st;
     }

@@ -224,7 +224,18 @@ fq_status fq_grad_ozaki(fq_plan* p, const double* d_f, const void* d_W, double* 
   cudaMemcpyAsync(w.ckpt(0).re, w.f[0].re, plane2, cudaMemcpyDeviceToDevice, s);
   std::vector<__nv_bfloat16*> left(L + 1);
   std::vector<int*> es(L + 1);
+  const size_t ss = w.slot_slice();
+  const int m_last = (w.nseg - 1) * S;  // first step of the last segment
   for (int m = 0; m < M; ++m) {
+    if (m >= m_last) {  // the last segment is walked back first: its slices are kept right away
+      if (m == m_last) r.slice(w.f[xb], 1.0, 0.0, Planes{nullptr, nullptr}, w.slot(0), ss, w.es_slot(0));
+      for (int l = 0; l <= L; ++l) {
+        left[l] = w.slot((m - m_last) * L + l);
+        es[l] = w.es_slot((m - m_last) * L + l);
+      }
+      if ((st = r.step(m, &xb, left.data(), es.data(), ss)) != FQ_OK) return st;
+      continue;
+    }
     for (int l = 0; l <= L; ++l) {
       left[l] = w.lsl[l & 1];
       es[l] = w.esl[l & 1];
@@ -246,14 +257,17 @@ fq_status fq_grad_ozaki(fq_plan* p, const double* d_f, const void* d_W, double* 
 
   // ---- backward, one checkpoint segment at a time
   const double cph_r = p->phase_re, cph_i = -p->phase_im;  // conj(e^{-i beta h})
-  const size_t ss = w.slot_slice();
   for (int k = w.nseg - 1; k >= 0; --k) {
     const int m0 = k * S, m1 = std::min(M, m0 + S);
-    // recompute the segment forward keeping the slices of every psi_l (slot st * L + l)
-    cudaMemcpyAsync(w.f[0].re, w.ckpt(k).re, plane2, cudaMemcpyDeviceToDevice, s);
-    r.slice(w.f[0], 1.0, 0.0, Planes{nullptr, nullptr}, w.slot(0), ss, w.es_slot(0));
-    xb = 0;
-    for (int st_ = 0; st_ < m1 - m0; ++st_) {
+    // recompute the segment forward keeping the slices of every psi_l (slot st * L + l); the forward
+    // sweep has done so for the last one
+    const int redo = k < w.nseg - 1 ? m1 - m0 : 0;
+    if (redo) {
+      cudaMemcpyAsync(w.f[0].re, w.ckpt(k).re, plane2, cudaMemcpyDeviceToDevice, s);
+      r.slice(w.f[0], 1.0, 0.0, Planes{nullptr, nullptr}, w.slot(0), ss, w.es_slot(0));
+      xb = 0;
+    }
+    for (int st_ = 0; st_ < redo; ++st_) {
       for (int l = 0; l <= L; ++l) {
         left[l] = w.slot(st_ * L + l);
         es[l] = w.es_slot(st_ * L + l);
