@@ -63,8 +63,9 @@ size_t res_smem(int nt, int ept) {
 }
 
 // Model of a pass (two products), for res_config: its latency is RES_LAT + RES_LAT_ROW EPT, and every
-// warp on the SM takes RES_WARP + RES_ROW EPT of its issue slots (fitted to shapes timed from 41 to
-// 9201 rows, in units of 1.8 cycles); registers of a thread by EPT / 2 - 1.
+// warp on the SM takes RES_WARP + RES_ROW EPT of its issue slots, a tenth more at 20 rows, which spill
+// (fitted to shapes timed from 41 to 9201 rows, in units of 1.8 cycles); registers of a thread by
+// EPT / 2 - 1.
 constexpr double RES_LAT = 284, RES_LAT_ROW = 22, RES_WARP = 24, RES_ROW = 4;
 constexpr int RES_REGS[] = {64, 88, 96, 104, 104, 112, 120, 120, 128, 128};
 
@@ -490,7 +491,7 @@ void res_config(int n, int nc, int* nt, int* ept) {
     // warps on an SM at a time, spread over its four schedulers
     const int fit = std::max(1, std::min(65536 / (RES_REGS[e / 2 - 1] * t), (int)(232448 / (res_smem(t, e) + 1024))));
     const double on = std::min(states, (double)std::min(fit, 2048 / t)) * w;
-    const double issue = states * w * (RES_WARP + RES_ROW * e) * (4.0 * std::ceil(on / 4.0) / on);
+    const double issue = states * w * (RES_WARP + RES_ROW * e) * (e == 20 ? 1.1 : 1.0) * (4.0 * std::ceil(on / 4.0) / on);
     const double c = std::hypot(RES_LAT + RES_LAT_ROW * e, issue);
     if (*nt == 0 || c < cost) {
       *nt = t;
