@@ -4,17 +4,26 @@
 // The per-term dense path launches one tiled GEMM per Chebyshev term; at N = 64 each of those
 // launches keeps only a handful of SMs busy and the chain is 1400 dependent launches long
 // (M = 200, L = 7).  Here the independence of the columns of U_T (Algorithm 1 propagates each
-// initial state on its own) is used instead: one cluster per state, each CTA owning 32 rows of
-// Omega~_m, so 64 states fill 128 SMs and the whole chunk is one launch.
+// initial state on its own) is used instead: one cluster per state, each CTA owning 16 or 32 rows of
+// Omega~_m, so 64 states fill the SMs and the whole chunk is one launch.
 //
 // Per step m (Eqs. 10-12): Phi_0 = X_{m-1}, Phi_1 = -i Omega~ Phi_0,
 // Phi_{l+1} = -2i Omega~ Phi_l + Phi_{l-1}, X_m = e^{-i beta h} sum_{l<=L} a_l Phi_l.
-// Each CTA keeps the full state vector Phi_l (N complex values) in shared memory, twice
-// (double-buffered); a thread pair (row i, k-group g) holds 8 entries of row i of S_m and A_m
-// (Omega~_m = S_m + i A_m) in registers, and the KG threads of a row reduce their partial
-// sums by shuffles.  The row's first thread advances the recurrence and the accumulator in
-// registers and writes the new entry of Phi into every CTA of the cluster (distributed shared
-// memory); one cluster barrier per product publishes the vector.
+//
+// FP64 (k_dense_resident).  GB300 runs one FP64 multiply-add every second cycle in each quarter of an
+// SM: an FP64 instruction of a warp takes 64 cycles of its quarter however many lanes it uses, so the
+// kernel is bound by their number in the busiest warp.  A CTA owns 16 rows and has 4 warps (8 above
+// N = 64) that share the values of k; lane (row, parity) holds up to 8 entries of its row of S_m and A_m
+// (Omega~_m = S_m + i A_m) in registers, the next step's loaded while this one runs.  A product is at
+// most 32 FP64 instructions a warp; the two parities of a row trade partial sums, one keeping Re y and
+// one Im y (one addition), and the first warp adds the warps' partials and advances the recurrence of
+// 16 complex rows on its 32 lanes (4 instructions at 4 warps).  The state vector Phi_l is kept whole in
+// every CTA's shared memory, twice; the first warp writes its new entries into every CTA of the cluster
+// (distributed shared memory), one cluster barrier per product publishes them, and the accumulator
+// and the bound check follow while it is under way.  (Eight lanes a row with a shuffle reduction and the
+// recurrence on every warp's leading lanes, 32 rows a CTA, took as many FP64 instructions again as the
+// products themselves.)  A product of all states in us before and now: N = 16 3.3 -> 0.9, 32 3.8 -> 1.4, 48 4.2 -> 2.5,
+// 64 4.2 -> 3.1, 100 23 -> 13, 128 31 -> 19.
 //
 // Omega~_m for the chunk's steps is formed beforehand in HBM (it is L2-resident: 64 steps x
 // 2 x N^2 doubles = 4 MB at N = 64) by one batched launch (order 4) or one launch per step
@@ -22,7 +31,9 @@
 //
 // FQ_DF32 runs the same chain in double-float arithmetic (dfl.cuh) on the FP32 pipes, which
 // GB300 runs at many times its FP64 rate: Omega~ is converted once per step to FP32 pairs, the
-// state lives in shared memory as packed complex pairs, and the states in HBM stay FP64.
+// state lives in shared memory as packed complex pairs, and the states in HBM stay FP64.  There a
+// thread pair (row i, k-group g) holds 8 entries of row i, and the KG threads of a row reduce their
+// partial sums by shuffles.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -34,8 +45,9 @@
 
 namespace {
 
-constexpr int DR_ROWS = 32;   // rows of Omega~ per CTA
+constexpr int DR_ROWS = 16;   // rows of Omega~ per CTA
 constexpr int DR_KPT = 8;     // entries of a row per thread
+constexpr int DR_MAXW = 8;    // FP64: most warps per CTA
 constexpr int DR_MAXN = 128;
 constexpr int DR_CHUNK = 64;  // steps per launch
 constexpr int DR_MAXL = 128;
@@ -54,97 +66,131 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// stores (x, y) at the same shared-memory offset as `local` in cluster CTA `rank`
-__device__ __forceinline__ void st_cluster_f64x2(const void* local, unsigned rank, double x, double y) {
+// the two halves of cluster_sync_all
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// stores x at the same shared-memory offset as `local` in cluster CTA `rank`
+__device__ __forceinline__ void st_cluster_f64(const double* local, unsigned rank, double x) {
   const unsigned la = (unsigned)__cvta_generic_to_shared(local);
   unsigned ra;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(rank));
-  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(ra), "d"(x), "d"(y) : "memory");
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(x) : "memory");
 }
 
 // S, A: [nsteps][n][n] (Omega~ of the chunk's steps); x: planar states [nc][n], updated in place.
-template <int ROWS, int KG>
-__global__ void __launch_bounds__(ROWS* KG)
+// C CTAs of W warps per state, warp w on the columns 2 KPT w .. 2 KPT (w + 1).
+template <int KPT>
+__global__ void __launch_bounds__(32 * DR_MAXW)
     k_dense_resident(const double* __restrict__ S, const double* __restrict__ A, int n, int nsteps, int L, int C,
                      DrCoef cf, double ph_re, double ph_im, double bound2, double* xr, double* xi,
                      unsigned* status) {
-  constexpr int NT = ROWS * KG;
-  constexpr int NV = KG * DR_KPT;  // vector length held per buffer (>= n)
-  __shared__ double2 phi[2][NV];
-  const int t = threadIdx.x, rl = t / KG, g = t % KG;
+  __shared__ double2 phi[2][DR_MAXN];
+  __shared__ double part[DR_MAXW][32];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, W = blockDim.x >> 5;
+  const int row = lane & 15, kh = lane >> 4;
   const unsigned rank = C > 1 ? cluster_rank() : 0u;
   const int j = blockIdx.x / C;  // the state this cluster carries
-  const int i = (int)rank * ROWS + rl;
-  const bool own = g == 0 && i < n;
-  for (int q = t; q < 2 * NV; q += NT) {
-    const int b = q / NV, k = q % NV;
+  const int i = (int)rank * DR_ROWS + row;
+  for (int q = t; q < 2 * DR_MAXN; q += 32 * W) {
+    const int b = q / DR_MAXN, k = q % DR_MAXN;
     phi[b][k] = b == 0 && k < n ? make_double2(xr[(size_t)j * n + k], xi[(size_t)j * n + k]) : make_double2(0.0, 0.0);
   }
   __syncthreads();
   if (C > 1) cluster_sync_all();  // every CTA of the cluster is running before remote stores
   const size_t nn = (size_t)n * n;
+  double s[KPT], a[KPT], sn[KPT], an[KPT];  // this step's entries and the next one's
+  auto load = [&](int m, double (&ls)[KPT], double (&la)[KPT]) {
+#pragma unroll
+    for (int q = 0; q < KPT; ++q) {
+      const int k = 2 * KPT * warp + 2 * q + kh;  // the parities interleave: no bank conflict on phi
+      const bool ok = m < nsteps && i < n && k < n;
+      ls[q] = ok ? S[m * nn + (size_t)i * n + k] : 0.0;
+      la[q] = ok ? A[m * nn + (size_t)i * n + k] : 0.0;
+    }
+  };
+  load(0, sn, an);
+  // first warp: lanes with kh = 0 sum Re y and carry the imaginary component of row i, the others
+  // the reverse (Phi_{l+1} = -2i y + Phi_{l-1})
+  double acc = 0.0, pv = 0.0;
   int buf = 0;
   bool bad = false;
   for (int m = 0; m < nsteps; ++m) {
-    double s[DR_KPT], a[DR_KPT];
 #pragma unroll
-    for (int q = 0; q < DR_KPT; ++q) {
-      const int k = g + KG * q;
-      const bool ok = i < n && k < n;
-      s[q] = ok ? S[m * nn + (size_t)i * n + k] : 0.0;
-      a[q] = ok ? A[m * nn + (size_t)i * n + k] : 0.0;
+    for (int q = 0; q < KPT; ++q) {
+      s[q] = sn[q];
+      a[q] = an[q];
     }
-    double accr = 0.0, acci = 0.0, pvr = 0.0, pvi = 0.0;
+    load(m + 1, sn, an);
     for (int l = 0; l < L; ++l) {
+      const double2* v = phi[buf] + 2 * KPT * warp + kh;
       double yr = 0.0, yi = 0.0;
 #pragma unroll
-      for (int q = 0; q < DR_KPT; ++q) {
-        const double2 v = phi[buf][g + KG * q];
-        yr = fma(s[q], v.x, fma(-a[q], v.y, yr));
-        yi = fma(s[q], v.y, fma(a[q], v.x, yi));
+      for (int q = 0; q < KPT; ++q) {
+        const double2 p = v[2 * q];
+        yr = fma(s[q], p.x, fma(-a[q], p.y, yr));
+        yi = fma(s[q], p.y, fma(a[q], p.x, yi));
       }
-#pragma unroll
-      for (int o = KG / 2; o > 0; o >>= 1) {
-        yr += __shfl_xor_sync(0xffffffffu, yr, o);
-        yi += __shfl_xor_sync(0xffffffffu, yi, o);
-      }
-      if (own) {
-        const double2 cur = phi[buf][i];
-        double nr, ni;
-        if (l == 0) {  // Phi_1 = -i y
-          nr = yi;
-          ni = -yr;
-          accr = fma(cf.a[1], nr, cf.a[0] * cur.x);
-          acci = fma(cf.a[1], ni, cf.a[0] * cur.y);
-        } else {       // Phi_{l+1} = -2i y + Phi_{l-1}
-          nr = fma(2.0, yi, pvr);
-          ni = fma(-2.0, yr, pvi);
-          accr = fma(cf.a[l + 1], nr, accr);
-          acci = fma(cf.a[l + 1], ni, acci);
-        }
-        pvr = cur.x;
-        pvi = cur.y;
-        bad |= !(nr * nr + ni * ni <= bound2);  // |T_l(Omega~) x| <= |x| inside the bounds
-        if (l == L - 1) {  // X_m = e^{-i beta h} acc
-          nr = ph_re * accr - ph_im * acci;
-          ni = ph_re * acci + ph_im * accr;
-        }
-        if (C > 1) {
-          for (int c = 0; c < C; ++c) st_cluster_f64x2(&phi[buf ^ 1][i], (unsigned)c, nr, ni);
+      const double other = __shfl_xor_sync(0xffffffffu, kh ? yr : yi, 16);
+      double y = (kh ? yi : yr) + other;
+      if (warp > 0) part[warp][lane] = y;
+      __syncthreads();
+      if (warp == 0) {
+        // the warps' partials (W is 4 or 8), added pairwise
+        const double y1 = part[2][lane] + part[3][lane];
+        y += part[1][lane];
+        if (W > 4) {
+          y += part[4][lane] + part[5][lane];
+          y += y1 + (part[6][lane] + part[7][lane]);
         } else {
-          phi[buf ^ 1][i] = make_double2(nr, ni);
+          y += y1;
         }
+        const double2 pc = phi[buf][i < n ? i : 0];
+        const double cur = kh ? pc.x : pc.y;
+        const double sy = kh ? y : -y;  // Phi_1 = -i y
+        double nx = l == 0 ? sy : fma(2.0, sy, pv);
+        const double psi = nx;
+        auto accumulate = [&] { acc = fma(cf.a[l + 1], psi, l == 0 ? cf.a[0] * cur : acc); };
+        if (l == L - 1) {  // X_m = e^{-i beta h} acc
+          accumulate();
+          const double ao = __shfl_xor_sync(0xffffffffu, acc, 16);
+          nx = fma(ph_re, acc, (kh ? -ph_im : ph_im) * ao);
+        }
+        if (i < n) {
+          double* dst = kh ? &phi[buf ^ 1][i].x : &phi[buf ^ 1][i].y;
+          if (C > 1) {
+            for (int c = 0; c < C; ++c) st_cluster_f64(dst, (unsigned)c, nx);
+          } else {
+            *dst = nx;
+          }
+        }
+        __syncwarp();
+        if (C > 1) cluster_arrive();
+        // what the peers do not wait for
+        pv = cur;
+        if (l < L - 1) accumulate();
+        // |T_l(Omega~) x| <= |x| inside the bounds; components below 2^-1/2 need no arithmetic
+        if (__any_sync(0xffffffffu, (__double2hiint(psi) & 0x7FFFFFFF) >= 0x3FE6A09E)) {
+          const double co = __shfl_xor_sync(0xffffffffu, psi, 16);
+          bad |= i < n && !(psi * psi + co * co <= bound2);
+        }
+      } else if (C > 1) {
+        cluster_arrive();
       }
-      if (C > 1) cluster_sync_all();
+      __syncwarp();
+      if (C > 1) cluster_wait();
       else __syncthreads();
       buf ^= 1;
     }
   }
-  if (own) {
-    xr[(size_t)j * n + i] = phi[buf][i].x;
-    xi[(size_t)j * n + i] = phi[buf][i].y;
+  if (warp == 0 && i < n) {
+    if (kh) xr[(size_t)j * n + i] = phi[buf][i].x;
+    else xi[(size_t)j * n + i] = phi[buf][i].y;
   }
   if (bad) atomicOr(status, FQ_BIT_BOUND);
+  __syncwarp();
   if (C > 1) cluster_sync_all();  // no CTA leaves while a peer could still address its memory
 }
 
@@ -275,6 +321,7 @@ __global__ void k_omega_dense_steps(const double* __restrict__ h0, const double*
   }
 }
 
+// FP64: KG = 0 (the warps share the values of k); double-float: KG threads per row
 template <int ROWS, int KG>
 cudaError_t launch_resident(const fq_plan* p, const double* S, const double* A, const float2* Sd, const float2* Ad,
                             int nsteps, double* xr, double* xi, int nc, cudaStream_t s) {
@@ -284,7 +331,8 @@ cudaError_t launch_resident(const fq_plan* p, const double* S, const double* A, 
   const double bound2 = 1.0 + 1e-9;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(nc * C));
-  cfg.blockDim = dim3(ROWS * KG);
+  const int W = p->n <= 64 ? 4 : DR_MAXW;  // FP64: warps
+  cfg.blockDim = dim3(KG ? ROWS * KG : 32 * W);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   if (C > 1) {
@@ -295,10 +343,15 @@ cudaError_t launch_resident(const fq_plan* p, const double* S, const double* A, 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
   }
-  if (p->precision == FQ_DF32)
+  if constexpr (KG > 0)
     return cudaLaunchKernelEx(&cfg, k_dense_resident_dfl<ROWS, KG>, (const float2*)Sd, (const float2*)Ad, p->n, nsteps,
                               p->L, C, cf, p->phase_re, p->phase_im, bound2, xr, xi, p->d_status);
-  return cudaLaunchKernelEx(&cfg, k_dense_resident<ROWS, KG>, S, A, p->n, nsteps, p->L, C, cf, p->phase_re,
+  const int need = (p->n + 2 * W - 1) / (2 * W);  // entries a lane
+  static constexpr decltype(&k_dense_resident<1>) kerns[DR_KPT] = {
+      k_dense_resident<1>, k_dense_resident<2>, k_dense_resident<3>, k_dense_resident<4>,
+      k_dense_resident<5>, k_dense_resident<6>, k_dense_resident<7>, k_dense_resident<8>};
+  const auto kern = kerns[need - 1];
+  return cudaLaunchKernelEx(&cfg, kern, S, A, p->n, nsteps, p->L, C, cf, p->phase_re,
                             p->phase_im, bound2, xr, xi, p->d_status);
 }
 
@@ -343,8 +396,7 @@ fq_status fq_dense_resident_chain(const fq_plan* p, double* xr, double* xi, int 
     cudaError_t e;
     if (p->precision == FQ_DF32 && n <= 64) e = launch_resident<16, 8>(p, S, A, Sd, Ad, cnt, xr, xi, nc, s);
     else if (p->precision == FQ_DF32) e = launch_resident<16, 16>(p, S, A, Sd, Ad, cnt, xr, xi, nc, s);
-    else if (n <= 64) e = launch_resident<DR_ROWS, 8>(p, S, A, Sd, Ad, cnt, xr, xi, nc, s);
-    else e = launch_resident<DR_ROWS, 16>(p, S, A, Sd, Ad, cnt, xr, xi, nc, s);
+    else e = launch_resident<DR_ROWS, 0>(p, S, A, Sd, Ad, cnt, xr, xi, nc, s);
     if (e != cudaSuccess) return fq_cuda_fail(e, "dense resident chain");
   }
   return FQ_OK;

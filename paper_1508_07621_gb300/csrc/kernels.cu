@@ -18,6 +18,8 @@ template <> struct vec2<double> { using t = double2; };
 template <> struct vec2<float> { using t = float2; };
 
 __device__ __forceinline__ void check_bound(double re, double im, const fq_term& t) {
+  // both parts below 2^-1/2 in magnitude (NaN and infinity are not): no FP64 arithmetic
+  if ((__double2hiint(re) & 0x7FFFFFFF) < 0x3FE6A09E && (__double2hiint(im) & 0x7FFFFFFF) < 0x3FE6A09E) return;
   if (!(re * re + im * im <= t.bound2)) atomicOr(t.status, FQ_BIT_BOUND);
 }
 
@@ -193,8 +195,8 @@ __global__ void k_frobenius(const double* __restrict__ a, size_t count, double* 
 // One Chebyshev term, dense FP64: Y^T[j][i] = sum_k Psi[j][k] (S[i][k] + i A[i][k]) (tile loop in
 // dense_core.cuh) followed by the fused recurrence / Bessel accumulation / step-close epilogue.
 // A == nullptr selects the real-operator variant (piecewise drives: c_m = 0).
-template <int BJ, int BI, int BK, int TJ, int TI, bool HAS_A>
-__global__ void __launch_bounds__((BJ / TJ) * (BI / TI))
+template <int BJ, int BI, int BK, int TJ, int TI, bool HAS_A, int KG = 1>
+__global__ void __launch_bounds__(KG * (BJ / TJ) * (BI / TI))
 k_term_dense_f64(const double* __restrict__ S, const double* __restrict__ A, int n,
                  const double* __restrict__ cur_re, const double* __restrict__ cur_im,
                  const double* prev_re, const double* prev_im, double* acc_re, double* acc_im,
@@ -203,7 +205,8 @@ k_term_dense_f64(const double* __restrict__ S, const double* __restrict__ A, int
   const int tx = threadIdx.x % NTX, ty = threadIdx.x / NTX;
   const int j0 = blockIdx.y * BJ, i0 = blockIdx.x * BI;
   double yr[TJ][TI], yi[TJ][TI];
-  dense_tile_f64<BJ, BI, BK, TJ, TI, HAS_A>(S, A, n, cur_re, cur_im, nc, j0, i0, yr, yi);
+  dense_tile_f64<BJ, BI, BK, TJ, TI, HAS_A, KG>(S, A, n, cur_re, cur_im, nc, j0, i0, yr, yi);
+  if (KG > 1 && threadIdx.x >= NTX * (BJ / TJ)) return;  // group 0 holds the sums
 #pragma unroll
   for (int u = 0; u < TJ; ++u)
 #pragma unroll
@@ -576,24 +579,27 @@ void fq_launch_frobenius(const double* a, size_t count, double* out, cudaStream_
 
 void fq_launch_term_dense_f64(const double* S, const double* A, int n, fq_blk<double> cur, fq_blk<double> prev,
                               fq_blk<double> acc, fq_blk<double> out, int nc, const fq_term& t, cudaStream_t s) {
-  // Smaller tiles when the grid would leave most of the 152 SMs idle (FP64 is ALU-bound).
-  const long big = (long)((n + 31) / 32) * ((nc + 31) / 32);
-  if (big >= 2 * 152) {
-    dim3 g((n + 31) / 32, (nc + 31) / 32);
-    if (A)
-      k_term_dense_f64<32, 32, 16, 2, 2, true><<<g, 256, 0, s>>>(S, A, n, cur.re, cur.im, prev.re, prev.im, acc.re,
-                                                                 acc.im, out.re, out.im, nc, t);
-    else
-      k_term_dense_f64<32, 32, 16, 2, 2, false><<<g, 256, 0, s>>>(S, A, n, cur.re, cur.im, prev.re, prev.im, acc.re,
-                                                                  acc.im, out.re, out.im, nc, t);
+  // FP64 is bound by its pipes.  32 x 32 tiles where they are at least two a SM, else 8 x 8 ones; below
+  // N = 545, where even the whole U_T has fewer, 4 x 8 tiles whose warps split K: a product of a few
+  // hundred levels is about one warp of outputs for each of the chip's 608 FP64 pipes, and many small
+  // pieces balance better and hide latency.  A product of all states (of an eighth of them) in us
+  // before, with 8 x 8 tiles, and now: N = 143 43.8 (39.6) -> 31.7 (15.0), 200 80.5 (52.9) -> 72.4 (23.2),
+  // 300 217 (71.8) -> 202 (41.4), 520 978 (161) -> 975 (148).  The rule looks at N alone, so that
+  // blocks of columns agree with the whole U_T bit for bit (both plain tiles add in the order of k).
+  const long ti = (n + 31) / 32, big = ti * ((nc + 31) / 32);
+  const dim3 g32((n + 31) / 32, (nc + 31) / 32), g8((n + 7) / 8, (nc + 7) / 8), g4((n + 7) / 8, (nc + 3) / 4);
+  auto launch = [&](auto kernel, dim3 g, int threads) {
+    kernel<<<g, threads, 0, s>>>(S, A, n, cur.re, cur.im, prev.re, prev.im, acc.re, acc.im, out.re, out.im, nc, t);
+  };
+  if (ti * ti < 2 * 152) {
+    if (A) launch(k_term_dense_f64<4, 8, 32, 1, 1, true, 4>, g4, 128);
+    else launch(k_term_dense_f64<4, 8, 32, 1, 1, false, 4>, g4, 128);
+  } else if (big >= 2 * 152) {
+    if (A) launch(k_term_dense_f64<32, 32, 16, 2, 2, true>, g32, 256);
+    else launch(k_term_dense_f64<32, 32, 16, 2, 2, false>, g32, 256);
   } else {
-    dim3 g((n + 7) / 8, (nc + 7) / 8);
-    if (A)
-      k_term_dense_f64<8, 8, 32, 1, 1, true><<<g, 64, 0, s>>>(S, A, n, cur.re, cur.im, prev.re, prev.im, acc.re,
-                                                              acc.im, out.re, out.im, nc, t);
-    else
-      k_term_dense_f64<8, 8, 32, 1, 1, false><<<g, 64, 0, s>>>(S, A, n, cur.re, cur.im, prev.re, prev.im, acc.re,
-                                                               acc.im, out.re, out.im, nc, t);
+    if (A) launch(k_term_dense_f64<8, 8, 32, 1, 1, true>, g8, 64);
+    else launch(k_term_dense_f64<8, 8, 32, 1, 1, false>, g8, 64);
   }
 }
 

@@ -468,6 +468,26 @@ def test_column_blocks_assemble_build_UT(fq, case):
 
 
 # ------------------------------------------------------------------ dense FP64, resident kernel
+@pytest.mark.parametrize("n", [1, 2, 8, 9, 15, 16, 17, 24, 31, 33, 48, 49, 63, 64, 65, 79, 81, 96, 97, 112, 113, 127, 128,
+                               129, 131, 136, 161, 300])
+def test_dense_fp64_sizes(fq, n):
+    """Every count of entries a lane and of CTAs a cluster of the resident kernel (N <= 128), and the
+    tiles with split K above it, at their edges: three states against the oracle, and the same bits
+    among all N states."""
+    import torch
+    M = 40
+    h0, h1 = fi.goe(n, 2501), fi.goe(n, 2502)
+    drv = fi.Drive(0.2, 1.3, 1.1, 0.6)
+    plan = fq.Plan.dense(h0, h1, omega=drv.omega, f_ac=drv.f_ac, f_dc=drv.f_dc, phi0=drv.phi0, steps=M)
+    x0 = _unit_states(n, n, 2503)
+    few = plan.propagate(cuda_c128(x0[-3:]), 3, 6)
+    X = plan.propagate(cuda_c128(x0), 3, 6)
+    assert plan.check_status() == fq.FQ_OK
+    assert torch.equal(X[-3:], few)
+    ref = o.propagate_dense(h0, h1, o.plan_for_drive_dense(h0, h1, drv, M), x0[-3:].T, 3, 6).T
+    assert np.max(np.abs(to_np(few) - ref)) <= 1e-12
+
+
 @pytest.mark.parametrize("n", [1, 5, 32, 33, 64, 65, 100, 128])
 def test_dense_fp64_resident_kernel(fq, n):
     """The small-N resident chain (clusters of ceil(N/32) CTAs, 64 steps per launch) against the
