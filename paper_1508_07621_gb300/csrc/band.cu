@@ -7,8 +7,8 @@
 // every state, each step
 //   1. forms the rows of P_m once (k_band_rows): in the real gauge frame Omega~ = D Omega' D^+
 //      (gauge.cuh), row i of P(Omega') is P(Omega') e_i (P(Omega') is complex symmetric), computed
-//      by Clenshaw's recurrence in double-float arithmetic on a 96-row window around i, which holds
-//      its support i +- L; then P_m[i][k] = e^{-i beta h} e^{i theta_i} v_k e^{-i theta_k} in FP64;
+//      by Clenshaw's recurrence in double-float arithmetic on a window of 32, 64 or 96 rows (by L) around
+//      i, which holds its support i +- L; then P_m[i][k] = e^{-i beta h} e^{i theta_i} v_k e^{-i theta_k} in FP64;
 //   2. multiplies every state, held as fixed-point BF16 slices (as FQ_OZAKI does for dense
 //      operators, ozaki_core.cuh), by the band on the tensor cores (k_oz_band): a tile of 64
 //      operator rows [i0, i0 + 64) needs only the state columns [i0 - kh, i0 + 64 + kh) (kh = L
@@ -32,7 +32,7 @@
 //              (the input, the output, and entries the slices cannot hold)
 //   left       OZ_S slices [2 npl][ncp] BF16: row k the real parts of component k of every
 //              state, row npl + k the imaginary parts
-//   right      OZ_S slices [nrows / 64][kw][192] BF16: per 64-row block b and window column
+//   right      OZ_S slices [steps ahead][nrows / 64][kw][192] BF16: per 64-row block b and window column
 //              c = k - (64 b - kh) the columns -Im, Re, Im of rows 64 b .. 64 b + 63 of P_m
 //   cf, rot    per step (2 d, 2 e') and (cos, sin) theta of the gauge frame, FP64, [nsteps][nrows]
 #include <atomic>
@@ -42,9 +42,11 @@
 
 namespace {
 
-constexpr int BAND_LANE_ROWS = 3;                       // window rows per lane
-constexpr int BAND_WIN = 32 * BAND_LANE_ROWS;           // 96-row window, centre at position 48
-constexpr int BAND_MAXL = BAND_WIN / 2 - 1;             // support i +- L inside the window
+constexpr int BAND_LANE_ROWS = 3;                       // most window rows per lane
+// window rows per lane for a series of L terms: the window of 32 rows a lane row, centre at its middle,
+// holds the support i +- L
+__host__ __device__ constexpr int band_lane_rows(int L) { return L / 16 + 1; }
+constexpr int BAND_MAXL = 16 * BAND_LANE_ROWS - 1;
 constexpr int BAND_KH = 48;                             // widest K half-width of a 64-row block's window
 constexpr int BAND_KW = OZ_BN + 2 * BAND_KH;            // at most 160 columns of K per tile (10 stages)
 constexpr int BAND_ROWS_PER_CTA = 8;                    // one warp per operator row
@@ -71,21 +73,21 @@ __device__ __forceinline__ dflc shfl_dflc(dflc a, int delta, bool up) {
   return r;
 }
 
-// One Clenshaw update on the lane's three window rows: out = (2 Omega' x) - out (HALF: the
+// One Clenshaw update on the lane's LR window rows: out = (2 Omega' x) - out (HALF: the
 // closing Omega' x - out), plus c_k at the centre row (c = cc or i cc for IM), double-float.
-template <bool IM, bool HALF>
-__device__ __forceinline__ void band_apply(const dflc (&x)[BAND_LANE_ROWS], dflc (&out)[BAND_LANE_ROWS],
-                                           const dfl (&d)[BAND_LANE_ROWS], const dfl (&e)[BAND_LANE_ROWS], dfl el0,
+template <int LR, bool IM, bool HALF>
+__device__ __forceinline__ void band_apply(const dflc (&x)[LR], dflc (&out)[LR],
+                                           const dfl (&d)[LR], const dfl (&e)[LR], dfl el0,
                                            dfl cc, int lane) {
   const dflc z = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  dflc left = shfl_dflc(x[BAND_LANE_ROWS - 1], 1, true);
+  dflc left = shfl_dflc(x[LR - 1], 1, true);
   dflc right = shfl_dflc(x[0], 1, false);
-  if (lane == 0) left = z;    // beyond the window: never reached by the support (L <= 47)
+  if (lane == 0) left = z;    // beyond the window: never reached by the support
   if (lane == 31) right = z;
 #pragma unroll
-  for (int q = 0; q < BAND_LANE_ROWS; ++q) {
+  for (int q = 0; q < LR; ++q) {
     const dflc xm = q == 0 ? left : x[q - 1];
-    const dflc xp = q == BAND_LANE_ROWS - 1 ? right : x[q + 1];
+    const dflc xp = q == LR - 1 ? right : x[q + 1];
     dfl dq = d[q], el = q == 0 ? el0 : e[q - 1], eh = e[q];
     if (HALF) {  // the stored operator is 2 Omega'; halving is exact
       dq = {0.5f * dq.h, 0.5f * dq.l};
@@ -93,7 +95,7 @@ __device__ __forceinline__ void band_apply(const dflc (&x)[BAND_LANE_ROWS], dflc
       eh = {0.5f * eh.h, 0.5f * eh.l};
     }
     dflc acc = dflc_fma(dq, x[q], dflc_fma(el, xm, dflc_fma(eh, xp, dflc_neg(out[q]))));
-    if (q == 0 && lane == BAND_WIN / 2 / BAND_LANE_ROWS) {  // centre row: + c_k e_i
+    if (q == 0 && lane == 16) {  // centre row: + c_k e_i
       const dflc c = IM ? dflc{make_float2(0.f, cc.h), make_float2(0.f, cc.l)}
                         : dflc{make_float2(cc.h, 0.f), make_float2(cc.l, 0.f)};
       acc = dflc_add(acc, c);
@@ -119,8 +121,10 @@ typedef __nv_bfloat16 BandStage[3][BAND_KW][BAND_ROWS_PER_CTA];  // one slice's 
 
 // One warp forms row i < nrows of P_m (zero for i >= n) into column r8 of the staged 8-row block
 // of the right operand slices, and its exponent et[i].
+template <int LR>
 __device__ __forceinline__ void band_form_row(const BandRows& a, const BandCoef& coef, int i, int r8,
                                               BandStage* stage, int lane) {
+  constexpr int BAND_WIN = 32 * LR;
   const int n = a.n, L = a.L, kh = a.kh;
   const double2* __restrict__ cf = a.cf;
   const double2* __restrict__ rot = a.rot;
@@ -128,11 +132,11 @@ __device__ __forceinline__ void band_form_row(const BandRows& a, const BandCoef&
   const int w0 = i - BAND_WIN / 2;  // row of window position 0
   const dfl zd = {0.f, 0.f};
   const dflc zc = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  dfl d[BAND_LANE_ROWS], e[BAND_LANE_ROWS];
-  dflc A[BAND_LANE_ROWS], B[BAND_LANE_ROWS];
+  dfl d[LR], e[LR];
+  dflc A[LR], B[LR];
 #pragma unroll
-  for (int q = 0; q < BAND_LANE_ROWS; ++q) {
-    const int k = w0 + BAND_LANE_ROWS * lane + q;
+  for (int q = 0; q < LR; ++q) {
+    const int k = w0 + LR * lane + q;
     if (live && k >= 0 && k < n) {
       const double2 c = cf[k];
       d[q] = dfl_of(c.x);
@@ -145,43 +149,43 @@ __device__ __forceinline__ void band_form_row(const BandRows& a, const BandCoef&
     B[q] = zc;
   }
   dfl el0;
-  el0.h = __shfl_up_sync(0xffffffffu, e[BAND_LANE_ROWS - 1].h, 1);
-  el0.l = __shfl_up_sync(0xffffffffu, e[BAND_LANE_ROWS - 1].l, 1);
+  el0.h = __shfl_up_sync(0xffffffffu, e[LR - 1].h, 1);
+  el0.l = __shfl_up_sync(0xffffffffu, e[LR - 1].l, 1);
   if (lane == 0) el0 = (live && w0 >= 1 && w0 - 1 < n) ? dfl_of(cf[w0 - 1].y) : zd;
 
   if (live) {
     // b_L = c_L e_i, b_{L+1} = 0; then b_k = c_k e_i + 2 Omega' b_{k+1} - b_{k+2}
-    if (lane == BAND_WIN / 2 / BAND_LANE_ROWS) {
+    if (lane == 16) {
       const dfl cL = coef.c[L];
       A[0] = (L & 1) ? dflc{make_float2(0.f, cL.h), make_float2(0.f, cL.l)}
                      : dflc{make_float2(cL.h, 0.f), make_float2(cL.l, 0.f)};
     }
     int k = L - 1;
     while (k >= 2) {
-      if (k & 1) band_apply<true, false>(A, B, d, e, el0, coef.c[k], lane);
-      else band_apply<false, false>(A, B, d, e, el0, coef.c[k], lane);
+      if (k & 1) band_apply<LR, true, false>(A, B, d, e, el0, coef.c[k], lane);
+      else band_apply<LR, false, false>(A, B, d, e, el0, coef.c[k], lane);
       --k;
-      if (k & 1) band_apply<true, false>(B, A, d, e, el0, coef.c[k], lane);
-      else band_apply<false, false>(B, A, d, e, el0, coef.c[k], lane);
+      if (k & 1) band_apply<LR, true, false>(B, A, d, e, el0, coef.c[k], lane);
+      else band_apply<LR, false, false>(B, A, d, e, el0, coef.c[k], lane);
       --k;
     }
     if (k == 1) {  // b_1 into B, then the sum c_0 e_i + Omega' b_1 - b_2 into A
-      band_apply<true, false>(A, B, d, e, el0, coef.c[1], lane);
-      band_apply<false, true>(B, A, d, e, el0, coef.c[0], lane);
+      band_apply<LR, true, false>(A, B, d, e, el0, coef.c[1], lane);
+      band_apply<LR, false, true>(B, A, d, e, el0, coef.c[0], lane);
     } else {  // b_1 in A, b_2 in B: the sum into B, then moved to A
-      band_apply<false, true>(A, B, d, e, el0, coef.c[0], lane);
+      band_apply<LR, false, true>(A, B, d, e, el0, coef.c[0], lane);
 #pragma unroll
-      for (int q = 0; q < BAND_LANE_ROWS; ++q) A[q] = B[q];
+      for (int q = 0; q < LR; ++q) A[q] = B[q];
     }
   }
   // P_m[i][k] = e^{-i beta h} e^{i theta_i} v_k e^{-i theta_k} in FP64, and the row's scale
-  double vr[BAND_LANE_ROWS], vi[BAND_LANE_ROWS];
+  double vr[LR], vi[LR];
   unsigned long long key = 0;
   const double2 ri = live ? rot[i] : make_double2(1.0, 0.0);
   const double wr = a.ph_re * ri.x - a.ph_im * ri.y, wi = a.ph_re * ri.y + a.ph_im * ri.x;  // e^{-i beta h} e^{i theta_i}
 #pragma unroll
-  for (int q = 0; q < BAND_LANE_ROWS; ++q) {
-    const int k = w0 + BAND_LANE_ROWS * lane + q;
+  for (int q = 0; q < LR; ++q) {
+    const int k = w0 + LR * lane + q;
     vr[q] = vi[q] = 0.0;
     if (live && k >= 0 && k < n) {
       const double2 rk = rot[k];
@@ -202,13 +206,13 @@ __device__ __forceinline__ void band_form_row(const BandRows& a, const BandCoef&
   const int E = oz_exponent(key);
   const int r = i % OZ_BN;
   const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
-  // window positions [p0, p1) (the row's band; L <= kh) go to tile columns c = r + p - 48 + kh
+  // window positions [p0, p1) (the row's band; L <= kh) go to tile columns c = r + p - BAND_WIN / 2 + kh
   const int kw = OZ_BN + 2 * kh;
   const int p0 = BAND_WIN / 2 - kh > 0 ? BAND_WIN / 2 - kh : 0;
   const int p1 = BAND_WIN / 2 + kh + 1 < BAND_WIN ? BAND_WIN / 2 + kh + 1 : BAND_WIN;
 #pragma unroll
-  for (int q = 0; q < BAND_LANE_ROWS; ++q) {
-    const int pos = BAND_LANE_ROWS * lane + q;
+  for (int q = 0; q < LR; ++q) {
+    const int pos = LR * lane + q;
     if (pos < p0 || pos >= p1) continue;
     __nv_bfloat16 sr[OZ_S], si[OZ_S];
     oz_digits(vr[q], E, sr);
@@ -238,6 +242,14 @@ __device__ __forceinline__ void band_form_row(const BandRows& a, const BandCoef&
   if (lane == 0) a.et[i] = E;
 }
 
+__device__ __forceinline__ void band_form_row(const BandRows& a, const BandCoef& coef, int i, int r8,
+                                              BandStage* stage, int lane) {
+  const int lr = band_lane_rows(a.L);
+  if (lr == 1) band_form_row<1>(a, coef, i, r8, stage, lane);
+  else if (lr == 2) band_form_row<2>(a, coef, i, r8, stage, lane);
+  else band_form_row<3>(a, coef, i, r8, stage, lane);
+}
+
 // The staged block of rows 8 b8 .. 8 b8 + 7 to the MN-major band: column c of part (-Im, Re, Im)
 // of 64-row block b, rows r0 .. r0 + 7, at [(b kw + c) 192 + 64 part + r0] as one 16-byte piece;
 // thread t of nt.
@@ -251,13 +263,20 @@ __device__ __forceinline__ void band_store_block(const BandRows& a, int b8, cons
   }
 }
 
-// Rows i < nrows of P_m (the first step of a call; later steps' bands are formed inside the
-// previous step's product, k_oz_band): one warp per row, 8 rows per CTA (nrows is a multiple of
-// 64, so the grid holds no partial CTA and a CTA's rows share one 64-row block), staged in shared
-// memory and written as 16-byte pieces of the MN-major band.
-__global__ void __launch_bounds__(32 * BAND_ROWS_PER_CTA) k_band_rows(const BandRows a, const BandCoef coef) {
+// Rows i < nrows of the bands of gridDim.y steps (consecutive gauge tables, and slots of the band
+// buffer): one warp per row, 8 rows per CTA (nrows is a multiple of 64, so the grid holds no partial
+// CTA and a CTA's rows share one 64-row block), staged in shared memory and written as 16-byte pieces
+// of the MN-major band.  One step's rows are a few dozen dependent products on a handful of CTAs (14
+// us at 101 rows, 26 at 1501), and no step's band depends on the states, so the steps run together.
+__global__ void __launch_bounds__(32 * BAND_ROWS_PER_CTA)
+    k_band_rows(const __grid_constant__ BandRows first, const __grid_constant__ BandCoef coef, size_t slot) {
   __shared__ __align__(16) BandStage stage[OZ_S];
   const int lane = threadIdx.x & 31, r8 = threadIdx.x >> 5;
+  BandRows a = first;
+  a.cf += (size_t)blockIdx.y * a.nrows;
+  a.rot += (size_t)blockIdx.y * a.nrows;
+  a.right += (size_t)blockIdx.y * slot;
+  a.et += (size_t)blockIdx.y * a.nrows;
   band_form_row(a, coef, blockIdx.x * BAND_ROWS_PER_CTA + r8, r8, stage, lane);
   __syncthreads();
   band_store_block(a, blockIdx.x, stage, threadIdx.x, blockDim.x);
@@ -277,10 +296,13 @@ __device__ __forceinline__ void two_sum2(float2& a, float2& b) {  // (a, b) <- (
 }
 
 // The OZ_S slices of v = a + b (a double-float pair, packed as (re, im), |v| < 1/2 in units of
-// the row scale), with FP32 instructions only: t_q = v rounded to a multiple of 2^(-8(q+1)) by
-// adding and subtracting 1.5 2^(15 - 8q) (exact for |v| < 2^(14 - 8q)), then v -= t_q (exact) and a
-// two-sum keeps the remainder as a normalised pair.  t_q = d_q 2^(-8(q+1)) with |d_q| <= 128 (a
-// remainder is at most half a grid step), exact in BF16; the part below 2^-49 is dropped.
+// the row scale), with FP32 instructions only: t_q = a rounded to a multiple of 2^(-8(q+1)) by
+// adding and subtracting 1.5 2^(15 - 8q) (exact for |a| < 2^(14 - 8q)), then a -= t_q (exact).  With
+// the pair normalised, |b| <= 2^-26 has no bit among the first three digits: it joins the remainder
+// (at most 2^-25) after them by a two-sum, whose error joins in turn after the fourth digit.
+// t_q = d_q 2^(-8(q+1)) with |d_q| <= 128 (192 for q = 3, whose pairs go to the rounded accumulator),
+// exact in BF16, so the upper half of its FP32 pattern is the BF16 number; the part below 2^-49 is
+// dropped.  (A two-sum after every digit took twice the instructions.)
 // Returns |t_0| <= 1/2 for both parts (false: the value broke the scale bound).
 __device__ __forceinline__ bool df_digits2(float2 a, float2 b, __nv_bfloat16 (&dr)[OZ_S], __nv_bfloat16 (&di)[OZ_S]) {
   two_sum2(a, b);
@@ -290,10 +312,11 @@ __device__ __forceinline__ bool df_digits2(float2 a, float2 b, __nv_bfloat16 (&d
     const float c = __int_as_float((127 + 15 - 8 * q) << 23) * 1.5f;
     const float2 t = __fadd2_rn(__fadd2_rn(a, make_float2(c, c)), make_float2(-c, -c));
     if (q == 0) ok = fabsf(t.x) <= 0.5f && fabsf(t.y) <= 0.5f;
-    dr[q] = __float2bfloat16_rn(t.x);
-    di[q] = __float2bfloat16_rn(t.y);
+    dr[q] = __ushort_as_bfloat16((unsigned short)(__float_as_uint(t.x) >> 16));
+    di[q] = __ushort_as_bfloat16((unsigned short)(__float_as_uint(t.y) >> 16));
     a = __fadd2_rn(a, neg2f(t));
-    two_sum2(a, b);
+    if (q == 2) two_sum2(a, b);
+    if (q == 3) a = __fadd2_rn(a, b);
   }
   return ok;
 }
@@ -440,6 +463,25 @@ __device__ __forceinline__ uint64_t band_desc(uint32_t saddr) {
   return d;
 }
 
+// W columns of this warp's tensor-memory lanes
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[16]) { tmem_ld16(taddr, v); }
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v[q] = __uint_as_float(r[q]);
+}
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[4]) {
+  uint32_t r[4];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] = __uint_as_float(r[q]);
+}
+
 struct BandEpi {
   float4* out;     // X_m, double-float [nc][ld]
   unsigned int* kmax;  // per row of X_m: largest |hi| of re or im as an FP32 key (atomicMax)
@@ -462,21 +504,30 @@ struct BandEpi {
 // TMA stages (K = 16 each, 128-byte MN-major box rows), warp 1 issues the MMAs of the 21 slice
 // pairs into the four accumulators (512 tensor-memory columns), warps 2-17 drain them once per
 // tile into double-float registers, release the tensor memory and write the tile's slices for the
-// next step (and, at the last step, its double-float states) while the next tile's MMAs run.  Every wait is bounded; a wait that gives up records FQ_BIT_TIMEOUT, drains this CTA's own
-// copies and MMAs, frees tensor memory and returns.
+// next step (and, at the last step, its double-float states) while the next tile's MMAs run.  Every
+// wait is bounded; a wait that gives up records FQ_BIT_TIMEOUT, drains this CTA's own copies and
+// MMAs, frees tensor memory and returns.
+// CW: where there are few tiles, 16 / CW CTAs each run a tile's MMAs and take every drain warp's share
+// of CW of its 16 columns: with one tile a CTA, the drain and the slicing of 16 columns a thread come
+// after the MMAs and took as long as they did.
+// kr0: first K row of the step's band in the maps' buffer of several steps.
 constexpr int BAND_FORM_WARPS = 2;                             // warps 18, 19 form the next step's band
 constexpr int BAND_THREADS = OZ_THREADS + 32 * BAND_FORM_WARPS;  // 20 warps x 96 registers: 5 per SM sub-partition
-// Forming the next band inside the product pays once the product outlasts it: with two warps per
-// SM the formation takes about a third of a 10001-state product at dim 10001, and both scale with
-// the band's rows, so the rule is a number of states.
+// Forming the next band inside the product pays where it hides behind many tiles (10001 states: 1700 us
+// a step, against 1834 with a launch before each product).  Below 4096 states the bands of several steps are
+// formed in one launch ahead of their products (4001 states: 295 us a step against 326 inside).  A step in us before (a launch per step below 4096 states, one CTA a tile) and now,
+// states x rows: 41 x 41 45 -> 24, 301 x 301 50 -> 27, 24 x 1501 61 -> 36, 1501 x 1501 83 -> 61, 3001 x
+// 3001 217 -> 185, 10001 x 10001 1757 -> 1700.
 constexpr int BAND_FORM_MIN_STATES = 4096;
 constexpr size_t BAND_SMEM = OzCfg::SMEM + OZ_S * sizeof(BandStage);
 static_assert(BAND_SMEM <= 232448, "stages and the band staging fit the 227 KB of shared memory a CTA may use");
 
+template <int CW>
 __global__ void __launch_bounds__(BAND_THREADS, 1)
-    k_oz_band(const __grid_constant__ OzMaps maps, int tiles_j, int tiles_i, int npl, int kh, BandEpi e,
+    k_oz_band(const __grid_constant__ OzMaps maps, int tiles_j, int tiles_i, int npl, int kh, int kr0, BandEpi e,
               const __grid_constant__ BandRows next, const __grid_constant__ BandCoef coef, int form_next) {
   using Cfg = OzCfg;
+  constexpr int SHARE = 16 / CW;  // CTAs of a tile
   constexpr int STAGES = Cfg::STAGES;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -491,10 +542,10 @@ __global__ void __launch_bounds__(BAND_THREADS, 1)
   const uint32_t tfull = smem_u32(bars + 2 * STAGES), tempty0 = smem_u32(bars + 2 * STAGES + 1);
   const uint32_t done = smem_u32(bars + 2 * STAGES + 5);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ntiles = tiles_i * tiles_j;
+  const int ntiles = tiles_i * tiles_j * SHARE;
   const int nk = (OZ_BN + 2 * kh) / OZ_BKE;  // K stages of the tile window
-  auto coords = [&](int t, int& j0, int& i0) {
-    const int per = BAND_RG * tiles_i, g = t / per;
+  auto coords = [&](int u, int& j0, int& i0) {
+    const int t = u / SHARE, per = BAND_RG * tiles_i, g = t / per;
     const int gj = min(BAND_RG, tiles_j - g * BAND_RG), r = t - g * per;
     j0 = (g * BAND_RG + r % gj) * BM;
     i0 = (r / gj) * OZ_BN;
@@ -540,7 +591,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 1)
           const uint32_t bar = full0 + 8 * s;
           mbar_expect_tx(bar, Cfg::STAGE_BYTES);
           const int kx = i0 - kh + kb * OZ_BKE;  // K row of the states (any row); negative at the first block
-          const int kr = (i0 / OZ_BN) * (OZ_BN + 2 * kh) + kb * OZ_BKE;  // K row of the band block
+          const int kr = kr0 + (i0 / OZ_BN) * (OZ_BN + 2 * kh) + kb * OZ_BKE;  // K row of the band block
 #pragma unroll
           for (int q = 0; q < OZ_S; ++q) {
 #pragma unroll
@@ -623,7 +674,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 1)
       }
   } else {  // ---------------- drain and epilogue warps 2-17
     const int quarter = warp & 3, part = (warp - 2) >> 2;
-    const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * 16);
+    const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * 16 + CW * (blockIdx.x % SHARE));
     bool bad = false, ok = true;
     int it = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++it) {
@@ -636,21 +687,21 @@ __global__ void __launch_bounds__(BAND_THREADS, 1)
         ok = false;
         break;
       }
-      float2 hr[8], lr[8], hi[8], li[8];  // double-float sums of columns (2p, 2p + 1)
+      float2 hr[CW / 2], lr[CW / 2], hi[CW / 2], li[CW / 2];  // double-float sums of columns (2p, 2p + 1)
 #pragma unroll
-      for (int q = 0; q < 8; ++q) hr[q] = lr[q] = hi[q] = li[q] = make_float2(0.f, 0.f);
+      for (int q = 0; q < CW / 2; ++q) hr[q] = lr[q] = hi[q] = li[q] = make_float2(0.f, 0.f);
       // accumulator 3 first (the MMAs of the next tile start with it), each released once read
 #pragma unroll
       for (int grp = 3; grp >= 0; --grp) {
 #pragma unroll
         for (int part_im = 0; part_im < 2; ++part_im) {
-          float v[16];
-          tmem_ld16(trow + grp * (2 * OZ_BN) + part_im * OZ_BN, v);
+          float v[CW];
+          tmem_ld(trow + grp * (2 * OZ_BN) + part_im * OZ_BN, v);
           tmem_wait_ld();
           float2* h = part_im ? hi : hr;
           float2* l = part_im ? li : lr;
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
+          for (int q = 0; q < CW / 2; ++q) {
             const float2 w = make_float2(v[2 * q], v[2 * q + 1]);
             if (grp < 3) dd_add2(h[q], l[q], w);
             else l[q] = w;  // below 2^-24 of the leading sum: the low word carries it
@@ -671,8 +722,8 @@ __global__ void __launch_bounds__(BAND_THREADS, 1)
         __nv_bfloat16* lcol = e.lnext + j;
         bool fit = true;
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const int i = i0 + part * 16 + c;
+        for (int c = 0; c < CW; ++c) {
+          const int i = i0 + part * 16 + CW * (blockIdx.x % SHARE) + c;
           if (i < e.n) {
             int ex = ej + e.et[i];
             ex = ex < -126 ? -126 : (ex > 127 ? 127 : ex);
@@ -768,16 +819,20 @@ __global__ void k_band_store_t(const float4* __restrict__ x, double2* __restrict
 struct BandWs {
   double2* cf;
   double2* rot;
-  __nv_bfloat16* right[2];  // the band a product reads and the one it forms for the next step
-  int* et[2];
+  __nv_bfloat16* right;  // bands of `slots` steps: OZ_S slices of [slots][nrows / 64][kw][192]
+  int* et;               // [slots][nrows]
   __nv_bfloat16* left[2];  // slices of the states a product reads (alternating per step)
   int* es[2];
   int* ovf;
   unsigned int* kmax[2];  // row maxima of the states a product writes (alternating per step)
   float4* x[2];
-  int nrows, npl, ncp, kh, kw;
-  size_t rstride, astride;
+  int nrows, npl, ncp, kh, kw, slots;
+  size_t slot, rstride, astride;  // elements of one step's band in a slice, of a slice, of a state slice
 };
+
+// Bytes of bands formed ahead of their products, and the least number of steps (the pair a product
+// reads and forms).
+constexpr size_t BAND_AHEAD_BYTES = (size_t)64 << 20;
 
 size_t up256b(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -790,7 +845,9 @@ size_t band_layout(const fq_plan* p, int nc, int nsteps, void* base, BandWs* out
   // coordinate of the MN-major boxes, so the window may start on any row)
   w.kh = std::min(BAND_KH, (p->L + 7) / 8 * 8);
   w.kw = OZ_BN + 2 * w.kh;
-  w.rstride = (size_t)3 * w.nrows * w.kw;
+  w.slot = (size_t)3 * w.nrows * w.kw;
+  w.slots = (int)std::min<size_t>(std::max(nsteps, 2), std::max<size_t>(2, BAND_AHEAD_BYTES / (2 * OZ_S * w.slot)));
+  w.rstride = w.slot * w.slots;
   w.astride = (size_t)w.ncp * 2 * w.npl;
   char* b = (char*)base;
   size_t off = 0;
@@ -801,8 +858,8 @@ size_t band_layout(const fq_plan* p, int nc, int nsteps, void* base, BandWs* out
   };
   w.cf = (double2*)take(sizeof(double2) * (size_t)nsteps * w.nrows);
   w.rot = (double2*)take(sizeof(double2) * (size_t)nsteps * w.nrows);
-  for (int q = 0; q < 2; ++q) w.right[q] = (__nv_bfloat16*)take(sizeof(__nv_bfloat16) * OZ_S * w.rstride);
-  for (int q = 0; q < 2; ++q) w.et[q] = (int*)take(sizeof(int) * w.nrows);
+  w.right = (__nv_bfloat16*)take(sizeof(__nv_bfloat16) * OZ_S * w.rstride);
+  w.et = (int*)take(sizeof(int) * (size_t)w.nrows * w.slots);
   for (int q = 0; q < 2; ++q) w.left[q] = (__nv_bfloat16*)take(sizeof(__nv_bfloat16) * OZ_S * w.astride);
   for (int q = 0; q < 2; ++q) w.es[q] = (int*)take(sizeof(int) * w.ncp);
   w.ovf = (int*)take(sizeof(int) * w.ncp);
@@ -836,14 +893,16 @@ fq_status fq_band_propagate(fq_plan* p, const double* x0, double* x, int nc, int
     for (int q = 0; q < OZ_S; ++q) {
       // MN-major: 64-element (128-byte) box rows, 16 K rows per box
       if ((st = make_map(&maps[b].a[q], w.left[b] + q * w.astride, 2 * w.npl, w.ncp, OZ_BKE, 64)) != FQ_OK) return st;
-      if ((st = make_map(&maps[b].r[q], w.right[b] + q * w.rstride, (w.nrows / OZ_BN) * w.kw, 3 * OZ_BN, OZ_BKE, 64)) !=
-          FQ_OK)
+      if ((st = make_map(&maps[b].r[q], w.right + q * w.rstride, w.slots * (w.nrows / OZ_BN) * w.kw, 3 * OZ_BN, OZ_BKE,
+                         64)) != FQ_OK)
         return st;
     }
   static std::atomic<unsigned> attr_set{0};
   if (fq_first_on_device(attr_set)) {
-    cudaError_t e = cudaFuncSetAttribute(k_oz_band, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BAND_SMEM);
-    if (e != cudaSuccess) return fq_cuda_fail(e, "band kernel shared-memory attribute");
+    for (auto k : {k_oz_band<16>, k_oz_band<8>, k_oz_band<4>}) {
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BAND_SMEM);
+      if (e != cudaSuccess) return fq_cuda_fail(e, "band kernel shared-memory attribute");
+    }
   }
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
@@ -888,13 +947,18 @@ fq_status fq_band_propagate(fq_plan* p, const double* x0, double* x, int nc, int
     k_band_slice<<<dim3(w.ncp / 64, w.npl / 16), 256, 0, s>>>(w.x[0], n, w.npl, nc, w.npl, w.ncp, w.astride,
                                                               w.left[0], w.es[0], w.kmax[1]);
   }
-  // step m's band (its gauge tables, its buffer of the pair)
+  const bool fold = nc >= BAND_FORM_MIN_STATES;  // the next band formed inside each product
+  const int slots = fold ? 2 : w.slots;
+  // CTAs of a tile: as many of 4, 2, 1 as keep a product within one wave
+  const int share = ntiles * 4 <= sms ? 4 : (ntiles * 2 <= sms ? 2 : 1);
+  const auto product = share == 4 ? k_oz_band<4> : (share == 2 ? k_oz_band<8> : k_oz_band<16>);
+  // step m's band (its gauge tables, its slot of the buffer)
   auto rows_of = [&](int m) {
     BandRows r{};
     r.cf = w.cf + (size_t)m * w.nrows;
     r.rot = w.rot + (size_t)m * w.nrows;
-    r.right = w.right[m & 1];
-    r.et = w.et[m & 1];
+    r.right = w.right + (size_t)(m % slots) * w.slot;
+    r.et = w.et + (size_t)(m % slots) * w.nrows;
     r.rstride = w.rstride;
     r.ph_re = p->phase_re;
     r.ph_im = p->phase_im;
@@ -904,14 +968,15 @@ fq_status fq_band_propagate(fq_plan* p, const double* x0, double* x, int nc, int
     r.kh = w.kh;
     return r;
   };
-  const bool fold = w.ncp >= BAND_FORM_MIN_STATES;  // the next band formed inside each product
   int cur = 0;
   for (int m = 0; m < nsteps; ++m) {
     const int b = m & 1, nb = b ^ 1;
-    if (m == 0 || !fold) k_band_rows<<<w.nrows / BAND_ROWS_PER_CTA, 32 * BAND_ROWS_PER_CTA, 0, s>>>(rows_of(m), coef);
+    const int ahead = fold ? (m == 0 ? 1 : 0) : (m % slots == 0 ? std::min(slots, nsteps - m) : 0);
+    if (ahead)
+      k_band_rows<<<dim3(w.nrows / BAND_ROWS_PER_CTA, ahead), 32 * BAND_ROWS_PER_CTA, 0, s>>>(rows_of(m), coef, w.slot);
     // X_m = P_m X_{m-1}, X_m's slices for the next step at the scales X_{m-1}'s maxima predict,
     // and P_{m+1} formed alongside when folded (into the other band buffer, which product m-1 read)
-    e.et = w.et[b];
+    e.et = w.et + (size_t)(m % slots) * w.nrows;
     e.out = w.x[cur ^ 1];
     e.kmax = w.kmax[b];
     e.es = w.es[b];
@@ -920,8 +985,9 @@ fq_status fq_band_propagate(fq_plan* p, const double* x0, double* x, int nc, int
     e.write_states = m == nsteps - 1;
     fq_ktimer_start(p, s, "k_oz_band");
     const int form = fold && m + 1 < nsteps;
-    k_oz_band<<<std::min(ntiles, sms), BAND_THREADS, BAND_SMEM, s>>>(maps[b], tiles_j, tiles_i, w.npl, w.kh, e,
-                                                                     rows_of(form ? m + 1 : m), coef, form);
+    product<<<std::min(ntiles * share, sms), BAND_THREADS, BAND_SMEM, s>>>(
+        maps[b], tiles_j, tiles_i, w.npl, w.kh, (m % slots) * (w.nrows / OZ_BN) * w.kw, e, rows_of(form ? m + 1 : m),
+        coef, form);
     fq_ktimer_stop(p, s);
     // the slice scales of X_m, and the states that outgrew their predicted scale cut again
     k_band_fixup<<<w.ncp / 8, 256, 0, s>>>(w.x[cur ^ 1], n, w.npl, nc, w.npl, w.ncp, w.astride, w.left[nb],

@@ -174,3 +174,48 @@ def test_fp32_digit_cut_reconstructs_the_pair():
             assert d.denominator == 1 and abs(d) <= 128
             assert float(np.float32(t)) == float(t)
         assert abs(sum(Fraction(float(t)) for t in ts) - exact) <= Fraction(1, 2 ** 49)
+
+
+def _df_digits_merged(a, b):
+    """The cut with the low word merged once (df_digits2 of the kernel): three digits from the high word,
+    a two-sum of its remainder with the low word, the fourth digit, then the two-sum's error."""
+    a, b = _two_sum(_f(a), _f(b))
+    ts = []
+    for q in range(6):
+        c = _f(1.5 * 2.0 ** (15 - 8 * q))
+        t = _f(_f(a + c) - c)
+        ts.append(t)
+        a = _f(a - t)
+        if q == 2:
+            a, b = _two_sum(a, b)
+        if q == 3:
+            a = _f(a + b)
+    return ts
+
+
+def test_merged_digit_cut_reconstructs_the_pair():
+    """Digits 0 to 2 (all that the exact accumulators see) are integers of at most 128, digit 3 of at
+    most 192, the rest of at most 128, each times 2^(-8(q+1)); the FP32 pattern of a digit's slice has
+    a zero lower half (its upper half is the BF16 number); and the slices sum to the pair's exact
+    value within 2^-49, for pairs of every magnitude below 1/2, low words of either sign at their
+    largest, and values next to rounding ties of the digits."""
+    rng = np.random.default_rng(18)
+    cases = []
+    for _ in range(3000):
+        x = float(rng.uniform(-0.5, 0.5) * 2.0 ** -rng.integers(0, 40))
+        a = np.float32(x)
+        cases.append((a, np.float32(x - float(a))))
+        u = np.spacing(np.float32(abs(a))) / 2
+        cases.append((a, np.float32(u * rng.choice([-1.0, 1.0]) * rng.uniform(0.9, 1.0))))
+        tie = np.float32((rng.integers(-120, 120) + 0.5) * 2.0 ** (-8 * rng.integers(1, 4)))
+        cases.append((tie, np.float32(np.spacing(abs(tie)) / 2 * rng.uniform(-1, 1))))
+    for a, b in cases:
+        if not abs(float(a) + float(b)) < 0.5:
+            continue
+        ts = _df_digits_merged(a, b)
+        exact = Fraction(float(a)) + Fraction(float(b))
+        for q, t in enumerate(ts):
+            d = Fraction(float(t)) * Fraction(2) ** (8 * (q + 1))
+            assert d.denominator == 1 and abs(d) <= (192 if q == 3 else 128)
+            assert np.float32(t).view(np.uint32) & 0xFFFF == 0
+        assert abs(sum(Fraction(float(t)) for t in ts) - exact) <= Fraction(1, 2 ** 49) + Fraction(1, 2 ** 57)

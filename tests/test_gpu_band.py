@@ -137,6 +137,29 @@ def test_band_next_band_formed_inside_the_product(fq):
     assert err <= 1e-10
 
 
+@pytest.mark.parametrize("nb,nc,steps", [(40, 41, 400), (100, 1, 400), (300, 301, 60), (600, 601, 30), (900, 130, 12),
+                                         (2000, 2001, 7)])
+def test_band_steps_ahead_and_shared_tiles(fq, nb, nc, steps):
+    """Bands of several steps formed in one launch (more steps than the buffer holds at 2001 rows, one
+    buffer at the others), windows of 32 to 64 rows, and tiles shared by four, two and one CTA: three
+    states match the oracle, and the same bits come back when they run alone."""
+    d = fi.config_dimer(nb=nb)
+    d.drive = fi.Drive(0.2, 1.5, 3.0, 0.4)
+    plan = band_plan(fq, d)
+    n = d.n
+    x0 = np.exp(2j * np.pi * fi.uniform(2711, n * nc)).reshape(nc, n) * (1.0 + fi.uniform(2712, n * nc).reshape(nc, n))
+    x0 /= np.linalg.norm(x0, axis=1, keepdims=True)
+    X = to_np(plan.propagate(cuda_c128(x0), 1, 1 + steps))
+    assert plan.check_status() == fq.FQ_OK
+    few = sorted({0, nc // 2, nc - 1})
+    ref = o.propagate_tridiag(d.h0_diag, d.h0_off, d.h1_diag,
+                              o.plan_for_drive_tridiag(d.h0_diag, d.h0_off, d.h1_diag, d.drive, d.steps),
+                              x0[few].T, 1, 1 + steps).T
+    assert np.max(np.abs(X[few] - ref)) <= 1e-10
+    alone = to_np(plan.propagate(cuda_c128(x0[few]), 1, 1 + steps))
+    assert np.array_equal(alone, X[few])
+
+
 def test_band_propagation_captured_in_a_cuda_graph(fq):
     """The band path on a capturing stream: floquet_propagate of 4096 states (so the product also
     forms the next band) through 3 steps, captured in a CUDA graph and replayed twice, equals the
