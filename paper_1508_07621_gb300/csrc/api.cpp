@@ -247,6 +247,32 @@ fq_status propagate_impl(fq_plan* p, const double* x0, double* x, int nc, int m_
   return cuda_ok(cudaGetLastError(), "propagation kernels");
 }
 
+}  // namespace
+
+bool fq_prepare_tables(const fq_plan* p, int nc, void* ws, cudaStream_t s) {
+  StateWs w;
+  const fq_tables t{0, p->steps};
+  layout(p, nc, p->steps, ws, &w);
+  if (p->path == PATH_TRI_RESIDENT) fq_resident_tables(p, nc, t, w.coeff, s);
+  else if (p->path == PATH_TRI_TILE) fq_tile_tables(p, t, w.coeff, s);
+  else if (p->path == PATH_TRI_BAND) fq_band_tables(p, nc, t, w.coeff, s);
+  else return false;
+  return true;
+}
+
+fq_status fq_step_with_tables(fq_plan* p, const double* x0, double* x, int nc, int m, void* ws, cudaStream_t s) {
+  StateWs w;
+  const fq_tables t{0, p->steps};
+  layout(p, nc, p->steps, ws, &w);
+  fq_status st = FQ_EUNSUPPORTED;
+  if (p->path == PATH_TRI_RESIDENT) st = fq_launch_resident(p, w.coeff, x0, x, 0, nc, m, m + 1, s, &t);
+  else if (p->path == PATH_TRI_TILE) st = fq_tile_propagate(p, x0, x, nc, m, m + 1, 0, 0, w.coeff, s, &t);
+  else if (p->path == PATH_TRI_BAND) st = fq_band_propagate(p, x0, x, nc, m, m + 1, 0, 0, w.coeff, s, &t);
+  return st == FQ_OK ? cuda_ok(cudaGetLastError(), "step with prepared tables") : st;
+}
+
+namespace {
+
 void free_plan(fq_plan* p) {
   if (!p) return;
   for (void* d : {(void*)p->d_h0, (void*)p->d_h1, (void*)p->d_k, (void*)p->d_h0o, (void*)p->d_scal,

@@ -877,8 +877,15 @@ int fq_band_supported(int L) { return L >= 1 && L <= BAND_MAXL; }
 
 size_t fq_band_workspace(const fq_plan* p, int nc, int nsteps) { return band_layout(p, nc, nsteps, nullptr, nullptr); }
 
+void fq_band_tables(const fq_plan* p, int nc, fq_tables t, void* ws, cudaStream_t s) {
+  BandWs w;
+  band_layout(p, nc, t.n, ws, &w);
+  GaugeArgs ga{p->n, p->steps, p->d_h0, p->d_h0o, p->d_h1, p->d_k, p->d_scal, p->sbeta};
+  k_gauge_tile<double><<<t.n, GAUGE_NT, 0, s>>>(ga, w.nrows, t.m0, w.cf, w.rot);
+}
+
 fq_status fq_band_propagate(fq_plan* p, const double* x0, double* x, int nc, int m_begin, int m_end, int identity,
-                            int transpose_out, void* ws, cudaStream_t s) {
+                            int transpose_out, void* ws, cudaStream_t s, const fq_tables* pre) {
   fq_status st = encode_fn();
   if (st != FQ_OK) return st;
   const int n = p->n, L = p->L, nsteps = m_end - m_begin;
@@ -887,7 +894,8 @@ fq_status fq_band_propagate(fq_plan* p, const double* x0, double* x, int nc, int
     return FQ_EUNSUPPORTED;
   }
   BandWs w;
-  band_layout(p, nc, nsteps, ws, &w);
+  const fq_tables tab = pre ? *pre : fq_tables{m_begin, nsteps};
+  band_layout(p, nc, tab.n, ws, &w);
   OzMaps maps[2];  // per step parity: the state slices and the band a product reads
   for (int b = 0; b < 2; ++b)
     for (int q = 0; q < OZ_S; ++q) {
@@ -918,8 +926,7 @@ fq_status fq_band_propagate(fq_plan* p, const double* x0, double* x, int nc, int
         ce = cudaMemsetAsync(w.left[1] + q * w.astride + (size_t)(part * w.npl + n) * w.ncp, 0,
                              sizeof(__nv_bfloat16) * (size_t)(w.npl - n) * w.ncp, s);
   if (ce != cudaSuccess) return fq_cuda_fail(ce, "band workspace clear");
-  GaugeArgs ga{p->n, p->steps, p->d_h0, p->d_h0o, p->d_h1, p->d_k, p->d_scal, p->sbeta};
-  k_gauge_tile<double><<<nsteps, GAUGE_NT, 0, s>>>(ga, w.nrows, m_begin, w.cf, w.rot);
+  if (!pre) fq_band_tables(p, nc, tab, ws, s);
   k_band_load<<<band_grid((size_t)nc * w.npl), 256, 0, s>>>(identity ? nullptr : (const double2*)x0, w.x[0], nc, n,
                                                             w.npl);
   BandCoef coef{};
@@ -955,8 +962,8 @@ fq_status fq_band_propagate(fq_plan* p, const double* x0, double* x, int nc, int
   // step m's band (its gauge tables, its slot of the buffer)
   auto rows_of = [&](int m) {
     BandRows r{};
-    r.cf = w.cf + (size_t)m * w.nrows;
-    r.rot = w.rot + (size_t)m * w.nrows;
+    r.cf = w.cf + (size_t)(m_begin - tab.m0 + m) * w.nrows;
+    r.rot = w.rot + (size_t)(m_begin - tab.m0 + m) * w.nrows;
     r.right = w.right + (size_t)(m % slots) * w.slot;
     r.et = w.et + (size_t)(m % slots) * w.nrows;
     r.rstride = w.rstride;

@@ -45,6 +45,12 @@ struct fq_tile_shape {
   int n, k;
 };
 
+// Gauge tables of steps [m0, m0 + n) that a caller has put into a tridiagonal path's workspace, laid out
+// for those n steps: a caller that walks the steps one call at a time forms them together.
+struct fq_tables {
+  int m0, n;
+};
+
 struct fq_plan {
   // problem
   int n = 0, steps = 0, format = 0, precision = 0, drive_kind = 0, stride = 16, L = 0;
@@ -220,14 +226,22 @@ size_t fq_tile_workspace(const fq_plan* p, int nc, int nsteps);
 int fq_band_supported(int L);
 size_t fq_band_workspace(const fq_plan* p, int nc, int nsteps);
 fq_status fq_band_propagate(fq_plan* p, const double* x0, double* x, int nc, int m_begin, int m_end, int identity,
-                            int transpose_out, void* ws, cudaStream_t s);
+                            int transpose_out, void* ws, cudaStream_t s, const fq_tables* pre = nullptr);
 fq_status fq_tile_propagate(fq_plan* p, const double* x0, double* x, int nc, int m_begin, int m_end, int identity,
-                            int transpose_out, void* ws, cudaStream_t s);
+                            int transpose_out, void* ws, cudaStream_t s, const fq_tables* pre = nullptr);
+// the gauge tables of steps [t.m0, t.m0 + t.n) into a workspace laid out for them (fq_tables)
+void fq_band_tables(const fq_plan* p, int nc, fq_tables t, void* ws, cudaStream_t s);
+void fq_tile_tables(const fq_plan* p, fq_tables t, void* ws, cudaStream_t s);
+void fq_resident_tables(const fq_plan* p, int nc, fq_tables t, void* coeff, cudaStream_t s);
+// Forms a tridiagonal plan's tables of every step in `ws` (sized by floquet_workspace_size); false for a
+// path without such tables.  Then one step on nc states with them (api.cpp).
+bool fq_prepare_tables(const fq_plan* p, int nc, void* ws, cudaStream_t s);
+fq_status fq_step_with_tables(fq_plan* p, const double* x0, double* x, int nc, int m, void* ws, cudaStream_t s);
 size_t fq_resident_coeff_bytes(int n, int steps);
 // per-step (2 d, 2 e') of the gauge-real operator and the frame rotations, into `coeff`
 void fq_launch_gauge_coeffs(const fq_plan* p, int nc, int m_begin, int nsteps, void* coeff, cudaStream_t s);
 fq_status fq_launch_resident(const fq_plan* p, const void* coeff, const double* x0, double* x, int transpose_out,
-                             int nc, int m_begin, int m_end, cudaStream_t s);
+                             int nc, int m_begin, int m_end, cudaStream_t s, const fq_tables* pre = nullptr);
 
 // FP64 emulation on the tensor cores (ozaki.cu, ozaki_grad.cu)
 size_t fq_grad_ozaki_workspace(const fq_plan* p);

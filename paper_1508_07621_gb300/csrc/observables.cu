@@ -6,6 +6,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "internal.h"
@@ -24,56 +25,89 @@ __device__ double block_sum(double v, double* red) {
   return s;  // valid in thread 0
 }
 
-// acc[r] += w <x_r| c0 H0 + c1 H1 |x_r>, tridiagonal H0 (diag, off), diagonal H1; one CTA per row.
-__global__ void k_expect_tri(const double2* __restrict__ x, int n, const double* __restrict__ h0d,
-                             const double* __restrict__ h0o, const double* __restrict__ h1d, double c0, double c1,
-                             double w, double* acc) {
-  __shared__ double red[32];
-  const double2* row = x + (size_t)blockIdx.x * n;
+constexpr int EXPECT_STATES = 4;  // states per CTA, a warp each
+constexpr int EXPECT_CHUNK = 512;  // tridiagonal: rows of H staged at a time
+constexpr int EXPECT_BLOCK = 32;   // dense: rows of H per CTA
+
+// acc[r] += w <x_r| c0 H0 + c1 H1 |x_r>, tridiagonal H0 (diag, off), diagonal H1:
+// sum_i d_i |x_i|^2 + 2 c0 o_i Re(conj(x_i) x_{i+1}), d = c0 diag + c1 H1.  Bound by the FP64 pipes (64
+// cycles a warp and instruction): 6 instructions an entry, d and o once for a CTA's states (one state per
+// CTA and both neighbours of every entry took 14).
+__global__ void __launch_bounds__(32 * EXPECT_STATES)
+    k_expect_tri(const double2* __restrict__ x, int nc, int n, const double* __restrict__ h0d,
+                 const double* __restrict__ h0o, const double* __restrict__ h1d, double c0, double c1, double w,
+                 double* acc) {
+  __shared__ double2 sh[EXPECT_CHUNK];  // (d_i, 2 c0 o_i)
+  const int lane = threadIdx.x & 31, r = blockIdx.x * EXPECT_STATES + (threadIdx.x >> 5);
+  const double2* row = x + (size_t)min(r, nc - 1) * n;
   double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double2 xi = row[i];
-    const double d = c0 * h0d[i] + c1 * h1d[i];
-    double yr = d * xi.x, yi = d * xi.y;
-    if (i > 0) {
-      const double2 xl = row[i - 1];
-      yr += c0 * h0o[i - 1] * xl.x;
-      yi += c0 * h0o[i - 1] * xl.y;
+  for (int i0 = 0; i0 < n; i0 += EXPECT_CHUNK) {
+    __syncthreads();
+    for (int q = threadIdx.x; q < EXPECT_CHUNK; q += 32 * EXPECT_STATES) {
+      const int i = i0 + q;
+      sh[q] = make_double2(i < n ? fma(c0, h0d[i], c1 * h1d[i]) : 0.0, i + 1 < n ? 2.0 * c0 * h0o[i] : 0.0);
     }
-    if (i + 1 < n) {
-      const double2 xr = row[i + 1];
-      yr += c0 * h0o[i] * xr.x;
-      yi += c0 * h0o[i] * xr.y;
+    __syncthreads();
+    const int m = min(EXPECT_CHUNK, n - i0);
+#pragma unroll 4
+    for (int q = lane; q < m; q += 32) {
+      const int i = i0 + q;
+      const double2 a = row[i], b = i + 1 < n ? row[i + 1] : make_double2(0.0, 0.0);
+      s = fma(sh[q].x, fma(a.x, a.x, a.y * a.y), fma(sh[q].y, fma(a.x, b.x, a.y * b.y), s));
     }
-    s += xi.x * yr + xi.y * yi;  // Re(conj(x_i) y_i)
   }
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) acc[blockIdx.x] += w * s;
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0 && r < nc) acc[r] += w * s;
 }
 
-// acc[r] += w <x_r| c0 H0 + c1 H1 |x_r>, dense real-symmetric H0, H1; one CTA per row, the row of
-// x staged in shared memory.
-__global__ void k_expect_dense(const double2* __restrict__ x, int n, const double* __restrict__ h0,
-                               const double* __restrict__ h1, double c0, double c1, double w, double* acc) {
-  extern __shared__ double2 xs[];
-  __shared__ double red[32];
-  const double2* row = x + (size_t)blockIdx.x * n;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) xs[k] = row[k];
-  __syncthreads();
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double* a = h0 + (size_t)i * n;
-    const double* b = h1 + (size_t)i * n;
-    double yr = 0.0, yi = 0.0;
-    for (int k = 0; k < n; ++k) {
-      const double hk = c0 * a[k] + c1 * b[k];
-      yr = fma(hk, xs[k].x, yr);
-      yi = fma(hk, xs[k].y, yi);
+// A = c0 H0 + c1 H1
+__global__ void k_expect_form(const double* __restrict__ h0, const double* __restrict__ h1, size_t nn, double c0,
+                              double c1, double* __restrict__ a) {
+  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < nn; q += (size_t)gridDim.x * blockDim.x)
+    a[q] = fma(c0, h0[q], c1 * h1[q]);
+}
+
+// acc[b][r] += w times the part of <x_r| A |x_r> (A dense real-symmetric) of the rows of block b: sum over
+// its rows i of x_i^* (A_ii x_i + 2 sum_{k < i} A_ik x_k), blockwise, so that only the blocks on and left of
+// the diagonal are visited.  Lane = row i, warp = state; the longest rows of blocks start first, and few
+// states a CTA balance the rest.  Bound by the FP64 pipes: half of the 2 N^2 multiply-adds a state.  (One
+// state per CTA, a thread per row of H walking it, formed A for every state on uncoalesced reads: 151 us
+// at N = 256 and 256 states, now 53 us.)
+__global__ void __launch_bounds__(32 * EXPECT_STATES)
+    k_expect_dense(const double2* __restrict__ x, int nc, int n, const double* __restrict__ A, double w, double* acc) {
+  __shared__ double sa[EXPECT_BLOCK][EXPECT_BLOCK + 1];      // [k][i]
+  __shared__ double2 sx[EXPECT_STATES][EXPECT_BLOCK];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = gridDim.y - 1 - blockIdx.y, i0 = b * EXPECT_BLOCK;
+  const int r = blockIdx.x * EXPECT_STATES + warp;
+  double yr = 0.0, yi = 0.0;
+  for (int kb = 0; kb <= b; ++kb) {
+    const int k0 = kb * EXPECT_BLOCK;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < EXPECT_BLOCK / EXPECT_STATES; ++q) {
+      const int ii = warp + EXPECT_STATES * q;
+      const bool in = i0 + ii < n && k0 + lane < n;
+      sa[lane][ii] = in ? A[(size_t)(i0 + ii) * n + k0 + lane] : 0.0;
     }
-    s += xs[i].x * yr + xs[i].y * yi;
+    sx[warp][lane] = r < nc && k0 + lane < n ? x[(size_t)r * n + k0 + lane] : make_double2(0.0, 0.0);
+    __syncthreads();
+    if (kb == b) {
+      yr += yr;
+      yi += yi;
+    }
+#pragma unroll 8
+    for (int kk = 0; kk < EXPECT_BLOCK; ++kk) {
+      const double a = sa[kk][lane];
+      const double2 v = sx[warp][kk];
+      yr = fma(a, v.x, yr);
+      yi = fma(a, v.y, yi);
+    }
   }
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) acc[blockIdx.x] += w * s;
+  const double2 v = sx[warp][lane];  // the diagonal block's entries: rows i0 + lane
+  double s = fma(v.x, yr, v.y * yi);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0 && r < nc) acc[(size_t)b * nc + r] += w * s;
 }
 
 // sigma[r] = |1 - e^{i eps_r T} <phi_r|moved_r>| (Eq. 20, reading R14), one CTA per state row.
@@ -99,17 +133,30 @@ __global__ void k_overlap_sigma(const double2* __restrict__ phi, const double2* 
   }
 }
 
-__global__ void k_scale_out(const double* acc, int nc, double s, double* out) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nc; q += gridDim.x * blockDim.x) out[q] = s * acc[q];
+// out[r] = s * (sum of the nb blocks' parts)
+__global__ void k_scale_out(const double* acc, int nc, int nb, double s, double* out) {
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nc; q += gridDim.x * blockDim.x) {
+    double t = 0.0;
+    for (int b = 0; b < nb; ++b) t += acc[(size_t)b * nc + q];
+    out[q] = s * t;
+  }
 }
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+
+// blocks of partial sums per state
+int expect_blocks(const fq_plan* p) { return p->format == FQ_DENSE ? (p->n + EXPECT_BLOCK - 1) / EXPECT_BLOCK : 1; }
+
+// the sums, and A of a dense plan
+size_t expect_bytes(const fq_plan* p, int32_t ncols) {
+  return up256((size_t)ncols * expect_blocks(p) * 8) + (p->format == FQ_DENSE ? up256((size_t)p->n * p->n * 8) : 0);
+}
 
 }  // namespace
 
 extern "C" size_t floquet_observable_workspace_size(const fq_plan* p, int32_t ncols) {
   if (!p || ncols < 1) return 0;
-  return up256((size_t)ncols * p->n * 16) + up256((size_t)ncols * 8) + floquet_workspace_size(p, ncols);
+  return up256((size_t)ncols * p->n * 16) + expect_bytes(p, ncols) + floquet_workspace_size(p, ncols);
 }
 
 static fq_status floquet_average_observable_body(fq_plan* p, const void* d_X0, int32_t ncols, double a0, double a1,
@@ -137,10 +184,12 @@ static fq_status floquet_average_observable_body(fq_plan* p, const void* d_X0, i
   char* b = (char*)d_ws;
   double* X = (double*)b;
   double* acc = (double*)(b + up256((size_t)ncols * n * 16));
-  void* inner = b + up256((size_t)ncols * n * 16) + up256((size_t)ncols * 8);
-  const size_t inner_bytes = ws_bytes - up256((size_t)ncols * n * 16) - up256((size_t)ncols * 8);
+  void* inner = b + up256((size_t)ncols * n * 16) + expect_bytes(p, ncols);
+  const size_t inner_bytes = ws_bytes - up256((size_t)ncols * n * 16) - expect_bytes(p, ncols);
+  const int nb = expect_blocks(p);
+  double* A = (double*)((char*)acc + up256((size_t)ncols * nb * 8));  // dense: c0 H0 + c1 H1
   cudaError_t e = cudaMemcpyAsync(X, d_X0, (size_t)ncols * n * 16, cudaMemcpyDeviceToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, (size_t)ncols * 8, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, (size_t)ncols * nb * 8, s);
   if (e != cudaSuccess) return fq_cuda_fail(e, "observable setup");
   const double h = p->h;
   std::vector<double> w(M + 1, h);
@@ -154,23 +203,26 @@ static fq_status floquet_average_observable_body(fq_plan* p, const void* d_X0, i
     const double t = m * h;
     const double f = fq_drive_f(0, p->f_dc, p->f_ac, p->omega, p->phi0, t);
     const double c0 = a0, c1 = a1 + s_drive * f;
-    if (p->format == FQ_TRIDIAG)
-      k_expect_tri<<<ncols, 256, 0, s>>>((const double2*)X, n, p->d_h0, p->d_h0o, p->d_h1, c0, c1, w[m], acc);
-    else
-      k_expect_dense<<<ncols, 256, (size_t)n * sizeof(double2), s>>>((const double2*)X, n, p->d_h0, p->d_h1, c0, c1,
-                                                                      w[m], acc);
+    const int groups = (ncols + EXPECT_STATES - 1) / EXPECT_STATES;
+    if (p->format == FQ_TRIDIAG) {
+      k_expect_tri<<<groups, 32 * EXPECT_STATES, 0, s>>>((const double2*)X, ncols, n, p->d_h0, p->d_h0o, p->d_h1, c0, c1,
+                                                         w[m], acc);
+    } else {
+      const size_t nn = (size_t)n * n;
+      k_expect_form<<<(int)std::min<size_t>((nn + 255) / 256, 152 * 16), 256, 0, s>>>(p->d_h0, p->d_h1, nn, c0, c1, A);
+      k_expect_dense<<<dim3(groups, nb), 32 * EXPECT_STATES, 0, s>>>((const double2*)X, ncols, n, A, w[m], acc);
+    }
   };
-  if (p->format == FQ_DENSE) {
-    e = cudaFuncSetAttribute(k_expect_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, n * (int)sizeof(double2));
-    if (e != cudaSuccess) return fq_cuda_fail(e, "observable smem attribute");
-  }
+  // a tridiagonal plan's gauge tables for all steps at once: one CTA forms a step's, for tens of us
+  const bool tables = fq_prepare_tables(p, ncols, inner, s);
   observe(0);
   for (int m = 0; m < M; ++m) {
-    fq_status st = floquet_propagate(p, X, X, ncols, m, m + 1, inner, inner_bytes, stream);
+    const fq_status st = tables ? fq_step_with_tables(p, X, X, ncols, m, inner, s)
+                                : floquet_propagate(p, X, X, ncols, m, m + 1, inner, inner_bytes, stream);
     if (st != FQ_OK) return st;
     observe(m + 1);
   }
-  k_scale_out<<<(ncols + 255) / 256, 256, 0, s>>>(acc, ncols, 1.0 / p->period, d_avg);
+  k_scale_out<<<(ncols + 255) / 256, 256, 0, s>>>(acc, ncols, nb, 1.0 / p->period, d_avg);
   e = cudaGetLastError();
   return e == cudaSuccess ? FQ_OK : fq_cuda_fail(e, "observable kernels");
 }

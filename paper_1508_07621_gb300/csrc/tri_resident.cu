@@ -76,11 +76,13 @@ __host__ __device__ __forceinline__ size_t res_index(int i, int nt, int ept) {
 }
 
 // CTA s < nsteps (step m = m_begin + s): cf[s][k] = (2 d_k, 2 e'_k) and
-//   rot[s][k] = e^{i (theta^{m-1}_k - theta^m_k)}  (theta^{m_begin - 1} := 0: input frame);
+//   rot[s][k] = e^{i (theta^{m-1}_k - theta^m_k)}  (theta^{m_begin - 1} := 0: input frame; with `apart`
+//   every step's theta^{m-1} := 0, for calls of one step each);
 // CTA s = nsteps: rot[nsteps][k] = e^{i theta^{m_end - 1}_k} (back to the original frame).
 // FP64 arithmetic throughout (the Magnus combination and rescaling stay FP64), FP32 stores.
-__global__ void __launch_bounds__(GAUGE_NT) k_gauge_coeffs(GaugeArgs p, int ld, int m_begin, int nsteps, int rnt,
-                                                           int rept, float2* __restrict__ cf, float2* __restrict__ rot) {
+__global__ void __launch_bounds__(GAUGE_NT) k_gauge_coeffs(GaugeArgs p, int ld, int m_begin, int nsteps, int apart,
+                                                           int rnt, int rept, float2* __restrict__ cf,
+                                                           float2* __restrict__ rot) {
   const size_t stride = (size_t)rnt * rept;  // one step, resident order; rows >= ld stay as set below
   __shared__ double sw[64];
   const int s = blockIdx.x;
@@ -90,7 +92,7 @@ __global__ void __launch_bounds__(GAUGE_NT) k_gauge_coeffs(GaugeArgs p, int ld, 
   if (s < nsteps) {
     const int m = m_begin + s;
     phases(p, m, ld, C, thA, sw);
-    phases(p, s == 0 ? -1 : m - 1, ld, C, thB, sw);
+    phases(p, s == 0 || apart ? -1 : m - 1, ld, C, thB, sw);
 #pragma unroll
     for (int q = 0; q < GAUGE_MAXC; ++q) {
       const int k = k0 + q;
@@ -312,7 +314,8 @@ struct Chain {
 
 template <int EPT, int FNT>
 __global__ void __launch_bounds__(FNT ? FNT : res_max_threads(EPT), 1)
-k_tri_resident(const float4* __restrict__ cf_all, const float4* __restrict__ rot_all, int n, int L, int nsteps,
+k_tri_resident(const float4* __restrict__ cf_all, const float4* __restrict__ rot_all,
+               const float4* __restrict__ rot_end, float end_sign, int n, int L, int nsteps,
                const double2* __restrict__ x0, double2* __restrict__ xout, int transpose_out, ResCoef coef,
                float ph_re, float ph_im, float clenshaw_bound, unsigned int* status) {
   using Ch = Chain<EPT, FNT>;
@@ -338,24 +341,30 @@ k_tri_resident(const float4* __restrict__ cf_all, const float4* __restrict__ rot
   const int i0 = t * EPT;
   const size_t stride = (size_t)NP * NT;  // one step of cf / rot, in float4
 
-  // initial state (registers) and its squared norm (unitarity bounds every later entry by it)
+  // position of row i among the float2 of the staged state (a row pair is a float4 of sv's layout)
+  float2* const stage = reinterpret_cast<float2*>(smem_raw);
+  auto slot = [](int i) {
+    const int th = i / EPT, q = i - th * EPT;
+    return 2 * (th * Ch::COL + (q >> 1) * Ch::ROW) + (q & 1);
+  };
+  // initial state (registers) and its squared norm (unitarity bounds every later entry by it); given
+  // states pass through shared memory, so that the threads read consecutive rows
   float2 A[EPT], B[EPT];
   float nrm = 0.f;
+  if (x0) {
+    for (int i = t; i < n; i += NT) {
+      const double2 zz = x0[(size_t)j * n + i];
+      stage[slot(i)] = make_float2((float)zz.x, (float)zz.y);
+    }
+    __syncthreads();
+  }
 #pragma unroll
   for (int q = 0; q < EPT; ++q) {
     const int i = i0 + q;
-    float a = 0.f, b = 0.f;
-    if (i < n) {
-      if (x0) {
-        const double2 zz = x0[(size_t)j * n + i];
-        a = (float)zz.x;
-        b = (float)zz.y;
-      } else {
-        a = i == j ? 1.f : 0.f;
-      }
-    }
-    A[q] = f2(a, b);
-    nrm = fmaf(a, a, fmaf(b, b, nrm));
+    float2 a = f2(0.f, 0.f);
+    if (i < n) a = x0 ? stage[slot(i)] : f2(i == j ? 1.f : 0.f, 0.f);
+    A[q] = a;
+    nrm = fmaf(a.x, a.x, fmaf(a.y, a.y, nrm));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
@@ -406,10 +415,11 @@ k_tri_resident(const float4* __restrict__ cf_all, const float4* __restrict__ rot
   // back to the original frame: X = D_last v; unitarity check on the state's norm (a spectral
   // bound that is too tight keeps the entries small but makes the truncated series non-unitary)
   float nrm_end = 0.f;
-  const size_t offr = (size_t)nsteps * stride;
 #pragma unroll
   for (int p = 0; p < NP; ++p) {
-    const float4 r = rot_all[offr + p * NT + t];
+    float4 r = rot_end[p * NT + t];
+    r.y *= end_sign;
+    r.w *= end_sign;
     const float2 a = A[2 * p], b = A[2 * p + 1];
     A[2 * p] = f2(r.x * a.x - r.y * a.y, r.x * a.y + r.y * a.x);
     A[2 * p + 1] = f2(r.z * b.x - r.w * b.y, r.z * b.y + r.w * b.x);
@@ -429,19 +439,26 @@ k_tri_resident(const float4* __restrict__ cf_all, const float4* __restrict__ rot
   }
   __syncthreads();
   if (t == 0 && C.sh->bad) atomicOr(status, FQ_BIT_BOUND);
+  if (transpose_out) {
 #pragma unroll
-  for (int q = 0; q < EPT; ++q) {
-    const int i = i0 + q;
-    if (i < n) {
-      const double2 x = make_double2((double)A[q].x, (double)A[q].y);
-      if (transpose_out) xout[(size_t)i * n + j] = x;
-      else xout[(size_t)j * n + i] = x;
+    for (int q = 0; q < EPT; ++q) {
+      const int i = i0 + q;
+      if (i < n) xout[(size_t)i * n + j] = make_double2((double)A[q].x, (double)A[q].y);
     }
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < EPT; ++q) stage[slot(i0 + q)] = A[q];  // the last step's state rows are read
+  __syncthreads();
+  for (int i = t; i < n; i += NT) {
+    const float2 a = stage[slot(i)];
+    xout[(size_t)j * n + i] = make_double2((double)a.x, (double)a.y);
   }
 }
 
 template <int EPT, int FNT>
-fq_status launch_cfg(const fq_plan* p, const float4* cf, const float4* rot, const double* x0, double* x,
+fq_status launch_cfg(const fq_plan* p, const float4* cf, const float4* rot, const float4* rot_end, float end_sign,
+                     const double* x0, double* x,
                      int transpose_out, int nc, int nsteps, const ResCoef& coef, float bcl, int nt, cudaStream_t s) {
   const size_t smem = res_smem(nt, EPT);
   static std::atomic<unsigned> attr_set{0};
@@ -451,7 +468,7 @@ fq_status launch_cfg(const fq_plan* p, const float4* cf, const float4* rot, cons
     if (e != cudaSuccess) return fq_cuda_fail(e, "resident kernel smem attribute");
   }
   fq_ktimer_start(p, s, "k_tri_resident");
-  k_tri_resident<EPT, FNT><<<nc, nt, smem, s>>>(cf, rot, p->n, p->L, nsteps, (const double2*)x0, (double2*)x, transpose_out,
+  k_tri_resident<EPT, FNT><<<nc, nt, smem, s>>>(cf, rot, rot_end, end_sign, p->n, p->L, nsteps, (const double2*)x0, (double2*)x, transpose_out,
                                            coef, (float)p->phase_re, (float)p->phase_im, bcl, p->d_status);
   fq_ktimer_stop(p, s);
   cudaError_t e = cudaGetLastError();
@@ -523,16 +540,33 @@ void fq_launch_gauge_coeffs(const fq_plan* p, int nc, int m_begin, int nsteps, v
   // and let the kernel overwrite every row < ld; rot padding only multiplies zeros.
   cudaMemsetAsync(coeff, 0, (2 * (size_t)nsteps + 1) * (size_t)nt * ept * sizeof(float2), s);
   GaugeArgs ga{p->n, p->steps, p->d_h0, p->d_h0o, p->d_h1, p->d_k, p->d_scal, p->sbeta};
-  k_gauge_coeffs<<<nsteps + 1, GAUGE_NT, 0, s>>>(ga, ld, m_begin, nsteps, nt, ept, cf, rot);
+  k_gauge_coeffs<<<nsteps + 1, GAUGE_NT, 0, s>>>(ga, ld, m_begin, nsteps, 0, nt, ept, cf, rot);
+}
+
+// Tables of steps taken one call at a time: each step enters from the original frame, and leaves by the
+// conjugate of the same rotation.
+void fq_resident_tables(const fq_plan* p, int nc, fq_tables t, void* coeff, cudaStream_t s) {
+  const int ld = (p->n + 3) & ~3;
+  int nt, ept;
+  res_config(p->n, nc, &nt, &ept);
+  const size_t rows = (size_t)nt * ept;
+  float2* cf = (float2*)coeff;
+  cudaMemsetAsync(coeff, 0, 2 * (size_t)t.n * rows * sizeof(float2), s);  // padding rows, as above
+  GaugeArgs ga{p->n, p->steps, p->d_h0, p->d_h0o, p->d_h1, p->d_k, p->d_scal, p->sbeta};
+  k_gauge_coeffs<<<t.n, GAUGE_NT, 0, s>>>(ga, ld, t.m0, t.n, 1, nt, ept, cf, cf + t.n * rows);
 }
 
 fq_status fq_launch_resident(const fq_plan* p, const void* coeff, const double* x0, double* x, int transpose_out,
-                             int nc, int m_begin, int m_end, cudaStream_t s) {
+                             int nc, int m_begin, int m_end, cudaStream_t s, const fq_tables* pre) {
   const int nsteps = m_end - m_begin;
   int nt, ept;
   res_config(p->n, nc, &nt, &ept);
-  const float4* cf = (const float4*)coeff;
-  const float4* rot = cf + (size_t)nsteps * nt * ept / 2;
+  const size_t stride = (size_t)nt * ept / 2;  // float4 of one step
+  const float4* cf = (const float4*)coeff + (pre ? (m_begin - pre->m0) * stride : 0);
+  const float4* rot = cf + (pre ? pre->n : nsteps) * stride;
+  // prepared tables hold single steps (nsteps = 1): out by the conjugate of the way in
+  const float4* rot_end = pre ? rot : rot + nsteps * stride;
+  const float end_sign = pre ? -1.f : 1.f;
   ResCoef coef;
   double bcl = 0.0;
   for (int k = 0; k <= p->L; ++k) bcl += (k + 1) * fabs(p->cheb[k]);
@@ -548,12 +582,12 @@ fq_status fq_launch_resident(const fq_plan* p, const void* coeff, const double* 
   }
   const float b = (float)bcl;
   if (nt == 512 && ept == 16)
-    return launch_cfg<16, 512>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
+    return launch_cfg<16, 512>(p, cf, rot, rot_end, end_sign, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
   if (nt == 512 && ept == 18)
-    return launch_cfg<18, 512>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
+    return launch_cfg<18, 512>(p, cf, rot, rot_end, end_sign, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
   switch (ept) {
 #define FQ_RES_CASE(E) \
-  case E: return launch_cfg<E, 0>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
+  case E: return launch_cfg<E, 0>(p, cf, rot, rot_end, end_sign, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
     FQ_RES_CASE(2)
     FQ_RES_CASE(4)
     FQ_RES_CASE(6)
@@ -564,7 +598,7 @@ fq_status fq_launch_resident(const fq_plan* p, const void* coeff, const double* 
     FQ_RES_CASE(16)
     FQ_RES_CASE(18)
     FQ_RES_CASE(20)
-    case 40: return launch_cfg<40, 256>(p, cf, rot, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
+    case 40: return launch_cfg<40, 256>(p, cf, rot, rot_end, end_sign, x0, x, transpose_out, nc, nsteps, coef, b, nt, s);
 #undef FQ_RES_CASE
     default: fq_set_error("resident kernel: n = %d too large", p->n); return FQ_EUNSUPPORTED;
   }

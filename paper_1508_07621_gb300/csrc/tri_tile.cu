@@ -425,16 +425,24 @@ k_tri_tile_dfl(const dfl2* __restrict__ cf, const dfl2* __restrict__ rot, const 
   if (bad) atomicOr(status, FQ_BIT_BOUND);
 }
 
+template <typename T>
+void gauge_tables(const fq_plan* p, fq_tables t, void* ws, cudaStream_t s) {
+  using T2 = typename V2<T>::t;
+  const int ld = (p->n + 3) & ~3;
+  GaugeArgs ga{p->n, p->steps, p->d_h0, p->d_h0o, p->d_h1, p->d_k, p->d_scal, p->sbeta};
+  k_gauge_tile<T><<<t.n, GAUGE_NT, 0, s>>>(ga, ld, t.m0, (T2*)ws, (T2*)ws + (size_t)t.n * ld);
+}
+
 fq_status dfl_chain(fq_plan* p, const double* x0, double* x, int nc, int m_begin, int m_end, int identity,
-                    int transpose_out, void* ws, cudaStream_t s) {
+                    int transpose_out, void* ws, cudaStream_t s, const fq_tables* pre) {
   const int n = p->n, ld = (n + 3) & ~3, nsteps = m_end - m_begin, L = p->L;
-  dfl2* cf = (dfl2*)ws;
-  dfl2* rot = cf + (size_t)nsteps * ld;
-  double* bufs = (double*)(rot + (size_t)nsteps * ld);
+  const fq_tables t = pre ? *pre : fq_tables{m_begin, nsteps};
+  if (!pre) fq_tile_tables(p, t, ws, s);
+  const dfl2* cf = (dfl2*)ws + (size_t)(m_begin - t.m0) * ld;
+  const dfl2* rot = cf + (size_t)t.n * ld;
+  double* bufs = (double*)((dfl2*)ws + 2 * (size_t)t.n * ld);
   const size_t plane = (size_t)nc * ld;
   fq_blk<double> b[2] = {{bufs, bufs + plane}, {bufs + 2 * plane, bufs + 3 * plane}};
-  GaugeArgs ga{p->n, p->steps, p->d_h0, p->d_h0o, p->d_h1, p->d_k, p->d_scal, p->sbeta};
-  k_gauge_tile<dfl><<<nsteps, GAUGE_NT, 0, s>>>(ga, ld, m_begin, cf, rot);
   if (identity) fq_launch_identity_f64(b[0], nc, n, ld, s);
   else fq_launch_load_states(x0, b[0], nc, n, ld, s);
   DflCoef coef{};
@@ -511,16 +519,16 @@ TileCoef<T> tile_coef(const fq_plan* p) {
 
 template <typename T>
 fq_status tile_chain(fq_plan* p, const double* x0, double* x, int nc, int m_begin, int m_end, int identity,
-                     int transpose_out, void* ws, cudaStream_t s) {
+                     int transpose_out, void* ws, cudaStream_t s, const fq_tables* pre) {
   using T2 = typename V2<T>::t;
   const int n = p->n, ld = (n + 3) & ~3, nsteps = m_end - m_begin, L = p->L;
-  T2* cf = (T2*)ws;
-  T2* rot = cf + (size_t)nsteps * ld;
-  T* bufs = (T*)(rot + (size_t)nsteps * ld);
+  const fq_tables t = pre ? *pre : fq_tables{m_begin, nsteps};
+  if (!pre) fq_tile_tables(p, t, ws, s);
+  const T2* cf = (T2*)ws + (size_t)(m_begin - t.m0) * ld;
+  const T2* rot = cf + (size_t)t.n * ld;
+  T* bufs = (T*)((T2*)ws + 2 * (size_t)t.n * ld);
   const size_t plane = (size_t)nc * ld;
   fq_blk<T> b[2] = {{bufs, bufs + plane}, {bufs + 2 * plane, bufs + 3 * plane}};
-  GaugeArgs ga{p->n, p->steps, p->d_h0, p->d_h0o, p->d_h1, p->d_k, p->d_scal, p->sbeta};
-  k_gauge_tile<T><<<nsteps, GAUGE_NT, 0, s>>>(ga, ld, m_begin, cf, rot);
   if (identity) identity_block(b[0], nc, n, ld, s);
   else load_block(x0, b[0], nc, n, ld, s);
   const TileCoef<T> coef = tile_coef<T>(p);
@@ -558,10 +566,16 @@ size_t fq_tile_workspace(const fq_plan* p, int nc, int nsteps) {
   return 2 * (size_t)nsteps * ld * 2 * es + 4 * (size_t)nc * ld * es;
 }
 
+void fq_tile_tables(const fq_plan* p, fq_tables t, void* ws, cudaStream_t s) {
+  if (p->precision == FQ_FP64) gauge_tables<double>(p, t, ws, s);
+  else if (p->precision == FQ_DF32) gauge_tables<dfl>(p, t, ws, s);
+  else gauge_tables<float>(p, t, ws, s);
+}
+
 fq_status fq_tile_propagate(fq_plan* p, const double* x0, double* x, int nc, int m_begin, int m_end, int identity,
-                            int transpose_out, void* ws, cudaStream_t s) {
+                            int transpose_out, void* ws, cudaStream_t s, const fq_tables* pre) {
   if (p->precision == FQ_FP64)
-    return tile_chain<double>(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s);
-  if (p->precision == FQ_DF32) return dfl_chain(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s);
-  return tile_chain<float>(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s);
+    return tile_chain<double>(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s, pre);
+  if (p->precision == FQ_DF32) return dfl_chain(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s, pre);
+  return tile_chain<float>(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s, pre);
 }

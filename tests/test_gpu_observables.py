@@ -115,6 +115,60 @@ def test_floquet_analysis_sorted_by_average_energy(fq):
     assert np.max(np.abs(res)) < 1e-9
 
 
+def _random_states(n, nc, seed):
+    import torch
+    x = np.exp(2j * np.pi * fi.uniform(seed, n * nc)).reshape(nc, n) * (0.1 + fi.uniform(seed + 1, n * nc).reshape(nc, n))
+    x /= np.linalg.norm(x, axis=1, keepdims=True)
+    return torch.from_numpy(x).cuda()
+
+
+@pytest.mark.parametrize("n,nc", [(1, 1), (2, 5), (31, 4), (32, 9), (33, 3), (64, 1), (65, 65), (100, 30), (161, 2)])
+def test_dense_averages_block_edges(fq, n, nc):
+    """Sizes around the 32-row blocks of H and the 4 states of a CTA, with an odd (trapezoid) and an
+    even number of steps, H0, H1 and the drive all weighted; FP64 against the oracle."""
+    h0, h1 = fi.goe(n, 1821), fi.goe(n, 1822)
+    drv = fi.Drive(0.3, 1.0, 1.4, 0.2)
+    states = _random_states(n, nc, 1823)
+    k = o.commutator_dense(h0, h1)
+    for M in (7, 10):
+        plan = fq.Plan.dense(h0, h1, omega=drv.omega, f_ac=drv.f_ac, f_dc=drv.f_dc, phi0=drv.phi0, steps=M)
+        avg = plan.average_observable(states, 0.7, -0.4, 1.3).cpu().numpy()
+        assert plan.check_status() == fq.FQ_OK
+        p = o.plan_for_drive_dense(h0, h1, drv, M)
+        step = lambda m, x: o.chebyshev_step(lambda v: o.omega_tilde_dense(h0, h1, k, p, m) @ v, x, p.coeffs, p.phase)
+        ref = o.average_observable(step, o.expect_dense(h0, h1, 0.7, -0.4, 1.3, drv), states.cpu().numpy().T, drv, M)
+        assert np.max(np.abs(avg - ref)) <= 1e-12
+
+
+@pytest.mark.parametrize("precision,kernel", [(0, 1), (0, 3), (1, 2), (1, 3), (4, 3), (5, 4)])
+@pytest.mark.parametrize("nb,nc", [(1, 1), (2, 5), (60, 61), (511, 3), (512, 6), (1100, 2)])
+def test_tridiagonal_averages_by_path(fq, precision, kernel, nb, nc):
+    """Averages on every tridiagonal kernel (those with gauge tables take all steps' tables from one
+    launch, each step then entering and leaving the original frame), around the 512-row chunks of H and
+    the 4 states of a CTA: against the averages of the same plan's own propagation, step by step, in
+    FP64 on the host."""
+    d = fi.config_dimer(nb=nb)
+    n, M = d.n, 5
+    h = 2 * math.pi / 3.0 / 2000
+    plan = fq.Plan.tridiag(d.h0_diag, d.h0_off, d.h1_diag, omega=3.0, f_ac=1.5, f_dc=0.2, phi0=0.3, steps=M,
+                           period=M * h, precision=precision, kernel=kernel)
+    states = _random_states(n, nc, 1831)
+    avg = plan.average_observable(states, 0.7, -0.4, 1.3).cpu().numpy()
+    assert plan.check_status() == fq.FQ_OK
+    x, ref, scale = states, 0.0, 0.0
+    for m in range(M + 1):
+        f = 0.2 + 1.5 * math.cos(3.0 * m * h + 0.3)
+        v = x.cpu().numpy()
+        dg = 0.7 * d.h0_diag + (-0.4 + 1.3 * f) * d.h1_diag
+        e = (np.abs(v) ** 2 @ dg) + 2 * 0.7 * np.real(np.conj(v[:, :-1]) * v[:, 1:]) @ d.h0_off
+        ref = ref + (0.5 if m in (0, M) else 1.0) * e / M
+        scale = max(scale, np.max(np.abs(dg)) + 2 * np.max(np.abs(d.h0_off), initial=0.0))
+        if m < M:
+            x = plan.propagate(x, m, m + 1)
+    # 64-bit sums of at most 1101 terms below the scale in magnitude
+    assert np.max(np.abs(avg - ref)) <= 4 * n * 2.0 ** -53 * scale + 1e-15
+
+
 @pytest.mark.parametrize("precision", [0, 2])
 def test_overlap_phase_error_matches_oracle(fq, precision):
     """Eq. 20 on the library (coarse chain applied to the fine Floquet states by
