@@ -699,8 +699,9 @@ fq_status floquet_unitarity_defect(const void* d_U, int32_t n, const int32_t* d_
   const size_t need = align_up(2 * sizeof(double) * (size_t)chunks * nb);
   if (!d_ws || ws_bytes < need) { fq_set_error("defect workspace too small (%zu < %zu)", ws_bytes, need); return FQ_EINVAL; }
   cudaStream_t s = (cudaStream_t)stream;
-  fq_launch_defect((const double*)d_U, n, d_cols, rows, (double*)d_ws, s);
-  std::vector<double> h(2 * (size_t)chunks * nb, 0.0);  // at most 2 * 16 * N / 256 doubles: N ~ 10^4 is 2.5 KB
+  const int parts = fq_launch_defect((const double*)d_U, n, d_cols, rows, (double*)d_ws,
+                                     ws_bytes / (2 * sizeof(double)), s);
+  std::vector<double> h(2 * (size_t)parts * nb, 0.0);
   cudaError_t e = cudaMemcpyAsync(h.data(), d_ws, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return fq_cuda_fail(e, "defect");

@@ -169,6 +169,26 @@ def test_tridiagonal_averages_by_path(fq, precision, kernel, nb, nc):
     assert np.max(np.abs(avg - ref)) <= 4 * n * 2.0 ** -53 * scale + 1e-15
 
 
+@pytest.mark.parametrize("n,k", [(1, 1), (5, 3), (31, 31), (32, 1), (33, 17), (255, 2), (256, 9), (257, 40), (520, 130)])
+def test_unitarity_defect_chunks(fq, n, k):
+    """The defect over listed columns (unsorted, one of them twice) at the edges of the 32- and 256-column
+    blocks and of every chunk size, against the same sums in numpy."""
+    import torch
+    rng = np.random.default_rng(1841)
+    u = fi.haar_unitary(n, 1842) + 1e-3 * (rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n)))
+    cols = rng.permutation(n)[:k]
+    cols[-1] = cols[0]
+    d = u[:, cols].conj().T @ u
+    d[np.arange(k), cols] -= 1.0
+    U = torch.from_numpy(np.ascontiguousarray(u)).cuda()
+    mx, fro = fq.api.unitarity_defect(U, torch.from_numpy(cols.astype(np.int32)).cuda())
+    assert abs(mx - np.max(np.abs(d))) <= 1e-14 * (1 + n) and abs(fro - np.linalg.norm(d) / math.sqrt(k)) <= 1e-14 * (1 + n)
+    full = u.conj().T @ u - np.eye(n)
+    mx, fro = fq.api.unitarity_defect(U)
+    assert abs(mx - np.max(np.abs(full))) <= 1e-14 * (1 + n)
+    assert abs(fro - np.linalg.norm(full) / math.sqrt(n)) <= 1e-14 * (1 + n)
+
+
 @pytest.mark.parametrize("precision", [0, 2])
 def test_overlap_phase_error_matches_oracle(fq, precision):
     """Eq. 20 on the library (coarse chain applied to the fine Floquet states by
