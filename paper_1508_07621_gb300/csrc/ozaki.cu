@@ -7,8 +7,8 @@
 namespace {
 
 struct OzWs {
-  __nv_bfloat16* left;   // OZ_S slices [ncp][2 np]
-  __nv_bfloat16* right;  // OZ_S slices [3 np][np]
+  __nv_bfloat16* left;   // OZ_S slices of [ncp][2 np], in pieces (OzOperands)
+  __nv_bfloat16* right;  // OZ_S slices of [3 np][np]
   int* es;               // [ncp]
   int* et;               // [np]
   double* m[3][2];       // FP64 state masters [nc][n], planar
@@ -74,16 +74,10 @@ size_t fq_ozaki_workspace(const fq_plan* p, int nc, void* base, void* out) {
 
 fq_status fq_ozaki_propagate(fq_plan* p, const double* x0, double* x, int nc, int m_begin, int m_end, int identity,
                              int transpose_out, void* ws, cudaStream_t s) {
-  fq_status st = encode_fn();
-  if (st != FQ_OK) return st;
   OzWs w;
   fq_ozaki_workspace(p, nc, ws, &w);
   const int n = p->n, L = p->L;
-  OzMaps maps;
-  for (int q = 0; q < OZ_S; ++q) {
-    if ((st = make_map(&maps.a[q], w.left + q * w.astride, w.ncp, 2 * w.np, BM, OZ_BKE)) != FQ_OK) return st;
-    if ((st = make_map(&maps.r[q], w.right + q * w.rstride, 3 * w.np, w.np, 3 * OZ_BN, OZ_BKE)) != FQ_OK) return st;
-  }
+  const OzOperands op{w.left, w.right};
   static std::atomic<unsigned> attr_set{0};
   if (fq_first_on_device(attr_set)) {
     cudaError_t e = cudaFuncSetAttribute(k_oz_term, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -95,8 +89,8 @@ fq_status fq_ozaki_propagate(fq_plan* p, const double* x0, double* x, int nc, in
   else fq_launch_load_states(x0, b0, nc, n, n, s);
   int xb = 0;
   if (m_end > m_begin)
-    k_oz_slice_left<<<w.ncp, 256, 0, s>>>(w.m[0][0], w.m[0][1], 1.0, 0.0, nullptr, nullptr, n, nc, w.np, w.astride,
-                                          w.left, w.es);
+    k_oz_slice_left<<<w.ncp, 256, 0, s>>>(w.m[0][0], w.m[0][1], 1.0, 0.0, nullptr, nullptr, n, nc, w.np, BM, w.left,
+                                          w.es);
   // output columns and values of k beyond N are zero: their tiles and stages are left out.  The
   // cluster size looks at N alone, so that a block of columns agrees with the whole U_T bit for bit.
   const int tiles_i = (n + OZ_BN - 1) / OZ_BN, tiles_j = w.ncp / BM;
@@ -110,7 +104,7 @@ fq_status fq_ozaki_propagate(fq_plan* p, const double* x0, double* x, int nc, in
   t.bound2 = 1.0 + 1e-9;
   t.status = p->d_status;
   for (int m = m_begin; m < m_end; ++m) {
-    k_oz_omega<<<w.np, 256, 0, s>>>(omega_args(p, m), n, w.np, w.rstride, w.right, w.et);
+    k_oz_omega<<<w.np, 256, 0, s>>>(omega_args(p, m), n, w.np, w.right, w.et);
     int cur = xb, nxt = (xb + 1) % 3, acc = (xb + 2) % 3, prv = -1;
     for (int l = 0; l < L; ++l) {
       t.first = l == 0;
@@ -131,11 +125,11 @@ fq_status fq_ozaki_propagate(fq_plan* p, const double* x0, double* x, int nc, in
       e.es = w.es;
       e.et = w.et;
       e.t = t;
-      cudaError_t le = cudaLaunchKernelEx(&launch.cfg, k_oz_term, maps, nk, tiles_j, tiles_i, w.np, csize, e);
+      cudaError_t le = cudaLaunchKernelEx(&launch.cfg, k_oz_term, op, nk, tiles_j, tiles_i, w.np, csize, e);
       if (le != cudaSuccess) return fq_cuda_fail(le, "FP64-emulation term launch");
       if (!(t.last && m == m_end - 1))
         k_oz_slice_left<<<w.ncp, 256, 0, s>>>(w.m[out][0], w.m[out][1], 1.0, 0.0, nullptr, nullptr, n, nc, w.np,
-                                              w.astride, w.left, w.es);
+                                              BM, w.left, w.es);
       if (t.last) {
         xb = out;
       } else {

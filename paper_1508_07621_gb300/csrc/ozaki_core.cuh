@@ -27,8 +27,8 @@
 // accumulation and the step phase in FP64, as the plain FP64 path does.  A separate pass slices
 // each new Psi_{l+1} (its row scales need the whole row).
 //
-// Kernel.  One 128-state x 64-column tile per CTA: warp 0 streams TMA stages (K = 16 per stage,
-// 32-byte rows with 32-byte swizzle), warp 1 issues the MMAs, warps 2-17 drain tensor memory
+// Kernel.  One 128-state x 64-column tile per CTA: warp 0 streams the stages (K = 16 each, 32-byte rows
+// with 32-byte swizzle, two bulk copies of operands stored in that order), warp 1 issues the MMAs, warps 2-17 drain tensor memory
 // (four warps per lane quarter, 16 complex columns each).  The 512 tensor-memory columns hold
 // the four accumulators (128 columns each), so the MMAs wait for each drain.  Every wait is
 // bounded; a wait that gives up records FQ_BIT_TIMEOUT, drains this CTA's own copies and MMAs,
@@ -76,10 +76,30 @@ struct OzCfg {
   static_assert((size_t)STAGES * STAGE_BYTES >= 4 * OZ_XS_PLANE * sizeof(float), "epilogue staging");
 };
 
+// Operand slices in global memory lie as the K stages lie in shared memory: per block of R rows and 16
+// values of k one contiguous piece, [slice][part][R rows][16] with 32-byte rows under the 32-byte swizzle.
+// Parts: Psi_r, Psi_i of the left operand; of the right one the rows -A, S, A of a 64-row block follow
+// one another (192 rows), or S alone for a real operator (ozaki_real.cuh).  A stage is then two plain
+// bulk copies.  (18 tensor-map boxes of 32-byte rows from row-major slices made a stage before: a term at
+// N = 777 139 -> 134 us, 1536 464 -> 433, 2600 2028 -> 1895.)
+struct OzOperands {
+  const __nv_bfloat16* left;   // [ncp / R][np / 16][OZ_S][2][R][16]
+  const __nv_bfloat16* right;  // [np / 64][np / 16][OZ_S][192 or 64][16]
+};
+
+// Element offset inside a piece's [rows][16] of row r, value k (multiples of 4 keep 8-byte pieces whole).
+__device__ __forceinline__ int oz_swizzled(int r, int k) { return r * 16 + ((((k >> 3) ^ (r >> 2)) & 1) << 3) + (k & 7); }
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+// Tensor maps of the band kernel's operands (band.cu).
 struct OzMaps {
-  CUtensorMap a[OZ_S];  // left slices [rows][2 np]: Psi_r in columns [0, np), Psi_i in [np, 2 np)
-  CUtensorMap r[OZ_S];  // right slices: [3 np][np] (per 64-row block of Omega~, rows -A, S, A), or
-                        // [np][np] for a real operator (ozaki_real.cuh)
+  CUtensorMap a[OZ_S];  // state slices
+  CUtensorMap r[OZ_S];  // band slices
 };
 
 // Epilogue of one product Y = Psi . Omega~^T (FP64 states, row stride n):
@@ -297,7 +317,7 @@ __device__ __forceinline__ uint2 pack4(__nv_bfloat16 a, __nv_bfloat16 b, __nv_bf
 
 __global__ void k_oz_slice_left(const double* __restrict__ re, const double* __restrict__ im, double cr, double ci,
                                 double* __restrict__ out_re, double* __restrict__ out_im, int n, int nc, int np,
-                                size_t astride, __nv_bfloat16* __restrict__ left, int* __restrict__ es) {
+                                int block, __nv_bfloat16* __restrict__ left, int* __restrict__ es) {
   __shared__ unsigned long long red[32];
   const int j = blockIdx.x;
   unsigned long long m = 0;
@@ -314,9 +334,10 @@ __global__ void k_oz_slice_left(const double* __restrict__ re, const double* __r
       m = b > m ? b : m;
     }
   const int e = oz_exponent(block_max_key(m, red));
-  __nv_bfloat16* row = left + (size_t)j * 2 * np;
-  // four consecutive columns per thread: one 8-byte store per slice and part (np % 4 == 0, and
-  // every slice row starts on an 8-byte boundary)
+  // the pieces of this row's block (`block` rows); four consecutive columns per thread: one 8-byte store
+  // per slice and part
+  const int r = j % block, piece = block * 16;
+  __nv_bfloat16* row = left + (size_t)(j / block) * (np / 16) * 2 * OZ_S * piece;
   for (int k0 = 4 * threadIdx.x; k0 < np; k0 += 4 * blockDim.x) {
     __nv_bfloat16 sr[4][OZ_S], si[4][OZ_S];
 #pragma unroll
@@ -328,8 +349,9 @@ __global__ void k_oz_slice_left(const double* __restrict__ re, const double* __r
     }
 #pragma unroll
     for (int q = 0; q < OZ_S; ++q) {
-      *reinterpret_cast<uint2*>(row + q * astride + k0) = pack4(sr[0][q], sr[1][q], sr[2][q], sr[3][q]);
-      *reinterpret_cast<uint2*>(row + q * astride + np + k0) = pack4(si[0][q], si[1][q], si[2][q], si[3][q]);
+      __nv_bfloat16* d = row + ((size_t)(k0 / 16) * 2 * OZ_S + 2 * q) * piece + oz_swizzled(r, k0 % 16);
+      *reinterpret_cast<uint2*>(d) = pack4(sr[0][q], sr[1][q], sr[2][q], sr[3][q]);
+      *reinterpret_cast<uint2*>(d + piece) = pack4(si[0][q], si[1][q], si[2][q], si[3][q]);
     }
   }
   if (threadIdx.x == 0) es[j] = e;
@@ -355,8 +377,8 @@ __device__ __forceinline__ void oz_omega_entry(const OzOmega& a, int n, int i, i
 }
 
 // Right slices of step m: one CTA per row i of the padded operator (rows >= n are zero).
-__global__ void k_oz_omega(const __grid_constant__ OzOmega a, int n, int np, size_t rstride,
-                           __nv_bfloat16* __restrict__ right, int* __restrict__ et) {
+__global__ void k_oz_omega(const __grid_constant__ OzOmega a, int n, int np, __nv_bfloat16* __restrict__ right,
+                           int* __restrict__ et) {
   __shared__ unsigned long long red[32];
   const int i = blockIdx.x;
   unsigned long long m = 0;
@@ -369,7 +391,8 @@ __global__ void k_oz_omega(const __grid_constant__ OzOmega a, int n, int np, siz
       m = y > m ? y : m;
     }
   const int e = oz_exponent(block_max_key(m, red));
-  const size_t rb = (size_t)(3 * OZ_BN) * (i / OZ_BN) + (i % OZ_BN);  // row of -A; S and A follow
+  constexpr int PIECE = 3 * OZ_BN * 16;
+  __nv_bfloat16* block = right + (size_t)(i / OZ_BN) * (np / 16) * OZ_S * PIECE;
   for (int k = threadIdx.x; k < np; k += blockDim.x) {
     double S = 0.0, A = 0.0;
     if (i < n && k < n) oz_omega_entry(a, n, i, k, S, A);
@@ -378,17 +401,18 @@ __global__ void k_oz_omega(const __grid_constant__ OzOmega a, int n, int np, siz
     oz_digits(A, e, sa);
 #pragma unroll
     for (int q = 0; q < OZ_S; ++q) {
-      __nv_bfloat16* base = right + q * rstride + k;
-      base[rb * np] = __hneg(sa[q]);
-      base[(rb + OZ_BN) * np] = ss[q];
-      base[(rb + 2 * OZ_BN) * np] = sa[q];
+      // rows i % 64 of the parts -A, S, A (64 rows apart: the same place in the swizzle)
+      __nv_bfloat16* d = block + ((size_t)(k / 16) * OZ_S + q) * PIECE + oz_swizzled(i % OZ_BN, k % 16);
+      d[0] = __hneg(sa[q]);
+      d[OZ_BN * 16] = ss[q];
+      d[2 * OZ_BN * 16] = sa[q];
     }
   }
   if (threadIdx.x == 0) et[i] = e;
 }
 
 // Slices of the real operator v = ((h0 ? h0 : 0) + c1 h1) inv - shift 1, c1 = f[m] (1 without f):
-// one CTA per row i of [np][np] (rows >= n are zero).  The adjoint's Omega~_m (piecewise-constant
+// one CTA per row i < np (rows >= n are zero).  The adjoint's Omega~_m (piecewise-constant
 // drive) and E = H1 / Delta E.
 __device__ __forceinline__ double oz_real_entry(const double* h0, const double* h1, double c1, double inv,
                                                 double shift, int n, int i, int k) {
@@ -397,8 +421,8 @@ __device__ __forceinline__ double oz_real_entry(const double* h0, const double* 
 }
 
 __global__ void k_oz_real(const double* __restrict__ h0, const double* __restrict__ h1, const double* __restrict__ f,
-                          int m, double inv, double shift, int n, int np, size_t rstride,
-                          __nv_bfloat16* __restrict__ right, int* __restrict__ et) {
+                          int m, double inv, double shift, int n, int np, __nv_bfloat16* __restrict__ right,
+                          int* __restrict__ et) {
   __shared__ unsigned long long red[32];
   const int i = blockIdx.x;
   const double c1 = f ? f[m] : 1.0;
@@ -418,7 +442,8 @@ __global__ void k_oz_real(const double* __restrict__ h0, const double* __restric
     }
 #pragma unroll
     for (int q = 0; q < OZ_S; ++q)
-      *reinterpret_cast<uint2*>(right + q * rstride + (size_t)i * np + k0) = pack4(sl[0][q], sl[1][q], sl[2][q], sl[3][q]);
+      *reinterpret_cast<uint2*>(right + (((size_t)(i / OZ_BN) * (np / 16) + k0 / 16) * OZ_S + q) * (OZ_BN * 16) +
+                                oz_swizzled(i % OZ_BN, k0 % 16)) = pack4(sl[0][q], sl[1][q], sl[2][q], sl[3][q]);
   }
   if (threadIdx.x == 0) et[i] = e;
 }
@@ -426,7 +451,7 @@ __global__ void k_oz_real(const double* __restrict__ h0, const double* __restric
 // One Chebyshev term (OZ_FWD) on a 128-state x 64-column tile per cluster of `csize` CTAs (see the
 // file comment).
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    k_oz_term(const __grid_constant__ OzMaps maps, int nk, int tiles_j, int tiles_i, int np, int csize, OzEpi e) {
+    k_oz_term(const OzOperands op, int nk, int tiles_j, int tiles_i, int np, int csize, OzEpi e) {
   using Cfg = OzCfg;
   constexpr int OZ_STAGES = Cfg::STAGES;
   constexpr int OZ_STAGE_BYTES = Cfg::STAGE_BYTES;
@@ -493,13 +518,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const uint32_t st = base + s * OZ_STAGE_BYTES;
         const uint32_t bar = full0 + 8 * s;
         mbar_expect_tx(bar, OZ_STAGE_BYTES);
-        const int kx = (kb0 + kb) * OZ_BKE;
-#pragma unroll
-        for (int q = 0; q < OZ_S; ++q) {
-          tma_load_2d(st + (2 * q) * OZ_A_BYTES, &maps.a[q], bar, kx, j0);           // Psi_r
-          tma_load_2d(st + (2 * q + 1) * OZ_A_BYTES, &maps.a[q], bar, np + kx, j0);  // Psi_i
-          tma_load_2d(st + 2 * OZ_S * OZ_A_BYTES + q * OZ_R_BYTES, &maps.r[q], bar, kx, 3 * i0);  // -A, S, A
-        }
+        const size_t kp = np / OZ_BKE, kx = kb0 + kb;  // K pieces of a block, and this one
+        bulk_load(st, op.left + ((size_t)(j0 / BM) * kp + kx) * (OZ_S * OZ_A_BYTES), 2 * OZ_S * OZ_A_BYTES, bar);
+        bulk_load(st + 2 * OZ_S * OZ_A_BYTES, op.right + ((size_t)(i0 / OZ_BN) * kp + kx) * (OZ_S * OZ_R_BYTES / 2),
+                  OZ_S * OZ_R_BYTES, bar);
         issued = kb + 1;
       }
       if (!ok) {

@@ -13,9 +13,9 @@
 //   dL/df_m = 2 Re sum_l w_l D_l  (w_1 = -i, w_l = -2i).
 // Every product's output is sliced again by k_oz_slice_left (row scales need whole rows).
 // Memory: FP64 checkpoints of X every s = checkpoint_stride steps; each segment is recomputed
-// once with the slices of every psi_l kept (the left operands of the dot products), slice-major
-// ([slice][slot][row][k]) so that the L dots of a step run as one product over L x Np stacked
-// rows against the stacked FP64 bbar_1 .. bbar_L.
+// once with the slices of every psi_l kept (the left operands of the dot products), one after another in
+// the blocks of OzOperands, so that the L dots of a step run as one product over L x Np stacked rows
+// against the stacked FP64 bbar_1 .. bbar_L.
 #include <vector>
 
 #include "ozaki_real.cuh"
@@ -36,7 +36,7 @@ struct OzGradWs {
   int* etE;
   __nv_bfloat16* lsl[2];  // left-operand ping-pong (forward sweep, adjoint terms)
   int* esl[2];
-  __nv_bfloat16* slots;   // psi_l slices of one recomputed segment: OZ_S x nslots x [ncp][2 np]
+  __nv_bfloat16* slots;   // psi_l slices of one segment: nslots x OZ_S x [ncp][2 np]
   int* es_slots;          // [nslots][ncp]
   Planes f[5];            // FP64 states [n][n]: forward cur / prev / acc; adjoint G and the next G
   Planes bbar;            // bbar_1 .. bbar_L of one step: L blocks of [ncp][n] (padding rows zero)
@@ -44,8 +44,7 @@ struct OzGradWs {
   double2* partial;       // (L + 1) x ncta
   double2* tau_partial;   // n
   double2* tau;
-  size_t slot_slice() const { return (size_t)nslots * astride; }
-  __nv_bfloat16* slot(int q) const { return slots + (size_t)q * astride; }
+  __nv_bfloat16* slot(int q) const { return slots + (size_t)q * OZ_S * astride; }
   int* es_slot(int q) const { return es_slots + (size_t)q * ncp; }
   Planes bbar_block(int l, int n) const {  // bbar_l, l = 1..L
     const size_t o = (size_t)(l - 1) * ncp * n;
@@ -103,16 +102,10 @@ size_t oz_grad_layout(const fq_plan* p, void* base, OzGradWs* out) {
   return off;
 }
 
-// One product Y = left . right^T (right real, [np][np] slices) with epilogue EPI over `rows` left rows.
+// One product Y = left . right^T (right real) with epilogue EPI over `rows` left rows.
 template <int EPI>
-fq_status oz_gemm(const OzGradWs& w, const __nv_bfloat16* left, size_t lstride, int rows, const __nv_bfloat16* right,
-                  const OzEpi& e, cudaStream_t s) {
-  OzMaps maps{};
-  fq_status st;
-  for (int q = 0; q < OZ_S; ++q) {
-    if ((st = make_map(&maps.a[q], left + q * lstride, rows, 2 * w.np, OZR_BM, OZ_BKE)) != FQ_OK) return st;
-    if ((st = make_map(&maps.r[q], right + q * w.rstride, w.np, w.np, OZ_BN, OZ_BKE)) != FQ_OK) return st;
-  }
+fq_status oz_gemm(const OzGradWs& w, const __nv_bfloat16* left, int rows, const __nv_bfloat16* right, const OzEpi& e,
+                  cudaStream_t s) {
   static std::atomic<unsigned> attr_set{0};
   if (fq_first_on_device(attr_set)) {
     cudaError_t r = cudaFuncSetAttribute(k_oz_real_term<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -127,7 +120,8 @@ fq_status oz_gemm(const OzGradWs& w, const __nv_bfloat16* left, size_t lstride, 
   const int nk = (e.n + OZ_BKE - 1) / OZ_BKE;
   const int csize = dot ? 1 : oz_cluster(tiles_i * tiles_j, nk);
   OzLaunch launch(tiles_i * tiles_j, csize, OZR_SMEM, s);
-  cudaError_t le = cudaLaunchKernelEx(&launch.cfg, k_oz_real_term<EPI>, maps, nk, tiles_j, tiles_i, w.np, csize, e);
+  cudaError_t le = cudaLaunchKernelEx(&launch.cfg, k_oz_real_term<EPI>, OzOperands{left, right}, nk, tiles_j, tiles_i, w.np,
+                                      csize, e);
   return le == cudaSuccess ? FQ_OK : fq_cuda_fail(le, "FP64-emulation gradient product");
 }
 
@@ -138,13 +132,11 @@ struct Runner {
   cudaStream_t s;
 
   void omega(int m) {
-    k_oz_real<<<w.np, 256, 0, s>>>(p->d_h0, p->d_h1, f, m, 1.0 / p->delta_e, p->sbeta, p->n, w.np, w.rstride, w.S,
-                                   w.etS);
+    k_oz_real<<<w.np, 256, 0, s>>>(p->d_h0, p->d_h1, f, m, 1.0 / p->delta_e, p->sbeta, p->n, w.np, w.S, w.etS);
   }
-  // slices of v = c x (x NULL: identity rows) into `left` (slice stride lstride) and es; FP64
-  // copy of v into `out` when given
-  void slice(Planes x, double cr, double ci, Planes out, __nv_bfloat16* left, size_t lstride, int* es) {
-    k_oz_slice_left<<<w.ncp, 256, 0, s>>>(x.re, x.im, cr, ci, out.re, out.im, p->n, p->n, w.np, lstride, left, es);
+  // slices of v = c x (x NULL: identity rows) into `left` and es; FP64 copy of v into `out` when given
+  void slice(Planes x, double cr, double ci, Planes out, __nv_bfloat16* left, int* es) {
+    k_oz_slice_left<<<w.ncp, 256, 0, s>>>(x.re, x.im, cr, ci, out.re, out.im, p->n, p->n, w.np, OZR_BM, left, es);
   }
   OzEpi epi() const {
     OzEpi e{};
@@ -156,7 +148,7 @@ struct Runner {
 
   // Step m of the forward chain: X_{m-1} in f[*xb] with slices left[0] -> X_m in one of f[0..2]
   // (returned through xb) with slices left[L]; left[l] receives the slices of psi_l.
-  fq_status step(int m, int* xb, __nv_bfloat16* const* left, int* const* es, size_t lstride) {
+  fq_status step(int m, int* xb, __nv_bfloat16* const* left, int* const* es) {
     const int L = p->L;
     omega(m);
     fq_term t{};
@@ -183,9 +175,9 @@ struct Runner {
       e.es = es[l];
       e.et = w.etS;
       e.t = t;
-      fq_status st = oz_gemm<OZ_FWD>(w, left[l], lstride, w.ncp, w.S, e, s);
+      fq_status st = oz_gemm<OZ_FWD>(w, left[l], w.ncp, w.S, e, s);
       if (st != FQ_OK) return st;
-      slice(w.f[out], 1.0, 0.0, Planes{nullptr, nullptr}, left[l + 1], lstride, es[l + 1]);
+      slice(w.f[out], 1.0, 0.0, Planes{nullptr, nullptr}, left[l + 1], es[l + 1]);
       if (t.last) {
         *xb = out;
       } else {
@@ -203,8 +195,7 @@ size_t fq_grad_ozaki_workspace(const fq_plan* p) { return oz_grad_layout(p, null
 
 fq_status fq_grad_ozaki(fq_plan* p, const double* d_f, const void* d_W, double* d_loss, double* d_grad, void* d_ws,
                         cudaStream_t s) {
-  fq_status st = encode_fn();
-  if (st != FQ_OK) return st;
+  fq_status st = FQ_OK;
   Runner r{};
   r.p = p;
   r.f = d_f;
@@ -216,31 +207,30 @@ fq_status fq_grad_ozaki(fq_plan* p, const double* d_f, const void* d_W, double* 
 
   // the stacked bbar blocks are written only in their first n rows: zero the padding once
   cudaMemsetAsync(w.bbar.re, 0, sizeof(double) * 2 * (size_t)L * w.ncp * n, s);
-  k_oz_real<<<w.np, 256, 0, s>>>(nullptr, p->d_h1, nullptr, 0, 1.0 / p->delta_e, 0.0, n, w.np, w.rstride, w.E, w.etE);
+  k_oz_real<<<w.np, 256, 0, s>>>(nullptr, p->d_h1, nullptr, 0, 1.0 / p->delta_e, 0.0, n, w.np, w.E, w.etE);
 
   // ---- forward sweep, checkpoints X_{kS}
   int xb = 0;
-  r.slice(Planes{nullptr, nullptr}, 1.0, 0.0, w.f[0], w.lsl[0], w.astride, w.esl[0]);
+  r.slice(Planes{nullptr, nullptr}, 1.0, 0.0, w.f[0], w.lsl[0], w.esl[0]);
   cudaMemcpyAsync(w.ckpt(0).re, w.f[0].re, plane2, cudaMemcpyDeviceToDevice, s);
   std::vector<__nv_bfloat16*> left(L + 1);
   std::vector<int*> es(L + 1);
-  const size_t ss = w.slot_slice();
   const int m_last = (w.nseg - 1) * S;  // first step of the last segment
   for (int m = 0; m < M; ++m) {
     if (m >= m_last) {  // the last segment is walked back first: its slices are kept right away
-      if (m == m_last) r.slice(w.f[xb], 1.0, 0.0, Planes{nullptr, nullptr}, w.slot(0), ss, w.es_slot(0));
+      if (m == m_last) r.slice(w.f[xb], 1.0, 0.0, Planes{nullptr, nullptr}, w.slot(0), w.es_slot(0));
       for (int l = 0; l <= L; ++l) {
         left[l] = w.slot((m - m_last) * L + l);
         es[l] = w.es_slot((m - m_last) * L + l);
       }
-      if ((st = r.step(m, &xb, left.data(), es.data(), ss)) != FQ_OK) return st;
+      if ((st = r.step(m, &xb, left.data(), es.data())) != FQ_OK) return st;
       continue;
     }
     for (int l = 0; l <= L; ++l) {
       left[l] = w.lsl[l & 1];
       es[l] = w.esl[l & 1];
     }
-    if ((st = r.step(m, &xb, left.data(), es.data(), w.astride)) != FQ_OK) return st;
+    if ((st = r.step(m, &xb, left.data(), es.data())) != FQ_OK) return st;
     // the last term's slices are in left[L]; the next step reads them from lsl[0]
     if (L & 1) {
       std::swap(w.lsl[0], w.lsl[1]);
@@ -264,7 +254,7 @@ fq_status fq_grad_ozaki(fq_plan* p, const double* d_f, const void* d_W, double* 
     const int redo = k < w.nseg - 1 ? m1 - m0 : 0;
     if (redo) {
       cudaMemcpyAsync(w.f[0].re, w.ckpt(k).re, plane2, cudaMemcpyDeviceToDevice, s);
-      r.slice(w.f[0], 1.0, 0.0, Planes{nullptr, nullptr}, w.slot(0), ss, w.es_slot(0));
+      r.slice(w.f[0], 1.0, 0.0, Planes{nullptr, nullptr}, w.slot(0), w.es_slot(0));
       xb = 0;
     }
     for (int st_ = 0; st_ < redo; ++st_) {
@@ -272,14 +262,14 @@ fq_status fq_grad_ozaki(fq_plan* p, const double* d_f, const void* d_W, double* 
         left[l] = w.slot(st_ * L + l);
         es[l] = w.es_slot(st_ * L + l);
       }
-      if ((st = r.step(m0 + st_, &xb, left.data(), es.data(), ss)) != FQ_OK) return st;
+      if ((st = r.step(m0 + st_, &xb, left.data(), es.data())) != FQ_OK) return st;
     }
     for (int st_ = m1 - m0 - 1; st_ >= 0; --st_) {
       const int m = m0 + st_;
       r.omega(m);
       // bbar_L = conj(phase) a_L G (FP64 in its stacked block, slices in lsl[0])
       const double aL = p->cheb[L];
-      r.slice(w.f[gi], cph_r * aL, cph_i * aL, w.bbar_block(L, n), w.lsl[0], w.astride, w.esl[0]);
+      r.slice(w.f[gi], cph_r * aL, cph_i * aL, w.bbar_block(L, n), w.lsl[0], w.esl[0]);
       int sl = 0;
       for (int l = L - 1; l >= 0; --l) {
         const double a = p->cheb[l];
@@ -297,8 +287,8 @@ fq_status fq_grad_ozaki(fq_plan* p, const double* d_f, const void* d_W, double* 
         e.cpa_im = cph_i * a;
         e.cw = l == 0 ? 1.0 : 2.0;
         e.t.bound2 = 1e300;  // NaN / overflow check only
-        if ((st = oz_gemm<OZ_ADJ>(w, w.lsl[sl], w.astride, w.ncp, w.S, e, s)) != FQ_OK) return st;
-        if (l >= 1) r.slice(out, 1.0, 0.0, Planes{nullptr, nullptr}, w.lsl[sl ^ 1], w.astride, w.esl[sl ^ 1]);
+        if ((st = oz_gemm<OZ_ADJ>(w, w.lsl[sl], w.ncp, w.S, e, s)) != FQ_OK) return st;
+        if (l >= 1) r.slice(out, 1.0, 0.0, Planes{nullptr, nullptr}, w.lsl[sl ^ 1], w.esl[sl ^ 1]);
         sl ^= 1;
       }
       // D_l = <bbar_l, E psi_{l-1}>, l = 1..L, as one product over the L stacked blocks:
@@ -310,7 +300,7 @@ fq_status fq_grad_ozaki(fq_plan* p, const double* d_f, const void* d_W, double* 
       d.es = w.es_slot(st_ * L);
       d.et = w.etE;
       d.partial = w.partial + w.ncta;  // block l at partial + l * ncta
-      if ((st = oz_gemm<OZ_DOT>(w, w.slot(st_ * L), ss, L * w.ncp, w.E, d, s)) != FQ_OK) return st;
+      if ((st = oz_gemm<OZ_DOT>(w, w.slot(st_ * L), L * w.ncp, w.E, d, s)) != FQ_OK) return st;
       fq_launch_grad_reduce(w.partial, w.ncta, L, d_grad + m, s);
       std::swap(gi, gn);  // bbar_0 is the next G
     }

@@ -9,8 +9,8 @@
 // the MMAs of chunk c + 1 run.  With one MMA per pair and value of k, a group's sum over 256
 // values of k is at most 3 pairs x 2^14 x 256 < 2^24 units: still exact.
 //
-// Warp 0 streams TMA stages (K = 16 per stage: the two 64-row halves of each left slice and the
-// 64 rows of each right slice), warp 1 issues the MMAs, warps 2-17 drain (four per lane quarter,
+// Warp 0 streams the stages (K = 16 each: the two 64-row halves of each left slice and the 64 rows of
+// each right slice, two bulk copies), warp 1 issues the MMAs, warps 2-17 drain (four per lane quarter,
 // 16 columns each) and finally run the FP64 epilogue.  Clusters split K where tiles are few, and the
 // epilogue is kept short, as in ozaki_core.cuh.  Every wait is bounded as in the other tensor-core
 // kernels.
@@ -33,7 +33,7 @@ static_assert((size_t)OZR_STAGES * OZR_STAGE_BYTES >= OZR_XS_BYTES + 16 * sizeof
 
 template <int EPI>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    k_oz_real_term(const __grid_constant__ OzMaps maps, int nk, int tiles_j, int tiles_i, int np, int csize, OzEpi e) {
+    k_oz_real_term(const OzOperands op, int nk, int tiles_j, int tiles_i, int np, int csize, OzEpi e) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -97,13 +97,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const uint32_t st = base + s * OZR_STAGE_BYTES;
         const uint32_t bar = full0 + 8 * s;
         mbar_expect_tx(bar, OZR_STAGE_BYTES);
-        const int kx = (kb0 + kb) * OZ_BKE;
-#pragma unroll
-        for (int q = 0; q < OZ_S; ++q) {
-          tma_load_2d(st + q * OZR_A_BYTES, &maps.a[q], bar, kx, j0);                                // Re rows
-          tma_load_2d(st + q * OZR_A_BYTES + OZR_BM * OZ_ROWB, &maps.a[q], bar, np + kx, j0);        // Im rows
-          tma_load_2d(st + OZ_S * OZR_A_BYTES + q * OZR_B_BYTES, &maps.r[q], bar, kx, i0);           // S rows
-        }
+        const size_t kp = np / OZ_BKE, kx = kb0 + kb;  // K pieces of a block, and this one
+        bulk_load(st, op.left + ((size_t)(j0 / OZR_BM) * kp + kx) * (OZ_S * OZR_A_BYTES / 2), OZ_S * OZR_A_BYTES, bar);
+        bulk_load(st + OZ_S * OZR_A_BYTES, op.right + ((size_t)(i0 / OZ_BN) * kp + kx) * (OZ_S * OZR_B_BYTES / 2),
+                  OZ_S * OZR_B_BYTES, bar);
         issued = kb + 1;
       }
       if (!ok) {
