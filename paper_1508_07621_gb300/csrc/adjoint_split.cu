@@ -375,7 +375,7 @@ struct Runner {
       e.out_im = w.f[out].im;
       e.slice_out = left[l + 1];
       e.slice_stride = stride;
-      e.t = t;
+      e.t = split_term(t);
       eps[l] = e;
       lefts[l] = Left{left[l], stride, w.ncp};
       if (t.last) {
@@ -481,7 +481,7 @@ fq_status fq_grad_split(fq_plan* p, const double* d_f, const void* d_W, double* 
         e.cpa_re = (float)(cph_r * a);
         e.cpa_im = (float)(cph_i * a);
         e.cw = l == 0 ? 1.f : 2.f;
-        e.t.bound2 = 1e30;  // NaN / overflow check only
+        e.t.bound2 = 1e30f;  // NaN / overflow check only
         aeps.push_back(e);
         alefts.push_back(Left{w.lsl[sl], w.astride, w.ncp});
         sl ^= 1;

@@ -203,7 +203,7 @@ static fq_status run_split(fq_plan* p, const double* x0, double* x, int nc, int 
       e.out_im = w.m[out][1];
       e.slice_out = w.a[av ^ 1];
       e.slice_stride = w.astride;
-      e.t = t;
+      e.t = split_term(t);
       left_of[l] = av;
       av ^= 1;
       if (t.last) {

@@ -59,8 +59,9 @@ struct ScanInst {  // 128-byte aligned through its tensor maps
   unsigned int* status;
   unsigned int* termcnt;   // [L][tiles_j]
   unsigned int* omegacnt;  // [2]: finished B-unit epilogue warps writing buffer 0 / 1
-  double cheb[SCAN_MAXL + 1];
-  double sbeta, ph_re, ph_im;
+  float cheb[SCAN_MAXL + 1];  // the terms' scalars, as SplitTerm's
+  float ph_re, ph_im;
+  double sbeta;
   size_t bstride, astride;
   int n, ldm, np, kp, L, tiles_i, tiles_j, nk, nblk, steps;
 };
@@ -169,7 +170,7 @@ __device__ __forceinline__ void scan_epi(const ScanInst& I, int m, int p, SplitE
   e.t.coef = I.cheb[p + 1];
   e.t.ph_re = I.ph_re;
   e.t.ph_im = I.ph_im;
-  e.t.bound2 = 1.0 + 2e-3;
+  e.t.bound2 = (float)(1.0 + 2e-3);
   e.t.status = I.status;
 }
 
@@ -469,9 +470,9 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_split_scan(const __grid_con
       }
       if (bad) atomicOr(I.status, FQ_BIT_BOUND);
       // this warp's stores of the tile made visible (to the async proxy too), then one release per
-      // warp: a state block is done when the epilogue warps of each of its tiles have counted
+      // warp, which covers the lanes' stores through the barrier: a state block is done when the epilogue
+      // warps of each of its tiles have counted
       fence_proxy_async_global();
-      __threadfence();
       __syncwarp();
       if (lane == 0) red_release_add(I.termcnt + (size_t)d.p * I.tiles_j + tj, 1u);
       ++k;
@@ -671,9 +672,9 @@ fq_status scan_capture(fq_plan* const* plans, int count, void* const* d_U, char*
     I.k = p->d_k;
     I.scal = p->d_scal;
     I.sbeta = p->sbeta;
-    I.ph_re = p->phase_re;
-    I.ph_im = p->phase_im;
-    for (int l = 0; l <= p->L; ++l) I.cheb[l] = p->cheb[l];
+    I.ph_re = (float)p->phase_re;
+    I.ph_im = (float)p->phase_im;
+    for (int l = 0; l <= p->L; ++l) I.cheb[l] = (float)p->cheb[l];
     I.status = p->d_status;
     I.u = (double2*)d_U[i];
     I.os_buf[0] = w.os;

@@ -138,6 +138,22 @@ __device__ __forceinline__ void split_f32(float x, __nv_bfloat16 (&s)[NS]) {
   }
 }
 
+// NS slices of two values, packed (a's in the low half): the slices of split_f32, two to a conversion
+// (a conversion takes as long as eight FP32 instructions; with one per slice they were a third of the
+// epilogue's arithmetic).  With this and SplitTerm a BF16X3 / X6 product of 64-wide tiles went from
+// 13.9 / 17.7 to 13.5 / 16.7 us at N = 200 and from 27.2 / 43.6 to 26.1 / 42.4 us at N = 1000, a gradient
+// step at N = 1024 from 589 to 576 us (X3).
+template <int NS>
+__device__ __forceinline__ void split_pair(float a, float b, uint32_t (&s)[NS]) {
+#pragma unroll
+  for (int t = 0; t < NS; ++t) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    s[t] = (uint32_t)__bfloat16_as_ushort(h.x) | ((uint32_t)__bfloat16_as_ushort(h.y) << 16);
+    a -= __uint_as_float(s[t] << 16);
+    b -= __uint_as_float(s[t] & 0xffff0000u);
+  }
+}
+
 template <int NS>
 __device__ __forceinline__ void split_f64(double x, __nv_bfloat16 (&s)[NS]) {
   double r = x;
@@ -220,6 +236,19 @@ enum SplitMode {
   EPI_DOT = 2,  // gradient dot: partial[cta] = sum over the tile of conj(b) Y
 };
 
+// A Chebyshev term's scalars in FP32 (converted once: FP64 conversions run at the FP64 rate, five of them
+// took 600 cycles of every 32 x 32 block).
+struct SplitTerm {
+  int first, last;
+  float coef0, coef, ph_re, ph_im, bound2;
+  unsigned int* status;
+};
+
+SplitTerm split_term(const fq_term& t) {
+  return SplitTerm{t.first,          t.last,           (float)t.coef0,   (float)t.coef,
+                   (float)t.ph_re,   (float)t.ph_im,   (float)t.bound2,  t.status};
+}
+
 struct SplitEpi {
   int n, nc, ldm, np;          // dims; ldm: FP32 master row stride; np: real part width in K'
   const float* cur_re;         // FWD: psi_l masters (first term: psi_0); ADJ: g; DOT: b
@@ -235,7 +264,7 @@ struct SplitEpi {
   int kp;
   float cpa_re, cpa_im, cw;    // ADJ coefficients
   double2* partial;            // DOT output, one per CTA
-  fq_term t;
+  SplitTerm t;
 };
 
 template <int NS, int BN, int BKE, bool HAS_A>
@@ -343,20 +372,18 @@ __device__ __forceinline__ void store_slices(const SplitEpi& e, int j, int ib, i
   const size_t srow = (size_t)j * e.kp + ib;
 #pragma unroll
   for (int part = 0; part < 2; ++part) {
-    __nv_bfloat16 s[4][NS];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) split_f32<NS>(part ? o_i[q] : o_r[q], s[q]);
+    uint32_t lo[NS], hi[NS];  // two bf16 per word
+    split_pair<NS>(part ? o_i[0] : o_r[0], part ? o_i[1] : o_r[1], lo);
+    split_pair<NS>(part ? o_i[2] : o_r[2], part ? o_i[3] : o_r[3], hi);
 #pragma unroll
     for (int t = 0; t < NS; ++t) {
       __nv_bfloat16* d = e.slice_out + t * e.slice_stride + srow + (part ? e.np : 0);
-      if (cnt >= 4) {  // two bf16 per word, element 2w in the low half
-        const uint32_t lo = (uint32_t)__bfloat16_as_ushort(s[0][t]) | ((uint32_t)__bfloat16_as_ushort(s[1][t]) << 16);
-        const uint32_t hi = (uint32_t)__bfloat16_as_ushort(s[2][t]) | ((uint32_t)__bfloat16_as_ushort(s[3][t]) << 16);
-        *reinterpret_cast<uint2*>(d) = make_uint2(lo, hi);
+      if (cnt >= 4) {
+        *reinterpret_cast<uint2*>(d) = make_uint2(lo[t], hi[t]);
       } else {
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          if (q < cnt) d[q] = s[q][t];
+          if (q < cnt) d[q] = __ushort_as_bfloat16((unsigned short)((q < 2 ? lo[t] : hi[t]) >> (16 * (q & 1))));
       }
     }
   }
@@ -411,13 +438,30 @@ __device__ __forceinline__ void split_load_y(uint32_t trow, int c0, float* stage
   }
 }
 
+// A Chebyshev term at one entry of Y: psi_{l+1} = -2i Y + psi_{l-1} (x; the first term, psi_1 = -i Y, has sg = 1
+// and x = 0) and z += a_{l+1} psi_{l+1} (the first term's z is a_0 psi_0).  Spelt out in FMAs so that every kernel
+// rounds alike.
+__device__ __forceinline__ void fwd_entry(float sg, float c, float yr, float yi, float xr, float xi, float& zr,
+                                          float& zi, float& nr, float& ni) {
+  nr = fmaf(sg, yi, xr);
+  ni = fmaf(-sg, yr, xi);
+  zr = fmaf(c, nr, zr);
+  zi = fmaf(c, ni, zi);
+}
+
+// X = e^{-i beta h} acc of one entry, the phase (pr, pi).
+__device__ __forceinline__ void fwd_phase(float pr, float pi, float ar, float ai, float& o_r, float& o_i) {
+  o_r = fmaf(pr, ar, -__fmul_rn(pi, ai));
+  o_i = fmaf(pr, ai, __fmul_rn(pi, ar));
+}
+
 // Epilogue of one 32-row x 32-column block (rows jb .., columns ib0 ..) in the layout of
 // epi_transpose; BATCH row groups' operands are loaded together.
 template <int NS, int EPI, int BATCH>
 __device__ __forceinline__ void epi_block(const SplitEpi& e, const float (&yr)[32], const float (&yi)[32], int jb,
                                           int ib0, int lane, bool& bad, double& dsr, double& dsi) {
-  const float c0f = (float)e.t.coef0, cf = (float)e.t.coef, pr_ = (float)e.t.ph_re, pi_ = (float)e.t.ph_im;
-  const float b2 = (float)e.t.bound2;
+  const float c0f = e.t.coef0, cf = e.t.coef, sg = e.t.first ? 1.f : 2.f;
+  const float b2 = e.t.bound2;
   const int ib = ib0 + 4 * (lane & 7), cnt = min(4, e.n - ib);
   if (cnt <= 0) return;
   // The operands are loaded without a branch: rows are clamped to the block, a row's four entries at ib
@@ -452,6 +496,14 @@ __device__ __forceinline__ void epi_block(const SplitEpi& e, const float (&yr)[3
 #pragma unroll
         for (int q = 0; q < 4; ++q) z_r[u][q] = z_i[u][q] = 0.f;
       }
+      if (first) {  // z holds psi_0
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          z_r[u][q] = __fmul_rn(c0f, z_r[u][q]);
+          z_i[u][q] = __fmul_rn(c0f, z_i[u][q]);
+          x_r[u][q] = x_i[u][q] = 0.f;
+        }
+      }
     }
 #pragma unroll
     for (int u = 0; u < BATCH; ++u) {
@@ -479,28 +531,12 @@ __device__ __forceinline__ void epi_block(const SplitEpi& e, const float (&yr)[3
       } else {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          float nr, ni, ar, ai;
-          if (e.t.first) {  // psi_1 = -i Y, acc = a_0 psi_0 + a_1 psi_1
-            nr = vi[q];
-            ni = -vr[q];
-            ar = c0f * x_r[u][q] + cf * nr;
-            ai = c0f * x_i[u][q] + cf * ni;
-          } else {  // psi_{l+1} = -2i Y + psi_{l-1}, acc += a_{l+1} psi_{l+1}
-            nr = 2.f * vi[q] + x_r[u][q];
-            ni = -2.f * vr[q] + x_i[u][q];
-            ar = z_r[u][q] + cf * nr;
-            ai = z_i[u][q] + cf * ni;
-          }
-          bad |= q < cnt && !(nr * nr + ni * ni <= b2);
-          if (e.t.last) {  // X = e^{-i beta h} (acc + a_L psi_L)
-            o_r[q] = pr_ * ar - pi_ * ai;
-            o_i[q] = pr_ * ai + pi_ * ar;
-          } else {
-            o_r[q] = nr;
-            o_i[q] = ni;
-          }
-          z_r[u][q] = ar;
-          z_i[u][q] = ai;
+          fwd_entry(sg, cf, vr[q], vi[q], x_r[u][q], x_i[u][q], z_r[u][q], z_i[u][q], o_r[q], o_i[q]);
+          bad |= q < cnt && !(o_r[q] * o_r[q] + o_i[q] * o_i[q] <= b2);
+        }
+        if (e.t.last) {  // X in place of psi_L
+#pragma unroll
+          for (int q = 0; q < 4; ++q) fwd_phase(e.t.ph_re, e.t.ph_im, z_r[u][q], z_i[u][q], o_r[q], o_i[q]);
         }
         if (!e.t.last) {
           store4(e.acc_re, idx, cnt, z_r[u]);
@@ -1016,9 +1052,9 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
         if (i0 + c0 < e.n) epi_block<NS, EPI, 4>(e, yr, yi, j0 + quarter * 32, i0 + c0, lane, bad, dsr, dsi);
       }
       // this warp's stores of the unit made visible (to the async proxy too), then one release per
-      // warp: a tile is done when its epilogue warps have counted
+      // warp, which covers the lanes' stores through the barrier: a tile is done when its epilogue warps
+      // have counted
       fence_proxy_async_global();
-      __threadfence();
       __syncwarp();
       if (lane == 0) red_release_add(args.flags + (size_t)p * args.tiles_j + tj, 1u);
     }
