@@ -228,7 +228,10 @@ static fq_status run_split(fq_plan* p, const double* x0, double* x, int nc, int 
       }
       cudaError_t ce = cudaMemsetAsync(w.flags, 0, sizeof(unsigned int) * (size_t)L * tiles_j, s);
       if (ce != cudaSuccess) return fq_cuda_fail(ce, "chain counters");
-      st = launch_chain<NS, BN, BKE, EPI_FWD, true>(ch, s);
+      st = FQ_EUNSUPPORTED;
+      if constexpr (Cfg::STACKED)  // one tile a CTA: its states stay on the SM (k_split_chain, KEEP)
+        if (tiles_i * tiles_j <= sms) st = launch_chain<NS, BN, BKE, EPI_FWD, true, true>(ch, s);
+      if (st == FQ_EUNSUPPORTED) st = launch_chain<NS, BN, BKE, EPI_FWD, true>(ch, s);
       if (st != FQ_OK && st != FQ_EUNSUPPORTED) return st;
     }
     if (st == FQ_EUNSUPPORTED)

@@ -123,6 +123,25 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
 }
 
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v[q] = __uint_as_float(r[q]);
+}
+
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float* v) {
+  uint32_t r[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) r[q] = __float_as_uint(v[q]);
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"r"(r[0]), "r"(r[1]),
+               "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(taddr)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -901,13 +920,162 @@ __device__ __forceinline__ bool wait_count(const unsigned int* p, unsigned int t
   return true;
 }
 
-template <int NS, int BN, int BKE, int EPI, bool HAS_A>
+// The FP32 side of a kept tile (KEEP chains): this warp's 32 rows (lane = row) x 32 columns of psi_l,
+// psi_{l-1} and acc over the products of a chain.  The two states stay in tensor memory, columns
+// KEEP_COL + 128 slot + 64 part (psi_l in slot l & 1), and acc in registers.
+constexpr uint32_t KEEP_COL = 256;
+template <int NS> constexpr int KEEP_STAGE_BYTES = 2 * NS * 1024;  // 16 columns of a warp's slices
+template <int NS>
+struct KeptTile {
+  float ar[32], ai[32];
+  int row, col;    // this lane's row, the warp's first column
+  uint32_t trow;   // the warp's tensor-memory lanes
+  unsigned char* stage;
+
+  // psi_0 from the masters of the first product (slot 0; slot 1 is the first term's zero), acc = a_0 psi_0
+  __device__ __forceinline__ void load(const SplitEpi& e, int half) {
+    const size_t base = (size_t)min(row, e.nc - 1) * e.ldm;
+#pragma unroll
+    for (int q = 0; q < 32; q += 4) {
+      float v[4] = {}, w[4] = {};
+      if (col + q < e.n) {  // ldm is a multiple of 4
+        load_f4(e.cur_re + base + col + q, v);
+        load_f4(e.cur_im + base + col + q, w);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        ar[q + u] = row < e.nc && col + q + u < e.n ? v[u] : 0.f;
+        ai[q + u] = row < e.nc && col + q + u < e.n ? w[u] : 0.f;
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 32; c += 8) {
+      const float zero[8] = {};
+      const uint32_t at = trow + KEEP_COL + 32 * half + c;
+      tmem_st8(at, ar + c);
+      tmem_st8(at + 64, ai + c);
+      tmem_st8(at + 128, zero);
+      tmem_st8(at + 192, zero);
+    }
+    tmem_wait_st();
+#pragma unroll
+    for (int q = 0; q < 32; ++q) {
+      ar[q] = __fmul_rn(e.t.coef0, ar[q]);
+      ai[q] = __fmul_rn(e.t.coef0, ai[q]);
+    }
+  }
+
+  // product p of the chain from the tile's sums (64 columns each: Psi_r.S, Psi_r.A, Psi_i.S, Psi_i.A):
+  // the new state, acc and the slices; `tempty` is signalled once the sums are read.
+  __device__ __forceinline__ void term(const SplitEpi& e, int p, int half, int lane, uint32_t tempty, bool& bad) {
+    const float cf = e.t.coef, sg = e.t.first ? 1.f : 2.f, b2 = e.t.bound2;
+    const bool last = e.t.last, edge = col + 32 > e.n;
+    const uint32_t psi = trow + KEEP_COL + 128 * ((p + 1) & 1) + 32 * half;  // psi_{l-1}, then psi_{l+1}
+#pragma unroll
+    for (int c = 0; c < 32; c += 8) {
+      float y[2][8], w[2][8], x[2][8];
+      const uint32_t sums = trow + 32 * half + c;
+      tmem_ld8(sums, y[0]);
+      tmem_ld8(sums + 192, w[0]);
+      tmem_ld8(sums + 64, y[1]);
+      tmem_ld8(sums + 128, w[1]);
+      tmem_ld8(psi + c, x[0]);
+      tmem_ld8(psi + 64 + c, x[1]);
+      tmem_wait_ld();
+      if (c == 24) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty);
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        float o_r, o_i;
+        fwd_entry(sg, cf, y[0][q] - w[0][q], y[1][q] + w[1][q], x[0][q], x[1][q], ar[c + q], ai[c + q], o_r, o_i);
+        bad |= !(o_r * o_r + o_i * o_i <= b2);  // zero beyond the block
+        y[0][q] = o_r;
+        y[1][q] = o_i;
+      }
+      if (last) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          fwd_phase(e.t.ph_re, e.t.ph_im, ar[c + q], ai[c + q], y[0][q], y[1][q]);
+          ar[c + q] = y[0][q];
+          ai[c + q] = y[1][q];
+        }
+      }
+      if (edge) {  // the slices' padding stays zero, also beside an entry that is not finite
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (col + c + q >= e.n) y[0][q] = y[1][q] = 0.f;
+      }
+      if (!last) {
+        tmem_st8(psi + c, y[0]);
+        tmem_st8(psi + 64 + c, y[1]);
+      }
+      // slices: 16 columns of a row, slice and part are 32 bytes, staged so that a warp's global stores
+      // take 16 whole rows each
+#pragma unroll
+      for (int part = 0; part < 2; ++part) {
+        uint32_t pk[4][NS];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) split_pair<NS>(y[part][2 * q], y[part][2 * q + 1], pk[q]);
+#pragma unroll
+        for (int t = 0; t < NS; ++t)
+          *reinterpret_cast<uint4*>(stage + (2 * t + part) * 1024 + lane * 32 +
+                                    16 * (((c >> 3) & 1) ^ ((lane >> 2) & 1))) =
+              make_uint4(pk[0][t], pk[1][t], pk[2][t], pk[3][t]);
+      }
+      if ((c & 8) == 0) continue;
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int r = 16 * k + (lane >> 1), u = lane & 1, j = row - lane + r;
+        if (j < e.nc) {
+          __nv_bfloat16* d = e.slice_out + (size_t)j * e.kp + col + (c - 8) + 8 * u;
+#pragma unroll
+          for (int t = 0; t < NS; ++t)
+#pragma unroll
+            for (int part = 0; part < 2; ++part)
+              *reinterpret_cast<uint4*>(d + t * e.slice_stride + part * e.np) =
+                  *reinterpret_cast<const uint4*>(stage + (2 * t + part) * 1024 + r * 32 + 16 * (u ^ ((r >> 2) & 1)));
+        }
+      }
+      __syncwarp();
+    }
+    tmem_wait_st();
+    if (last) {  // X to the masters
+      const int ib = col + 4 * (lane & 7), cnt = min(4, e.n - ib);
+#pragma unroll
+      for (int part = 0; part < 2; ++part) {
+        float u[32];
+        epi_transpose(reinterpret_cast<float*>(stage), lane, part ? ai : ar, u);
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+          const int j = row - lane + 4 * g + (lane >> 3);
+          const float v[4] = {u[4 * g], u[4 * g + 1], u[4 * g + 2], u[4 * g + 3]};
+          if (j < e.nc) store4(part ? e.out_im : e.out_re, (size_t)j * e.ldm + ib, cnt, v);
+        }
+      }
+    }
+  }
+};
+
+// KEEP: every CTA owns one tile for the whole chain (grid = tiles), and its states and accumulator stay
+// on the SM (KeptTile); only slices are exchanged.  A tile's epilogue otherwise reads 128 KB of FP32 masters
+// and writes as much, between the last MMA of a product and the first of the next.  The second buffer
+// of sums, which a CTA with one tile a product has no use for, makes room for the states.
+// BF16X3 / X6 products, masters in memory / kept: N = 64 9.8 / 7.9 and 11.5 / 9.8 us, N = 256 12.9 / 11.9 and
+// 17.5 / 16.8, N = 700 21.9 / 19.0 and 32.1 / 30.7, N = 1024 25.6 / 24.4 and 42.0 / 41.2.  What is left at N = 1000 is
+// the MMAs (80 cycles each for 64 at the tensor rate: 8 KB of operands from shared memory), 16 of
+// 24 us, then the epilogue (its arithmetic, 3 us), the release and the first stage's load.
+template <int NS, int BN, int BKE, int EPI, bool HAS_A, bool KEEP>
 __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_constant__ ChainArgs args) {
   static_assert(EPI != EPI_DOT, "chains of forward or adjoint terms only");
   using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
   constexpr int STAGES = Cfg::STAGES;
+  static_assert(!KEEP || (Cfg::STACKED && EPI == EPI_FWD), "kept tiles: 64-wide forward terms");
   constexpr uint32_t BUF_COLS = Cfg::ACC_COLS;
-  constexpr uint32_t TMEM_COLS = 2 * BUF_COLS;
+  constexpr uint32_t TMEM_COLS = 2 * BUF_COLS;  // two buffers of sums (KEEP: one, and the states)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -993,8 +1161,9 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
       int g = 0, i = 0;
       bool ok = true;
       for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x, ++i) {
-        const int b = i & 1;
-        if (i >= 2 && !(ok = mbar_wait(tempty0 + 8 * b, ((i >> 1) - 1) & 1))) break;
+        const int b = KEEP ? 0 : i & 1;
+        if (KEEP && i >= 1 && !(ok = mbar_wait(tempty0, (i - 1) & 1))) break;
+        if (!KEEP && i >= 2 && !(ok = mbar_wait(tempty0 + 8 * b, ((i >> 1) - 1) & 1))) break;
         const uint32_t acc = tmem + (uint32_t)b * BUF_COLS;
         for (int kb = 0; kb < args.nk; ++kb, ++g) {
           const int s = g % STAGES;
@@ -1025,31 +1194,46 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
     bool bad = false, ok = true;
     double dsr = 0.0, dsi = 0.0;
     int i = 0;
+    KeptTile<NS> kept;
+    const int half = (warp - 2) >> 2;
+    if constexpr (KEEP) {
+      int p, tj, j0, i0;
+      unit(blockIdx.x, p, tj, j0, i0);
+      kept.row = j0 + quarter * 32 + lane;
+      kept.col = i0 + 32 * half;
+      kept.trow = tmem + ((uint32_t)(quarter * 32) << 16);
+      kept.stage = gbase + STAGES * Cfg::STAGE_BYTES + Cfg::TAIL + (warp - 2) * KEEP_STAGE_BYTES<NS>;
+      kept.load(args.epi[0], half);
+    }
     for (int u = blockIdx.x; u < nunits; u += gridDim.x, ++i) {
       int p, tj, j0, i0;
       unit(u, p, tj, j0, i0);
-      const int b = i & 1;
-      bool go = mbar_wait(tfull0 + 8 * b, (i >> 1) & 1);
+      const int b = KEEP ? 0 : i & 1;
+      bool go = mbar_wait(tfull0 + 8 * b, KEEP ? i & 1 : (i >> 1) & 1);
       tc_fence_after();
       go = __all_sync(0xffffffffu, go && !*(volatile int*)abort_flag);
       if (!go) {
         ok = false;
         break;
       }
-      // the previous product's outputs this epilogue reads (prev, acc) were released with its counter
-      if (p > 0) ld_acquire_u32(args.flags + (size_t)(p - 1) * args.tiles_j + tj);
       const SplitEpi& e = args.epi[p];
-      const uint32_t trow = tmem + (uint32_t)b * BUF_COLS + ((uint32_t)(quarter * 32) << 16);
+      if constexpr (KEEP) {
+        kept.term(e, p, half, lane, tempty0, bad);
+      } else {
+        // the previous product's outputs this epilogue reads (prev, acc) were released with its counter
+        if (p > 0) ld_acquire_u32(args.flags + (size_t)(p - 1) * args.tiles_j + tj);
+        const uint32_t trow = tmem + (uint32_t)b * BUF_COLS + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
-      for (int c0 = epi_begin<BN>(warp), c1 = c0 + BN * 4 / EPI_WARPS; c0 < c1; c0 += 32) {
-        float yr[32], yi[32];
-        split_load_y<NS, BN, BKE, HAS_A>(trow, c0, stage, lane, yr, yi);
-        if (c0 + 32 >= c1) {  // this warp's sums are read: the buffer's next MMAs may start
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(tempty0 + 8 * b);
+        for (int c0 = epi_begin<BN>(warp), c1 = c0 + BN * 4 / EPI_WARPS; c0 < c1; c0 += 32) {
+          float yr[32], yi[32];
+          split_load_y<NS, BN, BKE, HAS_A>(trow, c0, stage, lane, yr, yi);
+          if (c0 + 32 >= c1) {  // this warp's sums are read: the buffer's next MMAs may start
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(tempty0 + 8 * b);
+          }
+          if (i0 + c0 < e.n) epi_block<NS, EPI, 4>(e, yr, yi, j0 + quarter * 32, i0 + c0, lane, bad, dsr, dsi);
         }
-        if (i0 + c0 < e.n) epi_block<NS, EPI, 4>(e, yr, yi, j0 + quarter * 32, i0 + c0, lane, bad, dsr, dsi);
       }
       // this warp's stores of the unit made visible (to the async proxy too), then one release per
       // warp, which covers the lanes' stores through the barrier: a tile is done when its epilogue warps
@@ -1075,22 +1259,24 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
 // Launches a chain cooperatively (all CTAs resident).  FQ_EUNSUPPORTED when that cannot be done
 // (a capturing stream, or the device refuses the cooperative launch): the caller then runs the
 // products one launch each.
-template <int NS, int BN, int BKE, int EPI, bool HAS_A>
+template <int NS, int BN, int BKE, int EPI, bool HAS_A, bool KEEP = false>
 fq_status launch_chain(const ChainArgs& args, cudaStream_t s) {
   using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
+  constexpr size_t SMEM = KEEP ? Cfg::SMEM + EPI_WARPS * (KEEP_STAGE_BYTES<NS> - EPI_STAGE_BYTES) : Cfg::SMEM;
+  static_assert(KEEP_STAGE_BYTES<NS> >= EPI_STAGE_BYTES && SMEM <= 232448, "shared memory of one CTA");
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return FQ_EUNSUPPORTED;
   static std::atomic<unsigned> attr_set{0};
   if (fq_first_on_device(attr_set)) {
-    cudaError_t e = cudaFuncSetAttribute(k_split_chain<NS, BN, BKE, EPI, HAS_A>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_split_chain<NS, BN, BKE, EPI, HAS_A, KEEP>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
     if (e != cudaSuccess) return fq_cuda_fail(e, "chain kernel shared-memory attribute");
   }
   const int tiles = args.tiles_i * args.tiles_j;
   const int grid = std::min(tiles, fq_sm_count());
   void* kargs[] = {(void*)&args};
-  cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_split_chain<NS, BN, BKE, EPI, HAS_A>, dim3(grid),
-                                              dim3(PTHREADS), kargs, Cfg::SMEM, s);
+  cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_split_chain<NS, BN, BKE, EPI, HAS_A, KEEP>, dim3(grid),
+                                              dim3(PTHREADS), kargs, SMEM, s);
   if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
     cudaGetLastError();
     return FQ_EUNSUPPORTED;

@@ -91,6 +91,46 @@ def test_split_default_tile(fq, prec):
     assert torch.equal(X.transpose(0, 1), U[:, 17:20])
 
 
+@pytest.mark.parametrize("prec", [2, 3])
+@pytest.mark.parametrize("n,nc", [(1, 1), (63, 5), (130, 129), (257, 200), (1024, 1024), (1100, 100)])
+def test_split_kept_tiles(fq, prec, n, nc):
+    """Chains whose tiles fit one to an SM keep states and accumulator on the SM, larger ones and a
+    captured stream's single products keep them in memory: the same bits.  n = 1100 has 162 tiles a
+    product for a whole build and 18 for 100 states."""
+    import torch
+    kw = dict(omega=1.3, f_ac=1.1, f_dc=0.2, phi0=0.4, steps=5, precision=prec, tile_n=64)
+    plan = fq.Plan.dense(fi.goe(n, 1315), fi.goe(n, 1316), **kw)
+    U = plan.build_UT()
+    X = plan.propagate(torch.eye(n, dtype=torch.complex128, device="cuda")[:nc].contiguous())
+    assert torch.equal(X.transpose(0, 1), U[:, :nc])
+    ws = fq.workspace(plan.workspace_size())
+    V = torch.empty_like(U)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        plan.build_UT(V, ws)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(U, V)
+    assert plan.check_status() == 0
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_split_kept_tiles_not_finite(fq, bad):
+    """A state with an entry that is not finite is reported and leaves the others as they are."""
+    import torch
+    n = 90
+    plan = fq.Plan.dense(fi.goe(n, 1317), fi.goe(n, 1318), omega=1.3, f_ac=1.1, steps=4, precision=2)
+    x = torch.eye(n, dtype=torch.complex128, device="cuda")[:40].contiguous()
+    clean = plan.propagate(x.clone())
+    assert plan.check_status() == 0
+    x[17, 3] = bad
+    X = plan.propagate(x)
+    keep = [j for j in range(40) if j != 17]
+    assert torch.equal(X[keep], clean[keep])
+    assert not torch.isfinite(X[17].abs()).any()
+    assert plan.check_status() != 0
+
+
 @pytest.mark.parametrize("prec,ns,tile,tk", SHAPES)
 def test_split_ragged_propagate(fq, prec, ns, tile, tk):
     """N = 200 (K' padded to 512, output tiles ragged), 37 states (one partial 128-row tile),
