@@ -234,7 +234,8 @@ fq_status gemm_cfg(const GemmCtx& c, Left left, const __nv_bfloat16* right, cons
     if (r != cudaSuccess) return fq_cuda_fail(r, "split gradient kernel shared-memory attribute");
   }
   const int sms = fq_sm_count();
-  const int tiles_i = c.np / BN, tiles_j = left.rows / BM, nk = c.np / BKE;
+  const int tiles_i = c.np / BN, tiles_j = left.rows / BM;
+  const int nk = (c.n + BKE - 1) / BKE;  // the operands' columns beyond N are zero
   if constexpr (persist)
     k_split_persist<NS, BN, BKE, EPI, false><<<std::min(tiles_i * tiles_j, sms), PTHREADS, Cfg::SMEM, s>>>(
         maps, nk, tiles_j, tiles_i, e);
@@ -269,12 +270,20 @@ fq_status chain_cfg(const GemmCtx& c, const Left* lefts, const SplitEpi* eps, in
     ch.epi[pp] = eps[pp];
   }
   ch.nprod = nprod;
-  ch.nk = c.np / BKE;
+  ch.nk = (c.n + BKE - 1) / BKE;  // the operands' columns beyond N are zero
   ch.tiles_i = c.np / BN;
   ch.tiles_j = lefts[0].rows / BM;
   ch.flags = flags;
   cudaError_t ce = cudaMemsetAsync(flags, 0, sizeof(unsigned int) * (size_t)nprod * ch.tiles_j, s);
   if (ce != cudaSuccess) return fq_cuda_fail(ce, "chain counters");
+  // one tile a CTA: the forward states stay on the SM (k_split_chain, KEEP), except in BF16X6, whose three
+  // K stages leave no room for the wider slice stage.  With K also cut at N a BF16X3 gradient step went from
+  // 199 to 161 us at N = 64, from 446 to 401 at N = 700 and from 570 to 552 at N = 1024.
+  if constexpr (EPI == EPI_FWD && BN == 64 && NS == 2)
+    if (ch.tiles_i * ch.tiles_j <= fq_sm_count()) {
+      st = launch_chain<NS, BN, BKE, EPI, false, true>(ch, s);
+      if (st != FQ_EUNSUPPORTED) return st;
+    }
   return launch_chain<NS, BN, BKE, EPI, false>(ch, s);
 }
 

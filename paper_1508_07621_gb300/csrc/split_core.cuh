@@ -925,7 +925,7 @@ __device__ __forceinline__ bool wait_count(const unsigned int* p, unsigned int t
 // KEEP_COL + 128 slot + 64 part (psi_l in slot l & 1), and acc in registers.
 constexpr uint32_t KEEP_COL = 256;
 template <int NS> constexpr int KEEP_STAGE_BYTES = 2 * NS * 1024;  // 16 columns of a warp's slices
-template <int NS>
+template <int NS, bool STACKED>
 struct KeptTile {
   float ar[32], ai[32];
   int row, col;    // this lane's row, the warp's first column
@@ -965,8 +965,8 @@ struct KeptTile {
     }
   }
 
-  // product p of the chain from the tile's sums (64 columns each: Psi_r.S, Psi_r.A, Psi_i.S, Psi_i.A):
-  // the new state, acc and the slices; `tempty` is signalled once the sums are read.
+  // product p of the chain from the tile's sums (64 columns each: Psi_r.S, Psi_r.A, Psi_i.S, Psi_i.A
+  // when STACKED, else Yr and Yi): the new state, acc and the slices; `tempty` is signalled once the sums are read.
   __device__ __forceinline__ void term(const SplitEpi& e, int p, int half, int lane, uint32_t tempty, bool& bad) {
     const float cf = e.t.coef, sg = e.t.first ? 1.f : 2.f, b2 = e.t.bound2;
     const bool last = e.t.last, edge = col + 32 > e.n;
@@ -976,9 +976,11 @@ struct KeptTile {
       float y[2][8], w[2][8], x[2][8];
       const uint32_t sums = trow + 32 * half + c;
       tmem_ld8(sums, y[0]);
-      tmem_ld8(sums + 192, w[0]);
       tmem_ld8(sums + 64, y[1]);
-      tmem_ld8(sums + 128, w[1]);
+      if (STACKED) {
+        tmem_ld8(sums + 192, w[0]);
+        tmem_ld8(sums + 128, w[1]);
+      }
       tmem_ld8(psi + c, x[0]);
       tmem_ld8(psi + 64 + c, x[1]);
       tmem_wait_ld();
@@ -990,7 +992,8 @@ struct KeptTile {
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         float o_r, o_i;
-        fwd_entry(sg, cf, y[0][q] - w[0][q], y[1][q] + w[1][q], x[0][q], x[1][q], ar[c + q], ai[c + q], o_r, o_i);
+        const float yr = STACKED ? y[0][q] - w[0][q] : y[0][q], yi = STACKED ? y[1][q] + w[1][q] : y[1][q];
+        fwd_entry(sg, cf, yr, yi, x[0][q], x[1][q], ar[c + q], ai[c + q], o_r, o_i);
         bad |= !(o_r * o_r + o_i * o_i <= b2);  // zero beyond the block
         y[0][q] = o_r;
         y[1][q] = o_i;
@@ -1073,9 +1076,9 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
   static_assert(EPI != EPI_DOT, "chains of forward or adjoint terms only");
   using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
   constexpr int STAGES = Cfg::STAGES;
-  static_assert(!KEEP || (Cfg::STACKED && EPI == EPI_FWD), "kept tiles: 64-wide forward terms");
+  static_assert(!KEEP || (BN == 64 && EPI == EPI_FWD), "kept tiles: 64-wide forward terms");
   constexpr uint32_t BUF_COLS = Cfg::ACC_COLS;
-  constexpr uint32_t TMEM_COLS = 2 * BUF_COLS;  // two buffers of sums (KEEP: one, and the states)
+  constexpr uint32_t TMEM_COLS = KEEP ? 512 : 2 * BUF_COLS;  // two buffers of sums (KEEP: one, and the states)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -1194,7 +1197,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
     bool bad = false, ok = true;
     double dsr = 0.0, dsi = 0.0;
     int i = 0;
-    KeptTile<NS> kept;
+    KeptTile<NS, Cfg::STACKED> kept;
     const int half = (warp - 2) >> 2;
     if constexpr (KEEP) {
       int p, tj, j0, i0;

@@ -136,6 +136,28 @@ def test_split_grad_matches_oracle(fq, prec, eps, n, M, stride, tile):
     assert abs(float(loss.item()) - ref_loss) <= 4 * (2 * M * plan.info.R * eps + 4 * math.sqrt(M * plan.info.L) * eps)
 
 
+@pytest.mark.parametrize("n,stride", [(1, 2), (63, 2), (130, 3), (700, 2), (1024, 2), (1100, 2)])
+def test_split_grad_kept_tiles(fq, n, stride):
+    """BF16X3 forward chains with at most one tile an SM (n <= 1024) keep their states on the SM; the
+    single products of a captured gradient keep them in memory: the same loss and gradient bit for bit."""
+    import torch
+    M = 4
+    fm = cuda(1.0 + 0.1 * fi.normal(1305, M))
+    w = cuda(fi.haar_unitary(n, 1306).astype(np.complex128))
+    plan = fq.Plan.piecewise(fi.goe(n, 1307), fi.goe(n, 1308), fm.cpu().numpy(), period=0.2, checkpoint_stride=stride,
+                             precision=fq.FQ_BF16X3, tile_n=64)
+    loss, g = plan.grad(fm, w)
+    ws = fq.workspace(fq.floquet_grad_workspace_size(plan.handle))
+    loss2, g2 = torch.zeros_like(loss), torch.zeros_like(g)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        fq.floquet_grad(plan.handle, fm, w, loss2, g2, ws)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(loss, loss2) and torch.equal(g, g2)
+    assert plan.check_status() == fq.FQ_OK
+
+
 def test_split_grad_config5_shape_vs_oracle(fq):
     """The adjoint workload's shape (M = 256, checkpoints every 16) at N = 128, BF16X3."""
     n, M = 128, 256
