@@ -37,7 +37,7 @@ STEPS = 2000
 FLOPS_PER_ELEMENT_TERM = 26   # complex tridiagonal apply 18 + recurrence 4 + Bessel accumulation 4
 SM_COUNT, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 # DRAM traffic of the resident kernel from one ncu capture of `--ncu-case resident` (152 states,
-# steps 0..19, k_tri_resident<256, 40>, the current kernel with its L2 prefetch): bytes read, of
+# steps 0..19, k_tri_resident<40, 256>, the current kernel with its L2 prefetch): bytes read, of
 # which the 152 initial states are a fixed part; the rest is the per-step (2d, 2e') and rotation
 # stream, which grows with waves x steps.  A build also writes U_T once.
 RES_NCU = {"read": 28515072.0, "x0": 152 * 10001 * 16, "states": 152, "steps": 20}
@@ -372,7 +372,7 @@ def run_reference(args):
 DIMER_PATHS = {
     # FP32 resident chain (one launch per U_T): 26 flop per element-term against the FP32 FMA peak
     "fp32": {"precision": "FQ_FP32", "kernel": "FQ_KERNEL_RESIDENT", "dtype": "f32", "level": "FP32",
-             "kernel_name": "k_tri_resident<256, 40>", "unit": "TFLOP/s", "per_unit": FLOPS_PER_ELEMENT_TERM,
+             "kernel_name": "k_tri_resident<40, 256>", "unit": "TFLOP/s", "per_unit": FLOPS_PER_ELEMENT_TERM,
              "launches_per_step": 2,
              "peak_note": "FP32 FMA: 152 SMs x 128 lanes x 2 flop x 2070 MHz (derived from unit counts and clocks)"},
     # double-float tiled chain (FP64-level, one launch per step): 4 double-float complex FMAs per
@@ -785,7 +785,7 @@ def run_dense(args):
     achieved = useful / avg / 1e12
     roofline = {"bound": "tensor", "achieved": achieved, "peak": peaks["bf16_sustained"], "unit": "TFLOP/s",
                 "frac": achieved / peaks["bf16_sustained"], "traffic": None,
-                "kernel": "k_oz_term" if prec == "ozaki" else "k_split_persist",
+                "kernel": "k_oz_term" if prec == "ozaki" else "k_split_chain",
                 "issued_tflops": issued / avg / 1e12, "issued_frac": issued / avg / 1e12 / peaks["bf16_sustained"],
                 "note": (f"achieved: useful 8 N^3 flop per term x M L terms per build; issued: the "
                          f"{SLICE_PRODUCTS[prec]} BF16 slice products each term runs; both over the build's "
@@ -803,7 +803,8 @@ def run_dense(args):
             got = plan.propagate(rows, 0, nst).cpu().numpy().T
             accuracy["sample_max_err_vs_oracle"] = float(np.max(np.abs(got - xs)))
             accuracy["sample"] = desc
-    launches = 2 + m.steps * (1 + (2 * L if prec == "ozaki" else L))
+    # a step: Omega~, then each term's product and slicing pass, or the split chain's one launch of up to 12 terms
+    launches = 2 + m.steps * (1 + (2 * L if prec == "ozaki" else 1 if L <= 12 else L))
     if paper:
         metric = (f"U_T builds/sec (the paper's Table 1 timing run: GOE N={n} with unit-variance entries, "
                   f"f = cos(pi t), M={m.steps}, L={L}, 6th-order Magnus)")
@@ -1097,7 +1098,7 @@ def run_adjoint(args):
     else:
         roofline = {"bound": "tensor", "achieved": achieved, "peak": peaks["bf16_sustained"], "unit": "TFLOP/s",
                     "frac": achieved / peaks["bf16_sustained"], "traffic": None,
-                    "kernel": "k_oz_real_term<*>" if prec == "ozaki" else "k_split_persist / k_split_term",
+                    "kernel": "k_oz_real_term<*>" if prec == "ozaki" else "k_split_chain / k_split_term",
                     "issued_tflops": issued / avg / 1e12,
                     "issued_frac": issued / avg / 1e12 / peaks["bf16_sustained"],
                     "note": (f"achieved: useful 4 M L x 4 N^3 flop per gradient; issued: x {SLICE_PRODUCTS[prec]} "
