@@ -296,7 +296,9 @@ struct SplitCfg {
   // 64-wide complex tiles multiply each left tile by the stacked [S; A] rows in one N = 128 MMA
   // (split_issue_stage); other tiles take S and A in MMAs of their own
   static constexpr bool STACKED = HAS_A && BN == 64;
-  static constexpr int ACC_COLS = STACKED ? 4 * BN : 2 * BN;  // tensor-memory columns of one tile's sums
+  // 64-wide real tiles multiply a left slice by the stacked rows of the two leading right slices
+  static constexpr bool SLICED = !HAS_A && BN == 64;
+  static constexpr int ACC_COLS = STACKED || SLICED ? 4 * BN : 2 * BN;  // tensor-memory columns of one tile's sums
   static constexpr int TMEM_COLS = ACC_COLS <= 128 ? 128 : 256;
   // stages, their alignment, barriers, then the epilogue warps' transposing stages
   static constexpr size_t TAIL = 256;
@@ -330,7 +332,12 @@ __device__ __forceinline__ void split_load_stage(uint32_t st, uint32_t bar, cons
 //    bytes a cycle of shared memory: 43 -> 35 us a product at N = 1000 (BF16X3, K stages of 64).
 //    split_load_y forms Yr and Yi from the four sums.
 //  other complex tiles: Yr += Psi_r.S - Psi_i.A, Yi += Psi_r.A + Psi_i.S (negate-A bit);
-//  real right operand: Yr += Psi_r.S, Yi += Psi_i.S.
+//  SLICED (real): a left slice that goes with both S_0 and S_1 takes them stacked, in one MMA of N = 128 onto
+//    2 BN columns (Psi_0, and Psi_1 in BF16X6); Psi_{NS-1}.S_0 and, in BF16X6, Psi_0.S_2 go onto one half, for
+//    Psi_r and, 2 BN columns on, for Psi_i; split_load_y adds the halves.  An MMA of N = 64 takes about 60
+//    cycles for its 6 KB of operands, one of N = 128 about 80: a gradient step at N = 1024 552 -> 496 us
+//    (BF16X3) and 890 -> 770 us (BF16X6).
+//  other real right operands: Yr += Psi_r.S, Yi += Psi_i.S.
 template <int NS, int BN, int BKE, bool HAS_A>
 __device__ __forceinline__ void split_issue_stage(uint32_t acc, uint32_t st, bool fresh) {
   using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
@@ -338,6 +345,28 @@ __device__ __forceinline__ void split_issue_stage(uint32_t acc, uint32_t st, boo
   constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(MN >> 3) << 17) |
                              ((uint32_t)(BM >> 4) << 24);
   constexpr uint32_t idesc_neg = idesc | (1u << 13);  // negate the left operand
+  if constexpr (Cfg::SLICED) {
+    constexpr uint32_t idesc2 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * BN) >> 3) << 17) |
+                                ((uint32_t)(BM >> 4) << 24);
+#pragma unroll
+    for (int kk = 0; kk < BKE / 16; ++kk) {
+      const uint64_t ds = smem_desc<Cfg::ROWB>(Cfg::right(st, 0, 0) + 32 * kk);
+      const uint32_t first = (fresh && kk == 0) ? 0u : 1u;
+#pragma unroll
+      for (int a = 0; a < NS; ++a)
+#pragma unroll
+        for (int part = 0; part < 2; ++part)
+          mma_bf16(acc + part * 2 * BN, smem_desc<Cfg::ROWB>(st + (part * NS + a) * Cfg::A_BYTES + 32 * kk), ds,
+                   a < NS - 1 ? idesc2 : idesc, a == 0 ? first : 1u);
+      if (NS == 3) {
+#pragma unroll
+        for (int part = 0; part < 2; ++part)
+          mma_bf16(acc + part * 2 * BN + BN, smem_desc<Cfg::ROWB>(st + part * NS * Cfg::A_BYTES + 32 * kk),
+                   smem_desc<Cfg::ROWB>(Cfg::right(st, NS - 1, 0) + 32 * kk), idesc, 1u);
+      }
+    }
+    return;
+  }
 #pragma unroll
   for (int p = 0; p < Pairs<NS>::N; ++p) {
     const uint32_t pr = st + Pairs<NS>::a(p) * Cfg::A_BYTES;
@@ -435,18 +464,21 @@ __device__ __forceinline__ void epi_transpose(float* stage, int lane, const floa
 template <int NS, int BN, int BKE, bool HAS_A>
 __device__ __forceinline__ void split_load_y(uint32_t trow, int c0, float* stage, int lane, float (&yr)[32],
                                              float (&yi)[32]) {
+  using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
 #pragma unroll
   for (int part = 0; part < 2; ++part) {
     float v[2][16];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) tmem_ld16(trow + part * BN + c0 + 16 * h, v[h]);
-    if constexpr (SplitCfg<NS, BN, BKE, HAS_A>::STACKED) {
-      float w[2][16];  // Psi_i.A for Yr, Psi_i.S for Yi
+    for (int h = 0; h < 2; ++h) tmem_ld16(trow + (Cfg::SLICED ? 2 * part : part) * BN + c0 + 16 * h, v[h]);
+    if constexpr (Cfg::STACKED || Cfg::SLICED) {
+      float w[2][16];  // STACKED: Psi_i.A for Yr, Psi_i.S for Yi; SLICED: the products with S_1
 #pragma unroll
-      for (int h = 0; h < 2; ++h) tmem_ld16(trow + (part ? 2 : 3) * BN + c0 + 16 * h, w[h]);
+      for (int h = 0; h < 2; ++h)
+        tmem_ld16(trow + (Cfg::SLICED ? 2 * part + 1 : part ? 2 : 3) * BN + c0 + 16 * h, w[h]);
       tmem_wait_ld();
 #pragma unroll
-      for (int q = 0; q < 32; ++q) v[q >> 4][q & 15] += part ? w[q >> 4][q & 15] : -w[q >> 4][q & 15];
+      for (int q = 0; q < 32; ++q)
+        v[q >> 4][q & 15] += part || Cfg::SLICED ? w[q >> 4][q & 15] : -w[q >> 4][q & 15];
     } else {
       tmem_wait_ld();
     }
@@ -965,8 +997,8 @@ struct KeptTile {
     }
   }
 
-  // product p of the chain from the tile's sums (64 columns each: Psi_r.S, Psi_r.A, Psi_i.S, Psi_i.A
-  // when STACKED, else Yr and Yi): the new state, acc and the slices; `tempty` is signalled once the sums are read.
+  // product p of the chain from the tile's sums (64 columns each: Psi_r.S, Psi_r.A, Psi_i.S, Psi_i.A when
+  // STACKED; the two parts of Yr, then of Yi, when the right operand is real): the new state, acc and the slices; `tempty` is signalled once the sums are read.
   __device__ __forceinline__ void term(const SplitEpi& e, int p, int half, int lane, uint32_t tempty, bool& bad) {
     const float cf = e.t.coef, sg = e.t.first ? 1.f : 2.f, b2 = e.t.bound2;
     const bool last = e.t.last, edge = col + 32 > e.n;
@@ -976,11 +1008,9 @@ struct KeptTile {
       float y[2][8], w[2][8], x[2][8];
       const uint32_t sums = trow + 32 * half + c;
       tmem_ld8(sums, y[0]);
-      tmem_ld8(sums + 64, y[1]);
-      if (STACKED) {
-        tmem_ld8(sums + 192, w[0]);
-        tmem_ld8(sums + 128, w[1]);
-      }
+      tmem_ld8(sums + (STACKED ? 192 : 64), w[0]);
+      tmem_ld8(sums + (STACKED ? 64 : 128), y[1]);
+      tmem_ld8(sums + (STACKED ? 128 : 192), w[1]);
       tmem_ld8(psi + c, x[0]);
       tmem_ld8(psi + 64 + c, x[1]);
       tmem_wait_ld();
@@ -992,8 +1022,8 @@ struct KeptTile {
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         float o_r, o_i;
-        const float yr = STACKED ? y[0][q] - w[0][q] : y[0][q], yi = STACKED ? y[1][q] + w[1][q] : y[1][q];
-        fwd_entry(sg, cf, yr, yi, x[0][q], x[1][q], ar[c + q], ai[c + q], o_r, o_i);
+        const float yr = STACKED ? y[0][q] - w[0][q] : y[0][q] + w[0][q];
+        fwd_entry(sg, cf, yr, y[1][q] + w[1][q], x[0][q], x[1][q], ar[c + q], ai[c + q], o_r, o_i);
         bad |= !(o_r * o_r + o_i * o_i <= b2);  // zero beyond the block
         y[0][q] = o_r;
         y[1][q] = o_i;
@@ -1076,9 +1106,9 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_split_chain(const __grid_consta
   static_assert(EPI != EPI_DOT, "chains of forward or adjoint terms only");
   using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
   constexpr int STAGES = Cfg::STAGES;
-  static_assert(!KEEP || (BN == 64 && EPI == EPI_FWD), "kept tiles: 64-wide forward terms");
+  static_assert(!KEEP || ((Cfg::STACKED || Cfg::SLICED) && EPI == EPI_FWD), "kept tiles: 64-wide forward terms");
   constexpr uint32_t BUF_COLS = Cfg::ACC_COLS;
-  constexpr uint32_t TMEM_COLS = KEEP ? 512 : 2 * BUF_COLS;  // two buffers of sums (KEEP: one, and the states)
+  constexpr uint32_t TMEM_COLS = 2 * BUF_COLS;  // two buffers of sums (KEEP: one, and the states)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
