@@ -1098,7 +1098,7 @@ def run_adjoint(args):
     else:
         roofline = {"bound": "tensor", "achieved": achieved, "peak": peaks["bf16_sustained"], "unit": "TFLOP/s",
                     "frac": achieved / peaks["bf16_sustained"], "traffic": None,
-                    "kernel": "k_oz_real_term<*>" if prec == "ozaki" else "k_split_chain / k_split_term",
+                    "kernel": "k_oz_real_term<*>" if prec == "ozaki" else "k_split_chain / k_split_persist",
                     "issued_tflops": issued / avg / 1e12,
                     "issued_frac": issued / avg / 1e12 / peaks["bf16_sustained"],
                     "note": (f"achieved: useful 4 M L x 4 N^3 flop per gradient; issued: x {SLICE_PRODUCTS[prec]} "

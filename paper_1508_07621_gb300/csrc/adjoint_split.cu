@@ -1,6 +1,6 @@
 // floquet_grad for BF16X3 / BF16X6 plans: the reverse-mode chain of adjoint.cu (loss
 // L = 1 - |Tr(W^+ U_T)|^2 / N^2, Clenshaw-form adjoint of Eqs. 10 and 12, dL/df_m from the kept
-// forward Chebyshev vectors) with every N x N x N product on the tensor cores (k_split_term).
+// forward Chebyshev vectors) with every N x N x N product on the tensor cores (k_split_persist, k_split_chain).
 //
 // Piecewise-constant f makes Omega~_m = (H0 + f_m H1 - beta) / Delta E real symmetric, so each
 // product is Y = X . S^T on the planar (re, im) state rows with a real right operand: two MMA
@@ -9,7 +9,7 @@
 //   forward term   (EPI_FWD): psi_{l+1} = -2i Y + psi_{l-1}, acc += a_{l+1} psi_{l+1}, phase;
 //   adjoint term   (EPI_ADJ): bbar_l = conj(e^{-i beta h}) a_l G + i cw Omega~ bbar_{l+1} + bbar_{l+2}
 //                             (cw = 2, and 1 for l = 0);
-//   gradient dot   (EPI_DOT): D_l = <bbar_l, E psi_{l-1}> with E = H1 / Delta E, per-CTA partials;
+//   gradient dot   (EPI_DOT): D_l = <bbar_l, E psi_{l-1}> with E = H1 / Delta E, partial sums per warp;
 //   dL/df_m = 2 Re sum_l w_l D_l  (w_1 = -i, w_l = -2i).
 // Memory: FP32 masters of X every s = checkpoint_stride steps; each segment is recomputed once
 // with the slices of every psi_l kept (they are the left operands of the dot products) and then
@@ -124,9 +124,16 @@ struct Master {
   float* im;
 };
 
+// A step's L gradient dots are one product of L Np rows.  They take 128-wide tiles once there is a wave of
+// them (152 SMs): a tile then reads 48 KB of operands from L2 for what two 64-wide ones read 80 KB each for,
+// and that feed bounds them.  A gradient step with 64- / 128-wide dots: N = 600 322 / 318 us, N = 1024
+// 478 / 454 us (BF16X3).  The rule looks at N and L alone.  (One CTA a tile, no overlap of its epilogue with
+// the next tile's MMAs: 496 us at N = 1024.)
+constexpr int DOT_WIDE_TILES = 152;
+
 // Workspace of the split gradient (all offsets 256-byte aligned).
 struct SplitGradWs {
-  int ns, np, kp, ldm, ncp, nseg, nslots, ncta;
+  int ns, np, kp, ldm, ncp, nseg, nslots, nsum, dot_bn;
   size_t bstride, astride;
   __nv_bfloat16* S;       // Omega~_m slices
   __nv_bfloat16* E;       // E = H1 / Delta E slices
@@ -135,7 +142,7 @@ struct SplitGradWs {
   Master f[5];            // FP32 masters: forward cur / prev / acc; adjoint G and the next G
   Master bbar;            // bbar_1 .. bbar_L of one step: L blocks of ncp rows (padding rows zero)
   float* ck_base;         // nseg checkpoints of X, each 2 planes [n][ldm]
-  double2* partial;       // (L + 1) x ncta
+  double2* partial;       // (L + 1) x nsum: the dot's partial sums of a step
   unsigned int* flags;    // chain counters [CHAIN_MAXP][row blocks]
   double2* tau_partial;   // n
   double2* tau;
@@ -165,8 +172,8 @@ size_t split_grad_layout(const fq_plan* p, void* base, SplitGradWs* out) {
   w.nslots = s * L + 1;
   w.bstride = (size_t)w.np * w.np;
   w.astride = (size_t)w.ncp * w.kp;
-  const int bn = fq_split_shape(p).n == 128 ? 128 : 64;
-  w.ncta = (w.np / bn) * (w.ncp / BM);
+  w.dot_bn = L * (w.np / 128) * (w.ncp / BM) >= DOT_WIDE_TILES ? 128 : fq_split_shape(p).n == 128 ? 128 : 64;
+  w.nsum = (w.np / w.dot_bn) * (w.ncp / BM) * EPI_WARPS;
   char* b = (char*)base;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -188,7 +195,7 @@ size_t split_grad_layout(const fq_plan* p, void* base, SplitGradWs* out) {
   float* bb = (float*)take(sizeof(float) * 2 * stacked);
   w.bbar = Master{bb, bb ? bb + stacked : nullptr};
   w.ck_base = (float*)take(sizeof(float) * 2 * plane * (size_t)w.nseg);
-  w.partial = (double2*)take(sizeof(double2) * (size_t)(L + 1) * w.ncta);
+  w.partial = (double2*)take(sizeof(double2) * (size_t)(L + 1) * (w.np / 64) * (w.ncp / BM) * EPI_WARPS);
   w.flags = (unsigned int*)take(sizeof(unsigned int) * CHAIN_MAXP * (size_t)(w.ncp / BM));
   w.tau_partial = (double2*)take(sizeof(double2) * n);
   w.tau = (double2*)take(sizeof(double2));
@@ -199,7 +206,7 @@ size_t split_grad_layout(const fq_plan* p, void* base, SplitGradWs* out) {
 // One split GEMM Y = left . right^T (right real) with epilogue EPI, for the plan's slice count
 // and tile width.
 struct GemmCtx {
-  int n, np, kp, ncp, ns, bn;
+  int n, np, kp, ncp, ns, bn, dot_bn;  // tile widths of the terms and of the gradient dots
   size_t bstride, astride;
 };
 
@@ -219,37 +226,26 @@ fq_status gemm_cfg(const GemmCtx& c, Left left, const __nv_bfloat16* right, cons
     if ((st = make_map(&maps.a[q], left.base + q * left.lstride, left.rows, c.kp, BM, BKE)) != FQ_OK) return st;
     if ((st = make_map(&maps.os[q], right + q * c.bstride, c.np, c.np, BN, BKE)) != FQ_OK) return st;
   }
-  // the forward and adjoint terms run persistently (epilogue overlapped with the next tile's
-  // MMAs); the gradient dot keeps one tile per CTA for its per-CTA partial sums
-  constexpr bool persist = EPI != EPI_DOT;
   static std::atomic<unsigned> attr_set{0};
   if (fq_first_on_device(attr_set)) {
-    cudaError_t r;
-    if constexpr (persist)
-      r = cudaFuncSetAttribute(k_split_persist<NS, BN, BKE, EPI, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)Cfg::SMEM);
-    else
-      r = cudaFuncSetAttribute(k_split_term<NS, BN, BKE, EPI, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)Cfg::SMEM);
+    const cudaError_t r = cudaFuncSetAttribute(k_split_persist<NS, BN, BKE, EPI, false>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     if (r != cudaSuccess) return fq_cuda_fail(r, "split gradient kernel shared-memory attribute");
   }
   const int sms = fq_sm_count();
   const int tiles_i = c.np / BN, tiles_j = left.rows / BM;
   const int nk = (c.n + BKE - 1) / BKE;  // the operands' columns beyond N are zero
-  if constexpr (persist)
-    k_split_persist<NS, BN, BKE, EPI, false><<<std::min(tiles_i * tiles_j, sms), PTHREADS, Cfg::SMEM, s>>>(
-        maps, nk, tiles_j, tiles_i, e);
-  else
-    k_split_term<NS, BN, BKE, EPI, false><<<tiles_i * tiles_j, NTHREADS, Cfg::SMEM, s>>>(maps, nk, tiles_j, tiles_i,
-                                                                                        e);
+  k_split_persist<NS, BN, BKE, EPI, false><<<std::min(tiles_i * tiles_j, sms), PTHREADS, Cfg::SMEM, s>>>(
+      maps, nk, tiles_j, tiles_i, e);
   return FQ_OK;
 }
 
 template <int EPI>
 fq_status gemm(const GemmCtx& c, Left left, const __nv_bfloat16* right, const SplitEpi& e, cudaStream_t s) {
+  const int bn = EPI == EPI_DOT ? c.dot_bn : c.bn;
   if (c.ns == 3)
-    return c.bn == 128 ? gemm_cfg<3, 128, 32, EPI>(c, left, right, e, s) : gemm_cfg<3, 64, 32, EPI>(c, left, right, e, s);
-  return c.bn == 128 ? gemm_cfg<2, 128, 32, EPI>(c, left, right, e, s) : gemm_cfg<2, 64, 64, EPI>(c, left, right, e, s);
+    return bn == 128 ? gemm_cfg<3, 128, 32, EPI>(c, left, right, e, s) : gemm_cfg<3, 64, 32, EPI>(c, left, right, e, s);
+  return bn == 128 ? gemm_cfg<2, 128, 32, EPI>(c, left, right, e, s) : gemm_cfg<2, 64, 64, EPI>(c, left, right, e, s);
 }
 
 // A chain of products with one right operand (the step's Omega~_m) as one cooperative launch
@@ -412,7 +408,7 @@ fq_status fq_grad_split(fq_plan* p, const double* d_f, const void* d_W, double* 
   r.s = s;
   split_grad_layout(p, d_ws, &r.w);
   SplitGradWs& w = r.w;
-  r.c = GemmCtx{p->n, w.np, w.kp, w.ncp, w.ns, fq_split_shape(p).n == 128 ? 128 : 64, w.bstride, w.astride};
+  r.c = GemmCtx{p->n, w.np, w.kp, w.ncp, w.ns, fq_split_shape(p).n == 128 ? 128 : 64, w.dot_bn, w.bstride, w.astride};
   const int n = p->n, M = p->steps, L = p->L, S = p->stride;
   const size_t plane_bytes = sizeof(float) * (size_t)n * w.ldm;
 
@@ -502,9 +498,9 @@ fq_status fq_grad_split(fq_plan* p, const double* d_f, const void* d_W, double* 
       d.nc = L * w.ncp;
       d.cur_re = w.bbar.re;
       d.cur_im = w.bbar.im;
-      d.partial = w.partial + w.ncta;  // block l at partial + l * ncta
+      d.partial = w.partial + w.nsum;  // block l at partial + l * nsum
       if ((st = gemm<EPI_DOT>(r.c, Left{w.slot(st_ * L), ss, L * w.ncp}, w.E, d, s)) != FQ_OK) return st;
-      fq_launch_grad_reduce(w.partial, w.ncta, L, d_grad + m, s);
+      fq_launch_grad_reduce(w.partial, w.nsum, L, d_grad + m, s);
       std::swap(gi, gn);  // bbar_0 is the next G
     }
   }

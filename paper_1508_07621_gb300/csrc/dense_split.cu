@@ -1,6 +1,6 @@
 // Split-precision dense Chebyshev chain (stages a2, a3, a5, a6, a8 on the tensor cores): per step
 // the S and A slices of Omega~_m (FP64 arithmetic, Eqs. 11 and 14), then L terms of Eq. 10 through
-// k_split_term (split_core.cuh) whose epilogue applies the recurrence, the Bessel accumulation
+// k_split_chain (split_core.cuh) whose epilogue applies the recurrence, the Bessel accumulation
 // of Eq. 12 and the step phase, and writes the next term's BF16 slices.
 #include <vector>
 

@@ -12,8 +12,7 @@
 // psi_{l-1}, Bessel accumulation and step phase on FP32 masters, Eqs. 10 and 12), the adjoint
 // term, or the gradient dot; the first two also write the next product's slices.
 //
-// k_split_term: one 128-row x BN-column tile per CTA of 128 threads.  k_split_persist: one CTA
-// per SM walks its tiles with a dedicated TMA warp, MMA warp and eight epilogue warps, and two
+// k_split_persist: one CTA per SM walks its tiles with a dedicated TMA warp, MMA warp and eight epilogue warps, and two
 // tensor-memory buffers so that a tile's epilogue overlaps the next tile's MMAs.  Tiles are
 // rasterized in groups of 8 row blocks so that co-running CTAs share operands in L2.  TMA loads
 // are K-major with 128- or 64-byte swizzle; stages and buffers are handed over by mbarriers.
@@ -35,7 +34,6 @@ namespace {
 
 
 constexpr int BM = 128;      // state rows per tile (tcgen05 M)
-constexpr int NTHREADS = 128;
 constexpr int RASTER_GROUP = 8;
 // Epilogue warps of the persistent kernels: two per tensor-memory lane quarter, each taking half of
 // the tile's columns, with a transposing stage (epi_transpose) of its own.
@@ -252,7 +250,7 @@ struct SplitMaps {
 enum SplitMode {
   EPI_FWD = 0,  // Chebyshev term: psi_{l+1} = -2i Y + psi_{l-1}, acc += a psi_{l+1}, phase at the last term
   EPI_ADJ = 1,  // adjoint term: out = cpa g + i cw Y + b2
-  EPI_DOT = 2,  // gradient dot: partial[cta] = sum over the tile of conj(b) Y
+  EPI_DOT = 2,  // gradient dot: partial[tile][epilogue warp] = sum of conj(b) Y over the warp's part of the tile
 };
 
 // A Chebyshev term's scalars in FP32 (converted once: FP64 conversions run at the FP64 rate, five of them
@@ -282,7 +280,7 @@ struct SplitEpi {
   size_t slice_stride;         // elements between slices
   int kp;
   float cpa_re, cpa_im, cw;    // ADJ coefficients
-  double2* partial;            // DOT output, one per CTA
+  double2* partial;            // DOT output, EPI_WARPS a tile
   SplitTerm t;
 };
 
@@ -299,7 +297,6 @@ struct SplitCfg {
   // 64-wide real tiles multiply a left slice by the stacked rows of the two leading right slices
   static constexpr bool SLICED = !HAS_A && BN == 64;
   static constexpr int ACC_COLS = STACKED || SLICED ? 4 * BN : 2 * BN;  // tensor-memory columns of one tile's sums
-  static constexpr int TMEM_COLS = ACC_COLS <= 128 ? 128 : 256;
   // stages, their alignment, barriers, then the epilogue warps' transposing stages
   static constexpr size_t TAIL = 256;
   static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + TAIL + EPI_WARPS * EPI_STAGE_BYTES;
@@ -605,150 +602,15 @@ __device__ __forceinline__ void epi_block(const SplitEpi& e, const float (&yr)[3
   }
 }
 
-// One split GEMM on a 128-row x BN-column tile of Y = left . right^T:
+// One split GEMM Y = left . right^T on 128-row x BN-column tiles:
 //   HAS_A:  Yr = Psi_r.S - Psi_i.A,  Yi = Psi_r.A + Psi_i.S   (right = S + i A)
 //   !HAS_A: Yr = Psi_r.S,            Yi = Psi_i.S             (right = S real)
-// followed by the epilogue EPI.
-template <int NS, int BN, int BKE, int EPI, bool HAS_A>
-__global__ void __launch_bounds__(NTHREADS, 1)
-k_split_term(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int tiles_i, SplitEpi e) {
-  using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
-  constexpr int STAGES = Cfg::STAGES;
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  // 1024-byte aligned stage buffers (swizzle atoms), then barriers
-  const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  unsigned char* gbase = smem_raw + (base - raw);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(gbase + STAGES * Cfg::STAGE_BYTES);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 1);
-  int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
-  double* red = reinterpret_cast<double*>(gbase + STAGES * Cfg::STAGE_BYTES + 128);  // DOT: 4 warps x 2
-  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES), done = smem_u32(bars + 2 * STAGES);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // grouped rasterization: RASTER_GROUP row blocks sweep the column blocks together
-  int tj, ti;
-  {
-    const int b = blockIdx.x, per = RASTER_GROUP * tiles_i, g = b / per;
-    const int gj = min(RASTER_GROUP, tiles_j - g * RASTER_GROUP), r = b - g * per;
-    tj = g * RASTER_GROUP + r % gj;
-    ti = r / gj;
-  }
-  const int j0 = tj * BM, i0 = ti * BN;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(full0 + 8 * s, 1);
-      mbar_init(empty0 + 8 * s, 1);
-    }
-    mbar_init(done, 1);
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"((uint32_t)Cfg::TMEM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-
-  if (warp == 0 && lane == 0) {
-    // ---------------- TMA producer
-    int issued = 0;
-    bool ok = true;
-    for (int kb = 0; kb < nk && ok; ++kb) {
-      const int s = kb % STAGES;
-      if (kb >= STAGES) {
-        ok = mbar_wait(empty0 + 8 * s, ((kb / STAGES) - 1) & 1);
-        if (!ok) break;
-      }
-      const uint32_t st = base + s * Cfg::STAGE_BYTES;
-      const uint32_t bar = full0 + 8 * s;
-      mbar_expect_tx(bar, Cfg::STAGE_BYTES);
-      const int kx = kb * BKE;
-      split_load_stage<NS, BN, BKE, HAS_A>(st, bar, maps.a, maps.os, maps.oa, kx, e.np, j0, i0);
-      issued = kb + 1;
-    }
-    if (!ok) {
-      atomicExch(abort_flag, 1);
-      atomicOr(e.t.status, FQ_BIT_TIMEOUT);
-    }
-    // drain: every copy this thread issued must have landed before the CTA may exit
-    for (int kb = max(0, issued - STAGES); kb < issued; ++kb) mbar_wait(full0 + 8 * (kb % STAGES), (kb / STAGES) & 1);
-  } else if (warp == 1 && lane == 0) {
-    // ---------------- MMA issuer
-    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                               ((uint32_t)(BM >> 4) << 24);
-    constexpr uint32_t idesc_neg = idesc | (1u << 13);  // negate the left operand
-    bool ok = true;
-    for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % STAGES;
-      ok = mbar_wait(full0 + 8 * s, (kb / STAGES) & 1);
-      if (!ok || *(volatile int*)abort_flag) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      const uint32_t st = base + s * Cfg::STAGE_BYTES;
-      split_issue_stage<NS, BN, BKE, HAS_A>(tmem, st, kb == 0);
-      mma_commit(empty0 + 8 * s);  // stage s free once these MMAs have read it
-    }
-    if (!ok) {
-      atomicExch(abort_flag, 1);
-      atomicOr(e.t.status, FQ_BIT_TIMEOUT);
-    }
-    mma_commit(done);  // arrives when every MMA issued above has completed
-  }
-  __syncwarp();
-
-  // ---------------- epilogue: all 128 threads, thread = state row j, 16 columns at a time
-  const bool got = mbar_wait(done, 0);
-  tc_fence_after();
-  if (!got) atomicOr(e.t.status, FQ_BIT_TIMEOUT);
-  const bool run = got && !*(volatile int*)abort_flag;
-  float* stage = reinterpret_cast<float*>(gbase + STAGES * Cfg::STAGE_BYTES + Cfg::TAIL + warp * EPI_STAGE_BYTES);
-  const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
-  bool bad = false;
-  double dsr = 0.0, dsi = 0.0;  // DOT partial of this thread
-#pragma unroll 1
-  for (int c0 = 0; c0 < BN; c0 += 32) {
-    float yr[32], yi[32];
-    split_load_y<NS, BN, BKE, HAS_A>(trow, c0, stage, lane, yr, yi);
-    if (!run || i0 + c0 >= e.n) continue;
-    epi_block<NS, EPI, 4>(e, yr, yi, j0 + warp * 32, i0 + c0, lane, bad, dsr, dsi);
-  }
-  if (bad) atomicOr(e.t.status, FQ_BIT_BOUND);
-  if (EPI == EPI_DOT) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      dsr += __shfl_xor_sync(0xffffffffu, dsr, o);
-      dsi += __shfl_xor_sync(0xffffffffu, dsi, o);
-    }
-    if (lane == 0) {
-      red[2 * warp] = dsr;
-      red[2 * warp + 1] = dsi;
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (EPI == EPI_DOT && threadIdx.x == 0)
-    e.partial[tj * tiles_i + ti] = make_double2(red[0] + red[2] + red[4] + red[6], red[1] + red[3] + red[5] + red[7]);
-  if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)Cfg::TMEM_COLS)
-                 : "memory");
-  }
-}
-
-// Persistent form of k_split_term for the forward and adjoint epilogues: one CTA per SM walks
-// the tiles blockIdx.x, blockIdx.x + gridDim.x, ...  Warp 0 (one thread) streams TMA stages,
-// warp 1 (one thread) issues the MMAs of tile i into tensor-memory buffer i & 1, and the
-// epilogue warps run the epilogue of tile i from its buffer while tile i + 1 accumulates in the other one.
-// Buffers are handed over by mbarriers (tfull: MMAs of a tile done; tempty: its accumulators
-// read).  Every wait is bounded as in k_split_term.
+// followed by the epilogue EPI.  One CTA per SM walks the tiles blockIdx.x, blockIdx.x + gridDim.x, ...
+// Warp 0 (one thread) streams TMA stages, warp 1 (one thread) issues the MMAs of tile i into
+// tensor-memory buffer i & 1, and the epilogue warps run the epilogue of tile i from its buffer while
+// tile i + 1 accumulates in the other one.  Buffers are handed over by mbarriers (tfull: MMAs of a tile
+// done; tempty: its accumulators read).  Every wait is bounded; one that gives up sets the abort flag
+// and FQ_BIT_TIMEOUT, and the CTA drains its own copies and MMAs before it returns.
 constexpr int PTHREADS = 64 + 32 * EPI_WARPS;
 // column range [begin, end) of epilogue warp `warp` (2 .. 1 + EPI_WARPS) of a BN-wide tile
 template <int BN>
@@ -757,7 +619,6 @@ __device__ __forceinline__ int epi_begin(int warp) { return ((warp - 2) >> 2) * 
 template <int NS, int BN, int BKE, int EPI, bool HAS_A>
 __global__ void __launch_bounds__(PTHREADS, 1)
 k_split_persist(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int tiles_i, SplitEpi e) {
-  static_assert(EPI != EPI_DOT, "the gradient dot keeps the one-tile kernel (per-CTA partials)");
   using Cfg = SplitCfg<NS, BN, BKE, HAS_A>;
   constexpr int STAGES = Cfg::STAGES;
   constexpr uint32_t BUF_COLS = Cfg::ACC_COLS;      // one tile's sums
@@ -894,6 +755,16 @@ k_split_persist(const __grid_constant__ SplitMaps maps, int nk, int tiles_j, int
           if (lane == 0) mbar_arrive(tempty0 + 8 * b);
         }
         if (i0 + c0 < e.n) epi_block<NS, EPI, 4>(e, yr, yi, j0 + quarter * 32, i0 + c0, lane, bad, dsr, dsi);
+      }
+      if (EPI == EPI_DOT) {  // a sum per warp: no barrier that a warp giving up could miss
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) {
+          dsr += __shfl_xor_sync(0xffffffffu, dsr, w);
+          dsi += __shfl_xor_sync(0xffffffffu, dsi, w);
+        }
+        if (lane == 0)
+          e.partial[((size_t)(j0 / BM) * tiles_i + i0 / BN) * EPI_WARPS + warp - 2] = make_double2(dsr, dsi);
+        dsr = dsi = 0.0;
       }
     }
     if (!ok) {
