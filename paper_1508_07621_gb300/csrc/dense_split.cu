@@ -76,8 +76,8 @@ static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Largest N whose default tile is 64 wide, for BF16X3 and BF16X6: up to there the 128-wide tiles of a
 // product are at most one wave (144 and 121 tiles on 152 SMs), and twice as many narrow ones fill the
-// chip better.  A product in us with 64- / 128-wide tiles: BF16X3 N = 400 18 / 29, 1000 28 / 48, 1536
-// 61 / 70, 2048 136 / 127; BF16X6 N = 1000 45 / 76, 1300 82 / 99, 1536 117 / 112.  The rule looks at N
+// chip better.  A product in us with 64- / 128-wide tiles: BF16X3 N = 256 11.5 / 21, 700 19 / 38, 1000 24 / 45,
+// 1536 61 / 69, 3000 435 / 385; BF16X6 N = 1000 41 / 73, 1300 82 / 98, 1536 116 / 110.  The rule looks at N
 // alone, so that a block of columns and the whole U_T take the same tiles and agree bit for bit.
 constexpr int SPLIT_NARROW_MAX_N_X3 = 1536;
 constexpr int SPLIT_NARROW_MAX_N_X6 = 1408;
