@@ -445,7 +445,9 @@ k_term_band6(const double* __restrict__ ore, const double* __restrict__ oim, int
 // D[c][j] = sum_i conj(U[i][c]) U[i][j] - delta_cj for KC listed columns c (chunk blockIdx.y) and the 256
 // columns j of a cluster of 8 CTAs: a CTA has 32 of them, one a lane, its 8 warps take every 8th row i,
 // and the chunk's entries of a row are loads of one address a warp.  Per cluster: the largest |D| and the
-// sum of |D|^2, in a fixed order (the CTAs' parts meet in the first one's shared memory).
+// sum of |D|^2, in a fixed order (the CTAs' parts meet in the first one's shared memory, which may be
+// written once that CTA runs: every CTA arrives at the cluster's barrier on entry and waits for the
+// others just before it stores, so the rows' sums hide the wait).
 // Bound by the FP64 pipes: 4 KC multiply-adds a lane and row; the chunk size fills the chip
 // (fq_launch_defect).  (One thread a column and a barrier pair a row kept N / 256 x k / 16 CTAs of one
 // row in flight each: N = 4096, 64 columns 19.6 ms, now 8.3 ms; N = 243, 40 columns 1.15 ms, now 0.08 ms.)
@@ -461,6 +463,7 @@ __global__ void __cluster_dims__(DEFECT_CTAS, 1, 1) __launch_bounds__(32 * DEFEC
   const int rank = blockIdx.x % DEFECT_CTAS;
   const int c0 = blockIdx.y * KC, kc = min(KC, k - c0);
   const int j = blockIdx.x * 32 + lane;
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   int col[KC];
 #pragma unroll
   for (int q = 0; q < KC; ++q) {
@@ -513,6 +516,7 @@ __global__ void __cluster_dims__(DEFECT_CTAS, 1, 1) __launch_bounds__(32 * DEFEC
     part[warp][1] = ss;
   }
   __syncthreads();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // the first CTA is running
   if (threadIdx.x == 0) {
     mx = ss = 0.0;
     for (int w = 0; w < DEFECT_WARPS; ++w) {
