@@ -701,8 +701,10 @@ fq_status floquet_unitarity_defect(const void* d_U, int32_t n, const int32_t* d_
   cudaStream_t s = (cudaStream_t)stream;
   const int parts = fq_launch_defect((const double*)d_U, n, d_cols, rows, (double*)d_ws,
                                      ws_bytes / (2 * sizeof(double)), s);
+  cudaError_t e = cudaGetLastError();  // a refused launch leaves the workspace as it was
+  if (e != cudaSuccess) return fq_cuda_fail(e, "defect launch");
   std::vector<double> h(2 * (size_t)parts * nb, 0.0);
-  cudaError_t e = cudaMemcpyAsync(h.data(), d_ws, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
+  e = cudaMemcpyAsync(h.data(), d_ws, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return fq_cuda_fail(e, "defect");
   double mx = 0.0, ss = 0.0;

@@ -325,6 +325,21 @@ def test_binding_refuses_bad_buffers(fq):
     assert e.value.status == fq.FQ_EINVAL
 
 
+def test_unitarity_defect_reports_a_refused_launch(fq):
+    """Where the kernel's launch is refused (here: there is no GPU) the call says so, before it reads the
+    workspace that the kernel never wrote."""
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("the launch is refused only where there is no GPU")
+    lib = ctypes.CDLL(LIB)
+    lib.floquet_last_error.restype = ctypes.c_char_p
+    u, ws = (ctypes.c_double * 72)(), (ctypes.c_double * 64)()
+    mx, fro = ctypes.c_double(), ctypes.c_double()
+    st = lib.floquet_unitarity_defect(u, 6, None, 6, ws, ctypes.c_size_t(512), None, ctypes.byref(mx), ctypes.byref(fro))
+    assert st == fq.FQ_ECUDA
+    assert lib.floquet_last_error().decode().startswith("defect launch")
+
+
 def test_host_quasienergies_concurrent_calls(fq):
     """Calls from several host threads at once (ctypes releases the GIL) each get their own
     worker pool and return exactly what a lone call returns."""
