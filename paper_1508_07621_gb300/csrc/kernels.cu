@@ -623,19 +623,25 @@ void fq_launch_term_dense_f64(const double* S, const double* A, int n, fq_blk<do
   // 300 217 (71.8) -> 202 (41.4), 520 978 (161) -> 975 (148).  The rule looks at N alone, so that
   // blocks of columns agree with the whole U_T bit for bit (both plain tiles add in the order of k).
   const long ti = (n + 31) / 32, big = ti * ((nc + 31) / 32);
-  const dim3 g32((n + 31) / 32, (nc + 31) / 32), g8((n + 7) / 8, (nc + 7) / 8), g4((n + 7) / 8, (nc + 3) / 4);
-  auto launch = [&](auto kernel, dim3 g, int threads) {
-    kernel<<<g, threads, 0, s>>>(S, A, n, cur.re, cur.im, prev.re, prev.im, acc.re, acc.im, out.re, out.im, nc, t);
+  auto launch = [&](auto kernel, int bj, int bi, int threads) {
+    const int most = 65535 * bj;  // states a launch: gridDim.y limit
+    for (long r0 = 0; r0 < nc; r0 += most) {
+      const int rows = nc - r0 < most ? (int)(nc - r0) : most;
+      const size_t o = (size_t)r0 * n;
+      kernel<<<dim3((n + bi - 1) / bi, (rows + bj - 1) / bj), threads, 0, s>>>(
+          S, A, n, cur.re + o, cur.im + o, prev.re + o, prev.im + o, acc.re + o, acc.im + o, out.re + o, out.im + o, rows,
+          t);
+    }
   };
   if (ti * ti < 2 * 152) {
-    if (A) launch(k_term_dense_f64<4, 8, 32, 1, 1, true, 4>, g4, 128);
-    else launch(k_term_dense_f64<4, 8, 32, 1, 1, false, 4>, g4, 128);
+    if (A) launch(k_term_dense_f64<4, 8, 32, 1, 1, true, 4>, 4, 8, 128);
+    else launch(k_term_dense_f64<4, 8, 32, 1, 1, false, 4>, 4, 8, 128);
   } else if (big >= 2 * 152) {
-    if (A) launch(k_term_dense_f64<32, 32, 16, 2, 2, true>, g32, 256);
-    else launch(k_term_dense_f64<32, 32, 16, 2, 2, false>, g32, 256);
+    if (A) launch(k_term_dense_f64<32, 32, 16, 2, 2, true>, 32, 32, 256);
+    else launch(k_term_dense_f64<32, 32, 16, 2, 2, false>, 32, 32, 256);
   } else {
-    if (A) launch(k_term_dense_f64<8, 8, 32, 1, 1, true>, g8, 64);
-    else launch(k_term_dense_f64<8, 8, 32, 1, 1, false>, g8, 64);
+    if (A) launch(k_term_dense_f64<8, 8, 32, 1, 1, true>, 8, 8, 64);
+    else launch(k_term_dense_f64<8, 8, 32, 1, 1, false>, 8, 8, 64);
   }
 }
 

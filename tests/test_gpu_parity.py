@@ -488,6 +488,20 @@ def test_dense_fp64_sizes(fq, n):
     assert np.max(np.abs(to_np(few) - ref)) <= 1e-12
 
 
+@pytest.mark.parametrize("n", [3, 130])
+def test_dense_fp64_more_states_than_a_launch(fq, n):
+    """The split-K tiles hold 4 states each and a launch 65535 of them: one state block beyond that, the
+    states of a second launch have the bits they have alone."""
+    import torch
+    nc = 4 * 65535 + 6
+    plan = fq.Plan.dense(fi.goe(n, 2511), fi.goe(n, 2512), omega=1.1, f_ac=1.3, steps=100, kernel=fq.FQ_KERNEL_STREAM)
+    x = cuda_c128(_unit_states(n, 7, 2513))
+    X = plan.propagate(x.repeat((nc + 6) // 7, 1)[:nc].contiguous(), 2, 3)
+    assert plan.check_status() == fq.FQ_OK
+    few = plan.propagate(x, 2, 3)
+    assert torch.equal(X, few.repeat((nc + 6) // 7, 1)[:nc])
+
+
 @pytest.mark.parametrize("n", [1, 5, 32, 33, 64, 65, 100, 128])
 def test_dense_fp64_resident_kernel(fq, n):
     """The small-N resident chain (clusters of ceil(N/32) CTAs, 64 steps per launch) against the
