@@ -34,16 +34,25 @@
 namespace {
 
 constexpr int TILE_NT = 256;  // most threads of a CTA
-constexpr int TILE_NW = TILE_NT / 32;
+constexpr int TILE_SLOTS = TILE_NT / 32 + 1;  // rows exchanged between warps, and a zero at the end
 constexpr int TILE_MAXL = 128;
 
-// Rows base .. a CTA holds and the rows [first, last) of them it writes, for segment blockIdx.x.
+// How the segments of a state lie: seg rows each, the tile of segment b from row b step - off on.
+struct TileSpan {
+  int seg, step, off;
+};
+
+// Rows base .. a CTA holds and the rows [first, last) of them it writes, for segment blockIdx.x.  LINEAR
+// takes the base from the span (it may be negative: those rows are zero).  The other form starts no tile
+// before row 0, as FP64 needs where the halos are as long as the state; the one-step FP32 kernel takes 8 % longer
+// with it (800 x 9001), and the double-float one spills more.
+template <bool LINEAR>
 struct TileRows {
   int first, last, base;
-  __device__ TileRows(int seg, int L, int n) {
-    first = blockIdx.x * seg;
-    last = min(first + seg, n);
-    base = max(0, first - L);
+  __device__ TileRows(TileSpan sp, int L, int n) {
+    first = blockIdx.x * sp.seg;
+    last = min(first + sp.seg, n);
+    base = LINEAR ? (int)blockIdx.x * sp.step - sp.off : max(0, first - L);
   }
 };
 
@@ -54,6 +63,8 @@ constexpr int F64_FLOOR_ROWS = 128;
 // Segments per state, threads per CTA and rows per thread.
 struct TileShape {
   int segs, seg, nt, ept;
+  // two segments have no halo on their outer sides, more have one on both
+  TileSpan span(int L) const { return segs <= 2 ? TileSpan{seg, segs == 1 ? 0 : seg - L, 0} : TileSpan{seg, seg, L}; }
 };
 
 // The shape for states of n rows, nc of them.  The arithmetic of a step is the rows the CTAs hold, halo
@@ -103,10 +114,20 @@ struct TileCoef {
 template <typename T, int TILE_EPT>
 struct Tile {
   using T2 = typename V2<T>::t;
-  static constexpr int NW = TILE_NW;
-  T2* slot_last;   // [2][NW]
-  T2* slot_first;  // [2][NW]
-  int lane, warp, warps;
+  T2* slot_last;   // [2][TILE_SLOTS]: entry w + 1 the last row of warp w, entry 0 zero
+  T2* slot_first;  // [2][TILE_SLOTS]: entry w the first row of warp w, the one after the last warp zero
+  int lane, warp;
+
+  __device__ __forceinline__ Tile(T2* slots) {
+    slot_last = slots;
+    slot_first = slots + 2 * TILE_SLOTS;
+    lane = threadIdx.x & 31;
+    warp = threadIdx.x >> 5;
+    if (threadIdx.x < 2) {  // visible from the first halo()'s barrier on
+      slot_last[threadIdx.x * TILE_SLOTS] = T2{0, 0};
+      slot_first[threadIdx.x * TILE_SLOTS + (blockDim.x >> 5)] = T2{0, 0};
+    }
+  }
 
   // rows i0 - 1 and i0 + EPT of x (neighbouring threads; zero beyond the tile)
   __device__ __forceinline__ void halo(const T2 (&x)[TILE_EPT], int par, T2& left, T2& right) {
@@ -114,16 +135,16 @@ struct Tile {
     T li = __shfl_up_sync(0xffffffffu, x[TILE_EPT - 1].y, 1);
     T rr = __shfl_down_sync(0xffffffffu, x[0].x, 1);
     T ri = __shfl_down_sync(0xffffffffu, x[0].y, 1);
-    if (lane == 31) slot_last[par * NW + warp] = x[TILE_EPT - 1];
-    if (lane == 0) slot_first[par * NW + warp] = x[0];
+    if (lane == 31) slot_last[par * TILE_SLOTS + warp + 1] = x[TILE_EPT - 1];
+    if (lane == 0) slot_first[par * TILE_SLOTS + warp] = x[0];
     __syncthreads();
     if (lane == 0) {
-      const T2 w = warp > 0 ? slot_last[par * NW + warp - 1] : T2{0, 0};
+      const T2 w = slot_last[par * TILE_SLOTS + warp];
       lr = w.x;
       li = w.y;
     }
     if (lane == 31) {
-      const T2 w = warp < warps - 1 ? slot_first[par * NW + warp + 1] : T2{0, 0};
+      const T2 w = slot_first[par * TILE_SLOTS + warp + 1];
       rr = w.x;
       ri = w.y;
     }
@@ -160,39 +181,34 @@ struct Tile {
   }
 };
 
-// `steps` steps of the chain (more than one only with a single segment per state).
-template <typename T, int TILE_EPT>
+// One step of the chain, or `steps` of them (MULTI: a single segment per state).
+template <typename T, int TILE_EPT, bool MULTI>
 __global__ void __launch_bounds__(TILE_NT)
 k_tri_tile(const typename V2<T>::t* __restrict__ cf, const typename V2<T>::t* __restrict__ rot,
            const T* __restrict__ xr, const T* __restrict__ xi, T* __restrict__ yr, T* __restrict__ yi, int n, int ld,
-           int L, int seg, int steps, TileCoef<T> coef, T ph_re, T ph_im, T bound2, unsigned int* status) {
+           int L, TileSpan span, int steps, TileCoef<T> coef, T ph_re, T ph_im, T bound2, unsigned int* status) {
   using T2 = typename V2<T>::t;
-  using Tl = Tile<T, TILE_EPT>;
-  __shared__ T2 slots[4 * Tl::NW];
-  Tl tl;
-  tl.slot_last = slots;
-  tl.slot_first = slots + 2 * Tl::NW;
-  tl.lane = threadIdx.x & 31;
-  tl.warp = threadIdx.x >> 5;
-  tl.warps = blockDim.x >> 5;
+  __shared__ T2 slots[4 * TILE_SLOTS];
+  Tile<T, TILE_EPT> tl(slots);
   const size_t j = blockIdx.y;
-  const TileRows rows(seg, L, n);
+  const TileRows<!MULTI> rows(span, L, n);
   const int i0 = rows.base + (int)threadIdx.x * TILE_EPT;
   T2 v[TILE_EPT], A[TILE_EPT], B[TILE_EPT];
   T d[TILE_EPT], e[TILE_EPT];
 #pragma unroll
   for (int q = 0; q < TILE_EPT; ++q) {
     const int i = i0 + q;
-    A[q] = i < n ? T2{xr[j * ld + i], xi[j * ld + i]} : T2{0, 0};
+    A[q] = (MULTI || i >= 0) && i < n ? T2{xr[j * ld + i], xi[j * ld + i]} : T2{0, 0};
   }
   bool bad = false;
   int par = 0;
   const T cL = coef.c[L];
-  for (int m = 0; m < steps; ++m, cf += ld, rot += ld) {
+  for (int m = 0; m < (MULTI ? steps : 1); ++m, cf += ld, rot += ld) {
 #pragma unroll
     for (int q = 0; q < TILE_EPT; ++q) {
       const int i = i0 + q;
-      const T2 r = i < n ? rot[i] : T2{0, 0}, c = i < n ? cf[i] : T2{0, 0};
+      const bool in = (MULTI || i >= 0) && i < n;
+      const T2 r = in ? rot[i] : T2{0, 0}, c = in ? cf[i] : T2{0, 0};
       v[q] = T2{fma(r.x, A[q].x, r.y * A[q].y), fma(r.x, A[q].y, -(r.y * A[q].x))};  // D^+ x
       d[q] = c.x;
       e[q] = c.y;
@@ -258,10 +274,21 @@ k_tri_tile(const typename V2<T>::t* __restrict__ cf, const typename V2<T>::t* __
 // SM: the double-float FMA chains are long, and latency, not the FP32 pipe, limits fewer warps.
 template <int DFL_EPT>
 struct DflTile {
-  static constexpr int NW = TILE_NW;
-  dflc* slot_last;   // [2][NW]
-  dflc* slot_first;  // [2][NW]
-  int lane, warp, warps;
+  dflc* slot_last;   // as Tile's
+  dflc* slot_first;
+  int lane, warp;
+
+  __device__ __forceinline__ DflTile(dflc* slots) {
+    const dflc z = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    slot_last = slots;
+    slot_first = slots + 2 * TILE_SLOTS;
+    lane = threadIdx.x & 31;
+    warp = threadIdx.x >> 5;
+    if (threadIdx.x < 2) {
+      slot_last[threadIdx.x * TILE_SLOTS] = z;
+      slot_first[threadIdx.x * TILE_SLOTS + (blockDim.x >> 5)] = z;
+    }
+  }
 
   __device__ __forceinline__ static dflc shfl(dflc a, bool up) {
     dflc r;
@@ -282,12 +309,11 @@ struct DflTile {
   __device__ __forceinline__ void halo(const dflc (&x)[DFL_EPT], int par, dflc& left, dflc& right) {
     dflc l = shfl(x[DFL_EPT - 1], true);
     dflc r = shfl(x[0], false);
-    if (lane == 31) slot_last[par * NW + warp] = x[DFL_EPT - 1];
-    if (lane == 0) slot_first[par * NW + warp] = x[0];
+    if (lane == 31) slot_last[par * TILE_SLOTS + warp + 1] = x[DFL_EPT - 1];
+    if (lane == 0) slot_first[par * TILE_SLOTS + warp] = x[0];
     __syncthreads();
-    const dflc z = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    if (lane == 0) l = warp > 0 ? slot_last[par * NW + warp - 1] : z;
-    if (lane == 31) r = warp < warps - 1 ? slot_first[par * NW + warp + 1] : z;
+    if (lane == 0) l = slot_last[par * TILE_SLOTS + warp];
+    if (lane == 31) r = slot_first[par * TILE_SLOTS + warp + 1];
     left = l;
     right = r;
   }
@@ -324,17 +350,11 @@ template <int DFL_EPT, bool MULTI>
 __global__ void __launch_bounds__(TILE_NT, 3)
 k_tri_tile_dfl(const dfl2* __restrict__ cf, const dfl2* __restrict__ rot, const double* __restrict__ xr,
                const double* __restrict__ xi, double* __restrict__ yr, double* __restrict__ yi, int n, int ld, int L,
-               int seg, int steps, DflCoef coef, double ph_re, double ph_im, double bound2, unsigned int* status) {
-  using Tl = DflTile<DFL_EPT>;
-  __shared__ dflc slots[4 * Tl::NW];
-  Tl tl;
-  tl.slot_last = slots;
-  tl.slot_first = slots + 2 * Tl::NW;
-  tl.lane = threadIdx.x & 31;
-  tl.warp = threadIdx.x >> 5;
-  tl.warps = blockDim.x >> 5;
+               TileSpan span, int steps, DflCoef coef, double ph_re, double ph_im, double bound2, unsigned int* status) {
+  __shared__ dflc slots[4 * TILE_SLOTS];
+  DflTile<DFL_EPT> tl(slots);
   const size_t j = blockIdx.y;
-  const TileRows rows(seg, L, n);
+  const TileRows<!MULTI> rows(span, L, n);
   const int i0 = rows.base + (int)threadIdx.x * DFL_EPT;
   const dfl zero = {0.f, 0.f};
   const dflc zc = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -356,7 +376,7 @@ k_tri_tile_dfl(const dfl2* __restrict__ cf, const dfl2* __restrict__ rot, const 
 #pragma unroll
     for (int q = 0; q < DFL_EPT; ++q) {
       const int i = i0 + q;
-      if (i < n) {
+      if ((MULTI || i >= 0) && i < n) {
         const dfl2 r = rot[i], c = cf[i];
         const double rc = dfl_value(r.x), rs = dfl_value(r.y);
         const double x_r = MULTI ? o_r[q] : xr[j * ld + i], x_i = MULTI ? o_i[q] : xi[j * ld + i];
@@ -475,8 +495,8 @@ fq_status dfl_chain(fq_plan* p, const double* x0, double* x, int nc, int m_begin
                         : sh.ept == 2 ? k_tri_tile_dfl<2, true>
                                       : k_tri_tile_dfl<4, true>;
       kern<<<dim3(sh.segs, rows), sh.nt, 0, s>>>(cf + (size_t)m * ld, rot + (size_t)m * ld, b[cur].re + o,
-                                                 b[cur].im + o, b[cur ^ 1].re + o, b[cur ^ 1].im + o, n, ld, L, sh.seg,
-                                                 per, coef, p->phase_re, p->phase_im, 1.0 + 1e-9, p->d_status);
+                                                 b[cur].im + o, b[cur ^ 1].re + o, b[cur ^ 1].im + o, n, ld, L,
+                                                 sh.span(L), per, coef, p->phase_re, p->phase_im, 1.0 + 1e-9, p->d_status);
       fq_ktimer_stop(p, s);
     }
     cur ^= 1;
@@ -541,10 +561,15 @@ fq_status tile_chain(fq_plan* p, const double* x0, double* x, int nc, int m_begi
     for (int r0 = 0; r0 < nc; r0 += 65535) {  // gridDim.y limit
       const int rows = nc - r0 < 65535 ? nc - r0 : 65535;
       const size_t o = (size_t)r0 * ld;
-      const auto kern = sh.ept == 2 ? k_tri_tile<T, 2> : (sh.ept == 4 ? k_tri_tile<T, 4> : k_tri_tile<T, 8>);
+      auto kern = sh.ept == 2 ? k_tri_tile<T, 2, true> : (sh.ept == 4 ? k_tri_tile<T, 4, true> : k_tri_tile<T, 8, true>);
+      // FP32 in several segments (8 rows a thread): the form for one step needs 80 registers instead of 115, and
+      // three CTAs share an SM instead of two.  Twelve steps of 4000 x 3001 3.07 ms against 3.91 on the form for
+      // many steps, 800 x 9001 3.07 against 3.46, 300 x 20001 3.81 against 4.26.
+      if constexpr (sizeof(T) == 4)
+        if (sh.segs > 1) kern = k_tri_tile<T, 8, false>;
       kern<<<dim3(sh.segs, rows), sh.nt, 0, s>>>(cf + (size_t)m * ld, rot + (size_t)m * ld, b[cur].re + o,
-                                                 b[cur].im + o, b[cur ^ 1].re + o, b[cur ^ 1].im + o, n, ld, L, sh.seg,
-                                                 per, coef, (T)p->phase_re, (T)p->phase_im, b2, p->d_status);
+                                                 b[cur].im + o, b[cur ^ 1].re + o, b[cur ^ 1].im + o, n, ld, L,
+                                                 sh.span(L), per, coef, (T)p->phase_re, (T)p->phase_im, b2, p->d_status);
     }
     cur ^= 1;
   }
