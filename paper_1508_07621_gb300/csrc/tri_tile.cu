@@ -474,13 +474,16 @@ fq_status dfl_chain(fq_plan* p, const double* x0, double* x, int nc, int m_begin
   }
   const int epts[] = {1, 2, 4};
   TileShape sh = pick_tile(n, nc, L, epts, 0);
-  // Three CTAs share an SM.  Where the CTAs are a wave and a part of one, segments as long as fit and a
-  // short last one (its FP64 rotations are few) fill the second wave better than equal ones: 160 x 3001
-  // 86 us a step against 95.
-  const double waves = (double)nc * sh.segs / (3.0 * fq_sm_count());
-  if (sh.segs > 1 && waves > 1.25 && waves < 2.0) {
-    sh.seg = 4 * TILE_NT - 2 * L;
-    sh.segs = (n + sh.seg - 1) / sh.seg;
+  // Four segments: where the CTAs are a few more than a whole number an SM, three segments as long as fit and
+  // a short last one (its FP64 rotations are few) spare the SMs that extra CTA.  The lines were drawn on a sweep
+  // of 28 lengths from 1051 to 7801 rows and 20 to 600 states: 120 x 3001 82 us a step against 90, 160 x 3001
+  // 96 against 103, 230 x 3101 129 against 135; beside these lines, and at other numbers of segments, equal
+  // ones take as long or up to 14 % less (320 x 1201).
+  const int longest = 4 * TILE_NT - 2 * L;
+  const double ctas = (double)nc * sh.segs / fq_sm_count();  // an SM
+  if (sh.segs == 4 && n - 3 * longest <= longest / 3 && ctas > 3.0 && ctas < 7.0 && ctas - std::floor(ctas) < 0.27) {
+    sh.seg = longest;
+    sh.segs = (n + longest - 1) / longest;
     sh.nt = TILE_NT;
   }
   const int per = sh.segs == 1 ? nsteps : 1;  // steps a launch

@@ -297,9 +297,8 @@ def _unit_states(n, count, seed):
 @pytest.mark.parametrize("nb", [1, 30, 63, 64, 127, 128, 255, 256, 511, 512, 600, 1023, 1024, 1500, 2047, 2048, 3000])
 def test_tiled_shapes_agree(fq, precision, nb):
     """Segments, threads and rows per thread follow the length and number of the states: one state, the
-    same state among 170 (at 3001 rows the double-float kernel's second wave), and step by step (one
-    launch runs every step where one CTA holds a state) give the same bits, at sizes around every rows-per-thread
-    limit, and the oracle's state."""
+    same state among 170, and step by step (one launch runs every step where one CTA holds a state) give
+    the same bits, at sizes around every rows-per-thread limit, and the oracle's state."""
     import torch
     d = _drive_models(nb)
     plan = dimer_plan(fq, d, precision, 3)
@@ -316,6 +315,23 @@ def test_tiled_shapes_agree(fq, precision, nb):
     ref = o.propagate_tridiag(d.h0_diag, d.h0_off, d.h1_diag, refp, x0[[0, 169]].T, 1, 4).T
     tol = tol_f32(3, plan.info.L, plan.info.R) if precision == 1 else 1e-12
     assert np.max(np.abs(to_np(many[[0, 169]]) - ref)) <= tol
+
+
+@pytest.mark.parametrize("nb,nc", [(2949, 118), (3000, 160), (3200, 120)])
+def test_tiled_dfl_short_last_segment(fq, nb, nc):
+    """Double-float states whose four segments run with a short last one (a few more CTAs than a whole
+    number an SM), which holds a handful of rows, an eighth and a quarter of a segment: the bits of a lone
+    state, whose segments are equal, and the oracle's."""
+    import torch
+    d = _drive_models(nb)
+    plan = dimer_plan(fq, d, 4, 3)
+    x0 = _unit_states(d.n, 2, 2305)
+    many = plan.propagate(cuda_c128(np.tile(x0, (nc // 2, 1))), 1, 4)
+    assert plan.check_status() == fq.FQ_OK
+    assert torch.equal(many[:1], plan.propagate(cuda_c128(x0[:1]), 1, 4)) and torch.equal(many[-2:], many[:2])
+    refp = o.plan_for_drive_tridiag(d.h0_diag, d.h0_off, d.h1_diag, d.drive, d.steps)
+    ref = o.propagate_tridiag(d.h0_diag, d.h0_off, d.h1_diag, refp, x0.T, 1, 4).T
+    assert np.max(np.abs(to_np(many[:2]) - ref)) <= 1e-12
 
 
 @pytest.mark.parametrize("nb", [1, 31, 63, 64, 100, 127, 200, 255, 320, 383, 500, 511, 512, 700, 1000, 1023, 1024, 1300,
