@@ -552,6 +552,11 @@ fq_status floquet_build_UT(fq_plan* p, void* d_U, void* d_ws, size_t ws_bytes, v
   return propagate_impl(p, nullptr, (double*)d_U, p->n, 0, p->steps, 1, 1, d_ws, ws_bytes, (cudaStream_t)stream);
 }
 
+// Least workspace of the defect over k of n columns: a pair of doubles per 16 of them and 256 columns
+static size_t defect_least_bytes(int n, int k) {
+  return align_up(2 * sizeof(double) * (size_t)((k + 15) / 16) * ((n + 255) / 256));
+}
+
 fq_status floquet_build_UT_report(fq_plan* p, void* d_U, void* d_ws, size_t ws_bytes, void* stream,
                                   int32_t defect_columns, fq_report* rep) {
   if (!p || !d_U || !rep) { fq_set_error("NULL plan, output or report"); return FQ_EINVAL; }
@@ -560,11 +565,12 @@ fq_status floquet_build_UT_report(fq_plan* p, void* d_U, void* d_ws, size_t ws_b
     fq_set_error("floquet_build_UT_report: defect_columns must be in [1, %d] (got %d)", n, defect_columns);
     return FQ_EINVAL;
   }
-  const size_t dws = floquet_defect_workspace_size(n), need = dws + align_up(4 * (size_t)defect_columns);
+  const size_t list = align_up(4 * (size_t)defect_columns), need = defect_least_bytes(n, n) + list;
   if (!d_ws || ws_bytes < need) {
     fq_set_error("floquet_build_UT_report: workspace must hold %zu bytes for the defect", need);
     return FQ_EINVAL;
   }
+  const size_t dws = std::min(floquet_defect_workspace_size(n), (ws_bytes - list) / kAlign * kAlign);
   return fq_guard("floquet_build_UT_report", [&]() -> fq_status {
     cudaStream_t s = (cudaStream_t)stream;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -686,7 +692,9 @@ fq_status floquet_build_UT_columns(fq_plan* p, int32_t j0, int32_t ncols, void* 
 
 size_t floquet_defect_workspace_size(int32_t n) {
   if (n < 1) return 0;
-  return align_up(2 * sizeof(double) * (size_t)((n + 15) / 16) * ((n + 255) / 256));
+  // a pair of doubles per 32 columns and 16 listed ones, and for small N per column, up to 2048 of them
+  const size_t blocks = (n + 31) / 32;
+  return align_up(2 * sizeof(double) * std::max((size_t)((n + 15) / 16) * blocks, std::min((size_t)n * blocks, (size_t)2048)));
 }
 
 fq_status floquet_unitarity_defect(const void* d_U, int32_t n, const int32_t* d_cols, int32_t k, void* d_ws,
@@ -694,16 +702,14 @@ fq_status floquet_unitarity_defect(const void* d_U, int32_t n, const int32_t* d_
   if (!d_U || n < 1 || !max_abs || !fro) { fq_set_error("bad defect arguments"); return FQ_EINVAL; }
   const int rows = d_cols ? k : n;
   if (rows < 1 || rows > n) { fq_set_error("defect: k must be in [1, n]"); return FQ_EINVAL; }
-  const int nb = (n + 255) / 256;
-  const int chunks = (rows + 15) / 16;
-  const size_t need = align_up(2 * sizeof(double) * (size_t)chunks * nb);
+  const size_t need = defect_least_bytes(n, rows);
   if (!d_ws || ws_bytes < need) { fq_set_error("defect workspace too small (%zu < %zu)", ws_bytes, need); return FQ_EINVAL; }
   cudaStream_t s = (cudaStream_t)stream;
   const int parts = fq_launch_defect((const double*)d_U, n, d_cols, rows, (double*)d_ws,
                                      ws_bytes / (2 * sizeof(double)), s);
   cudaError_t e = cudaGetLastError();  // a refused launch leaves the workspace as it was
   if (e != cudaSuccess) return fq_cuda_fail(e, "defect launch");
-  std::vector<double> h(2 * (size_t)parts * nb, 0.0);
+  std::vector<double> h(2 * (size_t)parts, 0.0);
   e = cudaMemcpyAsync(h.data(), d_ws, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return fq_cuda_fail(e, "defect");

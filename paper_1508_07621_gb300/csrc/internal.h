@@ -301,7 +301,7 @@ fq_status fq_grad_split(fq_plan* p, const double* d_f, const void* d_W, double* 
 fq_status fq_split_propagate(fq_plan* p, const double* x0, double* x, int nc, int m_begin, int m_end, int identity,
                              int transpose_out, void* ws, cudaStream_t s);
 
-// |D| partials (largest, sum of squares) of ceil(n / 256) column blocks x the returned number of chunks of the
-// k listed columns, at most `slots` pairs (at least ceil(n / 256) ceil(k / 16))
+// |D| partials (largest, sum of squares) of the k listed columns, the returned number of pairs: at most `slots`, of
+// which there are at least ceil(n / 256) ceil(k / 16)
 int fq_launch_defect(const double* u, int n, const int32_t* cols, int k, double* partial, size_t slots,
                      cudaStream_t s);

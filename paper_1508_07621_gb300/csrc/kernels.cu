@@ -442,69 +442,66 @@ k_term_band6(const double* __restrict__ ore, const double* __restrict__ oim, int
 }
 
 // ------------------------------------------------------------------ unitarity defect
-// D[c][j] = sum_i conj(U[i][c]) U[i][j] - delta_cj for KC listed columns c (chunk blockIdx.y) and the 256
-// columns j of a cluster of 8 CTAs: a CTA has 32 of them, one a lane, its 8 warps take every 8th row i,
-// and the chunk's entries of a row are loads of one address a warp.  Per cluster: the largest |D| and the
-// sum of |D|^2, in a fixed order (the CTAs' parts meet in the first one's shared memory, which may be
-// written once that CTA runs: every CTA arrives at the cluster's barrier on entry and waits for the
-// others just before it stores, so the rows' sums hide the wait).
+// D[c][j] = sum_i conj(U[i][c]) U[i][j] - delta_cj for KC listed columns c (chunk blockIdx.y) and the columns
+// j of `span` blocks of 32, one column a lane: the 8 warps take every 8th row i, and the chunk's entries of a row
+// are loads of one address a warp.  Per CTA: the largest |D| and the sum of |D|^2, in a fixed order.
 // Bound by the FP64 pipes: 4 KC multiply-adds a lane and row; the chunk size fills the chip
 // (fq_launch_defect).  (One thread a column and a barrier pair a row kept N / 256 x k / 16 CTAs of one
-// row in flight each: N = 4096, 64 columns 19.6 ms, now 8.3 ms; N = 243, 40 columns 1.15 ms, now 0.08 ms.)
-constexpr int DEFECT_CTAS = 8;   // CTAs of a cluster
+// row in flight each: N = 4096, 64 columns 19.1 ms, now 7.2 ms; N = 243, 40 columns 1.13 ms, now 0.06 ms.
+// Clusters of eight CTAs with one partial between them leave SMs idle that hold no whole cluster: 8.2 ms, and
+// 466 ms against 441 for all columns at N = 4096.)
 constexpr int DEFECT_WARPS = 8;
 
 template <int KC>
-__global__ void __cluster_dims__(DEFECT_CTAS, 1, 1) __launch_bounds__(32 * DEFECT_WARPS, KC > 8 ? 2 : 3)
-    k_defect(const double2* __restrict__ u, int n, const int32_t* __restrict__ cols, int k, double* partial) {
+__global__ void __launch_bounds__(32 * DEFECT_WARPS, KC > 8 ? 2 : 3)
+    k_defect(const double2* __restrict__ u, int n, const int32_t* __restrict__ cols, int k, int span, double* partial) {
   __shared__ double2 red[DEFECT_WARPS][KC][32];
-  __shared__ double part[DEFECT_WARPS][2], cta[DEFECT_CTAS][2];
+  __shared__ double part[DEFECT_WARPS][2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rank = blockIdx.x % DEFECT_CTAS;
   const int c0 = blockIdx.y * KC, kc = min(KC, k - c0);
-  const int j = blockIdx.x * 32 + lane;
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   int col[KC];
 #pragma unroll
   for (int q = 0; q < KC; ++q) {
     const int c = q < kc ? (cols ? cols[c0 + q] : c0 + q) : -1;
     col[q] = c < n ? c : -1;
   }
-  double sr[KC], si[KC];
+  const double2 zero = make_double2(0.0, 0.0);
+  double mx = 0.0, ss = 0.0;  // of |D|^2
+  for (int b = 0; b < span && (blockIdx.x * span + b) * 32 < n; ++b) {
+    const int j = (blockIdx.x * span + b) * 32 + lane;
+    double sr[KC], si[KC];
 #pragma unroll
-  for (int q = 0; q < KC; ++q) sr[q] = si[q] = 0.0;
-  if (blockIdx.x * 32 < n) {
-    const double2 zero = make_double2(0.0, 0.0);
+    for (int q = 0; q < KC; ++q) sr[q] = si[q] = 0.0;
 #pragma unroll(KC > 4 ? 1 : 2)
     for (int i = warp; i < n; i += DEFECT_WARPS) {
       const double2* row = u + (size_t)i * n;
-      const double2 b = j < n ? row[j] : zero;
+      const double2 v = j < n ? row[j] : zero;
       double2 a[KC];
 #pragma unroll
       for (int q = 0; q < KC; ++q) a[q] = col[q] >= 0 ? row[col[q]] : zero;
 #pragma unroll
       for (int q = 0; q < KC; ++q) {
-        sr[q] = fma(a[q].x, b.x, fma(a[q].y, b.y, sr[q]));
-        si[q] = fma(a[q].x, b.y, fma(-a[q].y, b.x, si[q]));
+        sr[q] = fma(a[q].x, v.x, fma(a[q].y, v.y, sr[q]));
+        si[q] = fma(a[q].x, v.y, fma(-a[q].y, v.x, si[q]));
       }
     }
-  }
+    if (b > 0) __syncthreads();  // the last block's sums are read
 #pragma unroll
-  for (int q = 0; q < KC; ++q) red[warp][q][lane] = make_double2(sr[q], si[q]);
-  __syncthreads();
-  double mx = 0.0, ss = 0.0;  // of |D|^2
-  for (int q = warp; q < kc; q += DEFECT_WARPS) {
-    double r = 0.0, m = 0.0;
-    for (int w = 0; w < DEFECT_WARPS; ++w) {
-      r += red[w][q][lane].x;
-      m += red[w][q][lane].y;
-    }
-    if (j < n) {
-      const int c = cols ? cols[c0 + q] : c0 + q;
-      if (c == j) r -= 1.0;
-      const double a2 = r * r + m * m;
-      mx = fmax(mx, a2);
-      ss += a2;
+    for (int q = 0; q < KC; ++q) red[warp][q][lane] = make_double2(sr[q], si[q]);
+    __syncthreads();
+    for (int q = warp; q < kc; q += DEFECT_WARPS) {
+      double r = 0.0, m = 0.0;
+      for (int w = 0; w < DEFECT_WARPS; ++w) {
+        r += red[w][q][lane].x;
+        m += red[w][q][lane].y;
+      }
+      if (j < n) {
+        const int c = cols ? cols[c0 + q] : c0 + q;
+        if (c == j) r -= 1.0;
+        const double a2 = r * r + m * m;
+        mx = fmax(mx, a2);
+        ss += a2;
+      }
     }
   }
   for (int o = 16; o > 0; o >>= 1) {
@@ -516,27 +513,13 @@ __global__ void __cluster_dims__(DEFECT_CTAS, 1, 1) __launch_bounds__(32 * DEFEC
     part[warp][1] = ss;
   }
   __syncthreads();
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // the first CTA is running
   if (threadIdx.x == 0) {
     mx = ss = 0.0;
     for (int w = 0; w < DEFECT_WARPS; ++w) {
       mx = fmax(mx, part[w][0]);
       ss += part[w][1];
     }
-    const unsigned la = (unsigned)__cvta_generic_to_shared(&cta[rank][0]);
-    unsigned ra;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(0));
-    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(ra), "d"(mx), "d"(ss) : "memory");
-  }
-  __syncwarp();
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-  if (rank == 0 && threadIdx.x == 0) {
-    mx = ss = 0.0;
-    for (int c = 0; c < DEFECT_CTAS; ++c) {
-      mx = fmax(mx, cta[c][0]);
-      ss += cta[c][1];
-    }
-    const size_t slot = (size_t)blockIdx.y * (gridDim.x / DEFECT_CTAS) + blockIdx.x / DEFECT_CTAS;
+    const size_t slot = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
     partial[2 * slot] = sqrt(mx);
     partial[2 * slot + 1] = ss;
   }
@@ -801,22 +784,26 @@ double fq_launch_fp32_probe(int packed, int iters, float* out, int blocks, cudaS
 }
 
 // Columns per chunk: the largest that gives the chip four CTAs a SM, or the smallest whose partials fit
-// `slots` (16 always fit) where none does.
+// `slots` where none does.  A workspace of the least size (a slot per 256 columns and chunk of 16) takes several
+// column blocks a CTA.
 int fq_launch_defect(const double* u, int n, const int32_t* cols, int k, double* partial, size_t slots,
                      cudaStream_t s) {
-  const int nb = (n + 255) / 256;
+  const size_t blocks = (n + 31) / 32;
   int kc = 16;
   while (kc > 1) {
-    const int chunks = (k + kc - 1) / kc, finer = (k + kc / 2 - 1) / (kc / 2);
-    if ((long long)DEFECT_CTAS * nb * chunks >= 4LL * fq_sm_count() || (size_t)finer * nb > slots || finer > 65535) break;
+    const size_t chunks = (k + kc - 1) / kc, finer = (k + kc / 2 - 1) / (kc / 2);
+    if (blocks * chunks >= 4 * (size_t)fq_sm_count() || finer * blocks > slots || finer > 65535) break;
     kc /= 2;
   }
-  const dim3 g(DEFECT_CTAS * nb, (k + kc - 1) / kc);
+  const size_t chunks = (k + kc - 1) / kc;
+  int span = 1;
+  while (span < 8 && (blocks + span - 1) / span * chunks > slots) ++span;
+  const dim3 g((unsigned)((blocks + span - 1) / span), (unsigned)chunks);
   const auto kern = kc == 16  ? k_defect<16>
                     : kc == 8 ? k_defect<8>
                     : kc == 4 ? k_defect<4>
                     : kc == 2 ? k_defect<2>
                               : k_defect<1>;
-  kern<<<g, 32 * DEFECT_WARPS, 0, s>>>((const double2*)u, n, cols, k, partial);
-  return (int)g.y;
+  kern<<<g, 32 * DEFECT_WARPS, 0, s>>>((const double2*)u, n, cols, k, span, partial);
+  return (int)(g.x * g.y);
 }

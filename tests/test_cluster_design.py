@@ -34,7 +34,7 @@ CLUSTERED = {name: body for name, body in _kernels() if REMOTE.search(body)}
 
 
 def test_clustered_kernels_are_found():
-    assert {"k_defect", "k_dense_resident", "k_dense_resident_dfl", "k_oz_term", "k_oz_real_term"} <= set(CLUSTERED)
+    assert {"k_dense_resident", "k_dense_resident_dfl", "k_oz_term", "k_oz_real_term"} <= set(CLUSTERED)
 
 
 @pytest.mark.parametrize("name", sorted(CLUSTERED))

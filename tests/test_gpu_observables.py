@@ -189,6 +189,24 @@ def test_unitarity_defect_chunks(fq, n, k):
     assert abs(fro - np.linalg.norm(full) / math.sqrt(n)) <= 1e-14 * (1 + n)
 
 
+@pytest.mark.parametrize("n,k", [(40, 40), (257, 33), (520, 520)])
+def test_unitarity_defect_least_workspace(fq, n, k):
+    """A workspace of the least accepted size (a pair of doubles per 16 listed columns and 256 columns) makes a
+    CTA take several column blocks: the defect of the queried size to rounding, and one alignment unit less is
+    refused."""
+    import torch
+    rng = np.random.default_rng(1851)
+    u = fi.haar_unitary(n, 1852) + 1e-3 * (rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n)))
+    U = torch.from_numpy(np.ascontiguousarray(u)).cuda()
+    cols = torch.from_numpy(rng.permutation(n)[:k].astype(np.int32)).cuda()
+    least = -(-16 * -(-k // 16) * -(-n // 256) // 256) * 256
+    mx, fro = fq.api.unitarity_defect(U, cols)
+    a, b = fq.floquet_unitarity_defect(U, n, cols, k, fq.workspace(least))
+    assert abs(a - mx) <= 1e-15 and abs(b - fro) <= 1e-14 * fro
+    with pytest.raises(fq.FloquetError):
+        fq.floquet_unitarity_defect(U, n, cols, k, fq.workspace(least - 256))
+
+
 @pytest.mark.parametrize("precision", [0, 2])
 def test_overlap_phase_error_matches_oracle(fq, precision):
     """Eq. 20 on the library (coarse chain applied to the fine Floquet states by
