@@ -25,39 +25,52 @@ __device__ double block_sum(double v, double* red) {
   return s;  // valid in thread 0
 }
 
-constexpr int EXPECT_STATES = 4;  // states per CTA, a warp each
-constexpr int EXPECT_CHUNK = 512;  // tridiagonal: rows of H staged at a time
+constexpr int EXPECT_STATES = 4;  // states per CTA (tridiagonal: one where they are few)
 constexpr int EXPECT_BLOCK = 32;   // dense: rows of H per CTA
+constexpr int EXPECT_WARPS = 8;    // tridiagonal: warps of a CTA
+// tridiagonal: up to this many states an SM, a CTA a state (500 x 1001 0.41 ms against 0.37 with four, 400 0.34 either
+// way, 300 0.32 against 0.35)
+constexpr int EXPECT_SINGLE = 3;
 
 // acc[r] += w <x_r| c0 H0 + c1 H1 |x_r>, tridiagonal H0 (diag, off), diagonal H1:
-// sum_i d_i |x_i|^2 + 2 c0 o_i Re(conj(x_i) x_{i+1}), d = c0 diag + c1 H1.  Bound by the FP64 pipes (64
-// cycles a warp and instruction): 6 instructions an entry, d and o once for a CTA's states (one state per
-// CTA and both neighbours of every entry took 14).
-__global__ void __launch_bounds__(32 * EXPECT_STATES)
+// sum_i d_i |x_i|^2 + 2 c0 o_i Re(conj(x_i) x_{i+1}), d = c0 diag + c1 H1, for S states a CTA.  Row i goes to lane
+// i % 32 of warp (i / 32) % 8; the warps, then the lanes are added pairwise, whatever S is.  Bound by the FP64
+// pipes (64 cycles a warp and instruction): 6 instructions an entry, and 4 for d and o, once for the S states.
+// (One state per CTA and both neighbours of every entry took 14 instructions; a warp a state, H staged for four of
+// them, left most FP64 pipes idle below a thousand states.)  Averages over ten FP32 steps in ms, a warp a state and
+// now, states x rows: 30 x 10001 2.06 -> 1.03, 100 x 1001 0.38 -> 0.28, 600 x 1001 0.43 -> 0.37, 1500 x 1001 0.69 ->
+// 0.70, 3000 x 301 0.43 -> 0.50 (more states than rows; two rounds of 256 rows for 301).
+template <int S>
+__global__ void __launch_bounds__(32 * EXPECT_WARPS)
     k_expect_tri(const double2* __restrict__ x, int nc, int n, const double* __restrict__ h0d,
                  const double* __restrict__ h0o, const double* __restrict__ h1d, double c0, double c1, double w,
                  double* acc) {
-  __shared__ double2 sh[EXPECT_CHUNK];  // (d_i, 2 c0 o_i)
-  const int lane = threadIdx.x & 31, r = blockIdx.x * EXPECT_STATES + (threadIdx.x >> 5);
-  const double2* row = x + (size_t)min(r, nc - 1) * n;
-  double s = 0.0;
-  for (int i0 = 0; i0 < n; i0 += EXPECT_CHUNK) {
-    __syncthreads();
-    for (int q = threadIdx.x; q < EXPECT_CHUNK; q += 32 * EXPECT_STATES) {
-      const int i = i0 + q;
-      sh[q] = make_double2(i < n ? fma(c0, h0d[i], c1 * h1d[i]) : 0.0, i + 1 < n ? 2.0 * c0 * h0o[i] : 0.0);
-    }
-    __syncthreads();
-    const int m = min(EXPECT_CHUNK, n - i0);
-#pragma unroll 4
-    for (int q = lane; q < m; q += 32) {
-      const int i = i0 + q;
-      const double2 a = row[i], b = i + 1 < n ? row[i + 1] : make_double2(0.0, 0.0);
-      s = fma(sh[q].x, fma(a.x, a.x, a.y * a.y), fma(sh[q].y, fma(a.x, b.x, a.y * b.y), s));
+  __shared__ double part[S][EXPECT_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r0 = blockIdx.x * S;
+  double sum[S];
+#pragma unroll
+  for (int q = 0; q < S; ++q) sum[q] = 0.0;
+#pragma unroll(S > 1 ? 2 : 4)
+  for (int i = threadIdx.x; i < n; i += 32 * EXPECT_WARPS) {
+    const bool right = i + 1 < n;
+    const double d = fma(c0, h0d[i], c1 * h1d[i]), o = right ? 2.0 * c0 * h0o[i] : 0.0;
+#pragma unroll
+    for (int q = 0; q < S; ++q) {
+      const double2* row = x + (size_t)min(r0 + q, nc - 1) * n;
+      const double2 a = row[i], b = right ? row[i + 1] : make_double2(0.0, 0.0);
+      sum[q] = fma(d, fma(a.x, a.x, a.y * a.y), fma(o, fma(a.x, b.x, a.y * b.y), sum[q]));
     }
   }
+#pragma unroll
+  for (int q = 0; q < S; ++q) part[q][warp][lane] = sum[q];
+  __syncthreads();
+  if (warp >= S) return;
+  double p[EXPECT_WARPS];
+#pragma unroll
+  for (int u = 0; u < EXPECT_WARPS; ++u) p[u] = part[warp][u][lane];
+  double s = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0 && r < nc) acc[r] += w * s;
+  if (lane == 0 && r0 + warp < nc) acc[r0 + warp] += w * s;
 }
 
 // A = c0 H0 + c1 H1
@@ -205,8 +218,10 @@ static fq_status floquet_average_observable_body(fq_plan* p, const void* d_X0, i
     const double c0 = a0, c1 = a1 + s_drive * f;
     const int groups = (ncols + EXPECT_STATES - 1) / EXPECT_STATES;
     if (p->format == FQ_TRIDIAG) {
-      k_expect_tri<<<groups, 32 * EXPECT_STATES, 0, s>>>((const double2*)X, ncols, n, p->d_h0, p->d_h0o, p->d_h1, c0, c1,
-                                                         w[m], acc);
+      const bool single = ncols <= EXPECT_SINGLE * fq_sm_count();
+      const auto kern = single ? k_expect_tri<1> : k_expect_tri<EXPECT_STATES>;
+      kern<<<single ? ncols : groups, 32 * EXPECT_WARPS, 0, s>>>((const double2*)X, ncols, n, p->d_h0, p->d_h0o, p->d_h1,
+                                                                 c0, c1, w[m], acc);
     } else {
       const size_t nn = (size_t)n * n;
       k_expect_form<<<(int)std::min<size_t>((nn + 255) / 256, 152 * 16), 256, 0, s>>>(p->d_h0, p->d_h1, nn, c0, c1, A);

@@ -169,6 +169,21 @@ def test_tridiagonal_averages_by_path(fq, precision, kernel, nb, nc):
     assert np.max(np.abs(avg - ref)) <= 4 * n * 2.0 ** -53 * scale + 1e-15
 
 
+@pytest.mark.parametrize("nb", [1, 30, 255, 256, 511, 512, 1100])
+def test_tridiagonal_averages_few_and_many_states(fq, nb):
+    """A CTA a state for up to three states an SM, four states a CTA for more: a state's average has the same bits
+    either way, at row counts around the 256-row rounds, with a partly filled last CTA."""
+    import torch
+    d = fi.config_dimer(nb=nb)
+    plan = fq.Plan.tridiag(d.h0_diag, d.h0_off, d.h1_diag, omega=3.0, f_ac=1.5, f_dc=0.2, phi0=0.3, steps=4,
+                           period=4 * 2 * math.pi / 6000, precision=fq.FQ_FP64)
+    x = _random_states(d.n, 5, 1835)
+    few = plan.average_observable(x, 0.7, -0.4, 1.3)
+    many = plan.average_observable(x.repeat(121, 1).contiguous(), 0.7, -0.4, 1.3)
+    assert plan.check_status() == fq.FQ_OK
+    assert torch.equal(many, few.repeat(121))
+
+
 @pytest.mark.parametrize("n,k", [(1, 1), (5, 3), (31, 31), (32, 1), (33, 17), (255, 2), (256, 9), (257, 40), (520, 130)])
 def test_unitarity_defect_chunks(fq, n, k):
     """The defect over listed columns (unsorted, one of them twice) at the edges of the 32- and 256-column
