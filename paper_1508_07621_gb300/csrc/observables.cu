@@ -86,8 +86,14 @@ __global__ void k_expect_form(const double* __restrict__ h0, const double* __res
 // states a CTA balance the rest.  Bound by the FP64 pipes: half of the 2 N^2 multiply-adds a state.  (One
 // state per CTA, a thread per row of H walking it, formed A for every state on uncoalesced reads: 151 us
 // at N = 256 and 256 states, now 53 us.)
+// FORM: A's entries are formed here from H0 and H1 (16 more instructions for a warp's 64 a block), without
+// k_expect_form's launch: up to N = 128, where every CTA has an SM to itself.  Averages over ten steps in ms, formed
+// before / here: FP64 N = 40 0.41 / 0.38, 128 1.39 / 1.38, BF16X3 64 0.68 / 0.66, 200 1.14 / 1.14, 400 (40 states) 1.29 /
+// 1.34, 1000 (16) 2.36 / 2.59: the CTA of the last rows forms all of them.
+template <bool FORM>
 __global__ void __launch_bounds__(32 * EXPECT_STATES)
-    k_expect_dense(const double2* __restrict__ x, int nc, int n, const double* __restrict__ A, double w, double* acc) {
+    k_expect_dense(const double2* __restrict__ x, int nc, int n, const double* __restrict__ A,
+                   const double* __restrict__ h1, double c0, double c1, double w, double* acc) {
   __shared__ double sa[EXPECT_BLOCK][EXPECT_BLOCK + 1];      // [k][i]
   __shared__ double2 sx[EXPECT_STATES][EXPECT_BLOCK];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -100,8 +106,10 @@ __global__ void __launch_bounds__(32 * EXPECT_STATES)
 #pragma unroll
     for (int q = 0; q < EXPECT_BLOCK / EXPECT_STATES; ++q) {
       const int ii = warp + EXPECT_STATES * q;
-      const bool in = i0 + ii < n && k0 + lane < n;
-      sa[lane][ii] = in ? A[(size_t)(i0 + ii) * n + k0 + lane] : 0.0;
+      const size_t at = (size_t)(i0 + ii) * n + k0 + lane;
+      double v = 0.0;
+      if (i0 + ii < n && k0 + lane < n) v = FORM ? fma(c0, A[at], c1 * h1[at]) : A[at];
+      sa[lane][ii] = v;
     }
     sx[warp][lane] = r < nc && k0 + lane < n ? x[(size_t)r * n + k0 + lane] : make_double2(0.0, 0.0);
     __syncthreads();
@@ -224,8 +232,12 @@ static fq_status floquet_average_observable_body(fq_plan* p, const void* d_X0, i
                                                                  c0, c1, w[m], acc);
     } else {
       const size_t nn = (size_t)n * n;
-      k_expect_form<<<(int)std::min<size_t>((nn + 255) / 256, 152 * 16), 256, 0, s>>>(p->d_h0, p->d_h1, nn, c0, c1, A);
-      k_expect_dense<<<dim3(groups, nb), 32 * EXPECT_STATES, 0, s>>>((const double2*)X, ncols, n, A, w[m], acc);
+      const bool form = nb <= 4 && groups * nb <= fq_sm_count();
+      if (!form)
+        k_expect_form<<<(int)std::min<size_t>((nn + 255) / 256, 152 * 16), 256, 0, s>>>(p->d_h0, p->d_h1, nn, c0, c1, A);
+      const auto kern = form ? k_expect_dense<true> : k_expect_dense<false>;
+      kern<<<dim3(groups, nb), 32 * EXPECT_STATES, 0, s>>>((const double2*)X, ncols, n, form ? p->d_h0 : A, p->d_h1, c0, c1,
+                                                           w[m], acc);
     }
   };
   // a tridiagonal plan's gauge tables for all steps at once: one CTA forms a step's, for tens of us

@@ -140,6 +140,19 @@ def test_dense_averages_block_edges(fq, n, nc):
         assert np.max(np.abs(avg - ref)) <= 1e-12
 
 
+@pytest.mark.parametrize("n", [1, 33, 100, 128])
+def test_dense_averages_few_and_many_states(fq, n):
+    """A formed inside the expectation kernel (few states) and by a launch of its own (more CTAs than SMs): the
+    same bits for every state."""
+    import torch
+    plan = fq.Plan.dense(fi.goe(n, 1824), fi.goe(n, 1825), omega=1.4, f_ac=1.0, f_dc=0.3, phi0=0.2, steps=5)
+    x = _random_states(n, 5, 1826)
+    few = plan.average_observable(x, 0.7, -0.4, 1.3)
+    many = plan.average_observable(x.repeat(130, 1).contiguous(), 0.7, -0.4, 1.3)
+    assert plan.check_status() == fq.FQ_OK
+    assert torch.equal(many, few.repeat(130))
+
+
 @pytest.mark.parametrize("precision,kernel", [(0, 1), (0, 3), (1, 2), (1, 3), (4, 3), (5, 4)])
 @pytest.mark.parametrize("nb,nc", [(1, 1), (2, 5), (60, 61), (511, 3), (512, 6), (1100, 2)])
 def test_tridiagonal_averages_by_path(fq, precision, kernel, nb, nc):
