@@ -337,10 +337,13 @@ fq_status floquet_build_UT_static(const fq_problem* problem, void* d_U, void* st
  *    tensor-core kernel (one CTA per SM) whose CTAs take work units from a device counter: per
  *    instance the blocks of Omega~_m's slices (Eqs. 11 and 14), and per step, term and output
  *    tile the Chebyshev term of Eq. 10 (state blocks of 128 columns advance independently, each
- *    unit waiting, with a bounded spin, only for the units it reads).  The tile width is the one
- *    the plans' own widths favour (tile_n or floquet_autotune), weighted by N^3 M L, with the
- *    width's default K stage; each U_T then equals the plan's own floquet_build_UT bit for bit
- *    when the tile shapes agree.  Other plans fall back to 8 lanes.
+ *    unit waiting, with a bounded spin, only for the units it reads).  One tile width runs all
+ *    plans, with its default K stage: the one that their widths favour, weighted by N^3 M L (a
+ *    plan's width is tile_n, floquet_autotune's, or the one of its size), or where no plan was
+ *    given or tuned to one, 128 if the size of any selects it or if BF16X6 products of the scan
+ *    fill the chip, else 64.  Each U_T then equals the plan's own floquet_build_UT bit for bit
+ *    when the tile shapes agree, and otherwise that of a plan with tile_n set to the scan's
+ *    width.  Other plans fall back to 8 lanes.
  *  - lanes = 1..32: floquet_build_UT of every plan captured on `lanes` concurrent graph
  *    branches, assigned longest-first by their cost N^3 M L.
  *  - A wait that gives up marks every plan's status word FQ_BIT_TIMEOUT (floquet_check_status

@@ -538,15 +538,31 @@ size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 int scan_ns(const fq_plan* p) { return p->precision == FQ_BF16X6 ? 3 : 2; }
 
-// Tile width of the scan: the one the plans' widths (their own or fq_split_shape's) favour, weighted
-// by their work.
+int np_of(int n) { return (n + 127) & ~127; }
+int tiles_j_of(int n) { return (n + BM - 1) / BM; }
+
+// Tile width of the scan.  Plans with a width (their own or floquet_autotune's) are asked for it, weighted by their
+// work; one without counts with the width of its size (fq_split_shape).  Where no plan has one, 128 as soon as a
+// plan's size asks for it, and in BF16X6, whose 64-wide stages feed the MMAs worse, where the 128-wide tiles of a
+// term fill the chip: 64- / 128-wide in ms a scan of 16 steps, tiles on 152 SMs: 4 x 896 (196) 13.1 / 16.5, 4 x 1024
+// (256) 18.2 / 19.7, 8 x 200 + 3 x 1200 (332) 23.9 / 24.2, 10 x 768 (360) 19.6 / 18.2, 3 x 1300 (363) 28.8 / 25.2,
+// 12 x 700 (432) 20.1 / 20.8, 8 x 1024 (512) 34.3 / 29.7, 12 x 1408 (1452) 128 / 110.  BF16X3 has 64-wide tiles within
+// 6 % even there (12 x 1408 67.7 / 64.4, 8 x 1024 20.0 / 21.5), and keeps those of the plans' own builds.
 int scan_bn(fq_plan* const* plans, int count) {
   double w128 = 0, w64 = 0;
+  bool own = false, wide = false;
+  long tiles = 0;  // 128-wide tiles of a term
   for (int i = 0; i < count; ++i) {
     const double c = (double)plans[i]->n * plans[i]->n * plans[i]->n * plans[i]->steps * plans[i]->L;
-    (fq_split_shape(plans[i]).n == 128 ? w128 : w64) += c;
+    const bool w = fq_split_shape(plans[i]).n == 128;
+    (w ? w128 : w64) += c;
+    own |= !plans[i]->tile_auto;
+    wide |= w;
+    tiles += (long)(np_of(plans[i]->n) / 128) * tiles_j_of(plans[i]->n);
   }
-  return w128 >= w64 ? 128 : 64;
+  if (own) return w128 >= w64 ? 128 : 64;
+  const bool full = 4 * tiles >= 9L * fq_sm_count();
+  return wide || (plans[0]->precision == FQ_BF16X6 && full) ? 128 : 64;
 }
 
 // Layout of the scan's own region (after the plans' workspaces): instance table, segment table,
@@ -563,9 +579,6 @@ struct ScanLayout {
 struct ScanShape {
   int n, L, ns;
 };
-
-int np_of(int n) { return (n + 127) & ~127; }
-int tiles_j_of(int n) { return (n + BM - 1) / BM; }
 
 std::vector<ScanShape> shapes_of(fq_plan* const* plans, int count) {
   std::vector<ScanShape> sh(count);

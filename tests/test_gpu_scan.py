@@ -72,6 +72,25 @@ def test_scan_matches_individual_builds(fq, precision, tile_n):
         assert torch.equal(u, p.build_UT()), (p.n, p.info.L)
 
 
+@pytest.mark.parametrize("precision,sizes,width", [
+    ("FQ_BF16X3", (150, 1600, 40, 1540), 128), ("FQ_BF16X6", (1450, 200), 128),   # sizes on both sides of the line
+    ("FQ_BF16X3", (1530, 150, 40), 64), ("FQ_BF16X6", (1000, 1400, 70), 64),      # all below it
+    ("FQ_BF16X6", (1200, 1100, 1280, 1000), 128)])                                # all below, and a full chip
+def test_scan_of_default_widths(fq, precision, sizes, width):
+    """The tile width of a scan of plans that were given none (the wide one with any plan above the line, as all
+    default plans ran before the width followed N): each U_T equals the build of a plan with that width, bit for
+    bit, on the second of two launches; below the line that is the plan's own build."""
+    import torch
+    models = [(fi.goe(n, 7100 + n), fi.goe(n, 7200 + n), fi.Drive(0.0, 1.2, 40.0)) for n in sizes]
+    plans = _plans(fq, models, 2, getattr(fq, precision), 0)
+    fixed = _plans(fq, models, 2, getattr(fq, precision), width)
+    outs = _scan(fq, plans)
+    for p, f, u in zip(plans, fixed, outs):
+        assert torch.equal(u, f.build_UT()), (p.n, p.info.L)
+        if width == 64:
+            assert torch.equal(u, p.build_UT()), (p.n, p.info.L)
+
+
 @pytest.mark.parametrize("steps", [1, 2, 3])
 def test_scan_short_scans(fq, steps):
     """Scans of 1 to 3 steps (no step reuses an Omega~ buffer before the third; the B units of
