@@ -158,6 +158,27 @@ def test_split_grad_kept_tiles(fq, n, stride):
     assert plan.check_status() == fq.FQ_OK
 
 
+@pytest.mark.parametrize("prec,eps,n,width", [("FQ_BF16X3", 2.0 ** -17, 1500, 64), ("FQ_BF16X3", 2.0 ** -17, 1550, 128),
+                                              ("FQ_BF16X6", 2.0 ** -23, 1390, 64), ("FQ_BF16X6", 2.0 ** -23, 1420, 128)])
+def test_split_grad_default_width(fq, prec, eps, n, width):
+    """A gradient plan without a tile width takes the one of its size: bit for bit the plan with that width, on
+    both sides of the line, and the FP64-emulated gradient to the arithmetic's bound."""
+    import torch
+    M = 3
+    h0, h1, fm = fi.goe(n, 1311), fi.goe(n, 1312), 1.0 + 0.1 * fi.normal(1313, M)
+    w = torch.eye(n, dtype=torch.complex128, device="cuda")
+    out = {}
+    for p, tile in ((prec, 0), (prec, width), ("FQ_OZAKI", 0)):
+        plan = fq.Plan.piecewise(h0, h1, fm, period=0.1, checkpoint_stride=2, precision=getattr(fq, p), tile_n=tile)
+        loss, g = plan.grad(cuda(fm), w)
+        assert plan.check_status() == fq.FQ_OK
+        out[p, tile] = plan, loss, g
+    plan, loss, g = out[prec, 0]
+    assert torch.equal(loss, out[prec, width][1]) and torch.equal(g, out[prec, width][2])
+    ref = out["FQ_OZAKI", 0]
+    assert float((g - ref[2]).abs().max()) <= split_grad_tol(plan, h1, eps, float(ref[1].item()))
+
+
 def test_split_grad_config5_shape_vs_oracle(fq):
     """The adjoint workload's shape (M = 256, checkpoints every 16) at N = 128, BF16X3."""
     n, M = 128, 256

@@ -284,3 +284,35 @@ def test_band_full_size_sampled_columns(fq):
     sample = torch.arange(0, d.n, 157, dtype=torch.int32, device="cuda")
     mx, fro = fq.api.unitarity_defect(U, sample)
     assert mx <= 1e-10
+
+
+@pytest.mark.parametrize("steps", [1, 3])
+def test_band_digit_cut_of_the_states(fq, steps):
+    """The kernel's own cut of the states into digits, to its last one.  A step this short is the identity to
+    1e-4, so every entry of X comes back as the sum of its own digits.  The states are multiples of a digit's half
+    step (rounding ties of the first three digits) with low words of either sign at their largest, on scales of
+    2^-20 to 1 in one batch.
+    Bound, in units of a state's largest entry: the digits leave 2^-49 of a scale of at most 4, the operator's
+    likewise over its 2 L + 1 entries of a row (a sum of absolute values below 2), the five slice pairs with
+    a + b = 6 that are not formed are below 16 * 2^-50 each, those beyond below 2^-48 together, and the
+    double-float sums and the states between steps are good to 2^-46: below 9 * 2^-46 a step.  Without the last
+    digit an entry would be off by up to 2^-40."""
+    nb, nc = 199, 96
+    d = fi.config_dimer(nb=nb)
+    rng = np.random.default_rng(2731)
+    shape = (2, nc, nb + 1)
+    part = (rng.integers(-120, 120, shape) + 0.5) * 2.0 ** (-8 * rng.integers(1, 4, shape))
+    half = np.spacing(np.abs(part).astype(np.float32)).astype(np.float64) / 2
+    part = part + half * rng.choice([-1.0, 1.0], shape) * rng.uniform(0.9, 1.0, shape)
+    x = (part[0] + 1j * part[1]) * 2.0 ** -rng.integers(0, 21, nc)[:, None]
+    d.drive = fi.Drive(0.2, 1.5, 2 * math.pi / 4e-6, 0.4)  # four steps of 1e-6
+    d.steps = 4
+    plan = band_plan(fq, d)
+    X = to_np(plan.propagate(cuda_c128(x), 0, steps))
+    assert plan.check_status() == fq.FQ_OK
+    p = o.plan_for_drive_tridiag(d.h0_diag, d.h0_off, d.h1_diag, d.drive, d.steps)
+    ref = o.propagate_tridiag(d.h0_diag, d.h0_off, d.h1_diag, p, x.T, 0, steps).T
+    largest = np.maximum(np.abs(x.real), np.abs(x.imag)).max(axis=1)
+    err = np.max(np.abs(X - ref).max(axis=1) / largest)
+    print(f"band digits, {steps} steps: {err * 2.0 ** 46:.2f} * 2^-46 of a state's largest entry")
+    assert err <= steps * 9 * 2.0 ** -46
