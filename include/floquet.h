@@ -105,14 +105,14 @@ typedef enum fq_kernel {
   FQ_KERNEL_AUTO = 0,       /* resident kernel when it applies, else tiled, else streaming */
   FQ_KERNEL_STREAM = 1,     /* tridiagonal: one launch per Chebyshev term, states in HBM;
                                dense FP64: one tiled GEMM launch per term (also for TILED) */
-  FQ_KERNEL_RESIDENT = 2,   /* tridiagonal FP32: one CTA per state (several small states a CTA)
+  FQ_KERNEL_RESIDENT = 2,   /* tridiagonal FP32: one CTA per state
                                runs the whole chain on chip (N <= 10240, L <= 128); dense FP64: a
                                cluster of ceil(N/16) CTAs per state runs 64 steps per launch on
                                chip (N <= 128, L <= 128); FQ_EUNSUPPORTED otherwise */
   FQ_KERNEL_TILED = 3,      /* tridiagonal FP64 or FP32, any N, L <= 128: each CTA runs a step's L
                                products on a segment of one state plus L halo rows a side, one
-                               launch per step, or per few steps where a segment holds the whole
-                               state; FQ_EUNSUPPORTED otherwise.  AUTO picks RESIDENT, then TILED,
+                               launch per step, or one for all steps of a call where a segment
+                               holds the whole state; FQ_EUNSUPPORTED otherwise.  AUTO picks RESIDENT, then TILED,
                                then STREAM. */
   FQ_KERNEL_BAND = 4        /* tridiagonal FQ_OZAKI (the only kernel for it; AUTO selects it),
                                L <= 47: per step the band matrix P_m = e^{-i beta h} sum_k c_k

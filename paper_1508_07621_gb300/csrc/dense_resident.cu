@@ -1,10 +1,10 @@
-// Resident dense chain for small N (FP64): a cluster of C = ceil(N/32) CTAs carries one state
+// Resident dense chain for small N (FP64): a cluster of C = ceil(N/16) CTAs carries one state
 // through every step of a chunk of the period, with the state on chip the whole time.
 //
 // The per-term dense path launches one tiled GEMM per Chebyshev term; at N = 64 each of those
 // launches keeps only a handful of SMs busy and the chain is 1400 dependent launches long
 // (M = 200, L = 7).  Here the independence of the columns of U_T (Algorithm 1 propagates each
-// initial state on its own) is used instead: one cluster per state, each CTA owning 16 or 32 rows of
+// initial state on its own) is used instead: one cluster per state, each CTA owning 16 rows of
 // Omega~_m, so 64 states fill the SMs and the whole chunk is one launch.
 //
 // Per step m (Eqs. 10-12): Phi_0 = X_{m-1}, Phi_1 = -i Omega~ Phi_0,

@@ -37,7 +37,11 @@ namespace {
 constexpr int SCAN_MAXL = 32;    // Chebyshev terms per step an instance may have
 constexpr int SCAN_RING = 8;     // units handed from the producer to the MMA thread and the warps
 constexpr int SCAN_BUILDERS = 4;  // warps of the B and W units
-constexpr int SCAN_THREADS = PTHREADS + 32 * SCAN_BUILDERS;  // producer, MMA, epilogue warps, builder warps
+// Producer, MMA, epilogue warps, builder warps: 14, four on one quarter of an SM, so that a thread has at most 128
+// registers.  The epilogue takes two row groups at a time (four in the chains) and still spills 84 bytes at width
+// 64 and 310 at width 128; with four epilogue warps (10 warps, 168 registers, no spills) it took longer: 8 plans of
+// N = 256 .. 1280, 12 steps, BF16X3 64-wide 15.4 ms against 12.7, 128-wide 14.8 against 13.4.
+constexpr int SCAN_THREADS = PTHREADS + 32 * SCAN_BUILDERS;
 constexpr int BLOCK_ROWS = 16;   // rows of a B or W unit
 constexpr int SCAN_TAIL = 512;   // barriers, tensor-memory slot, abort flag and ring after the stages
 

@@ -520,7 +520,7 @@ def test_dense_fp64_more_states_than_a_launch(fq, n):
 
 @pytest.mark.parametrize("n", [1, 5, 32, 33, 64, 65, 100, 128])
 def test_dense_fp64_resident_kernel(fq, n):
-    """The small-N resident chain (clusters of ceil(N/32) CTAs, 64 steps per launch) against the
+    """The small-N resident chain (clusters of ceil(N/16) CTAs, 64 steps per launch) against the
     oracle and against the per-term kernel: ragged row blocks (33, 65, 100), one to four CTAs per
     state, M = 70 crossing a launch boundary, a non-even drive."""
     M = 70
