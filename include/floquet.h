@@ -142,8 +142,9 @@ typedef struct fq_problem {
   int32_t kernel;           /* fq_kernel: which kernel family runs the chain (tridiagonal, and
                                dense FP64); ignored by the split precisions */
   int32_t tile_n;           /* split path: tensor-core output tile width 64 or 128; 0 = by N (64 where
-                               the 128-wide tiles of a product would leave SMs idle, else 128)
-                               until floquet_autotune picks one */
+                               the 128-wide tiles of a product would leave SMs idle, else 128;
+                               BF16X6 blocks of more than N states take 128 where those tiles
+                               fill the chip) until floquet_autotune picks one */
   int32_t magnus_order;     /* 4 (default, also 0) or 6: Eq. 14 in full with its alphas taken as
                                3-point Gauss-Legendre moments (nine commutators of H0, H1 computed
                                once: on the device for FQ_DENSE, on the host as bands for

@@ -77,16 +77,21 @@ static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 // Largest N whose default tile is 64 wide, for BF16X3 and BF16X6: up to there the 128-wide tiles of a
 // product are at most one wave (144 and 121 tiles on 152 SMs), and twice as many narrow ones fill the
 // chip better.  A product in us with 64- / 128-wide tiles: BF16X3 N = 256 11.5 / 21, 700 19 / 38, 1000 24 / 45,
-// 1536 61 / 69, 3000 435 / 385; BF16X6 N = 1000 41 / 73, 1300 82 / 98, 1536 116 / 110.  The rule looks at N
-// alone, so that a block of columns and the whole U_T take the same tiles and agree bit for bit.
+// 1536 61 / 69, 3000 435 / 385; BF16X6 N = 1000 41 / 73, 1300 82 / 98, 1536 116 / 110.  Up to N states the rule
+// looks at N alone, so that a block of columns and the whole U_T take the same tiles and agree bit for bit.
+// Blocks of more states in BF16X6 take the wide ones from a wave and a half of them on: four steps of states x N
+// in ms 3000 x 1000 (1.3 waves) 2.82 / 2.85, 4000 x 1000 3.75 / 3.47, 3600 x 900 3.08 / 2.99, 2800 x 1400 4.89 / 4.41,
+// 5600 x 1400 9.48 / 8.36.  (BF16X3 stays within a few per cent there.)
 constexpr int SPLIT_NARROW_MAX_N_X3 = 1536;
 constexpr int SPLIT_NARROW_MAX_N_X6 = 1408;
 
-// Tile shape of a split plan: its own (chosen by the caller or by floquet_autotune), or by size.
-fq_tile_shape fq_split_shape(const fq_plan* p) {
-  const int narrow = p->precision == FQ_BF16X6 ? SPLIT_NARROW_MAX_N_X6 : SPLIT_NARROW_MAX_N_X3;
-  if (p->tile_auto && p->n <= narrow) return fq_tile_shape{64, p->tile_k};
-  return fq_tile_shape{p->tile_n, p->tile_k};
+// Tile shape of a split plan for nc states: its own (chosen by the caller or by floquet_autotune), or by size.
+fq_tile_shape fq_split_shape(const fq_plan* p, int nc) {
+  const bool x6 = p->precision == FQ_BF16X6;
+  const int narrow = x6 ? SPLIT_NARROW_MAX_N_X6 : SPLIT_NARROW_MAX_N_X3;
+  if (!p->tile_auto || p->n > narrow) return fq_tile_shape{p->tile_n, p->tile_k};
+  const long wide = (long)((p->n + 127) / 128) * ((nc + BM - 1) / BM);  // 128-wide tiles
+  return x6 && nc > p->n && 2 * wide >= 3L * fq_sm_count() ? fq_tile_shape{128, 0} : fq_tile_shape{64, p->tile_k};
 }
 
 size_t fq_split_workspace(const fq_plan* p, int nc, void* base, void* out) {
@@ -256,7 +261,7 @@ fq_status fq_split_propagate(fq_plan* p, const double* x0, double* x, int nc, in
                              int transpose_out, void* ws, cudaStream_t s) {
   // (slices, tile width, K per stage): 64-byte swizzle stages where 128-byte ones would not fit
   // more than two stages in shared memory
-  const fq_tile_shape shape = fq_split_shape(p);
+  const fq_tile_shape shape = fq_split_shape(p, nc);
   const bool wide = shape.n == 128;
   if (p->precision == FQ_BF16X6)
     return wide ? run_split<3, 128, 32>(p, x0, x, nc, m_begin, m_end, identity, transpose_out, ws, s)

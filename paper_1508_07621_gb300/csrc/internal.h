@@ -257,7 +257,7 @@ fq_status fq_ozaki_propagate(fq_plan* p, const double* x0, double* x, int nc, in
                              int transpose_out, void* ws, cudaStream_t s);
 // split-precision dense path (dense_split.cu)
 size_t fq_split_workspace(const fq_plan* p, int nc, void* base, void* out);
-fq_tile_shape fq_split_shape(const fq_plan* p);
+fq_tile_shape fq_split_shape(const fq_plan* p, int nc = 0);
 // batched scan as one persistent launch (scan.cu): whether the plans qualify, the bytes it needs
 // beyond the plans' own workspaces, and the graph (counter reset + the launch) writing d_U[i];
 // plan i's workspace at ws + off[i], the scan's region at ws + extra_off

@@ -91,6 +91,20 @@ def test_split_default_tile(fq, prec):
     assert torch.equal(X.transpose(0, 1), U[:, 17:20])
 
 
+@pytest.mark.parametrize("prec,n,nc,width", [(3, 700, 700, 64), (3, 700, 3900, 64), (3, 700, 5000, 128), (2, 700, 5000, 64)])
+def test_split_default_tile_of_many_states(fq, prec, n, nc, width):
+    """More states than levels: BF16X6 plans without a tile width run the wide tiles from a wave and a half of
+    them on (228 on 152 SMs: 38 blocks of 128 states at n = 700), bit for bit as a plan that asks for them."""
+    import torch
+    kw = dict(omega=1.3, f_ac=1.1, steps=64, precision=prec)
+    h0, h1 = fi.goe(n, 1319), fi.goe(n, 1320)
+    x = torch.eye(n, dtype=torch.complex128, device="cuda").repeat((nc + n - 1) // n, 1)[:nc].contiguous()
+    plan = fq.Plan.dense(h0, h1, **kw)
+    X = plan.propagate(x, 3, 5)
+    assert plan.check_status() == 0
+    assert torch.equal(X, fq.Plan.dense(h0, h1, tile_n=width, **kw).propagate(x, 3, 5))
+
+
 @pytest.mark.parametrize("prec", [2, 3])
 @pytest.mark.parametrize("n,nc", [(1, 1), (63, 5), (130, 129), (257, 200), (1024, 1024), (1100, 100)])
 def test_split_kept_tiles(fq, prec, n, nc):
