@@ -486,14 +486,18 @@ fq_status dfl_chain(fq_plan* p, const double* x0, double* x, int nc, int m_begin
     sh.segs = (n + longest - 1) / longest;
     sh.nt = TILE_NT;
   }
-  const int per = sh.segs == 1 ? nsteps : 1;  // steps a launch
+  // At four rows a thread the form for one step spills less: it takes over where a launch is long beside its
+  // gap, from twenty states an SM on.  Twelve steps in ms, all in one launch / one each, states x rows: 2000 x 516 1.45 /
+  // 1.48, 2000 x 801 2.12 / 2.07, 4000 x 516 2.68 / 2.71, 4000 x 801 3.99 / 3.81, 10000 x 601 6.58 / 6.28.
+  const bool one = sh.segs > 1 || (sh.ept == 4 && nc > 20 * fq_sm_count());
+  const int per = one ? 1 : nsteps;  // steps a launch
   int cur = 0;
   for (int m = 0; m < nsteps; m += per) {
     for (int r0 = 0; r0 < nc; r0 += 65535) {  // gridDim.y limit
       const int rows = nc - r0 < 65535 ? nc - r0 : 65535;
       const size_t o = (size_t)r0 * ld;
       fq_ktimer_start(p, s, "k_tri_tile_dfl");
-      const auto kern = sh.segs > 1   ? k_tri_tile_dfl<4, false>
+      const auto kern = one           ? k_tri_tile_dfl<4, false>
                         : sh.ept == 1 ? k_tri_tile_dfl<1, true>
                         : sh.ept == 2 ? k_tri_tile_dfl<2, true>
                                       : k_tri_tile_dfl<4, true>;

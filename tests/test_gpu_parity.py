@@ -334,6 +334,20 @@ def test_tiled_dfl_short_last_segment(fq, nb, nc):
     assert np.max(np.abs(to_np(many[:2]) - ref)) <= 1e-12
 
 
+@pytest.mark.parametrize("nb", [515, 800, 1023])
+def test_tiled_dfl_one_step_launches(fq, nb):
+    """Double-float states of one segment: more than twenty states an SM run a launch a step, fewer all steps in one;
+    the same bits."""
+    import torch
+    d = _drive_models(nb)
+    plan = dimer_plan(fq, d, 4, 3)
+    x = cuda_c128(_unit_states(d.n, 4, 2307))
+    few = plan.propagate(x, 1, 4)
+    many = plan.propagate(x.repeat(800, 1).contiguous(), 1, 4)
+    assert plan.check_status() == fq.FQ_OK
+    assert torch.equal(many, few.repeat(800, 1))
+
+
 @pytest.mark.parametrize("nb", [1, 31, 63, 64, 100, 127, 200, 255, 320, 383, 500, 511, 512, 700, 1000, 1023, 1024, 1300,
                                 1600, 2047, 2048, 2600, 3500, 5000, 6500, 8191, 8192, 9215])
 def test_resident_shapes_agree(fq, nb):
