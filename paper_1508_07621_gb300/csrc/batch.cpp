@@ -103,8 +103,10 @@ static fq_status floquet_batch_create_body(fq_batch** out, fq_plan* const* plans
   for (int k = 0; k < count && st == FQ_OK; ++k) {
     const int i = order[k];
     plans[i]->grid_cap = cap;
+    plans[i]->lanes = std::min(lanes, (int)count);
     st = floquet_build_UT(plans[i], d_U[i], (char*)d_ws + off[i], ws_bytes - off[i], ls[lane_of[i]]);
     plans[i]->grid_cap = 0;
+    plans[i]->lanes = 1;
   }
   for (int l = 0; l < lanes && capturing; ++l) {
     cudaEventRecord(joins[l], ls[l]);

@@ -95,6 +95,7 @@ struct fq_plan {
   // dense split path: per-plan constants prepared once
   void* split = nullptr;
   fq_ktimer* ktimer = nullptr;  // owned; NULL until floquet_kernel_timing
+  int lanes = 1;     // products side by side on the chip (> 1 while a batch graph captures the plan)
   int grid_cap = 0;  // > 0: CTAs of a persistent split product (while a batch graph captures the plan)
 };
 

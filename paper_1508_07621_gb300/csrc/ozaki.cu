@@ -80,7 +80,10 @@ fq_status fq_ozaki_propagate(fq_plan* p, const double* x0, double* x, int nc, in
   const OzOperands op{w.left, w.right};
   static std::atomic<unsigned> attr_set{0};
   if (fq_first_on_device(attr_set)) {
-    cudaError_t e = cudaFuncSetAttribute(k_oz_term, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_oz_term<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)OzCfg::SMEM);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_oz_term<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)OzCfg::SMEM);
     if (e != cudaSuccess) return fq_cuda_fail(e, "Ozaki kernel shared-memory attribute");
   }
@@ -92,11 +95,13 @@ fq_status fq_ozaki_propagate(fq_plan* p, const double* x0, double* x, int nc, in
     k_oz_slice_left<<<w.ncp, 256, 0, s>>>(w.m[0][0], w.m[0][1], 1.0, 0.0, nullptr, nullptr, n, nc, w.np, BM, w.left,
                                           w.es);
   // output columns and values of k beyond N are zero: their tiles and stages are left out.  The
-  // cluster size looks at N alone up to N states, so that a block of columns agrees with the whole U_T bit for
-  // bit; more states have tiles enough (three steps of 13248 states at N = 414 10.7 ms, in clusters of four 20.8).
+  // ranges of k look at N alone, so that blocks of any number of states agree bit for bit
   const int tiles_i = (n + OZ_BN - 1) / OZ_BN, tiles_j = w.ncp / BM;
   const int nk = (n + OZ_BKE - 1) / OZ_BKE;
-  const int csize = oz_cluster(tiles_i * std::max((n + BM - 1) / BM, tiles_j), nk);
+  const int ranges = oz_cluster(tiles_i * ((n + BM - 1) / BM), nk);
+  const bool shared = oz_shared(tiles_i * tiles_j, nk, ranges, p->lanes);
+  const int csize = shared ? ranges : 1;
+  const auto term = ranges > 1 && !shared ? k_oz_term<true> : k_oz_term<false>;
   OzLaunch launch(tiles_i * tiles_j, csize, OzCfg::SMEM, s);
   fq_term t{};
   t.coef0 = p->cheb[0];
@@ -126,7 +131,7 @@ fq_status fq_ozaki_propagate(fq_plan* p, const double* x0, double* x, int nc, in
       e.es = w.es;
       e.et = w.et;
       e.t = t;
-      cudaError_t le = cudaLaunchKernelEx(&launch.cfg, k_oz_term, op, nk, tiles_j, tiles_i, w.np, csize, e);
+      cudaError_t le = cudaLaunchKernelEx(&launch.cfg, term, op, nk, tiles_j, tiles_i, w.np, csize, ranges, e);
       if (le != cudaSuccess) return fq_cuda_fail(le, "FP64-emulation term launch");
       if (!(t.last && m == m_end - 1))
         k_oz_slice_left<<<w.ncp, 256, 0, s>>>(w.m[out][0], w.m[out][1], 1.0, 0.0, nullptr, nullptr, n, nc, w.np,

@@ -34,10 +34,12 @@
 // bounded; a wait that gives up records FQ_BIT_TIMEOUT, drains this CTA's own copies and MMAs,
 // frees tensor memory and returns.
 //
-// Split K.  Where a product has fewer tiles than half the SMs (oz_cluster), a cluster of 2 or 4 CTAs
-// shares a tile: each takes a range of k, the double-float sums stay in shared memory, and each
-// CTA folds all of them (double-float again, as the chunks of one CTA are folded) for its share of
-// the 64 columns and runs the epilogue there.
+// Split K.  Where a product of N states has fewer tiles than half the SMs (oz_cluster), k is summed in 2 or 4
+// ranges, and a cluster of as many CTAs shares a tile: each takes a range, the double-float sums stay in
+// shared memory, and each CTA folds all of them (double-float again, as the chunks of one CTA are folded)
+// for its share of the 64 columns and runs the epilogue there.  Where the clusters would not run at once
+// (many more states than N, products of several lanes side by side; oz_shared), one CTA takes a tile's ranges
+// one after another (SERIAL) and folds them in the same order: the same bits.
 //
 // Epilogue.  GB300 runs 2 FP64 multiply-adds a cycle and SM, so an FP64 instruction of a warp costs
 // 16 cycles and the epilogue is bound by their number: it had 15 a complex entry (30 us a tile) and
@@ -448,10 +450,43 @@ __global__ void k_oz_real(const double* __restrict__ h0, const double* __restric
   if (threadIdx.x == 0) et[i] = e;
 }
 
-// One Chebyshev term (OZ_FWD) on a 128-state x 64-column tile per cluster of `csize` CTAs (see the
-// file comment).
+// Folds the double-float sums of 16 columns into the running totals `tot` of the ranges before, as oz_fold does
+// with the sums of a cluster.  The totals wait in local memory (an index that the compiler cannot see through keeps
+// them there): registers hold one range's sums.
+__device__ __forceinline__ void oz_carry(float (&tot)[64], bool first, bool last, float2 (&hr)[8], float2 (&lr)[8],
+                                         float2 (&hi)[8], float2 (&li)[8]) {
+  int at = 0;
+  asm volatile("" : "+r"(at));
+#pragma unroll
+  for (int part_im = 0; part_im < 2; ++part_im) {
+    float2* h = part_im ? hi : hr;
+    float2* l = part_im ? li : lr;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int o = at + 32 * part_im + 4 * q;
+      if (!first) {
+        float2 th = make_float2(tot[o], tot[o + 1]), tl = make_float2(tot[o + 2], tot[o + 3]);
+        dd_add(th.x, tl.x, h[q].x, l[q].x);
+        dd_add(th.y, tl.y, h[q].y, l[q].y);
+        h[q] = th;
+        l[q] = tl;
+      }
+      if (!last) {
+        tot[o] = h[q].x;
+        tot[o + 1] = h[q].y;
+        tot[o + 2] = l[q].x;
+        tot[o + 3] = l[q].y;
+        h[q] = l[q] = make_float2(0.f, 0.f);
+      }
+    }
+  }
+}
+
+// One Chebyshev term (OZ_FWD) on a 128-state x 64-column tile per cluster of `csize` CTAs, k in `ranges` ranges:
+// one a CTA of the cluster, or all on the one CTA (SERIAL) (see the file comment).
+template <bool SERIAL>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    k_oz_term(const OzOperands op, int nk, int tiles_j, int tiles_i, int np, int csize, OzEpi e) {
+    k_oz_term(const OzOperands op, int nk, int tiles_j, int tiles_i, int np, int csize, int ranges, OzEpi e) {
   using Cfg = OzCfg;
   constexpr int OZ_STAGES = Cfg::STAGES;
   constexpr int OZ_STAGE_BYTES = Cfg::STAGE_BYTES;
@@ -471,7 +506,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   // this CTA's K stages kb0 .. kb0 + nkr
   const int rank = blockIdx.x % csize;
   const int kb0 = nk * rank / csize, nkr = nk * (rank + 1) / csize - kb0;
-  const int nchunks = (nkr + OZ_KB_PER_DRAIN - 1) / OZ_KB_PER_DRAIN;
+  // its ranges, and where range r ends
+  const int nranges = SERIAL ? ranges : 1;
+  auto range_end = [&](int r) { return SERIAL ? nk * (r + 1) / ranges : nkr; };
 
   int tj, ti;
   {
@@ -536,9 +573,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * OZ_BN) >> 3) << 17) |
                                  ((uint32_t)(BM >> 4) << 24);
       bool ok = true;
-      int kb = 0;
-      for (int c = 0; c < nchunks && ok; ++c) {
-        for (int kq = 0; kq < OZ_KB_PER_DRAIN && kb < nkr; ++kq, ++kb) {
+      int kb = 0, r = 0;
+      for (int c = 0; kb < nkr && ok; ++c) {
+        const int end = range_end(r);
+        for (int kq = 0; kq < OZ_KB_PER_DRAIN && kb < end; ++kq, ++kb) {
           const int s = kb % OZ_STAGES;
           ok = mbar_wait(full0 + 8 * s, (kb / OZ_STAGES) & 1);
           if (!ok || *(volatile int*)abort_flag) {
@@ -575,6 +613,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           mma_commit(empty0 + 8 * s);
         }
         if (!ok) break;
+        if (kb == end) ++r;
         mma_commit(tfull);
       }
       if (!ok) {
@@ -590,8 +629,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     float2 hr[8], lr[8], hi[8], li[8];  // double-float sums of columns (2p, 2p + 1)
 #pragma unroll
     for (int q = 0; q < 8; ++q) hr[q] = lr[q] = hi[q] = li[q] = make_float2(0.f, 0.f);
+    float tot[SERIAL ? 64 : 1];
     bool ok = true;
-    for (int c = 0; c < nchunks; ++c) {
+    int kb = 0, r = 0;
+    for (int c = 0; kb < nkr; ++c) {
       bool go = mbar_wait(tfull, c & 1);
       tc_fence_after();
       go = __all_sync(0xffffffffu, go && !*(volatile int*)abort_flag);
@@ -620,6 +661,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(tempty0 + 8 * g);  // the next chunk's MMAs into it may start
+      }
+      const int end = range_end(r);
+      kb = min(kb + OZ_KB_PER_DRAIN, end);
+      if constexpr (SERIAL) {
+        if (kb == end) {
+          oz_carry(tot, r == 0, r == nranges - 1, hr, lr, hi, li);
+          ++r;
+        }
       }
     }
     if (!ok) {
@@ -711,7 +760,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   if (csize > 1) oz_cluster_sync();  // no CTA leaves while a peer may still read its sums
 }
 
-// CTAs that share a tile's K range: as many of 4, 2, 1 as keep a product of `tiles` tiles within one
+// Ranges of k: as many of 4, 2, 1 as keep the clusters of a product of `tiles` tiles within one
 // wave, and no more than its K stages.  A term (product and slicing pass) in us before and now, the
 // shorter epilogue included: N = 64 56 -> 32 and 200 94 -> 48 and 414 121 -> 58 (clusters of four), 777
 // 175 -> 139, 1536 546 -> 464 and 2600 2287 -> 2028 (no clusters: more tiles than half the SMs; a
@@ -719,6 +768,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 int oz_cluster(int tiles, int nk) {
   const int sms = fq_sm_count();
   return tiles * 4 <= sms && nk >= 4 ? 4 : (tiles * 2 <= sms && nk >= 2 ? 2 : 1);
+}
+
+// Whether clusters share the tiles of a product summed in `ranges` ranges, or one CTA takes each tile's ranges: fewer
+// waves of longer CTAs.  A CTA's time is modelled as 46 us and 1.9 for each of its K stages (fitted to the terms
+// above), and `lanes` products side by side as a share of the chip each, with half of a lane's time in gaps.  Three
+// steps in ms, clusters / one CTA a tile, states x N: 828 x 414 1.93 / 2.02, 3312 x 414 5.64 / 4.25, 9600 x 300 10.9 /
+// 6.5, 6400 x 200 5.5 / 3.7; lane graphs of 8 builds of 8 steps, 2 lanes of N = 414 15.6 / 20.3, 600 24.0 / 26.1,
+// 8 lanes of 200 3.7 / 4.0, 414 15.0 / 8.9, 600 23.1 / 19.0.
+bool oz_shared(int tiles, int nk, int ranges, int lanes) {
+  const int sms = std::max(1, lanes > 1 ? 2 * fq_sm_count() / lanes : fq_sm_count());
+  auto waves = [&](int ctas) { return (ctas + sms - 1) / sms; };
+  return ranges > 1 && waves(tiles * ranges) * (46.0 + 1.9 * nk / ranges) <= waves(tiles) * (46.0 + 1.9 * nk);
 }
 
 // Launch configuration of `tiles` tiles of `csize` CTAs.

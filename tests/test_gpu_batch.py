@@ -62,6 +62,26 @@ def test_batch_matches_individual_builds(fq):
     assert np.max(np.abs(outs[0].cpu().numpy() - ref)) <= tol
 
 
+@pytest.mark.parametrize("lanes,sizes", [(8, (414, 500, 130, 320, 600, 414, 300, 70)), (2, (200, 414))])
+def test_lanes_of_emulated_builds(fq, lanes, sizes):
+    """FP64-emulated builds side by side: with eight lanes one CTA takes the K ranges of a tile that a lone build
+    shares between the CTAs of a cluster.  The same bits."""
+    import torch
+    plans = [fq.Plan.dense(fi.goe(n, 5100 + n), fi.goe(n, 5200 + n), omega=1.0, f_ac=1.0, steps=3, period=0.1,
+                           precision=fq.FQ_OZAKI) for n in sizes]
+    outs = [torch.empty((p.n, p.n), dtype=torch.complex128, device="cuda") for p in plans]
+    handles = [p.handle for p in plans]
+    ws = fq.workspace(fq.floquet_batch_workspace_size(handles))
+    b = fq.floquet_batch_create(handles, outs, ws, lanes)
+    try:
+        fq.floquet_batch_launch(b)
+        torch.cuda.synchronize()
+    finally:
+        fq.floquet_batch_destroy(b)
+    for p, u in zip(plans, outs):
+        assert torch.equal(u, p.build_UT()) and p.check_status() == fq.FQ_OK
+
+
 def test_autotune_picks_a_tile_and_stays_correct(fq):
     m = fi.config_goe64()
     plan = fq.Plan.dense(m.h0, m.h1, omega=1.0, f_ac=1.0, steps=m.steps, precision=fq.FQ_BF16X3)
